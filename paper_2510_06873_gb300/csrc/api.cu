@@ -329,6 +329,7 @@ metad_status validate(const metad_params *p, std::string &why)
     return METAD_OK;
 }
 
+constexpr double kLog2e = 1.4426950408889634073599246810019;
 constexpr double kTwoPi = 6.283185307179586476925286766559;  // the period of a torsion angle
 
 // CVs the hills see: the per-atom CVs, then the three box lengths when they
@@ -411,7 +412,12 @@ metad_status setup_system(metad_ctx *c)
     if (c->p.n_cv == 2) y.sigma[1] = c->p.sigma[1];
     if (c->p.lattice_cvs)
         for (int a = 0; a < 3; ++a) y.sigma[c->p.n_cv + a] = c->p.sigma_lattice[a];
-    for (int d = 0; d < metad::kMaxCv; ++d) y.inv2v[d] = 0.5 / (y.sigma[d] * y.sigma[d]);
+    for (int d = 0; d < metad::kMaxCv; ++d) {
+        y.inv2v[d] = 0.5 / (y.sigma[d] * y.sigma[d]);
+        y.k2v[d] = kLog2e * y.inv2v[d];
+        y.half[d] = 0.5 * y.period[d];
+        y.three_half[d] = 1.5 * y.period[d];
+    }
     y.w0 = c->p.w0;
     y.kbdt = c->p.kB * c->p.temperature * (c->p.biasfactor - 1.0);
     y.grid_on = c->p.grid_on;

@@ -19,20 +19,18 @@ namespace {
 
 // V and dV/ds at s.bias_x into s.bias_out; with s.deposit, also appends the
 // well-tempered hill there as hill s.K.
-__device__ __forceinline__ void bias(const Sys &s, Blk blk) { hill_sum(s, blk, s.bias_x, s.bias_out, s.deposit); }
-
-__global__ void __launch_bounds__(kBlockBias) k_bias(Sys s) { bias(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockBias) k_bias(Sys s)
+{
+    hill_sum<kMaxCv>(s, own_blk(), s.bias_x, s.bias_out, s.deposit);
+}
 
 // Batched: every system evaluates at its own CVs (deposit 0) or deposits a
 // hill there (deposit 1; only systems with s.deposit have blocks).
 __global__ void __launch_bounds__(kBlockBias) kb_bias(BatchView v, int deposit)
 {
     Blk k;
-    Sys s = v.sys[batch_system(v, k)];
-    s.bias_x = s.scal + kS0;
-    s.bias_out = s.scal + (deposit ? kDepV : kV);
-    s.deposit = deposit;
-    bias(s, k);
+    const Sys &s = v.sys[batch_system(v, k)];
+    hill_sum<kMaxCv>(s, k, s.scal + kS0, s.scal + (deposit ? kDepV : kV), deposit);
 }
 
 // One thread per system: s1, s2 (0 with one per-atom CV), V and the error
@@ -59,7 +57,7 @@ __global__ void k_grid_fold(Sys s, int K)
     double f = 0.0, fx = 0.0, fy = 0.0, fxy = 0.0;
     for (int k = 0; k < K; ++k) {
         const double dx = x - s.hc[(size_t)s.hstride * k], dy = y - s.hc[(size_t)s.hstride * k + 1];
-        const double g = s.hw[k] * exp(-(dx * dx / (2.0 * v0) + dy * dy / (2.0 * v1)));
+        const double g = s.hw[k] * exp2_neg(dx * dx * s.k2v[0] + dy * dy * s.k2v[1]);
         f += g;
         fx -= g * dx / v0;
         fy -= g * dy / v1;
@@ -74,11 +72,13 @@ __global__ void k_grid_fold(Sys s, int K)
 
 }  // namespace
 
-// About kHillsPerBlock hills per block (one per thread).  Fewer hills per
-// block spread one system's FP64 work over more SMs (a lone 10,000-hill
-// walker's step: 22.5 -> 18.4 us at 64 per block) but halve the throughput
-// of batched walkers, whose blocks fill the GPU anyway; a system's grid must
+// About kHillsPerBlock hills per block (two per thread).  Fewer hills per
+// block spread one system's FP64 work over more SMs, more of them share the
+// block's fixed work (the CVs of a fused small-system step, the block sums)
+// in batched walkers, whose blocks fill the GPU anyway; a system's grid must
 // not depend on whether it is batched, or the two would round differently.
+// Measured at 256 / 512 / 1024: a lone 10,000-hill torsion walker's step
+// 12.3 / 14.3 / 16.4 us, 256 such walkers batched 447 / 360 / 320 us.
 int bias_blocks(int K)
 {
     int b = (K + kHillsPerBlock - 1) / kHillsPerBlock;

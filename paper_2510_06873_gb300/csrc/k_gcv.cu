@@ -38,14 +38,42 @@ __device__ __forceinline__ double min_image(double d, double L)
     return d;
 }
 
-// Caller atom i, wrapped into the box, in FP64; flags a non-finite input.
-__device__ __forceinline__ void atom_pos(const Sys &s, int i, double p[3], bool &bad)
+// Caller atom i, wrapped into the box; flags a non-finite input.
+__device__ __forceinline__ void atom_posf(const Sys &s, int i, float p[3], bool &bad)
 {
     const float4 q = __ldg(s.pos_in + i);
     bad |= !(isfinite(q.x) && isfinite(q.y) && isfinite(q.z));
-    p[0] = (double)wrap_coord(isfinite(q.x) ? q.x : 0.0f, s.Lin[0], s.L[0]);
-    p[1] = (double)wrap_coord(isfinite(q.y) ? q.y : 0.0f, s.Lin[1], s.L[1]);
-    p[2] = (double)wrap_coord(isfinite(q.z) ? q.z : 0.0f, s.Lin[2], s.L[2]);
+    p[0] = wrap_coord(isfinite(q.x) ? q.x : 0.0f, s.Lin[0], s.L[0]);
+    p[1] = wrap_coord(isfinite(q.y) ? q.y : 0.0f, s.Lin[1], s.L[1]);
+    p[2] = wrap_coord(isfinite(q.z) ? q.z : 0.0f, s.Lin[2], s.L[2]);
+}
+
+// The same in FP64.
+__device__ __forceinline__ void atom_pos(const Sys &s, int i, double p[3], bool &bad)
+{
+    float f[3];
+    atom_posf(s, i, f, bad);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[k] = (double)f[k];
+}
+
+// One component of the minimum-image bond from pi to pj: the exact FP64
+// difference rounded to `real`.  In FP32 a difference clear of half the box
+// needs no image and is the float32 difference itself, so the usual bond
+// takes no FP64 instruction (each holds a warp for 64 cycles here).
+template <typename real>
+__device__ __forceinline__ real bond_comp(const Sys &s, float pi, float pj, int k);
+template <>
+__device__ __forceinline__ double bond_comp<double>(const Sys &s, float pi, float pj, int k)
+{
+    return min_image((double)pj - (double)pi, s.L[k]);
+}
+template <>
+__device__ __forceinline__ float bond_comp<float>(const Sys &s, float pi, float pj, int k)
+{
+    const float d = pj - pi;
+    if (fabsf(d) < 0.999f * s.halfL[k]) return d;
+    return (float)bond_comp<double>(s, pi, pj, k);
 }
 
 // Minimum-image displacement r_j - r_i.
@@ -98,19 +126,17 @@ template <typename real>
 __device__ void torsion(const Sys &s, int d, bool &bad, double *xo, double *go)
 {
     const int *q = s.cv_atoms + 4 * d;
-    double ra[3], rb[3], rc[3], rd[3], e1[3], e2[3], e3[3];
-    atom_pos(s, q[0], ra, bad);
-    atom_pos(s, q[1], rb, bad);
-    atom_pos(s, q[2], rc, bad);
-    atom_pos(s, q[3], rd, bad);
-    disp(s, ra, rb, e1);
-    disp(s, rb, rc, e2);
-    disp(s, rc, rd, e3);
+    float ra[3], rb[3], rc[3], rd[3];
+    atom_posf(s, q[0], ra, bad);
+    atom_posf(s, q[1], rb, bad);
+    atom_posf(s, q[2], rc, bad);
+    atom_posf(s, q[3], rd, bad);
     real b1[3], b2[3], b3[3];
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        b1[k] = (real)e1[k];
-        b2[k] = (real)e2[k];
-        b3[k] = (real)e3[k];
+        b1[k] = bond_comp<real>(s, ra[k], rb[k], k);
+        b2[k] = bond_comp<real>(s, rb[k], rc[k], k);
+        b3[k] = bond_comp<real>(s, rc[k], rd[k], k);
     }
     real n1[3], n2[3], n3[3];
     cross3(b1, b2, n1);
@@ -297,9 +323,14 @@ __device__ void gcv_forces(const Sys &s, Blk blk, const double *gterms)
             const double dv = s.scal[kDV0 + d];
             const double *g = gterms + 16 * d;
             if (s.kind == kKindTorsion) {
+                // an atom sits in a quadruplet at most once: find its place,
+                // then one set of FP64 terms for the whole warp
+                int at = -1;
+#pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (s.cv_atoms[4 * d + q] == i)
-                        for (int k = 0; k < 3; ++k) f[k] -= dv * g[3 * q + k];
+                    if (s.cv_atoms[4 * d + q] == i) at = q;
+                if (at >= 0)
+                    for (int k = 0; k < 3; ++k) f[k] -= dv * g[3 * at + k];
                 continue;
             }
             if (s.cv_atoms[d] == i)
@@ -352,7 +383,7 @@ __device__ void gcv_step(const Sys &s, Blk blk)
         if (threadIdx.x < kMaxCv) s.scal[kS0 + threadIdx.x] = xs[threadIdx.x];
         if (threadIdx.x < 16 * s.ncv) s.gcv[threadIdx.x] = gs[threadIdx.x];
     }
-    if (!hill_sum(s, blk, xs, s.scal + kV, s.deposit)) return;
+    if (!hill_sum<2>(s, blk, xs, s.scal + kV, s.deposit)) return;
     __syncthreads();  // thread 0 of this block wrote dV/ds
     gcv_forces(s, Blk{0, 1}, gs);
 }
@@ -361,7 +392,7 @@ template <typename real>
 __global__ void __launch_bounds__(kGcvThreads) k_gcv_step(Sys s) { gcv_step<real>(s, own_blk()); }
 
 template <typename real>
-__global__ void __launch_bounds__(kGcvThreads) kb_gcv_step(BatchView v)
+__global__ void __launch_bounds__(kGcvThreads, 4) kb_gcv_step(BatchView v)
 {
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];

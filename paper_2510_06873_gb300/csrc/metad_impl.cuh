@@ -14,7 +14,7 @@ constexpr int kNY = 13;          // real Y_6^m, m = -6..6
 constexpr int kBlockAtoms = 128; // threads per block of the per-atom kernels
 constexpr int kBlockBias = 256;  // threads per block of the hill kernels
 constexpr int kMaxBiasBlocks = 304;  // two per SM
-constexpr int kHillsPerBlock = 256;  // hill kernel: blocks of kBlockBias threads take this many hills each
+constexpr int kHillsPerBlock = 512;  // hill kernel: blocks of kBlockBias threads take this many hills each
 constexpr int kMaxCv = 5;        // CN, Q6 and the three lattice parameters
 
 enum ErrBits : int {
@@ -122,6 +122,7 @@ struct Sys {
     int hill_cap;
     double sigma[kMaxCv];  // per CV (the lattice CVs last)
     double inv2v[kMaxCv];  // 0.5 / sigma^2 per CV
+    double k2v[kMaxCv];    // log2(e) / (2 sigma^2) per CV
     int D;                 // CVs the hills see: ncv (+ 3 lattice parameters)
     int hstride;           // doubles per hill centre: max(D, 2)
     int lattice;           // 1: the box lengths are CVs ncv .. ncv + 2
@@ -142,6 +143,7 @@ struct Sys {
     // torsion and nearest-distance families (no neighbour list)
     double period[kMaxCv];      // 0, or the period of a periodic CV (2 pi for a torsion)
     double inv_period[kMaxCv];  // 1 / period (0 when not periodic)
+    double half[kMaxCv], three_half[kMaxCv];  // 1/2 and 3/2 periods
     const int *cv_atoms;   // torsion: [ncv][4]; nearest: [ncv] references, then n_cand candidates
     const int *cand_slot;  // nearest: [n] position of each atom in the candidate group, or -1
     int n_cand;

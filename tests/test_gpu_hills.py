@@ -1,0 +1,86 @@
+"""Hill sums at the sizes where their kernels change shape, against plain
+numpy in FP64: the integer exponential over its whole argument range, the
+nearest image of far hill centres and the block edges of the hill kernel."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53  # one rounding, relative
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_06873_gb300 import build
+    build.build()
+    d = torch.device("cuda:0")
+    torch.cuda.set_stream(torch.cuda.Stream(d))
+    return d
+
+
+def _ctx(dev, n_cv, sigma, **kw):
+    from paper_2510_06873_gb300 import metad
+    return metad.Metad(metad.params_for(8, [23.0, 23.0, 23.0], n_cv=n_cv, sigma=sigma,
+                                        stream=torch.cuda.current_stream(dev).cuda_stream, **kw))
+
+
+def test_one_hill_over_the_whole_argument_range(dev):
+    """V = exp(-e) of a single hill: the exponent takes six roundings
+    (sigma^2, 1/2 over it, log2 e, its product, two squares), the exponential
+    and the reference one each."""
+    ctx = _ctx(dev, 1, (1.0,))
+    ctx.load_hills([[0.0]], [1.0])
+    s = np.concatenate([np.linspace(0.0, 2.0, 97), np.geomspace(1e-160, 37.6, 200), [37.2, 37.3, 38.5, 38.7, 40.0, 1e3]])
+    for x in s:
+        V, _ = ctx.bias_eval([x])
+        e = 0.5 * x * x
+        ref = math.exp(-e)
+        # below the normal range the reference itself is a multiple of 2^-1074
+        assert abs(V - ref) <= (6.0 * e + 3.0) * U * ref + 2.0 ** -1074, (x, V, ref)
+    ctx.load_hills([[math.inf]], [1.0])
+    assert ctx.bias_eval([0.0])[0] == 0.0
+
+
+@pytest.mark.parametrize("n_cv", [1, 2])
+@pytest.mark.parametrize("K", [1, 31, 255, 256, 257, 1023, 1025, 2500, 10000])
+def test_hill_sum_block_edges(dev, n_cv, K):
+    r = np.random.default_rng(K + n_cv)
+    sig = np.array([0.05, 0.02])[:n_cv]
+    ctr = np.array([2.0, 0.3])[:n_cv]
+    c, w = ctr + sig * r.uniform(-6, 6, (K, n_cv)), r.uniform(0.1, 1.0, K)
+    ctx = _ctx(dev, n_cv, sig)
+    ctx.load_hills(c, w)
+    V, g = ctx.bias_eval(ctr)
+    d = ctr - c
+    t = w * np.exp(-(d * d / (2 * sig**2)).sum(1))
+    ref_g = -(t[:, None] * d / sig**2).sum(0)
+    # each term within (6 e + 8) roundings with e <= 36, sums of K terms pairwise-like (<= 30 levels)
+    tol = (6 * 36 + 8 + 30) * U
+    assert abs(V - t.sum()) <= tol * t.sum()
+    assert np.all(np.abs(g - ref_g) <= tol * (t[:, None] * np.abs(d) / sig**2).sum(0))
+
+
+def test_far_periodic_centres_wrap_to_the_nearest_image(dev):
+    from paper_2510_06873_gb300 import metad
+    p = metad.params_for(22, [24.0] * 3, n_cv=2, sigma=(0.35, 0.6), cv_kind="torsion", biasfactor=math.inf,
+                         stream=torch.cuda.current_stream(dev).cuda_stream)
+    ctx = metad.Metad(p)
+    ctx.set_cv_atoms([2, 3, 4, 5, 3, 4, 5, 6])
+    r = np.random.default_rng(3)
+    c, w = r.uniform(-16.0, 16.0, (3000, 2)), r.uniform(0.1, 1.0, 3000)
+    ctx.load_hills(c, w)
+    sig = np.array([0.35, 0.6])
+    for s in r.uniform(-math.pi, math.pi, (20, 2)):
+        V, g = ctx.bias_eval(s)
+        d = s - c
+        d -= 2 * math.pi * np.rint(d / (2 * math.pi))
+        t = w * np.exp(-(d * d / (2 * sig**2)).sum(1))
+        # an image shift leaves an absolute rounding of 16 U in d: 2 d 16 U / (2 sigma^2) in the exponent
+        tol = (6 * 60 + 40 + 2 * math.pi * 16 / 0.35**2) * U
+        assert abs(V - t.sum()) <= tol * t.sum()
+        assert np.all(np.abs(g + (t[:, None] * d / sig**2).sum(0)) <= 4 * tol * (t[:, None] * np.abs(d) / sig**2).sum(0))
