@@ -51,6 +51,11 @@ struct metad_ctx {
     std::vector<int> prof_stage;
     int64_t launches = 0;
     int64_t device_bytes = 0;  // requested by cudaMalloc for this context
+    // workspace of the fold and free-energy passes: grown on use, kept up to
+    // kScratchKeep bytes, freed with the context
+    static constexpr size_t kScratchKeep = 256u << 20;
+    double *scratch = nullptr;
+    size_t scratch_doubles = 0;
     // metad_step as captured CUDA graphs, each valid for the flags and hill
     // count it was captured with; a few are kept (least recently used
     // replaced).  When every kernel node takes only the descriptor, a graph
@@ -209,6 +214,31 @@ metad_status dalloc(metad_ctx *c, T **ptr, size_t count)
     c->device_bytes += (int64_t)bytes;
     *ptr = static_cast<T *>(p);
     return METAD_OK;
+}
+
+// The context's workspace with room for `doubles`, or NULL: more than is kept,
+// no memory, or a growth asked for while the stream is being captured.  Work
+// on it is ordered by the context stream; growing frees the old one, which
+// waits for the device.
+double *kept_scratch(metad_ctx *c, size_t doubles)
+{
+    if (doubles <= c->scratch_doubles) return c->scratch;
+    if (doubles * sizeof(double) > metad_ctx::kScratchKeep) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    void *p = nullptr;
+    if (cudaMalloc(&p, doubles * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (c->scratch) cudaFree(c->scratch);
+    c->device_bytes += (int64_t)((doubles - c->scratch_doubles) * sizeof(double));
+    c->scratch = static_cast<double *>(p);
+    c->scratch_doubles = doubles;
+    return c->scratch;
 }
 
 // s_raw(x) = S_n(x) / S_m(x), S_k = 1 + x + ... + x^(k-1) (the device form).
@@ -628,6 +658,7 @@ metad_status metad_destroy(metad_ctx *c)
     if (c->stream) cudaStreamSynchronize(c->stream);
     for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
     for (void *ptr : c->allocs) cudaFree(ptr);
+    if (c->scratch) cudaFree(c->scratch);
     if (c->host_pinned) cudaFreeHost(c->host_pinned);
     if (c->err_pinned) cudaFreeHost(c->err_pinned);
     for (auto &g : c->graphs) drop_graph(g);
@@ -1110,8 +1141,16 @@ metad_status metad_fold_hills(metad_ctx *c)
     if (s) return s;
     if (!c->p.grid_on) return fail(c, METAD_ERR_INVALID, "fold_hills needs grid_on");
     if (c->K > 0) {
-        StageScope t(c, ST_OTHER, 1);
-        metad::launch_grid_fold(c->sys, c->K, c->stream);
+        // the contraction needs a workspace; without one (see kept_scratch)
+        // every node evaluates every hill
+        double *work = kept_scratch(c, metad::fold_doubles(c->sys, c->K));
+        StageScope t(c, ST_OTHER, 0);
+        if (work) {
+            c->launches += metad::launch_fold_separable(c->sys, c->K, work, c->stream);
+        } else {
+            metad::launch_grid_fold(c->sys, c->K, c->stream);
+            c->launches += 1;
+        }
     }
     s = launched(c, "fold_hills");
     if (s) return s;
@@ -1763,6 +1802,17 @@ struct Scratch {
     }
 };
 
+// A workspace for one synchronising call: the kept one, or a buffer of the
+// call's own.
+cudaError_t call_scratch(metad_ctx *c, size_t doubles, Scratch &own, double **out)
+{
+    *out = kept_scratch(c, doubles);
+    if (*out) return cudaSuccess;
+    const cudaError_t e = cudaMalloc(&own.p, sizeof(double) * doubles);
+    *out = static_cast<double *>(own.p);
+    return e;
+}
+
 }  // namespace
 
 metad_status metad_fes_grid(metad_ctx *c, const double *lo, const double *hi, const int32_t *n, double *F_host)
@@ -1772,15 +1822,21 @@ metad_status metad_fes_grid(metad_ctx *c, const double *lo, const double *hi, co
     int64_t bins = 0;
     if ((s = fes_grid_args(c, lo, hi, n, bins))) return s;
     if (!F_host) return fail(c, METAD_ERR_INVALID, "F_host is NULL");
-    Scratch buf;
-    if ((s = cuda_check(c, cudaMalloc(&buf.p, sizeof(double) * 2 * bins), "fes buffer"))) return s;
-    double *V = static_cast<double *>(buf.p), *F = V + bins;
     const int nn[2] = {n[0], c->p.n_cv == 2 ? n[1] : 1};
+    Scratch own;
+    double *work = nullptr;
+    bool separable = metad::fes_separable(c->sys, c->K, nn);
+    if (separable && call_scratch(c, metad::fes_points_doubles(c->sys, c->K, nn, true), own, &work) != cudaSuccess) {
+        cudaGetLastError();
+        separable = false;
+    }
+    if (!separable && (s = cuda_check(c, call_scratch(c, metad::fes_points_doubles(c->sys, c->K, nn, false), own, &work),
+                                      "fes buffer")))
+        return s;
     const double fac = std::isinf(c->p.biasfactor) ? 1.0 : c->p.biasfactor / (c->p.biasfactor - 1.0);
-    metad::launch_fes_points(c->sys, c->K, lo, hi, nn, V, F, fac, c->stream);
-    c->launches += 2;
+    c->launches += metad::launch_fes_points(c->sys, c->K, lo, hi, nn, work, separable, fac, c->stream);
     if ((s = launched(c, "fes_grid"))) return s;
-    if ((s = cuda_check(c, cudaMemcpyAsync(F_host, F, sizeof(double) * bins, cudaMemcpyDeviceToHost, c->stream),
+    if ((s = cuda_check(c, cudaMemcpyAsync(F_host, work, sizeof(double) * bins, cudaMemcpyDeviceToHost, c->stream),
                         "fes copy")))
         return s;
     return sync_and_check(c);
@@ -1795,10 +1851,18 @@ metad_status metad_fes_reweight(metad_ctx *c, const double *samples_host, const 
     if ((s = fes_grid_args(c, lo, hi, n, bins))) return s;
     if (T < 1 || !samples_host || !V_host || !F_host) return fail(c, METAD_ERR_INVALID, "bad samples");
     const int ncv = c->p.n_cv;
-    Scratch buf;
-    const size_t doubles = (size_t)T * (ncv + 1) + 1 + 2 * (size_t)bins;
-    if ((s = cuda_check(c, cudaMalloc(&buf.p, sizeof(double) * doubles), "reweight buffer"))) return s;
-    double *S = static_cast<double *>(buf.p), *V = S + (size_t)T * ncv, *scratch = V + T, *F = scratch + 1 + bins;
+    constexpr size_t kRows = 8u << 20;  // 64 MB of chunk rows
+    size_t rows = kRows;
+    Scratch own;
+    double *S = nullptr;
+    if (call_scratch(c, metad::reweight_doubles(T, ncv, (int)bins, rows), own, &S) != cudaSuccess) {
+        cudaGetLastError();
+        rows = 0;  // one row
+        if ((s = cuda_check(c, call_scratch(c, metad::reweight_doubles(T, ncv, (int)bins, rows), own, &S),
+                            "reweight buffer")))
+            return s;
+    }
+    double *V = S + (size_t)T * ncv, *F = V + T, *work = F + bins;
     if ((s = cuda_check(c, cudaMemcpyAsync(S, samples_host, sizeof(double) * T * ncv, cudaMemcpyHostToDevice,
                                            c->stream), "sample upload")) ||
         (s = cuda_check(c, cudaMemcpyAsync(V, V_host, sizeof(double) * T, cudaMemcpyHostToDevice, c->stream),
@@ -1806,8 +1870,7 @@ metad_status metad_fes_reweight(metad_ctx *c, const double *samples_host, const 
         return s;
     const int nn[2] = {n[0], ncv == 2 ? n[1] : 1};
     const double beta = 1.0 / (c->p.kB * c->p.temperature);
-    metad::launch_fes_reweight(S, V, T, ncv, lo, hi, nn, beta, scratch, F, c->stream);
-    c->launches += 3;
+    c->launches += metad::launch_fes_reweight(S, V, T, ncv, lo, hi, nn, beta, rows, work, F, c->stream);
     if ((s = launched(c, "fes_reweight"))) return s;
     if ((s = cuda_check(c, cudaMemcpyAsync(F_host, F, sizeof(double) * bins, cudaMemcpyDeviceToHost, c->stream),
                         "fes copy")))

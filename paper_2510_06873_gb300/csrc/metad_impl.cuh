@@ -281,12 +281,21 @@ void launch_batch_gcv_step(const BatchView &hills, int hill_total, int fp64, cud
 int bias_blocks(int K);
 
 // Free-energy passes (k_fes.cu): F at the bin centres of a regular grid from
-// the hills (and grid), and F reweighted from biased samples.  V, F:
-// device [prod n]; scratch: device [1 + prod n].
-void launch_fes_points(const Sys &s, int K, const double *lo, const double *hi, const int *n, double *V, double *F,
-                       double fac, cudaStream_t st);
-void launch_fes_reweight(const double *S, const double *V, long long T, int ncv, const double *lo, const double *hi,
-                         const int *n, double beta, double *scratch, double *F, cudaStream_t st);
+// the hills (and grid), and F reweighted from biased samples; F: device
+// [prod n].  Each takes a workspace of *_doubles() doubles (launch_fes_points
+// leaves F at its start) and returns the kernels launched.  fes_separable:
+// whether the contraction form serves this grid.
+bool fes_separable(const Sys &s, int K, const int *n);
+size_t fes_points_doubles(const Sys &s, int K, const int *n, bool separable);
+int launch_fes_points(const Sys &s, int K, const double *lo, const double *hi, const int *n, double *scratch,
+                      bool separable, double fac, cudaStream_t st);
+// rows: doubles the chunks' rows of bins may take (at least one row is used).
+size_t reweight_doubles(long long T, int ncv, int nbins, size_t rows);
+int launch_fes_reweight(const double *S, const double *V, long long T, int ncv, const double *lo, const double *hi,
+                        const int *n, double beta, size_t rows, double *work, double *F, cudaStream_t st);
+// Fold of the live hills into the grid through the contraction.
+size_t fold_doubles(const Sys &s, int K);
+int launch_fold_separable(const Sys &s, int K, double *work, cudaStream_t st);
 
 // ----------------------------------------------------------------- device math
 __device__ __forceinline__ float mi_f(float d, float halfL, float Lhi, float Llo)

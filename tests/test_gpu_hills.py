@@ -1,6 +1,8 @@
 """Hill sums at the sizes where their kernels change shape, against plain
 numpy in FP64: the integer exponential over its whole argument range, the
-nearest image of far hill centres and the block edges of the hill kernel."""
+nearest image of far hill centres, block and slice edges of the hill kernel,
+the per-axis contraction (free-energy grids, fold) and the chunked
+reweighting sums."""
 import math
 
 import numpy as np
@@ -84,3 +86,77 @@ def test_far_periodic_centres_wrap_to_the_nearest_image(dev):
         tol = (6 * 60 + 40 + 2 * math.pi * 16 / 0.35**2) * U
         assert abs(V - t.sum()) <= tol * t.sum()
         assert np.all(np.abs(g + (t[:, None] * d / sig**2).sum(0)) <= 4 * tol * (t[:, None] * np.abs(d) / sig**2).sum(0))
+
+
+@pytest.mark.parametrize("n", [(7, 40), (8, 8), (16, 16), (17, 33), (101, 9), (300, 8)])
+@pytest.mark.parametrize("K", [0, 1, 33, 65, 700])
+def test_free_energy_grid_tile_edges(dev, n, K):
+    r = np.random.default_rng(n[0] + K)
+    sig, ctr = np.array([0.05, 0.02]), np.array([2.0, 0.3])
+    c, w = ctr + sig * r.uniform(-6, 6, (K, 2)), r.uniform(0.1, 1.0, K)
+    ctx = _ctx(dev, 2, sig)
+    ctx.load_hills(c, w)
+    lo, hi = ctr - 8 * sig, ctr + 7 * sig
+    F = ctx.fes_grid(lo, hi, n)
+    ax = [lo[d] + (np.arange(n[d]) + 0.5) * ((hi[d] - lo[d]) / n[d]) for d in range(2)]
+    e = [(ax[d][:, None] - c[None, :, d]) ** 2 / (2 * sig[d] ** 2) for d in range(2)]
+    V = (w * np.exp(-(e[0][:, None, :] + e[1][None, :, :]))).sum(2)
+    ref = -(10.0 / 9.0) * V
+    # every term within (6 e + 10) roundings, e <= 2 * 14^2 / 2, weighed by the whole sum
+    assert np.abs(F - (ref - ref.min())).max() <= 2 * (6 * 196 + 10 + 40) * U * max(np.abs(ref).max(), 1e-300)
+    assert F.min() == 0.0
+
+
+@pytest.mark.parametrize("n", [(2, 2), (16, 17), (60, 35)])
+@pytest.mark.parametrize("K", [1, 33, 600])
+def test_fold_tile_edges(dev, n, K):
+    """Node values, first and mixed derivatives of the folded hills, folded
+    twice (the second fold adds to the first)."""
+    r = np.random.default_rng(n[0] + K)
+    sig, ctr = np.array([0.05, 0.02]), np.array([2.0, 0.3])
+    lo, hi = ctr - 8 * sig, ctr + 8 * sig
+    ctx = _ctx(dev, 2, sig, grid=(n, lo, hi))
+    ref = np.zeros((*n, 4))
+    scale = np.zeros((*n, 4))
+    ax = [lo[d] + np.arange(n[d]) * ((hi[d] - lo[d]) / (n[d] - 1)) for d in range(2)]
+    for _ in range(2):
+        c, w = ctr + sig * r.uniform(-6, 6, (K, 2)), r.uniform(0.1, 1.0, K)
+        ctx.load_hills(c, w)
+        ctx.fold_hills()
+        dx = [ax[d][:, None] - c[None, :, d] for d in range(2)]
+        e = [dx[d] ** 2 / (2 * sig[d] ** 2) for d in range(2)]
+        g = w * np.exp(-(e[0][:, None, :] + e[1][None, :, :]))
+        u, v = (dx[0] / sig[0] ** 2)[:, None, :], (dx[1] / sig[1] ** 2)[None, :, :]
+        for q, t in enumerate((g, -g * u, -g * v, g * u * v)):
+            ref[..., q] += t.sum(2)
+            scale[..., q] += np.abs(t).sum(2)
+    G = ctx.get_grid()
+    # (6 e + 10) roundings a term, e <= 2 * 14^2 / 2, and the sums; the node
+    # positions differ by a rounding of 2.0, 16 sigma: e changes by 14 * 2 U 2.4 / sigma
+    tol = (6 * 196 + 60 + 14 * 2 * 2.4 / 0.05 * 2) * U
+    assert np.all(np.abs(G - ref) <= tol * scale + 1e-300)
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 64, 65, 5000])
+@pytest.mark.parametrize("n", [(1,), (20,), (9, 7)])
+def test_reweight_chunk_edges(dev, T, n):
+    k = len(n)
+    r = np.random.default_rng(T + k)
+    S = np.column_stack([r.normal(2.0, 0.1, T), r.normal(0.3, 0.03, T)])[:, :k]
+    V = r.uniform(0.0, 15.0, T)
+    lo, hi = np.array([1.8, 0.22])[:k], np.array([2.2, 0.38])[:k]
+    ctx = _ctx(dev, k, (0.05, 0.02)[:k])
+    F = ctx.fes_reweight(S, V, lo, hi, n)
+    h = (hi - lo) / np.array(n)
+    idx = np.floor((S - lo) / h).astype(int)
+    ok = np.all((S >= lo) & (S < hi) & (idx < np.array(n)), axis=1)
+    beta = 1.0 / (0.0083144626 * 300.0)
+    acc = np.zeros(n)
+    np.add.at(acc, tuple(idx[ok].T), np.exp(beta * (V[ok] - V.max())))
+    assert np.array_equal(np.isinf(F), acc == 0.0)
+    if acc.any():
+        with np.errstate(divide="ignore"):
+            ref = -np.log(acc / acc.sum()) / beta
+        ref -= ref.min()
+        fin = acc > 0
+        assert np.allclose(F[fin], ref[fin], rtol=1e-11, atol=1e-11)
