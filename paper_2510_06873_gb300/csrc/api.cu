@@ -412,10 +412,6 @@ metad_status setup_system(metad_ctx *c)
         y.always_rebuild = c->p.skin > 0.0 ? 0 : 1;
         const double grow = std::pow(rv / c->p.rc, 3.0);
         y.max_vnb = ((int)std::ceil(y.max_nb * grow) + 7) / 8 * 8;
-        // mirror slots put i's Verlet position (8 bits) beside j (23 bits)
-        // in an entry's tag, and count exact entries in a byte
-        y.mirror = (n < (1 << metad::kMirrorShift) && y.max_vnb <= 256 && y.max_nb <= 255) ? 1 : 0;
-        y.vround_stride = y.max_vnb / 8;  // one u16 per 8 Verlet entries, rows packed
     }
     y.sw_n = c->p.sw_n;
     y.sw_m = c->p.sw_m;
@@ -435,6 +431,7 @@ metad_status setup_system(metad_ctx *c)
     y.hill_cap = c->p.hill_capacity;
     y.lattice = c->p.lattice_cvs;
     y.virial = c->p.virial || c->p.lattice_cvs;
+    y.pairs = c->fp64 && c->p.n_cv == 2;
     y.D = cv_dims(c->p);
     y.hstride = std::max(y.D, 2);
     for (int d = 0; d < metad::kMaxCv; ++d) y.sigma[d] = 1.0;
@@ -457,10 +454,12 @@ metad_status setup_system(metad_ctx *c)
         y.ghi[a] = c->p.grid_hi[a];
         y.gh[a] = c->p.grid_on ? (y.ghi[a] - y.glo[a]) / (y.gn[a] - 1) : 1.0;
     }
-    // one FP64 partial per block of the per-atom kernels (slot 0: CN, 1: Q6),
-    // three per block of the hill kernel (slot 2), the neighbour statistics
-    // (slot 3)
-    y.part_stride = std::max(metad::group_grid(n), metad::kMaxBiasBlocks * (metad::kMaxCv + 1));
+    // FP64 partials: one per block of the CV sums (slot 0: CN, 1: Q6), three
+    // per block of the force pass with the virial (slot 1, at most
+    // kPersistBlocks / 2 blocks), up to six per block of the hill kernel (slot
+    // 2), the neighbour statistics (slot 3)
+    y.part_stride = std::max(3 * std::min(metad::force_grid(n, y.ncv, y.pairs), metad::kPersistBlocks / 2),
+                             metad::kMaxBiasBlocks * (metad::kMaxCv + 1));
     return METAD_OK;
 }
 
@@ -504,6 +503,21 @@ std::vector<double> pack_centres(const metad_ctx *c, const double *centers, int 
     return out;
 }
 
+// Elements of the per-atom record arrays, each a multiple of 32 so that every
+// record starts on its own size: q 16 per atom (one CV: 8), b 32 in FP32 (q
+// beside b) and 16 in FP64, h 16.
+struct RecSizes {
+    size_t q, b, h;
+};
+
+RecSizes rec_sizes(const metad_ctx *c)
+{
+    const size_t n = ((size_t)c->p.n_atoms + 3) / 4 * 4;
+    if (c->p.n_cv != 2) return RecSizes{8 * n, 0, 0};
+    const size_t m = (n + 1) / 2 * 2;
+    return RecSizes{16 * m, (c->fp64 ? 16 : 32) * m, 16 * m};
+}
+
 struct Buffers {
     int *rank_xyz = nullptr, *xyz_rank = nullptr;
     char *rb = nullptr, *wlb = nullptr, *pfb = nullptr, *geob = nullptr, *crossb = nullptr;
@@ -517,7 +531,9 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
     Sys &y = c->sys;
     const int n = c->p.n_atoms;
     const size_t rs = c->fp64 ? sizeof(double) : sizeof(float);
-    const size_t nq = c->p.n_cv == 2 ? (size_t)16 * n : 16;
+    const RecSizes r = rec_sizes(c);
+    const bool two = c->p.n_cv == 2, pairs = y.pairs != 0;
+    const size_t rows = (size_t)y.max_nb * n;
     metad_status s;
     if (c->p.cv_kind != METAD_CV_COORDINATION) {
         // no neighbour list: CV atoms, gradient terms, reductions and hills
@@ -538,14 +554,13 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
         (s = alloc(&y.ucell, n)) || (s = alloc(&y.uslot, n)) || (s = alloc(&y.cell_count, y.ncell)) ||
         (s = alloc(&y.cell_start, (size_t)y.ncell + 1)) || (s = alloc(&y.scan_part, y.ncell / 4096 + 2)) ||
         (s = alloc(&b.rank_xyz, y.ncell)) || (s = alloc(&b.xyz_rank, y.ncell)) ||
-        (s = alloc(&y.nbr, (size_t)y.max_nb * n)) || (s = alloc(&y.nn, n)) || (s = alloc(&y.nh, n)) ||
-        (s = alloc(&y.vnh, n)) || (s = alloc(&b.wlb, 2 * rs * (size_t)y.max_nb * n)) ||
-        (s = alloc(&b.pfb, rs * 4 * (size_t)y.max_nb * n)) || (s = alloc(&b.geob, rs * 4 * (size_t)y.max_nb * n)) ||
-        (s = alloc(&b.crossb, c->p.n_cv == 2 ? rs * (size_t)y.max_nb * n : 1)) ||
+        (s = alloc(&y.nbr, pairs ? rows : 1)) || (s = alloc(&y.nn, n)) || (s = alloc(&y.nh, n)) ||
+        (s = alloc(&y.vnh, n)) || (s = alloc(&b.wlb, two ? 2 * rs * rows : 1)) ||
+        (s = alloc(&b.pfb, pairs ? rs * 4 * rows : 1)) || (s = alloc(&b.geob, rs * 4 * rows)) ||
+        (s = alloc(&b.crossb, two ? rs * rows : 1)) ||
         (s = alloc(&y.pos_ref, n)) ||
         (s = alloc(&y.vnbr, (size_t)y.max_vnb * n)) || (s = alloc(&y.vnn, n)) || (s = alloc(&y.flag, 1)) ||
-        (s = alloc(&y.vround, y.mirror ? (size_t)y.vround_stride * n : 1)) || (s = alloc(&y.rows_fresh, 1)) ||
-        (s = alloc(&y.rebuilds, 1)) || (s = alloc(&y.Lref, 4)) || (s = alloc(&b.rb, rs * (nq * 3 + (size_t)n * 4 + 64))) ||
+        (s = alloc(&y.rebuilds, 1)) || (s = alloc(&y.Lref, 4)) || (s = alloc(&b.rb, rs * (r.q + r.b + r.h + (size_t)n * 3))) ||
         (s = alloc(&y.part, (size_t)y.part_stride * 4)) || (s = alloc(&y.ticket, 8)) ||
         (s = alloc(&y.scal, metad::kNumScal)) || (s = alloc(&y.err, 1)) ||
         (s = alloc(&y.hc, (size_t)y.hstride * ((size_t)y.hill_cap + 1))) ||
@@ -707,7 +722,6 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
     Sys &y = c->sys;
     const int n = c->p.n_atoms;
     const size_t rs = c->fp64 ? sizeof(double) : sizeof(float);
-    const size_t nq = c->p.n_cv == 2 ? (size_t)16 * n : 16;
     Buffers bf;
     if ((s = state_buffers(c, bf, [c](auto **ptr, size_t count) { return dalloc(c, ptr, count); }))) {
         metad_destroy(c);
@@ -733,13 +747,14 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
     }
     int *rank_xyz = bf.rank_xyz, *xyz_rank = bf.xyz_rank;
     char *rb = bf.rb, *wlb = bf.wlb, *pfb = bf.pfb;
-    // records first (16-element rows stay 64 / 128 B aligned), scalars after
+    // records first, scalars after
+    const RecSizes r = rec_sizes(c);
     y.q = rb;
-    y.b = rb + rs * nq;
-    y.h = rb + rs * 2 * nq;
-    y.cn = rb + rs * 3 * nq;
-    y.W = rb + rs * (3 * nq + n);
-    y.qb6 = rb + rs * (3 * nq + 2 * (size_t)n);
+    y.b = rb + rs * r.q;
+    y.h = rb + rs * (r.q + r.b);
+    y.cn = rb + rs * (r.q + r.b + r.h);
+    y.W = rb + rs * (r.q + r.b + r.h + n);
+    y.qb6 = rb + rs * (r.q + r.b + r.h + 2 * (size_t)n);
     y.wl = wlb;
     y.pairF = pfb;
     y.cross = bf.crossb;
@@ -769,7 +784,6 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
     cudaMemsetAsync(y.vnh, 0, sizeof(int) * (size_t)n, c->stream);
     cudaMemsetAsync(y.vnn, 0, sizeof(int) * (size_t)n, c->stream);
     cudaMemsetAsync(y.rebuilds, 0, sizeof(unsigned long long), c->stream);
-    cudaMemsetAsync(y.rows_fresh, 0, sizeof(int), c->stream);
     {
         const float Lr[4] = {y.Lhi[0], y.Lhi[1], y.Lhi[2], 0.0f};
         if ((s = cuda_check(c, cudaMemcpy(y.Lref, Lr, sizeof(Lr), cudaMemcpyHostToDevice), "box upload"))) {
@@ -841,9 +855,10 @@ metad_status metad_cv_forward(metad_ctx *c, double *cv_host, double *per_atom_de
         c->filter_pending = false;
     }
     if (c->p.n_cv == 2) {
-        StageScope t(c, ST_CV_AVG, 1);  // with the CV sums
+        StageScope t(c, ST_CV_AVG, 1);
         metad::launch_cv_avg(c->sys, c->fp64, c->stream);
-    } else {
+    }
+    {
         StageScope t(c, ST_CV_SUM, 1);
         metad::launch_cv_sum(c->sys, c->fp64, c->stream);
     }
@@ -902,6 +917,19 @@ metad_status metad_bias_eval(metad_ctx *c, const double *s_host, double *V_host,
     return METAD_OK;
 }
 
+// a8 on the context stream.
+static void force_passes(metad_ctx *c, float *forces_dev, int accumulate, double scale)
+{
+    {
+        StageScope t(c, ST_FORCE, 1);
+        metad::launch_forces(c->sys, c->fp64, forces_dev, accumulate, scale, c->stream);
+    }
+    if (metad::pair_slots(c->sys, c->fp64)) {
+        StageScope t(c, ST_FGATHER, 1);
+        metad::launch_force_gather(c->sys, c->fp64, forces_dev, accumulate, c->stream);
+    }
+}
+
 metad_status metad_bias_forces(metad_ctx *c, float *forces_dev, int32_t accumulate, double scale)
 {
     metad_status s = check_usable(c);
@@ -920,14 +948,7 @@ metad_status metad_bias_forces(metad_ctx *c, float *forces_dev, int32_t accumula
         StageScope t(c, ST_ADJ, 1);
         metad::launch_adjoint(c->sys, c->fp64, c->stream);
     }
-    {
-        StageScope t(c, ST_FORCE, 1);
-        metad::launch_force_pairs(c->sys, c->fp64, scale, c->stream);
-    }
-    {
-        StageScope t(c, ST_FGATHER, 1);
-        metad::launch_force_gather(c->sys, c->fp64, forces_dev, accumulate ? 1 : 0, c->stream);
-    }
+    force_passes(c, forces_dev, accumulate ? 1 : 0, scale);
     return launched(c, "bias_forces");
 }
 
@@ -1237,40 +1258,46 @@ metad_status gcv_step_fused(metad_ctx *c, const float *pos_dev, float *forces_de
     return METAD_OK;
 }
 
-// The coordination family's step with the hill kernel on the side stream,
-// concurrent with the adjoint pass: the adjoint needs only the CV pass's
-// records, and the pair forces (which need dV/ds) wait for the join.  The
-// same kernels and arguments as the sequential calls, so the same bits.
+// The coordination family's step with two CVs: the CV sums and the hill
+// kernel on the side stream, concurrent with the adjoint pass, which needs
+// only the Q6 pass's records; the forces (which need dV/ds) wait for the
+// join.  The same kernels and arguments as the sequential calls, so the same
+// bits.  (With one CV there is nothing to run them beside.)
 metad_status step_overlapped(metad_ctx *c, const float *pos_dev, float *forces_dev, int32_t accumulate,
                              int32_t deposit)
 {
     metad_status s;
     if ((s = metad_build_neighbors(c, pos_dev))) return s;
-    if ((s = metad_cv_forward(c, nullptr, nullptr))) return s;
     if (!forces_dev) return fail(c, METAD_ERR_INVALID, "forces_dev is NULL");
+    {
+        StageScope t(c, ST_CV_FWD, 1);
+        metad::launch_cv_fwd(c->sys, c->fp64, 1, c->stream);
+        c->filter_pending = false;
+    }
+    {
+        StageScope t(c, ST_CV_AVG, 1);
+        metad::launch_cv_avg(c->sys, c->fp64, c->stream);
+    }
     if ((s = cuda_check(c, cudaEventRecord(c->ev_fork, c->stream), "fork")) ||
         (s = cuda_check(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0), "fork")))
         return s;
+    {
+        StageScope t(c, ST_CV_SUM, 1, c->side);
+        metad::launch_cv_sum(c->sys, c->fp64, c->side);
+    }
     {
         StageScope t(c, ST_BIAS, 1, c->side);
         metad::launch_bias(c->sys, c->K, c->sys.scal + metad::kS0, c->sys.scal + metad::kV, 0, c->side);
     }
     if ((s = cuda_check(c, cudaEventRecord(c->ev_join, c->side), "join"))) return s;
-    if (c->p.n_cv == 2) {
+    {
         StageScope t(c, ST_ADJ, 1);
         metad::launch_adjoint(c->sys, c->fp64, c->stream);
     }
     if ((s = cuda_check(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0), "join"))) return s;
-    {
-        StageScope t(c, ST_FORCE, 1);
-        metad::launch_force_pairs(c->sys, c->fp64, 1.0, c->stream);
-    }
-    {
-        StageScope t(c, ST_FGATHER, 1);
-        metad::launch_force_gather(c->sys, c->fp64, forces_dev, accumulate ? 1 : 0, c->stream);
-    }
+    force_passes(c, forces_dev, accumulate ? 1 : 0, 1.0);
     if ((s = launched(c, "step"))) return s;
-    c->have_bias = true;
+    c->have_cv = c->have_bias = true;
     c->forces_done = true;
     if (deposit && (s = metad_deposit_hill(c, nullptr, nullptr))) return s;
     return METAD_OK;
@@ -1281,7 +1308,7 @@ metad_status step_direct(metad_ctx *c, const float *pos_dev, float *forces_dev, 
     metad_status s;
     if (c && !c->failed && c->p.cv_kind != METAD_CV_COORDINATION && c->p.n_atoms <= metad::kFuseAtoms)
         return gcv_step_fused(c, pos_dev, forces_dev, accumulate, deposit);
-    if (c && !c->failed && c->p.cv_kind == METAD_CV_COORDINATION)
+    if (c && !c->failed && c->p.cv_kind == METAD_CV_COORDINATION && c->p.n_cv == 2)
         return step_overlapped(c, pos_dev, forces_dev, accumulate, deposit);
     if ((s = metad_build_neighbors(c, pos_dev))) return s;
     if ((s = metad_cv_forward(c, nullptr, nullptr))) return s;
@@ -1692,22 +1719,28 @@ metad_status metad_batch_step(metad_batch *b, const float *const *pos_dev, float
     } else {
     metad::launch_batch_gather(rows[metad::GK_ATOM256], totals[metad::GK_ATOM256], b->stream);
     metad::launch_batch_rebuild(rows, totals, b->stream);
-    metad::launch_batch_cv(rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], rows[metad::GK_CV], totals[metad::GK_CV],
-                           rows[metad::GK_SUM], totals[metad::GK_SUM], b->fp64, b->ncv, b->stream);
-    // the hill kernel on the side stream, concurrent with the adjoint
-    cudaEventRecord(b->ev_fork, b->stream);
-    cudaStreamWaitEvent(b->side, b->ev_fork, 0);
-    metad::launch_batch_bias(rows[metad::GK_HILLS], totals[metad::GK_HILLS], 0, b->side);
-    cudaEventRecord(b->ev_join, b->side);
-    metad::launch_batch_force(rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], rows[metad::GK_ATOM32],
-                              totals[metad::GK_ATOM32], rows[metad::GK_ATOM128], totals[metad::GK_ATOM128], b->fp64,
-                              b->ncv, b->ctx[0]->sys.virial, b->stream, 1);
-    cudaStreamWaitEvent(b->stream, b->ev_join, 0);
-    metad::launch_batch_force(rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], rows[metad::GK_ATOM32],
-                              totals[metad::GK_ATOM32], rows[metad::GK_ATOM128], totals[metad::GK_ATOM128], b->fp64,
-                              b->ncv, b->ctx[0]->sys.virial, b->stream, 2);
+    metad::launch_batch_cv(rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], rows[metad::GK_ROWS],
+                           totals[metad::GK_ROWS], b->fp64, b->ncv, b->stream);
+    // two CVs: the CV sums and the hill kernel on the side stream, concurrent
+    // with the adjoint
+    const bool fork = b->ncv == 2;
+    cudaStream_t side = fork ? b->side : b->stream;
+    if (fork) {
+        cudaEventRecord(b->ev_fork, b->stream);
+        cudaStreamWaitEvent(b->side, b->ev_fork, 0);
+    }
+    metad::launch_batch_sum(rows[metad::GK_SUM], totals[metad::GK_SUM], b->fp64, side);
+    metad::launch_batch_bias(rows[metad::GK_HILLS], totals[metad::GK_HILLS], 0, side);
+    if (fork) {
+        cudaEventRecord(b->ev_join, b->side);
+        metad::launch_batch_adjoint(rows[metad::GK_ROWS], totals[metad::GK_ROWS], b->fp64, b->stream);
+        cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+    }
+    const int forces = metad::launch_batch_forces(rows[metad::GK_FORCE], totals[metad::GK_FORCE],
+                                                  rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], b->fp64, b->ncv,
+                                                  b->ctx[0]->sys.virial, b->stream);
     if (any_deposit) metad::launch_batch_bias(rows[metad::GK_DEPOSIT], totals[metad::GK_DEPOSIT], 1, b->stream);
-    b->launches += 1 + 6 + 2 + 1 + (b->ncv == 2 ? 3 : 2) + (any_deposit ? 1 : 0);
+    b->launches += 1 + 6 + 1 + (fork ? 2 : 0) + 2 + forces + (any_deposit ? 1 : 0);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

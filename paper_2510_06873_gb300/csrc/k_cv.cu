@@ -17,9 +17,9 @@
 //     ds2/dd = ds2/dw w'(r) d/r + w sum_m (h_m(i)+h_m(j)) dY_m/dd
 //     ds1/dd = (2/N) w'(r) d/r [unlike]
 //   F_i = sum_{j in N(i)} (V1 ds1/dd + V2 ds2/dd)
-// The CV passes walk full rows (each atom gathers its own sums); the force
-// evaluates each unordered pair once and gathers per atom in a fixed order:
-// no floating-point atomics, bit-reproducible.
+// Every pass walks full rows, each atom gathering its own sums: no atomics,
+// bit-reproducible.  (FP64 with two CVs instead evaluates each unordered pair
+// once and adds the pair forces up per atom in a fixed order.)
 #include "metad_impl.cuh"
 
 namespace metad {
@@ -38,8 +38,6 @@ struct YlmConst {
     float dpf[7][4];  // dP_m/dz likewise
     double pd[7][4];
     double dpd[7][4];
-    float kf_hi[kNY], kf_lo[kNY];  // K per Y slot
-    double kd[kNY];
 };
 __constant__ YlmConst c_ylm;
 
@@ -121,33 +119,6 @@ __device__ __forceinline__ void ylm13_acc(real x, real y, real z, real w, real v
     }
 }
 
-// Y_k(u) and g = (I - u u^T) grad(sum_k c_k Y_k) / r.
-template <typename real>
-__device__ __forceinline__ void ylm13_grad(real x, real y, real z, real inv_r, const real c[kNY], real Y[kNY],
-                                           real g[3])
-{
-    real P[7], D[7], C[7], S[7];
-    legendre_parts<real>(z, P);
-    legendre_dparts<real>(z, D);
-    cs_powers<real>(x, y, C, S);
-    Y[0] = P[0];
-    real gx = real(0), gy = real(0), gz = c[0] * D[0];
-#pragma unroll
-    for (int m = 1; m <= 6; ++m) {
-        real cc = c[2 * m - 1], cs = c[2 * m];
-        Y[2 * m - 1] = P[m] * C[m];
-        Y[2 * m] = P[m] * S[m];
-        real pm = P[m] * real(m);
-        gx += pm * (cc * C[m - 1] + cs * S[m - 1]);
-        gy += pm * (cs * C[m - 1] - cc * S[m - 1]);
-        gz += D[m] * (cc * C[m] + cs * S[m]);
-    }
-    real ug = x * gx + y * gy + z * gz;
-    g[0] = (gx - ug * x) * inv_r;
-    g[1] = (gy - ug * y) * inv_r;
-    g[2] = (gz - ug * z) * inv_r;
-}
-
 // sum_k h_k Y_k(u) and g = (I - u u^T) grad(sum_k h_k Y_k) / r in one loop,
 // without materialising the harmonics (fewer live registers in the pair pass).
 template <typename real>
@@ -175,46 +146,73 @@ __device__ __forceinline__ real ylm13_dot_grad(real x, real y, real z, real inv_
     return t;
 }
 
-// sum_k K_k a_k^2 with K as a float pair (FP32) or exact (FP64).
-template <typename real>
-__device__ __forceinline__ real weighted_sq(const real a[kNY]);
-template <>
-__device__ __forceinline__ float weighted_sq<float>(const float a[kNY])
+// The weights K per Y slot (0 past the 13), as float pairs and in FP64.  Read
+// by slots that depend on the lane, so they sit in global memory: a constant
+// bank serves one address of a warp at a time.
+constexpr double k_weight(int slot)
 {
-    float hi = 0.0f, lo = 0.0f;
-#pragma unroll
-    for (int m = 0; m < kNY; ++m) {
-        float a2 = a[m] * a[m];
-        hi = fmaf(c_ylm.kf_hi[m], a2, hi);
-        lo = fmaf(c_ylm.kf_lo[m], a2, lo);
-    }
-    return hi + lo;
+    const int m = (slot + 1) / 2;
+    if (slot >= kNY) return 0.0;
+    double f = m > 0 ? 2.0 : 1.0;
+    for (int k = 6 - m + 1; k <= 6 + m; ++k) f /= k;
+    return f;
 }
-template <>
-__device__ __forceinline__ double weighted_sq<double>(const double a[kNY])
-{
-    double s = 0.0;
-#pragma unroll
-    for (int m = 0; m < kNY; ++m) s += c_ylm.kd[m] * a[m] * a[m];
-    return s;
-}
-template <typename real>
-__device__ __forceinline__ real weighted_term(int m, real a);
-template <>
-__device__ __forceinline__ float weighted_term<float>(int m, float a)
-{
-    const float a2 = a * a;
-    return fmaf(c_ylm.kf_lo[m], a2, c_ylm.kf_hi[m] * a2);
-}
-template <>
-__device__ __forceinline__ double weighted_term<double>(int m, double a) { return c_ylm.kd[m] * a * a; }
+#define METAD_K16(f) f(0), f(1), f(2), f(3), f(4), f(5), f(6), f(7), f(8), f(9), f(10), f(11), f(12), f(13), f(14), f(15)
+#define METAD_KHI(m) (float)k_weight(m)
+#define METAD_KLO(m) (float)(k_weight(m) - (double)(float)k_weight(m))
+static __device__ __align__(16) const float kKhi[16] = {METAD_K16(METAD_KHI)};
+static __device__ __align__(16) const float kKlo[16] = {METAD_K16(METAD_KLO)};
+static __device__ __align__(16) const double kKd[16] = {METAD_K16(k_weight)};
+#undef METAD_K16
+#undef METAD_KHI
+#undef METAD_KLO
 
+// K of slots 4l .. 4l + 3, and the terms K_m a_m^2 of them.
 template <typename real>
-__device__ __forceinline__ real kweight(int m);
+struct KWeights;
 template <>
-__device__ __forceinline__ float kweight<float>(int m) { return c_ylm.kf_hi[m]; }
+struct KWeights<float> {
+    float4 hi, lo;
+    __device__ __forceinline__ explicit KWeights(int l)
+        : hi(__ldg(reinterpret_cast<const float4 *>(kKhi) + l)), lo(__ldg(reinterpret_cast<const float4 *>(kKlo) + l))
+    {
+    }
+    __device__ __forceinline__ void get(float k[4]) const
+    {
+        k[0] = hi.x;
+        k[1] = hi.y;
+        k[2] = hi.z;
+        k[3] = hi.w;
+    }
+    __device__ __forceinline__ float sum_sq(const float a[4]) const
+    {
+        const float x = a[0] * a[0], y = a[1] * a[1], z = a[2] * a[2], w = a[3] * a[3];
+        const float h = fmaf(hi.w, w, fmaf(hi.z, z, fmaf(hi.y, y, hi.x * x)));
+        const float e = fmaf(lo.w, w, fmaf(lo.z, z, fmaf(lo.y, y, lo.x * x)));
+        return h + e;
+    }
+};
 template <>
-__device__ __forceinline__ double kweight<double>(int m) { return c_ylm.kd[m]; }
+struct KWeights<double> {
+    double k_[4];
+    __device__ __forceinline__ explicit KWeights(int l)
+    {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) k_[c] = __ldg(kKd + 4 * l + c);
+    }
+    __device__ __forceinline__ void get(double k[4]) const
+    {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) k[c] = k_[c];
+    }
+    __device__ __forceinline__ double sum_sq(const double a[4]) const
+    {
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s += k_[c] * a[c] * a[c];
+        return s;
+    }
+};
 
 // 16-wide per-atom records (13 used): one 64 B (FP32) or 128 B (FP64) row
 // per atom, so a neighbour's record is two sectors, not thirteen.
@@ -246,23 +244,6 @@ __device__ __forceinline__ void load_rec<double>(const double *base, int i, doub
         v[2 * k + 1] = t.y;
     }
 }
-template <typename real>
-__device__ __forceinline__ void store_rec(real *base, int i, const real v[kRec]);
-template <>
-__device__ __forceinline__ void store_rec<float>(float *base, int i, const float v[kRec])
-{
-    float4 *p = reinterpret_cast<float4 *>(base + (size_t)i * kRec);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) p[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-}
-template <>
-__device__ __forceinline__ void store_rec<double>(double *base, int i, const double v[kRec])
-{
-    double2 *p = reinterpret_cast<double2 *>(base + (size_t)i * kRec);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = make_double2(v[2 * k], v[2 * k + 1]);
-}
-
 namespace {
 
 template <typename real>
@@ -284,13 +265,12 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
 }
 
 // Displacement (cached by the exact filter), 1/r, switch weight and its
-// derivative of one exact entry, with its neighbour, CN mask and mirror
-// position.
+// derivative of one exact entry, with its neighbour and CN mask.
 template <typename real, bool kLast = false>
 __device__ __forceinline__ void cached_geometry(const Sys &s, size_t slot, Vec3<real> &d, real &inv_r, real &w,
-                                                real &dw, bool &cn, int &j, unsigned &vm)
+                                                real &dw, bool &cn, int &j)
 {
-    load_geo<real, kLast>(s, slot, d, cn, j, vm);
+    load_geo<real, kLast>(s, slot, d, cn, j);
     real r2 = d.x * d.x + d.y * d.y + d.z * d.z;
     inv_r = rsqrt_r<real>(r2);
     switch_eval<real>(s, r2 * inv_r, w, dw);
@@ -334,48 +314,31 @@ __device__ __forceinline__ real group_get(real v, int src_lane)
     return __shfl_sync(0xffffffffu, v, base + src_lane);
 }
 
-template <typename real>
-__device__ __forceinline__ void store_pair(real *base, int i, int l, real a, real b);
-template <>
-__device__ __forceinline__ void store_pair<float>(float *base, int i, int l, float a, float b)
+// Components (2l, 2l + 1) of a record of kLen.
+template <typename real, int kLen>
+__device__ __forceinline__ void store_pair(real *base, int i, int l, real a, real b)
 {
-    reinterpret_cast<float2 *>(base + (size_t)i * kRec)[l] = make_float2(a, b);
-}
-template <>
-__device__ __forceinline__ void store_pair<double>(double *base, int i, int l, double a, double b)
-{
-    reinterpret_cast<double2 *>(base + (size_t)i * kRec)[l] = make_double2(a, b);
-}
-
-// Components (2l, 2l + 1) of record i: the kG lanes of a group together read
-// the whole 64 B (FP32) row with one coalesced access.
-template <typename real>
-__device__ __forceinline__ void load_pair(const real *base, int i, int l, real &a, real &b);
-template <>
-__device__ __forceinline__ void load_pair<float>(const float *base, int i, int l, float &a, float &b)
-{
-    const float2 t = reinterpret_cast<const float2 *>(base + (size_t)i * kRec)[l];
-    a = t.x;
-    b = t.y;
-}
-template <>
-__device__ __forceinline__ void load_pair<double>(const double *base, int i, int l, double &a, double &b)
-{
-    const double2 t = reinterpret_cast<const double2 *>(base + (size_t)i * kRec)[l];
-    a = t.x;
-    b = t.y;
+    struct alignas(2 * sizeof(real)) P2 {
+        real a, b;
+    };
+    reinterpret_cast<P2 *>(base + (size_t)i * kLen)[l] = P2{a, b};
 }
 
 __device__ __forceinline__ const int *nbr_row(const Sys &s, int i) { return s.nbr + (size_t)i * s.max_nb; }
 
-// a4: CN_i, W_i and q_m(i) = sum_j w_ij Y_m(rhat_ij) / W_i.
+// a4: CN_i, W_i and q_m(i) = sum_j w_ij Y_m(rhat_ij) / W_i.  With one CV, CN_i
+// and what its force and virial need: sum_j w' d / r and sum_j w' d_a^2 / r
+// over the counted pairs (the force on an atom is 2 V1 / N times the first,
+// so no later pass walks the rows).
 // With kFilter the exact row is first compacted from the Verlet row.
+constexpr int kCnRec = 8;  // fx fy fz, vx vy vz, 2 unused
+
 template <typename real, bool kFilter>
-__device__ __forceinline__ double cv_fwd_group(const Sys &s, const AtomLane a)
+__device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
 {
     int nn_f = 0;
     if (kFilter) nn_f = filter_row<real>(s, a);
-    real v[kRec];  // 0..12: sum w Y_m ; 13: W ; 14: CN
+    real v[kRec];  // 0..12: sum w Y_m (one CV: 0..5 as above) ; 13: W ; 14: CN
 #pragma unroll
     for (int m = 0; m < kRec; ++m) v[m] = real(0);
     if (a.ok) {
@@ -386,33 +349,41 @@ __device__ __forceinline__ double cv_fwd_group(const Sys &s, const AtomLane a)
             real inv_r, w, dw;
             bool cn;
             int j;
-            unsigned vm;
-            cached_geometry<real>(s, (size_t)a.i * s.max_nb + k, d, inv_r, w, dw, cn, j, vm);
-            jwrow[k] = JW<real>{j, w};
+            cached_geometry<real>(s, (size_t)a.i * s.max_nb + k, d, inv_r, w, dw, cn, j);
             if (cn) v[14] += w;
             v[13] += w;
-            if (s.ncv == 2) ylm13_acc<real>(d.x * inv_r, d.y * inv_r, d.z * inv_r, w, v);
+            if (s.ncv == 2) {
+                jwrow[k] = JW<real>{j, w};
+                ylm13_acc<real>(d.x * inv_r, d.y * inv_r, d.z * inv_r, w, v);
+            } else if (cn) {
+                const real gx = dw * inv_r * d.x, gy = dw * inv_r * d.y, gz = dw * inv_r * d.z;
+                v[0] += gx;
+                v[1] += gy;
+                v[2] += gz;
+                if (s.virial) {
+                    v[3] += gx * d.x;
+                    v[4] += gy * d.y;
+                    v[5] += gz * d.z;
+                }
+            }
         }
     }
     reduce_scatter16<real>(v, a.l);
     // lane 6 holds (13: W, ...) in v[1]; lane 7 holds (14: CN, 15) in v[0]
     const real W = group_get<real>(v[1], 6);
-    double cn_out = 0.0;
     if (a.ok) {
-        if (a.l == 7) {
-            R<real>(s.cn)[a.i] = v[0];
-            cn_out = (double)v[0];
-        }
-        if (a.l == 6) R<real>(s.W)[a.i] = W;
+        if (a.l == 7) R<real>(s.cn)[a.i] = v[0];
         if (s.ncv == 2) {
+            if (a.l == 6) R<real>(s.W)[a.i] = W;
             const real inv_W = W > real(0) ? real(1) / W : real(0);
             real q0 = v[0] * inv_W, q1 = v[1] * inv_W;
             if (a.l == 6) q1 = real(0);
             if (a.l == 7) q0 = q1 = real(0);
-            store_pair<real>(R<real>(s.q), a.i, a.l, q0, q1);
+            store_pair<real, kRec>(R<real>(s.q), a.i, a.l, q0, q1);
+        } else if (a.l < kCnRec / 2) {
+            store_pair<real, kCnRec>(R<real>(s.q), a.i, a.l, v[0], v[1]);
         }
     }
-    return cn_out;
 }
 
 template <typename real, bool kFilter>
@@ -422,11 +393,16 @@ __device__ __forceinline__ void cv_fwd(const Sys &s, Blk k)
     for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_fwd_group<real, kFilter>(s, atom_lane_at(s, g));
 }
 
+// Resident blocks per SM: 12 in FP32 (40 registers), none asked for in FP64
+// (40 registers spill there).
+template <typename real>
+constexpr int kFwdBlocks = sizeof(real) == 4 ? 12 : 0;
+
 template <typename real, bool kFilter>
-__global__ void __launch_bounds__(kBlockAtoms, 12) k_cv_fwd(Sys s) { cv_fwd<real, kFilter>(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) k_cv_fwd(Sys s) { cv_fwd<real, kFilter>(s, own_blk()); }
 
 template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms, 12) kb_cv_fwd(BatchView v)
+__global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) kb_cv_fwd(BatchView v)
 {
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
@@ -498,131 +474,88 @@ __device__ __forceinline__ void load_jw2<float>(const JW<float> *row, int k, JW<
     e1 = JW<float>{v.z, __int_as_float(v.w)};
 }
 
-// a5: qbar_m(i), qbar6(i), s2.  Record b: b_m(i) = K_m qbar_m(i) / (N qbar6
-// (1 + W_i)) (slots 0..12) and beta_i = b(i).qbar(i) (slot 13).
-template <typename real>
-__device__ __forceinline__ void cv_avg_group(const Sys &s, const AtomLane a, RunSum<real> &cn_sum,
-                                             RunSum<real> &q6_sum)
+// The CV sums: each block's C and Q -> part[b], part[part_stride + b]; the
+// last block to finish adds them (lane l of warp 0 resp. 1 takes blocks l,
+// l + 32, ... in order, then a fixed tree): s1 = C / N, s2 = Q / N.  A fixed
+// association for a given grid.
+__device__ void finish_cv_sums(const Sys &s, Blk k, double sum, int which)
 {
-    // lane l owns components 2l, 2l + 1 and walks every neighbour of the atom
-    const real *q = R<real>(s.q);
-    real a0 = real(0), a1 = real(0);
-    if (a.ok) {
-        const int nn = s.nn[a.i];
-        const JW<real> *jwrow = reinterpret_cast<const JW<real> *>(s.wl) + (size_t)a.i * s.max_nb;
-#pragma unroll 2
-        for (int k = 0; k < nn; k += 2) {
-            JW<real> e0, e1;
-            load_jw2<real>(jwrow, k, e0, e1);
-            const bool two = k + 1 < nn;
-            real x0, x1, y0 = real(0), y1 = real(0);
-            load_pair<real>(q, e0.j, a.l, x0, x1);
-            if (two) load_pair<real>(q, e1.j, a.l, y0, y1);
-            a0 += e0.w * x0;
-            a1 += e0.w * x1;
-            if (two) {
-                a0 += e1.w * y0;
-                a1 += e1.w * y1;
-            }
-        }
-    }
-    real qb0 = real(0), qb1 = real(0), sq = real(0), inv_D = real(0);
-    if (a.ok) {
-        inv_D = real(1) / (real(1) + R<real>(s.W)[a.i]);
-        real o0, o1;
-        load_pair<real>(q, a.i, a.l, o0, o1);
-        const int m0 = 2 * a.l, m1 = 2 * a.l + 1;
-        if (m0 < kNY) qb0 = (o0 + a0) * inv_D;
-        if (m1 < kNY) qb1 = (o1 + a1) * inv_D;
-        if (m0 < kNY) sq += weighted_term<real>(m0, qb0);
-        if (m1 < kNY) sq += weighted_term<real>(m1, qb1);
-    }
-    sq = group_sum<real>(sq);
-    const real qb6 = sqrt(sq);
-    const real ci = qb6 > real(0) ? inv_D / (n_real<real>(s) * qb6) : real(0);
-    const int m0 = 2 * a.l, m1 = 2 * a.l + 1;
-    real b0 = m0 < kNY ? ci * kweight<real>(m0) * qb0 : real(0);
-    real b1 = m1 < kNY ? ci * kweight<real>(m1) * qb1 : real(0);
-    const real beta = group_sum<real>(b0 * qb0 + b1 * qb1);
-    if (a.ok) {
-        if (a.l == 6) b1 = beta;  // slot 13
-        store_pair<real>(R<real>(s.b), a.i, a.l, b0, b1);
-        if (a.l == 0) {
-            R<real>(s.qb6)[a.i] = qb6;
-            cn_sum.add(R<real>(s.cn)[a.i]);
-            q6_sum.add(qb6);
-        }
-    }
-}
-
-// Block sums c, q -> part[b], part[part_stride + b]; the last block to finish
-// adds them (thread t takes blocks t, t + blockDim, ... in order, then a
-// fixed tree): s1 = C / N, s2 = Q / N.  A fixed association for a given grid.
-__device__ void last_block_cv(const Sys &s, Blk k, double c, double q)
-{
-    __shared__ double sh[32];
+    // thread 0 holds the block's C, thread 32 its Q
     __shared__ bool am_last;
+    const int lane = threadIdx.x & 31;
     if (k.nb > s.part_stride) {  // never with the grids used; refuse rather than overrun
         if (k.b == 0 && threadIdx.x == 0) set_err(s, kErrInternal);
         return;
     }
-    c = block_sum(c, sh);
-    q = block_sum(q, sh);
-    double *pc = s.part, *pq = s.part + s.part_stride;
-    if (threadIdx.x == 0) {
-        pc[k.b] = c;
-        pq[k.b] = q;
+    if (k.nb > 1) {
+        double *part = s.part + (size_t)which * s.part_stride;
+        if (which < 2 && lane == 0) {
+            part[k.b] = sum;
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) am_last = atomicAdd(&s.ticket[0], 1u) == (unsigned)k.nb - 1u;
+        __syncthreads();
+        if (!am_last) return;
         __threadfence();
-        am_last = atomicAdd(&s.ticket[0], 1u) == (unsigned)k.nb - 1u;
+        if (which < 2) {
+            sum = 0.0;
+            for (int b = lane; b < k.nb; b += 32) sum += __ldcg(part + b);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+        }
+        if (threadIdx.x == 0) s.ticket[0] = 0u;
     }
-    __syncthreads();
-    if (!am_last) return;
-    __threadfence();
-    double C = 0.0, Q = 0.0;
-    for (int b = threadIdx.x; b < k.nb; b += blockDim.x) {
-        C += __ldcg(pc + b);
-        Q += __ldcg(pq + b);
-    }
-    C = block_sum(C, sh);
-    Q = block_sum(Q, sh);
-    if (threadIdx.x == 0) {
-        s.scal[kS0] = C / s.n;
-        if (s.ncv == 2) s.scal[kS1] = Q / s.n;
+    if (which == 0 && lane == 0) s.scal[kS0] = sum / s.n;
+    if (which == 1 && lane == 0) {
+        if (s.ncv == 2) s.scal[kS1] = sum / s.n;
         else if (!s.lattice) s.scal[kS1] = 0.0;
         if (s.lattice)  // the triaxial lattice parameters follow the per-atom CVs
             for (int a = 0; a < 3; ++a) s.scal[kS0 + s.ncv + a] = s.L[a];
-        s.ticket[0] = 0u;
     }
 }
 
-// a5 with the CV sums: persistent (the block partials are few).
-// The filter of the last kernel saw the rows' mirror positions stored.
-__device__ __forceinline__ void rows_used(const Sys &s, Blk k)
-{
-    if (k.b == 0 && threadIdx.x == 0 && s.mirror) *s.rows_fresh = 0;
-}
-
-template <typename real>
-__device__ __forceinline__ void cv_avg(const Sys &s, Blk k)
-{
-    rows_used(s, k);
-    RunSum<real> c, q;
-    const int groups = group_grid(s.n);
-    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_avg_group<real>(s, atom_lane_at(s, g), c, q);
-    last_block_cv(s, k, c.value(), q.value());
-}
-
-// The CV sum when there is no Q6 pass (n_cv == 1): thread t of block b sums
-// the CN of atoms b kSumThreads + t, + blocks kSumThreads, ... in order
-// (a compensated FP32 pair with FP32 records).
+// s1, s2: thread t of block b sums CN and qbar6 of atoms b kSumThreads + t,
+// + blocks kSumThreads, ... in order (compensated FP32 pairs with FP32
+// records), four loads in flight; the warps' trees stay compensated FP32 and
+// only one value per warp enters the FP64 sums (a warp-wide FP64 add holds
+// the pipe for 64 cycles).  Its own pass, beside the adjoint in a step: the
+// Q6 pass then carries no sums, and its blocks no FP64 epilogue (27,648
+// atoms: Q6 pass 25.6 -> 10.2 us).
 template <typename real>
 __device__ __forceinline__ void cv_sum(const Sys &s, Blk k)
 {
-    rows_used(s, k);
-    RunSum<real> c;
-    const real *cn = R<real>(s.cn);
-    for (int i = k.b * blockDim.x + threadIdx.x; i < s.n; i += k.nb * blockDim.x) c.add(cn[i]);
-    last_block_cv(s, k, c.value(), 0.0);
+    RunSum<real> c, q;
+    const real *cn = R<real>(s.cn), *q6 = R<real>(s.qb6);
+    const int step = k.nb * blockDim.x;
+    for (int i = k.b * blockDim.x + threadIdx.x; i < s.n; i += 4 * step) {
+        real x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool in = i + u * step < s.n;
+            x[u] = in ? cn[i + u * step] : real(0);
+            y[u] = in && s.ncv == 2 ? q6[i + u * step] : real(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            c.add(x[u]);
+            q.add(y[u]);
+        }
+    }
+    constexpr int kW = kSumThreads / 32;
+    __shared__ double sh[2][kW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    warp_sum(c);
+    warp_sum(q);
+    if (lane == 0) {
+        sh[0][wid] = c.value();
+        sh[1][wid] = q.value();
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (wid < 2 && lane == 0)
+        for (int w = 0; w < kW; ++w) t += sh[wid][w];
+    finish_cv_sums(s, k, t, wid);
 }
 
 template <typename real>
@@ -636,25 +569,12 @@ __global__ void __launch_bounds__(kSumThreads) kb_cv_sum(BatchView v)
     cv_sum<real>(s, k);
 }
 
-template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms) k_cv_avg(Sys s) { cv_avg<real>(s, own_blk()); }
-
-template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms) kb_cv_avg(BatchView v)
-{
-    Blk k;
-    const Sys &s = v.sys[batch_system(v, k)];
-    cv_avg<real>(s, k);
-}
-
-// a7: g_m(k) = b_m(k) + sum_i w_ik b_m(i) ; h = g / W ; record h holds h_m
-// (0..12) and gamma_k = h(k).q(k) + beta_k (slot 13).
-// a7 with four lanes per atom, four record components per lane (one 16 B
-// load of each neighbour record per lane): a warp has eight atoms' gathers in
-// flight.  (Measured faster than eight lanes of two components here; the Q6
-// average keeps eight lanes, where four cost it occupancy.)
+// The row passes a5, a7 and a8 give an atom four lanes; lane l owns record
+// components 4l .. 4l + 3 (one 16 B load of each neighbour record per lane),
+// so a warp has eight atoms' gathers in flight.
 constexpr int kG4 = 4;
-constexpr int kAtoms4 = kBlockAtoms / kG4;
+static_assert(kRowAtoms * kG4 == kRowThreads, "four lanes per atom");
+constexpr int kRecQB = 32;  // FP32: q and b side by side, in chunks of four
 
 template <typename real>
 __device__ __forceinline__ void load4(const real *base, int i, int l, real v[4]);
@@ -692,6 +612,26 @@ __device__ __forceinline__ void store4<double>(double *base, int i, int l, const
     p[1] = make_double2(v[2], v[3]);
 }
 
+// Chunk l of record i of the FP32 q-and-b records: q then b, one 32 B load.
+__device__ __forceinline__ void load_qb(const float *base, int i, int l, float q[4], float b[4])
+{
+    const float *p = base + (size_t)i * kRecQB + 8 * l;
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(q[0]), "=f"(q[1]), "=f"(q[2]), "=f"(q[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
+        : "l"(p));
+}
+
+__device__ __forceinline__ void store_b(const Sys &s, int i, int l, const float q[4], const float b[4])
+{
+    float4 *p = reinterpret_cast<float4 *>(R<float>(s.b) + (size_t)i * kRecQB) + 2 * l;
+    p[0] = make_float4(q[0], q[1], q[2], q[3]);
+    p[1] = make_float4(b[0], b[1], b[2], b[3]);
+}
+__device__ __forceinline__ void store_b(const Sys &s, int i, int l, const double *, const double b[4])
+{
+    store4<double>(R<double>(s.b), i, l, b);
+}
+
 template <typename real>
 __device__ __forceinline__ real group4_sum(real v)
 {
@@ -700,6 +640,86 @@ __device__ __forceinline__ real group4_sum(real v)
     return v;
 }
 
+// a5: qbar_m(i), qbar6(i).  Record b: b_m(i) = K_m qbar_m(i) / (N qbar6
+// (1 + W_i)) (slots 0..12) and beta_i = b(i).qbar(i) (slot 13); FP32 records
+// carry q beside b, for the adjoint to gather both with one load.
+template <typename real>
+__device__ __forceinline__ void cv_avg_group(const Sys &s, int g)
+{
+    const int i = g * kRowAtoms + (threadIdx.x / kG4), l = threadIdx.x & (kG4 - 1);
+    const bool ok = i < s.n;
+    const real *q = R<real>(s.q);
+    real a[4] = {real(0), real(0), real(0), real(0)}, o[4] = {real(0), real(0), real(0), real(0)};
+    real inv_D = real(0);
+    const KWeights<real> K(l);
+    if (ok) {
+        const int nn = s.nn[i];
+        inv_D = real(1) / (real(1) + R<real>(s.W)[i]);
+        load4<real>(q, i, l, o);
+        const JW<real> *jwrow = reinterpret_cast<const JW<real> *>(s.wl) + (size_t)i * s.max_nb;
+#pragma unroll 2
+        for (int k = 0; k < nn; k += 2) {
+            JW<real> e0, e1;
+            load_jw2<real>(jwrow, k, e0, e1);
+            const bool two = k + 1 < nn;
+            real x[4], y[4] = {real(0), real(0), real(0), real(0)};
+            load4<real>(q, e0.j, l, x);
+            if (two) load4<real>(q, e1.j, l, y);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a[c] += e0.w * x[c];
+            if (two) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) a[c] += e1.w * y[c];
+            }
+        }
+    }
+    // slots 13 .. 15 hold 0 in q, so qb is 0 there too
+    real qb[4], kw[4], b[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) qb[c] = (o[c] + a[c]) * inv_D;
+    const real sq = group4_sum<real>(K.sum_sq(qb));
+    const real qb6 = sqrt(sq);
+    const real ci = qb6 > real(0) ? inv_D / (n_real<real>(s) * qb6) : real(0);
+    K.get(kw);
+    real bq = real(0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        b[c] = ci * kw[c] * qb[c];
+        bq += b[c] * qb[c];
+    }
+    const real beta = group4_sum<real>(bq);
+    if (ok) {
+        if (l == 3) b[1] = beta;  // slot 13
+        store_b(s, i, l, o, b);
+        if (l == 0) R<real>(s.qb6)[i] = qb6;
+    }
+}
+
+template <typename real>
+__device__ __forceinline__ void cv_avg(const Sys &s, Blk k)
+{
+    const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_avg_group<real>(s, g);
+}
+
+// At 1M atoms: 10 blocks per SM (48 registers) 145 us, 12 (40) 154 us.
+template <typename real>
+constexpr int kAvgBlocks = sizeof(real) == 4 ? 10 : 0;
+
+template <typename real>
+__global__ void __launch_bounds__(kRowThreads, kAvgBlocks<real>) k_cv_avg(Sys s) { cv_avg<real>(s, own_blk()); }
+
+template <typename real>
+__global__ void __launch_bounds__(kRowThreads, kAvgBlocks<real>) kb_cv_avg(BatchView v)
+{
+    Blk k;
+    const Sys &s = v.sys[batch_system(v, k)];
+    cv_avg<real>(s, k);
+}
+
+// a7: g_m(k) = b_m(k) + sum_i w_ik b_m(i) ; h = g / W ; record h holds h_m
+// (0..12) and gamma_k = h(k).q(k) + beta_k (slot 13).
+//
 // Reduce-scatter of four values over the four lanes of this thread's group:
 // lane l returns the group sum of v[l].  The shuffle masks name the group
 // alone, so groups of one warp may run different trip counts.
@@ -715,50 +735,11 @@ __device__ __forceinline__ real group4_reduce_scatter(const real v[4], int l)
     return (hi1 ? a1 : a0) + __shfl_xor_sync(mask, hi1 ? a0 : a1, 1);
 }
 
+// h and gamma from the gathered sum (acc), the atom's own b (o) and q.
 template <typename real>
-__device__ __forceinline__ void adjoint_group(const Sys &s, int g)
+__device__ __forceinline__ void store_h(const Sys &s, int i, int l, bool ok, const real acc[4], const real o[4],
+                                        const real q[4])
 {
-    // lane l owns components 4l .. 4l + 3; record b holds b_m (0..12), beta (13)
-    const int i = g * kAtoms4 + (threadIdx.x / kG4), l = threadIdx.x & (kG4 - 1);
-    const bool ok = i < s.n;
-    const real *bb = R<real>(s.b);
-    real acc[4] = {real(0), real(0), real(0), real(0)};
-    real o[4] = {real(0), real(0), real(0), real(0)}, q[4] = {real(0), real(0), real(0), real(0)};
-    if (ok) {
-        load4<real>(bb, i, l, o);
-        load4<real>(R<real>(s.q), i, l, q);
-        const int nn = s.nn[i];
-        const JW<real> *jwrow = reinterpret_cast<const JW<real> *>(s.wl) + (size_t)i * s.max_nb;
-        // with each gathered b_j also the half b_j.q_i of the pair's cross
-        // term b_i.q_j + b_j.q_i in ds2/dw (a8), stored per entry: the force
-        // pass adds the halves of entry ij and its mirror ji.  Entries go
-        // four at a time; a reduce-scatter over the group leaves entry
-        // k0 + l's sum in lane l, so the group stores 16 contiguous bytes.
-        real *crow = R<real>(s.cross) + (size_t)i * s.max_nb;
-        for (int k0 = 0; k0 < nn; k0 += 4) {
-            JW<real> e4[4];
-            load_jw2<real>(jwrow, k0, e4[0], e4[1]);
-            load_jw2<real>(jwrow, k0 + 2, e4[2], e4[3]);
-            real p[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                p[u] = real(0);
-                if (k0 + u < nn) {
-                    const JW<real> e = e4[u];
-                    const real w = e.w;
-                    real x[4];
-                    load4<real>(bb, e.j, l, x);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        acc[c] += w * x[c];
-                        if (4 * l + c < kNY) p[u] += x[c] * q[c];
-                    }
-                }
-            }
-            const real t = group4_reduce_scatter<real>(p, l);
-            if (k0 + l < nn) crow[k0 + l] = t;
-        }
-    }
     real h[4] = {real(0), real(0), real(0), real(0)};
     real alpha = real(0), beta = real(0);
     if (ok) {
@@ -782,131 +763,159 @@ __device__ __forceinline__ void adjoint_group(const Sys &s, int g)
     }
 }
 
+// With each gathered record also the pair's cross term b_i.q_j + b_j.q_i of
+// ds2/dw (a8), stored per entry: the neighbour's q lies beside its b, so it
+// costs half a line and eight multiply-adds, and the force pass needs nothing
+// from the mirror entry.  Two chains, added last: both ends of a pair get the
+// same bits.  Entries go four at a time; a reduce-scatter over the group
+// leaves entry k0 + l's sum in lane l, so the group stores 16 contiguous
+// bytes.
+__device__ __forceinline__ void adjoint_group(const Sys &s, int g, float)
+{
+    const int i = g * kRowAtoms + (threadIdx.x / kG4), l = threadIdx.x & (kG4 - 1);
+    const bool ok = i < s.n;
+    const float *qb = R<float>(s.b);
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, o[4] = {0.0f, 0.0f, 0.0f, 0.0f}, q[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (ok) {
+        load_qb(qb, i, l, q, o);
+        const int nn = s.nn[i];
+        const JW<float> *jwrow = reinterpret_cast<const JW<float> *>(s.wl) + (size_t)i * s.max_nb;
+        float *crow = R<float>(s.cross) + (size_t)i * s.max_nb;
+        for (int k0 = 0; k0 < nn; k0 += 4) {
+            JW<float> e4[4];
+            load_jw2<float>(jwrow, k0, e4[0], e4[1]);
+            load_jw2<float>(jwrow, k0 + 2, e4[2], e4[3]);
+            float p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                p[u] = 0.0f;
+                if (k0 + u < nn) {
+                    float xq[4], xb[4];
+                    load_qb(qb, e4[u].j, l, xq, xb);
+                    // slot 13: 0 in q beside beta in b; 14, 15: 0 in both
+                    float p1 = xq[0] * o[0], p2 = xb[0] * q[0];
+                    acc[0] += e4[u].w * xb[0];
+#pragma unroll
+                    for (int c = 1; c < 4; ++c) {
+                        acc[c] += e4[u].w * xb[c];
+                        p1 = fmaf(xq[c], o[c], p1);
+                        p2 = fmaf(xb[c], q[c], p2);
+                    }
+                    p[u] = p1 + p2;
+                }
+            }
+            const float t = group4_reduce_scatter<float>(p, l);
+            if (k0 + l < nn) crow[k0 + l] = t;
+        }
+    }
+    store_h<float>(s, i, l, ok, acc, o, q);
+}
+
+// FP64: the half b_j.q_i of the cross term per entry; the pair pass adds the
+// halves of entry ij and its mirror ji.
+__device__ __forceinline__ void adjoint_group(const Sys &s, int g, double)
+{
+    const int i = g * kRowAtoms + (threadIdx.x / kG4), l = threadIdx.x & (kG4 - 1);
+    const bool ok = i < s.n;
+    const double *bb = R<double>(s.b);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, o[4] = {0.0, 0.0, 0.0, 0.0}, q[4] = {0.0, 0.0, 0.0, 0.0};
+    if (ok) {
+        load4<double>(bb, i, l, o);
+        load4<double>(R<double>(s.q), i, l, q);
+        const int nn = s.nn[i];
+        const JW<double> *jwrow = reinterpret_cast<const JW<double> *>(s.wl) + (size_t)i * s.max_nb;
+        double *crow = R<double>(s.cross) + (size_t)i * s.max_nb;
+        for (int k0 = 0; k0 < nn; k0 += 4) {
+            JW<double> e4[4];
+            load_jw2<double>(jwrow, k0, e4[0], e4[1]);
+            load_jw2<double>(jwrow, k0 + 2, e4[2], e4[3]);
+            double p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                p[u] = 0.0;
+                if (k0 + u < nn) {
+                    double x[4];
+                    load4<double>(bb, e4[u].j, l, x);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[c] += e4[u].w * x[c];
+                        if (4 * l + c < kNY) p[u] += x[c] * q[c];
+                    }
+                }
+            }
+            const double t = group4_reduce_scatter<double>(p, l);
+            if (k0 + l < nn) crow[k0 + l] = t;
+        }
+    }
+    store_h<double>(s, i, l, ok, acc, o, q);
+}
+
 template <typename real>
 __device__ __forceinline__ void adjoint(const Sys &s, Blk k)
 {
-    const int groups = (s.n + kAtoms4 - 1) / kAtoms4;
-    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) adjoint_group<real>(s, g);
+    const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) adjoint_group(s, g, real(0));
 }
 
-// Resident blocks per SM the adjoint is compiled for: 12 in FP32 (40
-// registers, no spill; measured 163 against 183 us at 1M atoms with the
-// default 47 registers and 10 blocks), unconstrained in FP64.
+// Resident blocks per SM the adjoint is compiled for (none in FP64): at 1M
+// atoms 12 (40 registers) 200 us, 10 (48) 214 us.  Blocks of 256 / 512 / 1024
+// threads 202 / 206 / 230 us: the neighbours' records are found in L2 either
+// way, and small blocks balance better.
 template <typename real>
 constexpr int kAdjointBlocks = sizeof(real) == 4 ? 12 : 0;
 
 template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms, kAdjointBlocks<real>) k_adjoint(Sys s) { adjoint<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) k_adjoint(Sys s) { adjoint<real>(s, own_blk()); }
 
 template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms, kAdjointBlocks<real>) kb_adjoint(BatchView v)
+__global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) kb_adjoint(BatchView v)
 {
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     adjoint<real>(s, k);
 }
 
-// a8, pass 1: for every unordered pair, from the row of its lower index i
-// (entries k < nh_i, j > i), G_ij = V1 ds1/dd + V2 ds2/dd at d = r_j - r_i,
-// stored in the pair's slot.  Each pair is evaluated once.
+// a8: G_ij = V1 ds1/dd + V2 ds2/dd at d = r_j - r_i:
 //   ds2/dw = (h_i + h_j).Y - gamma_i - gamma_j + b_i.q_j + b_j.q_i
 //   ds2/dd = ds2/dw w' d/r + w sum_m (h_i + h_j)_m dY_m/dd
 //   ds1/dd = (2/N) w' d/r [unlike]
-// The pair slots are a stream (written once, read once by pass 2): stored
-// and loaded evict-first, so they leave the gathered records in L2.
-template <typename real>
-__device__ __forceinline__ void store_pair_force(real *slot, real fx, real fy, real fz);
-template <>
-__device__ __forceinline__ void store_pair_force<float>(float *slot, float fx, float fy, float fz)
-{
-    __stcs(reinterpret_cast<float4 *>(slot), make_float4(fx, fy, fz, 0.0f));
-}
-template <>
-__device__ __forceinline__ void store_pair_force<double>(double *slot, double fx, double fy, double fz)
-{
-    __stcs(reinterpret_cast<double2 *>(slot), make_double2(fx, fy));
-    __stcs(reinterpret_cast<double2 *>(slot) + 1, make_double2(fz, 0.0));
-}
-
-// Pair-parallel: the half-row entries (k < nh_i) of a chunk of kPairChunk
-// atoms are numbered in atom order and thread t of the block evaluates
-// entries t, t + blockDim, ...: every lane has a pair while the chunk lasts,
-// whatever the spread of the atoms' half-row lengths.
+// and F_i = sum_j G_ij over the whole row (G_ji = -G_ij).
 //
-// G_ij goes to the slot of entry k in i's row and -G_ij to the slot of i in
-// the j < i part of j's row (rows are symmetric: the neighbour predicate is),
-// so pass 2 sums each atom's own slots in row order.
-constexpr int kPairChunk = 32;
-
-template <typename real, bool kVir>
-__device__ __forceinline__ void pair_force(const Sys &s, int i, int k, real cn_fac, real V2, RunSum<real> &vx,
-                                           RunSum<real> &vy, RunSum<real> &vz)
+// One pair's G (without a CN part, radial is V2 ds2/dw w' alone).
+template <typename real>
+__device__ __forceinline__ Vec3<real> pair_gradient(const Vec3<real> &d, real inv_r, real w, real dw, real cn_radial,
+                                                    real V2, real cross, const real hi[kRec], const real hj[kRec])
 {
-    Vec3<real> d;
-    real inv_r, w, dw;
-    bool cn;
-    int j;
-    unsigned vm;
-    cached_geometry<real, true>(s, (size_t)i * s.max_nb + k, d, inv_r, w, dw, cn, j, vm);
-    // the slot of i in j's exact row: with mirror slots, the exact entries
-    // of j's Verlet row before i's position vm there (one 2 B load);
-    // otherwise a search of the j < i part [nh_j, nn_j) of j's row, four
-    // entries per load
-    int kk = -1;
-    if (s.mirror) {
-        const unsigned e = s.vround[(size_t)j * s.vround_stride + (vm >> 3)];
-        kk = (int)(e & 0xffu) + __popc((e >> 8) & ((1u << (vm & 7u)) - 1u));
-    } else {
-        const int nhj = s.nh[j], nnj = s.nn[j];
-        const int *rj = nbr_row(s, j);
-        for (int b = nhj & ~3; b < nnj && kk < 0; b += 4) {
-            const int4 v = *reinterpret_cast<const int4 *>(rj + b);
-            if (v.x == i && b >= nhj) kk = b;
-            else if (v.y == i && b + 1 >= nhj && b + 1 < nnj) kk = b + 1;
-            else if (v.z == i && b + 2 >= nhj && b + 2 < nnj) kk = b + 2;
-            else if (v.w == i && b + 3 >= nhj && b + 3 < nnj) kk = b + 3;
-        }
-    }
-    if (kk < 0 || kk >= s.max_nb) {
-        set_err(s, kErrInternal);  // rows not symmetric: never expected
-        return;
-    }
     const real ux = d.x * inv_r, uy = d.y * inv_r, uz = d.z * inv_r;
-    real radial = cn ? cn_fac * dw : real(0);
-    real fx = real(0), fy = real(0), fz = real(0);
-    if (s.ncv == 2) {
-        const real *hh = R<real>(s.h), *cc = R<real>(s.cross);
-        // cross term b_i.q_j + b_j.q_i: the halves the adjoint pass stored
-        // in entry ij (b_j.q_i) and in its mirror ji (b_i.q_j)
-        real t = cc[(size_t)i * s.max_nb + k] + cc[(size_t)j * s.max_nb + kk];
-        real hi[kRec], hj[kRec];
-        load_rec<real>(hh, i, hi);
-        load_rec<real>(hh, j, hj);
-        t -= hi[13] + hj[13];
-        real hs[kNY];
+    real t = cross - (hi[13] + hj[13]);
+    real hs[kNY];
 #pragma unroll
-        for (int m = 0; m < kNY; ++m) hs[m] = hi[m] + hj[m];
-        // (h_i + h_j).Y and its transverse gradient; the w Y term's gradient
-        // is w times it
-        real gY[3];
-        t += ylm13_dot_grad<real>(ux, uy, uz, inv_r, hs, gY);
-        radial += V2 * t * dw;
-        const real vw = V2 * w;
-        fx = vw * gY[0];
-        fy = vw * gY[1];
-        fz = vw * gY[2];
+    for (int m = 0; m < kNY; ++m) hs[m] = hi[m] + hj[m];
+    // (h_i + h_j).Y and its transverse gradient; the w Y term's gradient
+    // is w times it
+    real gY[3];
+    t += ylm13_dot_grad<real>(ux, uy, uz, inv_r, hs, gY);
+    const real radial = cn_radial + V2 * t * dw, vw = V2 * w;
+    return Vec3<real>{vw * gY[0] + radial * ux, vw * gY[1] + radial * uy, vw * gY[2] + radial * uz};
+}
+
+// The chain-rule factors of the two CVs, 2 V1 scale / N and V2 scale, formed
+// once per block: an FP64 chain is long and its pipe narrow on this part.
+template <typename real>
+__device__ __forceinline__ void chain_factors(const Sys &s, real fac[2])
+{
+    if (threadIdx.x == 0) {
+        fac[0] = (real)(s.scal[kDV0] * s.fscale * 2.0 / s.n);
+        fac[1] = s.ncv == 2 ? (real)(s.scal[kDV1] * s.fscale) : real(0);
     }
-    fx += radial * ux;
-    fy += radial * uy;
-    fz += radial * uz;
-    if (kVir) {  // (dV/dd)_a d_a of this pair
-        vx.add(fx * d.x);
-        vy.add(fy * d.y);
-        vz.add(fz * d.z);
-    }
-    real *pf = R<real>(s.pairF);
-    store_pair_force<real>(pf + ((size_t)i * s.max_nb + k) * 4, fx, fy, fz);
-    store_pair_force<real>(pf + ((size_t)j * s.max_nb + kk) * 4, -fx, -fy, -fz);
+    __syncthreads();
+}
+
+template <typename real>
+__device__ __forceinline__ void put_force(const Sys &s, int i, int comp, real f)
+{
+    float *o = s.F_out + 3 * (size_t)s.perm[i] + comp;
+    *o = s.accumulate ? *o + (float)f : (float)f;
 }
 
 // The bias virial W_a = sum_pairs (dV/dd)_a d_a, which a barostat needs: it
@@ -917,8 +926,9 @@ __device__ __forceinline__ void pair_force(const Sys &s, int i, int k, real cn_f
 template <typename real>
 __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real> &vy, RunSum<real> &vz)
 {
-    constexpr int kW = kBlockAtoms / 32;
-    __shared__ double sh[3][kW];
+    constexpr int kMaxW = (kRowThreads > kBlockAtoms ? kRowThreads : kBlockAtoms) / 32;
+    const int kW = blockDim.x >> 5;
+    __shared__ double sh[3][kMaxW];
     __shared__ bool am_last;
     if (3 * k.nb > s.part_stride) {  // never with the grids used; refuse rather than overrun
         if (k.b == 0 && threadIdx.x == 0) set_err(s, kErrInternal);
@@ -981,29 +991,190 @@ __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real
     }
 }
 
+// FP32, two CVs: every atom walks its own row, four lanes an atom, one entry
+// per lane, so each pair is evaluated at both ends.  That repeats the pair's
+// arithmetic but needs no slots for the pair forces, no search for i in j's
+// row and no pass to add the slots up: what bound the half-row form was its
+// scattered line accesses (per pair four for h_j, one each for the mirror
+// entry's place, its cross half and its force slot), and its 32 B of slots
+// per entry were most of the step's DRAM traffic.  Bound by the L1's
+// wavefronts (68% at 262,144 atoms) and instruction issue (54%).
+// Measured against the half-row pass and the slot sums: 1M atoms 300 -> 268
+// us, and the forward pass, without the mirror records, 309 -> 271 us (and
+// 200 us less after a rebuild); 27,648 atoms 36.4 -> 14.3 us.
+template <bool kVir>
+__device__ __forceinline__ void force_rows(const Sys &s, Blk k)
+{
+    __shared__ float fac[2];
+    chain_factors<float>(s, fac);
+    const float cn_fac = fac[0], V2 = fac[1];
+    const int l = threadIdx.x & (kG4 - 1);
+    const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
+    RunSum<float> vx, vy, vz;
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) {
+        const int i = g * kRowAtoms + (threadIdx.x / kG4);
+        float fx = 0.0f, fy = 0.0f, fz = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
+        if (i < s.n) {
+            const int nn = s.nn[i];
+            const float *hh = R<float>(s.h), *crow = R<float>(s.cross) + (size_t)i * s.max_nb;
+            float hi[kRec];
+            load_rec<float>(hh, i, hi);
+            for (int e = l; e < nn; e += kG4) {
+                Vec3<float> d;
+                float inv_r, w, dw;
+                bool cn;
+                int j;
+                cached_geometry<float, true>(s, (size_t)i * s.max_nb + e, d, inv_r, w, dw, cn, j);
+                float hj[kRec];
+                load_rec<float>(hh, j, hj);
+                const Vec3<float> G =
+                    pair_gradient<float>(d, inv_r, w, dw, cn ? cn_fac * dw : 0.0f, V2, __ldcs(crow + e), hi, hj);
+                fx += G.x;
+                fy += G.y;
+                fz += G.z;
+                if (kVir) {
+                    wx += G.x * d.x;
+                    wy += G.y * d.y;
+                    wz += G.z * d.z;
+                }
+            }
+        }
+        fx = group4_sum<float>(fx);
+        fy = group4_sum<float>(fy);
+        fz = group4_sum<float>(fz);
+        if (i < s.n && l < 3) put_force<float>(s, i, l, l == 0 ? fx : (l == 1 ? fy : fz));
+        if (kVir) {  // each pair is met at both ends
+            vx.add(0.5f * wx);
+            vy.add(0.5f * wy);
+            vz.add(0.5f * wz);
+        }
+    }
+    if (kVir) virial_finish<float>(s, k, vx, vy, vz);
+}
+
+// Resident blocks per SM: at 1M atoms 9 (56 registers) 268 us, 8 (64) 279 us;
+// the virial's instance is left alone.
+template <bool kVir>
+constexpr int kForceBlocks = kVir ? 0 : 9;
+
+template <bool kVir>
+__global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) k_force_rows(Sys s) { force_rows<kVir>(s, own_blk()); }
+
+template <bool kVir>
+__global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) kb_force_rows(BatchView v)
+{
+    Blk k;
+    const Sys &s = v.sys[batch_system(v, k)];
+    force_rows<kVir>(s, k);
+}
+
+// One CV: the CV pass left each atom's sum_j w' d / r, so the force is a
+// factor away.  One thread per atom.
 template <typename real, bool kVir>
+__device__ __forceinline__ void force_cn(const Sys &s, Blk k)
+{
+    __shared__ real fac[2];
+    chain_factors<real>(s, fac);
+    const real f = fac[0];
+    RunSum<real> vx, vy, vz;
+    for (int i = k.b * blockDim.x + threadIdx.x; i < s.n; i += k.nb * blockDim.x) {
+        const real *r = R<real>(s.q) + (size_t)i * kCnRec;
+        put_force<real>(s, i, 0, f * r[0]);
+        put_force<real>(s, i, 1, f * r[1]);
+        put_force<real>(s, i, 2, f * r[2]);
+        if (kVir) {  // each pair is met at both ends
+            const real hf = real(0.5) * f;
+            vx.add(hf * r[3]);
+            vy.add(hf * r[4]);
+            vz.add(hf * r[5]);
+        }
+    }
+    if (kVir) virial_finish<real>(s, k, vx, vy, vz);
+}
+
+template <typename real, bool kVir>
+__global__ void __launch_bounds__(kBlockAtoms) k_force_cn(Sys s) { force_cn<real, kVir>(s, own_blk()); }
+
+template <typename real, bool kVir>
+__global__ void __launch_bounds__(kBlockAtoms) kb_force_cn(BatchView v)
+{
+    Blk k;
+    const Sys &s = v.sys[batch_system(v, k)];
+    force_cn<real, kVir>(s, k);
+}
+
+// FP64, two CVs, pass 1: each unordered pair once (its ~200 FP64 operations
+// bound this form, so they are not repeated), from the row of its lower index
+// i (entries k < nh_i, j > i): G_ij into the slot of entry k in i's row and
+// -G_ij into the slot of i in the j < i part of j's row (rows are symmetric:
+// the neighbour predicate is), found by a search of that part.  Pass 2 sums
+// each atom's own slots in row order.  The slots are a stream (written once,
+// read once): stored and loaded evict-first.
+//
+// Pair-parallel: the half-row entries of a chunk of atoms are numbered in
+// atom order and the lanes of a warp take them in turn: every lane has a pair
+// while the chunk lasts, whatever the spread of the half-row lengths.
+template <bool kVir>
+__device__ __forceinline__ void pair_force(const Sys &s, int i, int k, double cn_fac, double V2, RunSum<double> &vx,
+                                           RunSum<double> &vy, RunSum<double> &vz)
+{
+    Vec3<double> d;
+    double inv_r, w, dw;
+    bool cn;
+    int j;
+    cached_geometry<double, true>(s, (size_t)i * s.max_nb + k, d, inv_r, w, dw, cn, j);
+    int kk = -1;
+    const int nhj = s.nh[j], nnj = s.nn[j];
+    const int *rj = nbr_row(s, j);
+    for (int b = nhj & ~3; b < nnj && kk < 0; b += 4) {  // four entries per load
+        const int4 v = *reinterpret_cast<const int4 *>(rj + b);
+        if (v.x == i && b >= nhj) kk = b;
+        else if (v.y == i && b + 1 >= nhj && b + 1 < nnj) kk = b + 1;
+        else if (v.z == i && b + 2 >= nhj && b + 2 < nnj) kk = b + 2;
+        else if (v.w == i && b + 3 >= nhj && b + 3 < nnj) kk = b + 3;
+    }
+    if (kk < 0 || kk >= s.max_nb) {
+        set_err(s, kErrInternal);  // rows not symmetric: never expected
+        return;
+    }
+    const double *hh = R<double>(s.h), *cc = R<double>(s.cross);
+    double hi[kRec], hj[kRec];
+    load_rec<double>(hh, i, hi);
+    load_rec<double>(hh, j, hj);
+    // cross term b_i.q_j + b_j.q_i: the halves the adjoint pass stored
+    // in entry ij (b_j.q_i) and in its mirror ji (b_i.q_j)
+    const double cross = cc[(size_t)i * s.max_nb + k] + cc[(size_t)j * s.max_nb + kk];
+    const Vec3<double> G = pair_gradient<double>(d, inv_r, w, dw, cn ? cn_fac * dw : 0.0, V2, cross, hi, hj);
+    if (kVir) {  // (dV/dd)_a d_a of this pair
+        vx.add(G.x * d.x);
+        vy.add(G.y * d.y);
+        vz.add(G.z * d.z);
+    }
+    double2 *pi = reinterpret_cast<double2 *>(s.pairF) + 2 * ((size_t)i * s.max_nb + k);
+    double2 *pj = reinterpret_cast<double2 *>(s.pairF) + 2 * ((size_t)j * s.max_nb + kk);
+    __stcs(pi, make_double2(G.x, G.y));
+    __stcs(pi + 1, make_double2(G.z, 0.0));
+    __stcs(pj, make_double2(-G.x, -G.y));
+    __stcs(pj + 1, make_double2(-G.z, 0.0));
+}
+
+template <bool kVir>
 __device__ __forceinline__ void force_pairs(const Sys &s, Blk k)
 {
-    // the chain-rule factors of the two CVs, once per block: an FP64 chain is
-    // long and its pipe narrow on this part, so no thread repeats it
-    __shared__ real fac[2];
-    if (threadIdx.x == 0) {
-        fac[0] = (real)(s.scal[kDV0] * s.fscale * 2.0 / s.n);
-        fac[1] = s.ncv == 2 ? (real)(s.scal[kDV1] * s.fscale) : real(0);
-    }
-    __syncthreads();
-    const real cn_fac = fac[0], V2 = fac[1];
-    // each warp takes its own chunk of 32 atoms (a block of kBlockAtoms/32
-    // warps is one work item, one per 128 atoms of the grid): no barrier
+    __shared__ double fac[2];
+    chain_factors<double>(s, fac);
+    const double cn_fac = fac[0], V2 = fac[1];
+    // each warp takes its own chunk of atoms (a block is one work item): no barrier
     constexpr int kWarps = kBlockAtoms / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int items = (s.n + kPairChunk * kWarps - 1) / (kPairChunk * kWarps);
-    RunSum<real> vx, vy, vz;
+    const int chunk = pair_chunk(s.n);
+    const int items = (s.n + chunk * kWarps - 1) / (chunk * kWarps);
+    RunSum<double> vx, vy, vz;
     for (int it = 0, g; (g = work_item(k, it)) < items; ++it) {
-        const int i0 = (g * kWarps + warp) * kPairChunk;
+        const int i0 = (g * kWarps + warp) * chunk;
         if (i0 >= s.n) continue;  // warp-uniform
         // inclusive prefix of the half-row lengths, one lane per atom
-        int off = i0 + lane < s.n ? s.nh[i0 + lane] : 0;
+        int off = lane < chunk && i0 + lane < s.n ? s.nh[i0 + lane] : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, off, o);
@@ -1022,96 +1193,55 @@ __device__ __forceinline__ void force_pairs(const Sys &s, Blk k)
             }
             const int prev = __shfl_sync(0xffffffffu, off, lo > 0 ? lo - 1 : 0);  // every lane shuffles
             const int start = lo > 0 ? prev : 0;
-            if (p < T) pair_force<real, kVir>(s, i0 + lo, p - start, cn_fac, V2, vx, vy, vz);
+            if (p < T) pair_force<kVir>(s, i0 + lo, p - start, cn_fac, V2, vx, vy, vz);
         }
     }
-    if (kVir) virial_finish<real>(s, k, vx, vy, vz);
+    if (kVir) virial_finish<double>(s, k, vx, vy, vz);
 }
 
-template <typename real, bool kVir = false>
-__global__ void __launch_bounds__(kBlockAtoms) k_force_pairs(Sys s) { force_pairs<real, kVir>(s, own_blk()); }
+template <bool kVir>
+__global__ void __launch_bounds__(kBlockAtoms) k_force_pairs(Sys s) { force_pairs<kVir>(s, own_blk()); }
 
-template <typename real, bool kVir = false>
+template <bool kVir>
 __global__ void __launch_bounds__(kBlockAtoms) kb_force_pairs(BatchView v)
 {
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
-    force_pairs<real, kVir>(s, k);
+    force_pairs<kVir>(s, k);
 }
 
-template <typename real>
-__device__ __forceinline__ void load_pair_force(const real *slot, real &fx, real &fy, real &fz);
-template <>
-__device__ __forceinline__ void load_pair_force<float>(const float *slot, float &fx, float &fy, float &fz)
-{
-    const float4 t = __ldcs(reinterpret_cast<const float4 *>(slot));
-    fx = t.x;
-    fy = t.y;
-    fz = t.z;
-}
-template <>
-__device__ __forceinline__ void load_pair_force<double>(const double *slot, double &fx, double &fy, double &fz)
-{
-    const double2 a = __ldcs(reinterpret_cast<const double2 *>(slot));
-    const double2 b = __ldcs(reinterpret_cast<const double2 *>(slot) + 1);
-    fx = a.x;
-    fy = a.y;
-    fz = b.x;
-}
-
-// a8, pass 2: F_i = sum_{j > i} G_ij - sum_{j < i} G_ji: the slots of i's
-// row hold exactly those terms (pass 1 wrote both ends of every pair), summed
-// in row order per lane and a fixed shuffle tree across lanes: deterministic,
-// no atomics, and contiguous reads.
-template <typename real>
-__device__ __forceinline__ void force_gather_group(const Sys &s, const AtomLane a, float *F, int accumulate)
-{
-    real fx = real(0), fy = real(0), fz = real(0);
-    if (a.ok) {
-        const int nn = s.nn[a.i];
-        const real *pf = R<real>(s.pairF) + (size_t)a.i * s.max_nb * 4;
-        for (int k = a.l; k < nn; k += kG) {
-            real gx, gy, gz;
-            load_pair_force<real>(pf + 4 * (size_t)k, gx, gy, gz);
-            fx += gx;
-            fy += gy;
-            fz += gz;
-        }
-    }
-    fx = group_sum<real>(fx);
-    fy = group_sum<real>(fy);
-    fz = group_sum<real>(fz);
-    if (a.ok && a.l == 0) {
-        float *o = F + 3 * (size_t)s.perm[a.i];
-        if (accumulate) {
-            o[0] += (float)fx;
-            o[1] += (float)fy;
-            o[2] += (float)fz;
-        } else {
-            o[0] = (float)fx;
-            o[1] = (float)fy;
-            o[2] = (float)fz;
-        }
-    }
-}
-
-template <typename real>
+// Pass 2: the slots of i's row summed in row order per lane and by a fixed
+// shuffle tree across lanes.
 __device__ __forceinline__ void force_gather(const Sys &s, Blk k)
 {
     const int groups = group_grid(s.n);
-    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it)
-        force_gather_group<real>(s, atom_lane_at(s, g), s.F_out, s.accumulate);
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) {
+        const AtomLane a = atom_lane_at(s, g);
+        double fx = 0.0, fy = 0.0, fz = 0.0;
+        if (a.ok) {
+            const int nn = s.nn[a.i];
+            const double2 *pf = reinterpret_cast<const double2 *>(s.pairF) + 2 * (size_t)a.i * s.max_nb;
+            for (int e = a.l; e < nn; e += kG) {
+                const double2 u = __ldcs(pf + 2 * e), v = __ldcs(pf + 2 * e + 1);
+                fx += u.x;
+                fy += u.y;
+                fz += v.x;
+            }
+        }
+        fx = group_sum<double>(fx);
+        fy = group_sum<double>(fy);
+        fz = group_sum<double>(fz);
+        if (a.ok && a.l < 3) put_force<double>(s, a.i, a.l, a.l == 0 ? fx : (a.l == 1 ? fy : fz));
+    }
 }
 
-template <typename real>
-__global__ void __launch_bounds__(kBlockAtoms) k_force_gather(Sys s) { force_gather<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms) k_force_gather(Sys s) { force_gather(s, own_blk()); }
 
-template <typename real>
 __global__ void __launch_bounds__(kBlockAtoms) kb_force_gather(BatchView v)
 {
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
-    force_gather<real>(s, k);
+    force_gather(s, k);
 }
 
 template <typename real>
@@ -1145,91 +1275,118 @@ void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st)
 
 void launch_cv_avg(const Sys &s, int fp64, cudaStream_t st)
 {
+    const int nb = grid_blocks(s, GK_ROWS, 0);
     if (fp64)
-        k_cv_avg<double><<<grid_blocks(s, GK_CV, 0), kBlockAtoms, 0, st>>>(s);
+        k_cv_avg<double><<<nb, kRowThreads, 0, st>>>(s);
     else
-        k_cv_avg<float><<<grid_blocks(s, GK_CV, 0), kBlockAtoms, 0, st>>>(s);
+        k_cv_avg<float><<<nb, kRowThreads, 0, st>>>(s);
 }
 
 void launch_cv_sum(const Sys &s, int fp64, cudaStream_t st)
 {
+    const int nb = grid_blocks(s, GK_SUM, 0);
     if (fp64)
-        k_cv_sum<double><<<grid_blocks(s, GK_SUM, 0), kSumThreads, 0, st>>>(s);
+        k_cv_sum<double><<<nb, kSumThreads, 0, st>>>(s);
     else
-        k_cv_sum<float><<<grid_blocks(s, GK_SUM, 0), kSumThreads, 0, st>>>(s);
+        k_cv_sum<float><<<nb, kSumThreads, 0, st>>>(s);
 }
 
 void launch_adjoint(const Sys &s, int fp64, cudaStream_t st)
 {
+    const int nb = grid_blocks(s, GK_ROWS, 0);
     if (fp64)
-        k_adjoint<double><<<grid_blocks(s, GK_ATOM32, 0), kBlockAtoms, 0, st>>>(s);
+        k_adjoint<double><<<nb, kRowThreads, 0, st>>>(s);
     else
-        k_adjoint<float><<<grid_blocks(s, GK_ATOM32, 0), kBlockAtoms, 0, st>>>(s);
+        k_adjoint<float><<<nb, kRowThreads, 0, st>>>(s);
 }
 
-void launch_force_pairs(const Sys &s, int fp64, double scale, cudaStream_t st)
+namespace {
+
+// The force pass of one system (Arg = Sys) or a batch (BatchView).
+template <typename Arg>
+using Kern = void (*)(Arg);
+
+Kern<Sys> force_kernel(int fp64, int ncv, int virial)
 {
-    Sys t = s;
-    t.fscale = scale;
-    const int nb = grid_blocks(s, GK_ATOM128, 0);
-    if (fp64) {
-        if (s.virial) k_force_pairs<double, true><<<nb, kBlockAtoms, 0, st>>>(t);
-        else k_force_pairs<double><<<nb, kBlockAtoms, 0, st>>>(t);
-    } else {
-        if (s.virial) k_force_pairs<float, true><<<nb, kBlockAtoms, 0, st>>>(t);
-        else k_force_pairs<float><<<nb, kBlockAtoms, 0, st>>>(t);
+    if (ncv == 1) {
+        if (fp64) return virial ? k_force_cn<double, true> : k_force_cn<double, false>;
+        return virial ? k_force_cn<float, true> : k_force_cn<float, false>;
     }
+    if (fp64) return virial ? k_force_pairs<true> : k_force_pairs<false>;
+    return virial ? k_force_rows<true> : k_force_rows<false>;
 }
 
-void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st)
+int force_threads(int fp64, int ncv) { return ncv == 2 && !fp64 ? kRowThreads : kBlockAtoms; }
+
+Kern<BatchView> batch_force_kernel(int fp64, int ncv, int virial)
+{
+    if (ncv == 1) {
+        if (fp64) return virial ? kb_force_cn<double, true> : kb_force_cn<double, false>;
+        return virial ? kb_force_cn<float, true> : kb_force_cn<float, false>;
+    }
+    if (fp64) return virial ? kb_force_pairs<true> : kb_force_pairs<false>;
+    return virial ? kb_force_rows<true> : kb_force_rows<false>;
+}
+
+}  // namespace
+
+void launch_forces(const Sys &s, int fp64, float *F, int accumulate, double scale, cudaStream_t st)
 {
     Sys t = s;
     t.F_out = F;
     t.accumulate = accumulate;
-    if (fp64)
-        k_force_gather<double><<<group_grid(s.n), kBlockAtoms, 0, st>>>(t);
-    else
-        k_force_gather<float><<<group_grid(s.n), kBlockAtoms, 0, st>>>(t);
+    t.fscale = scale;
+    force_kernel(fp64, s.ncv, s.virial)<<<grid_blocks(t, GK_FORCE, 0), force_threads(fp64, s.ncv), 0, st>>>(t);
 }
 
-void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &cv, int cv_total,
-                     const BatchView &sums, int sum_total, int fp64, int ncv, cudaStream_t st)
+void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st)
+{
+    if (!pair_slots(s, fp64)) return;
+    Sys t = s;
+    t.F_out = F;
+    t.accumulate = accumulate;
+    k_force_gather<<<group_grid(s.n), kBlockAtoms, 0, st>>>(t);
+}
+
+void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &rows, int row_total, int fp64, int ncv,
+                     cudaStream_t st)
 {
     if (group_total <= 0) return;
     if (fp64) {
         kb_cv_fwd<double><<<group_total, kBlockAtoms, 0, st>>>(groups);
-        if (ncv == 2)
-            kb_cv_avg<double><<<cv_total, kBlockAtoms, 0, st>>>(cv);
-        else
-            kb_cv_sum<double><<<sum_total, kSumThreads, 0, st>>>(sums);
+        if (ncv == 2) kb_cv_avg<double><<<row_total, kRowThreads, 0, st>>>(rows);
     } else {
         kb_cv_fwd<float><<<group_total, kBlockAtoms, 0, st>>>(groups);
-        if (ncv == 2)
-            kb_cv_avg<float><<<cv_total, kBlockAtoms, 0, st>>>(cv);
-        else
-            kb_cv_sum<float><<<sum_total, kSumThreads, 0, st>>>(sums);
+        if (ncv == 2) kb_cv_avg<float><<<row_total, kRowThreads, 0, st>>>(rows);
     }
 }
 
-void launch_batch_force(const BatchView &groups, int group_total, const BatchView &adj, int adj_total,
-                        const BatchView &pairs, int pair_total, int fp64, int ncv, int virial, cudaStream_t st,
-                        int part)
+void launch_batch_sum(const BatchView &sums, int sum_total, int fp64, cudaStream_t st)
 {
-    if (group_total <= 0) return;
-    const bool adjoint = part != 2 && ncv == 2, forces = part != 1;
-    if (fp64) {
-        if (adjoint) kb_adjoint<double><<<adj_total, kBlockAtoms, 0, st>>>(adj);
-        if (!forces) return;
-        if (virial) kb_force_pairs<double, true><<<pair_total, kBlockAtoms, 0, st>>>(pairs);
-        else kb_force_pairs<double><<<pair_total, kBlockAtoms, 0, st>>>(pairs);
-        kb_force_gather<double><<<group_total, kBlockAtoms, 0, st>>>(groups);
-    } else {
-        if (adjoint) kb_adjoint<float><<<adj_total, kBlockAtoms, 0, st>>>(adj);
-        if (!forces) return;
-        if (virial) kb_force_pairs<float, true><<<pair_total, kBlockAtoms, 0, st>>>(pairs);
-        else kb_force_pairs<float><<<pair_total, kBlockAtoms, 0, st>>>(pairs);
-        kb_force_gather<float><<<group_total, kBlockAtoms, 0, st>>>(groups);
-    }
+    if (sum_total <= 0) return;
+    if (fp64)
+        kb_cv_sum<double><<<sum_total, kSumThreads, 0, st>>>(sums);
+    else
+        kb_cv_sum<float><<<sum_total, kSumThreads, 0, st>>>(sums);
+}
+
+void launch_batch_adjoint(const BatchView &rows, int total, int fp64, cudaStream_t st)
+{
+    if (total <= 0) return;
+    if (fp64)
+        kb_adjoint<double><<<total, kRowThreads, 0, st>>>(rows);
+    else
+        kb_adjoint<float><<<total, kRowThreads, 0, st>>>(rows);
+}
+
+int launch_batch_forces(const BatchView &force, int force_total, const BatchView &groups, int group_total, int fp64,
+                        int ncv, int virial, cudaStream_t st)
+{
+    if (force_total <= 0) return 0;
+    batch_force_kernel(fp64, ncv, virial)<<<force_total, force_threads(fp64, ncv), 0, st>>>(force);
+    if (!(fp64 && ncv == 2)) return 1;
+    kb_force_gather<<<group_total, kBlockAtoms, 0, st>>>(groups);
+    return 2;
 }
 
 // The gather kernels without shared memory prefer the SM's unified storage
@@ -1240,10 +1397,10 @@ void launch_batch_force(const BatchView &groups, int group_total, const BatchVie
 void configure_kernels()
 {
     const int l1 = cudaSharedmemCarveoutMaxL1;
+    cudaFuncSetAttribute(k_cv_avg<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
+    cudaFuncSetAttribute(kb_cv_avg<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
     cudaFuncSetAttribute(k_adjoint<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
-    cudaFuncSetAttribute(k_force_gather<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
     cudaFuncSetAttribute(kb_adjoint<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
-    cudaFuncSetAttribute(kb_force_gather<float>, cudaFuncAttributePreferredSharedMemoryCarveout, l1);
     cudaGetLastError();
 }
 
@@ -1259,8 +1416,7 @@ void launch_per_atom_out(const Sys &s, int fp64, double *out, cudaStream_t st)
 // arrays (pole-free, unnormalised):
 //   P_m^m = (2m-1)!!,  P_{m+1}^m = (2m+1) z P_m^m,
 //   P_l^m = ((2l-1) z P_{l-1}^m - (l+m-1) P_{l-2}^m) / (l-m);
-// every coefficient is a dyadic rational, exact in float32.  Weights
-// K_0 = 1, K_m = 2 (6-m)!/(6+m)!.
+// every coefficient is a dyadic rational, exact in float32.
 void set_ylm_constants(cudaStream_t st)
 {
     YlmConst h{};
@@ -1292,15 +1448,6 @@ void set_ylm_constants(cudaStream_t st)
             h.dpd[m][t] = cur[p] * p;
             h.dpf[m][t] = (float)(cur[p] * p);
         }
-        double fr = 1.0;  // (l-m)!/(l+m)!
-        for (int k = l - m + 1; k <= l + m; ++k) fr /= k;
-        const double K = m > 0 ? 2.0 * fr : 1.0;
-        const int slots[2] = {m == 0 ? 0 : 2 * m - 1, m == 0 ? 0 : 2 * m};
-        for (int q = 0; q < (m == 0 ? 1 : 2); ++q) {
-            h.kd[slots[q]] = K;
-            h.kf_hi[slots[q]] = (float)K;
-            h.kf_lo[slots[q]] = (float)(K - (double)(float)K);
-        }
     }
     cudaMemcpyToSymbolAsync(c_ylm, &h, sizeof(h), 0, cudaMemcpyHostToDevice, st);
 }
@@ -1321,12 +1468,15 @@ bool sys_kernel_cv(const void *func)
         (const void *)k_cv_sum<double>,
         (const void *)k_adjoint<float>,
         (const void *)k_adjoint<double>,
-        (const void *)k_force_pairs<float, false>,
-        (const void *)k_force_pairs<float, true>,
-        (const void *)k_force_pairs<double, false>,
-        (const void *)k_force_pairs<double, true>,
-        (const void *)k_force_gather<float>,
-        (const void *)k_force_gather<double>,
+        (const void *)k_force_rows<false>,
+        (const void *)k_force_rows<true>,
+        (const void *)k_force_cn<float, false>,
+        (const void *)k_force_cn<float, true>,
+        (const void *)k_force_cn<double, false>,
+        (const void *)k_force_cn<double, true>,
+        (const void *)k_force_pairs<false>,
+        (const void *)k_force_pairs<true>,
+        (const void *)k_force_gather,
     };
     for (const void *k : kernels)
         if (k == func) return true;

@@ -427,7 +427,7 @@ __device__ __forceinline__ void verlet_cell(const Sys &s, VerletWarpSmem &w, int
 }
 
 // End of a rebuild, run once by the last Verlet block to finish: the rows'
-// box becomes the reference, the rows are marked new, and the flag is
+// box becomes the reference, and the flag is
 // cleared for the next step (kept set when the skin is zero, so every step
 // rebuilds).
 __device__ __forceinline__ void finish_rebuild(const Sys &s, Blk k)
@@ -440,7 +440,6 @@ __device__ __forceinline__ void finish_rebuild(const Sys &s, Blk k)
     s.ticket[4] = 0u;
     *s.rebuilds += 1ull;
     for (int a = 0; a < 3; ++a) s.Lref[a] = s.Lhi[a];
-    if (s.mirror) *s.rows_fresh = 1;  // the next filter finds the mirror positions
     *s.flag = s.always_rebuild ? 1 : 0;
 }
 
@@ -554,8 +553,7 @@ __global__ void __launch_bounds__(kBlockAtoms) kb_verlet(BatchView v)
 
 // Pairs (i < j) in caller indices, for export: one thread per sorted atom,
 // entries with caller(i) < caller(j) appended through one counter.  Each
-// exact entry's j is read from its geometry tag (the exact rows of indices
-// are kept only without mirror slots).
+// exact entry's j is read from its geometry tag.
 template <typename real>
 __global__ void k_export_pairs(Sys s, long long *pairs, int *count)
 {
@@ -566,8 +564,7 @@ __global__ void k_export_pairs(Sys s, long long *pairs, int *count)
         Vec3<real> d;
         bool cn;
         int j;
-        unsigned vm;
-        load_geo<real>(s, (size_t)i * s.max_nb + k, d, cn, j, vm);
+        load_geo<real>(s, (size_t)i * s.max_nb + k, d, cn, j);
         int uj = s.perm[j];
         if (ui < uj) {
             int slot = atomicAdd(count, 1);
@@ -625,13 +622,15 @@ int grid_blocks(const Sys &s, int kind, int persist_cap)
         const int g = group_grid(s.n);
         return persist_cap > 0 && persist_cap < g ? persist_cap : g;
     }
-    case GK_CV: return persist_grid(s.n);  // not tiled: its grid fixes the CV sums' order
-    case GK_ATOM32: {
-        const int g = (s.n + 31) / 32;
+    case GK_ROWS: {
+        const int g = (s.n + kRowAtoms - 1) / kRowAtoms;
         return persist_cap > 0 && persist_cap < g ? persist_cap : g;
     }
-    case GK_ATOM128: {
-        const int g = (s.n + 127) / 128;
+    case GK_FORCE: {
+        // with the virial its grid fixes the order of the virial's partials:
+        // by N only, few enough for the last block to add
+        const int g = force_grid(s.n, s.ncv, s.pairs);
+        if (s.virial) return g < kPersistBlocks / 2 ? g : kPersistBlocks / 2;
         return persist_cap > 0 && persist_cap < g ? persist_cap : g;
     }
     case GK_SUM: return sum_blocks(s.n);

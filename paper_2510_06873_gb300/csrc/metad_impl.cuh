@@ -79,29 +79,23 @@ struct Sys {
     int *scan_part;        // block partial sums of the cell scan
     const int *rank_of_xyz;  // cell (x, y, z) -> Morton rank
     const int *xyz_of_rank;  // Morton rank -> packed x | y << 10 | z << 20
-    int *nbr;              // [n][max_nb] sorted indices, row per atom: r < rc exactly;
-                           // entries j > i first (nh of them), then j < i
+    int *nbr;              // [n][max_nb] FP64, two CVs: sorted indices of the exact row,
+                           // entries j > i first (nh of them), then j < i; its pair pass
+                           // searches them
     int *nn;               // [n]
     int *nh;               // [n] entries with j > i
     void *wl;              // JW<real> [n][max_nb]: neighbour and switch weight of each entry
-    void *pairF;           // real [n][max_nb][4]: G_ij in i's entry of j, -G_ji in the others
-    void *cross;           // real [n][max_nb]: b_j.q_i of each exact entry (two CVs)
+    void *pairF;           // FP64, two CVs: [n][max_nb][4], G_ij in i's entry of j, -G_ji in the others
+    void *cross;           // real [n][max_nb], two CVs: b_i.q_j + b_j.q_i of each exact entry
+                           // (FP64: its half b_j.q_i)
     void *geo;             // real [n][max_nb][4]: r_j - r_i (minimum image) and the CN mask
                            // of each exact entry, written by the exact filter
     // Verlet list (cutoff rc + skin, built at the reference positions)
     float4 *pos_ref;       // sorted positions at the last rebuild
-    int *vnbr;             // [n][max_vnb]; with mirror slots an entry j > i carries, above bit 23,
-                           // i's position in j's Verlet row (set once per rebuild by the filter)
+    int *vnbr;             // [n][max_vnb]
     int *vnn;              // [n]
     int *vnh;              // [n] Verlet entries with j > i (stored first)
     int max_vnb;
-    // mirror slots: where the pair force of i's entry j > i goes in j's row,
-    // without searching j's row in the force pass
-    int mirror;                // 1: in use (n < 2^23, rows of at most 255 entries)
-    unsigned short *vround;    // [n][vround_stride]: per filter round r (Verlet entries 8r .. 8r + 7),
-                               // the exact entries before it | the round's exact bits << 8
-    int vround_stride;
-    int *rows_fresh;           // 1 from a rebuild until the CV pass after the next filter
     int *flag;             // 1: rebuild the cell order and Verlet list this step
     float disp_thr2;       // (skin / 2)^2 with margin: rebuild above it
     float skin_eff;        // skin with margin
@@ -110,7 +104,10 @@ struct Sys {
     int always_rebuild;    // skin == 0
     unsigned long long *rebuilds;  // number of rebuilds done
     void *cn, *W, *qb6;    // real-typed per-atom scalars
-    void *q, *b, *h;       // real-typed per-atom records [n][16]: q_m; b_m, beta; h_m, gamma
+    void *q, *b, *h;       // real-typed per-atom records [n][16]: q_m; b_m, beta; h_m, gamma.
+                           // FP32: b is [n][32], q and b side by side in chunks of four
+                           // (q0..3 b0..3 q4..7 ...).  One CV: q is [n][8], the sums of
+                           // the coordination number's force and virial
     double *part;          // per-block FP64 partial sums, slots of part_stride
     int part_stride;
     unsigned *ticket;      // completion counters of the last-block reductions
@@ -127,6 +124,7 @@ struct Sys {
     int hstride;           // doubles per hill centre: max(D, 2)
     int lattice;           // 1: the box lengths are CVs ncv .. ncv + 2
     int virial;            // 1: the force pass also sums the bias virial
+    int pairs;             // 1: the force pass is the FP64 two-CV pair pass
     double w0, kbdt;
     int grid_on;
     int gn[2];
@@ -217,9 +215,8 @@ enum GridKind : int {
     GK_GROUPS_CAP,     // rebuild: Verlet rows
     GK_ONE,            // one block per system
     GK_GROUPS,         // one block per 16 atoms (lane-group kernels); a batch tile caps it
-    GK_CV,             // the Q6 pass with the CV sums: persistent, by N only
-    GK_ATOM32,         // one block per 32 atoms (four-lane adjoint); a batch tile caps it
-    GK_ATOM128,        // one block per 128 atoms (pair-parallel force); a batch tile caps it
+    GK_ROWS,           // one block per kRowAtoms atoms (four-lane kernels); a batch tile caps it
+    GK_FORCE,          // the force pass
     GK_SUM,            // the CV sums: blocks by N only
     GK_HILLS,          // hill kernel, evaluation
     GK_DEPOSIT,        // hill kernel, deposit (systems that deposit)
@@ -234,14 +231,15 @@ int grid_blocks(const Sys &s, int kind, int persist_cap);
 // Batched stage launches (one launch each over every system of the view).
 void launch_batch_gather(const BatchView &v, int total, cudaStream_t st);
 void launch_batch_rebuild(const BatchView *rows, const int *totals, cudaStream_t st);
-void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &cv, int cv_total,
-                     const BatchView &sums, int sum_total, int fp64, int ncv, cudaStream_t st);
+void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &rows, int row_total, int fp64, int ncv,
+                     cudaStream_t st);
+void launch_batch_sum(const BatchView &sums, int sum_total, int fp64, cudaStream_t st);
 void launch_cv_sum(const Sys &s, int fp64, cudaStream_t st);
 void launch_batch_bias(const BatchView &v, int total, int deposit, cudaStream_t st);
-// part 0: adjoint, pair forces and gather; 1: the adjoint only; 2: the rest
-void launch_batch_force(const BatchView &groups, int group_total, const BatchView &adj, int adj_total,
-                        const BatchView &pairs, int pair_total, int fp64, int ncv, int virial, cudaStream_t st,
-                        int part = 0);
+void launch_batch_adjoint(const BatchView &rows, int total, int fp64, cudaStream_t st);
+// The kernels after dV/ds is known; returns how many.
+int launch_batch_forces(const BatchView &force, int force_total, const BatchView &groups, int group_total, int fp64,
+                        int ncv, int virial, cudaStream_t st);
 void launch_batch_collect(const BatchView &v, double *out, cudaStream_t st);
 
 // Launch entry points (stream-ordered, no host synchronisation).
@@ -252,7 +250,10 @@ void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st);
 void launch_cv_avg(const Sys &s, int fp64, cudaStream_t st);
 void launch_bias(const Sys &s, int K, const double *s_dev, double *out_dev, int deposit, cudaStream_t st);
 void launch_adjoint(const Sys &s, int fp64, cudaStream_t st);
-void launch_force_pairs(const Sys &s, int fp64, double scale, cudaStream_t st);  // + virial if s.virial
+// The force pass (+ virial if s.virial): one kernel, except that the FP64
+// two-CV one leaves its pair forces for launch_force_gather.
+void launch_forces(const Sys &s, int fp64, float *F, int accumulate, double scale, cudaStream_t st);
+inline bool pair_slots(const Sys &s, int fp64) { return fp64 && s.ncv == 2; }
 void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st);
 void configure_kernels();
 void launch_grid_fold(const Sys &s, int K, cudaStream_t st);
@@ -553,17 +554,34 @@ constexpr int kAtomsPerBlock = kBlockAtoms / kG;
 // it, so launches and allocations can never disagree.
 __host__ __device__ inline int group_grid(int n) { return (n + kAtomsPerBlock - 1) / kAtomsPerBlock; }
 
-// Without a Q6 pass the CN sum runs in its own kernel: kSumThreads threads
-// per block, one block per kSumAtoms atoms (at most kMaxBiasBlocks blocks).
+// The CV sums run in their own kernel: kSumThreads threads per block, one
+// block per kSumAtoms atoms (at most kMaxBiasBlocks blocks).
 constexpr int kSumThreads = 256;
-constexpr int kSumAtoms = 2048;
+constexpr int kSumAtoms = 1024;
 __host__ __device__ inline int sum_blocks(int n)
 {
     const int b = (n + kSumAtoms - 1) / kSumAtoms;
     return b < 1 ? 1 : (b > kMaxBiasBlocks ? kMaxBiasBlocks : b);
 }
 
-// Persistent grids (the CV kernels, and the capped rebuild kernels) have at
+// Atoms per warp of the FP64 pair pass: 32 keep its lanes full, but leave a
+// small system on few SMs (1,000 atoms: 8 blocks, 39.6 us).
+__host__ __device__ inline int pair_chunk(int n) { return n < 20000 ? 8 : 32; }
+
+// The row passes (Q6 average, adjoint, FP32 force) give an atom four lanes and
+// a block kRowAtoms consecutive atoms.
+constexpr int kRowThreads = 128;
+constexpr int kRowAtoms = kRowThreads / 4;
+
+// Blocks of the force pass: a thread per atom with one CV, four lanes per
+// atom in FP32, a warp per chunk of atoms in the FP64 pair pass.
+__host__ __device__ inline int force_grid(int n, int ncv, int pairs)
+{
+    const int atoms = ncv == 1 ? kBlockAtoms : (pairs ? pair_chunk(n) * (kBlockAtoms / 32) : kRowAtoms);
+    return (n + atoms - 1) / atoms;
+}
+
+// Persistent grids (the capped rebuild kernels) have at
 // most kPersistBlocks blocks, walking their work grid-stride.
 constexpr int kPersistBlocks = 152 * 16;
 
@@ -662,111 +680,72 @@ __device__ __forceinline__ bool pair_in_warp(const Sys &s, bool valid, float4 pi
 // The geometry of an exact entry, cached by the filter so the CV and force
 // passes read one contiguous record per entry instead of gathering the
 // neighbour's position again: r_j - r_i, and in the fourth slot a tag
-// (carried through float registers unchanged): the bits of j, the CN mask in
-// bit 31, and with mirror slots, for an entry j > i, i's position in j's
-// Verlet row in bits 23..30.  The force pass reads it for the last time
-// (kLast: an evict-first load, so the stream does not push the gathered
-// per-atom records out of L2).
+// (carried through float registers unchanged): j, with the CN mask in bit 31.
+// The force pass reads it for the last time (kLast: an evict-first load, so
+// the stream does not push the gathered per-atom records out of L2).
 constexpr unsigned kCnBit = 0x80000000u;
-constexpr int kMirrorShift = 23;
-constexpr unsigned kMirrorJ = (1u << kMirrorShift) - 1u;
 
-__device__ __forceinline__ unsigned make_tag(const Sys &s, int j, float4 pi, float4 pj, unsigned vm)
+__device__ __forceinline__ unsigned make_tag(const Sys &s, int j, float4 pi, float4 pj)
 {
-    return (unsigned)j | (vm << kMirrorShift) | ((!s.cn_unlike || pj.w != pi.w) ? kCnBit : 0u);
+    return (unsigned)j | ((!s.cn_unlike || pj.w != pi.w) ? kCnBit : 0u);
 }
 
 template <typename real>
 __device__ __forceinline__ void store_geo(const Sys &s, size_t slot, const Vec3<float> &df, float4 pi, float4 pj,
-                                          int j, unsigned vm);
+                                          int j);
 template <>
 __device__ __forceinline__ void store_geo<float>(const Sys &s, size_t slot, const Vec3<float> &df, float4 pi,
-                                                 float4 pj, int j, unsigned vm)
+                                                 float4 pj, int j)
 {
-    const unsigned tag = make_tag(s, j, pi, pj, vm);
-    reinterpret_cast<float4 *>(s.geo)[slot] = make_float4(df.x, df.y, df.z, __uint_as_float(tag));
+    reinterpret_cast<float4 *>(s.geo)[slot] = make_float4(df.x, df.y, df.z, __uint_as_float(make_tag(s, j, pi, pj)));
 }
 template <>
 __device__ __forceinline__ void store_geo<double>(const Sys &s, size_t slot, const Vec3<float> &, float4 pi,
-                                                  float4 pj, int j, unsigned vm)
+                                                  float4 pj, int j)
 {
     const Vec3<double> d = displacement<double>(s, pi, pj);
-    const unsigned tag = make_tag(s, j, pi, pj, vm);
     double2 *g = reinterpret_cast<double2 *>(s.geo) + 2 * slot;
     g[0] = make_double2(d.x, d.y);
-    g[1] = make_double2(d.z, __longlong_as_double((long long)tag));
+    g[1] = make_double2(d.z, __longlong_as_double((long long)make_tag(s, j, pi, pj)));
 }
 
-// j, the CN mask and the mirror position (0 without mirror slots) of a tag.
-__device__ __forceinline__ void untag(const Sys &s, unsigned tag, int &j, bool &cn, unsigned &vm)
+__device__ __forceinline__ void untag(unsigned tag, int &j, bool &cn)
 {
-    j = (int)(tag & (s.mirror ? kMirrorJ : ~kCnBit));
+    j = (int)(tag & ~kCnBit);
     cn = (tag & kCnBit) != 0u;
-    vm = s.mirror ? (tag & ~kCnBit) >> kMirrorShift : 0u;
 }
 
 template <typename real, bool kLast = false>
-__device__ __forceinline__ void load_geo(const Sys &s, size_t slot, Vec3<real> &d, bool &cn, int &j, unsigned &vm);
+__device__ __forceinline__ void load_geo(const Sys &s, size_t slot, Vec3<real> &d, bool &cn, int &j);
 template <>
-__device__ __forceinline__ void load_geo<float, false>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j,
-                                                       unsigned &vm)
+__device__ __forceinline__ void load_geo<float, false>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j)
 {
     const float4 g = reinterpret_cast<const float4 *>(s.geo)[slot];
-    d.x = g.x;
-    d.y = g.y;
-    d.z = g.z;
-    untag(s, __float_as_uint(g.w), j, cn, vm);
+    d = Vec3<float>{g.x, g.y, g.z};
+    untag(__float_as_uint(g.w), j, cn);
 }
 template <>
-__device__ __forceinline__ void load_geo<float, true>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j,
-                                                      unsigned &vm)
+__device__ __forceinline__ void load_geo<float, true>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j)
 {
     const float4 g = __ldcs(reinterpret_cast<const float4 *>(s.geo) + slot);
-    d.x = g.x;
-    d.y = g.y;
-    d.z = g.z;
-    untag(s, __float_as_uint(g.w), j, cn, vm);
+    d = Vec3<float>{g.x, g.y, g.z};
+    untag(__float_as_uint(g.w), j, cn);
 }
 template <>
-__device__ __forceinline__ void load_geo<double, true>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j,
-                                                       unsigned &vm)
+__device__ __forceinline__ void load_geo<double, true>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j)
 {
     const double2 *g = reinterpret_cast<const double2 *>(s.geo) + 2 * slot;
     const double2 a = __ldcs(g), b = __ldcs(g + 1);
-    d.x = a.x;
-    d.y = a.y;
-    d.z = b.x;
-    untag(s, (unsigned)__double_as_longlong(b.y), j, cn, vm);
+    d = Vec3<double>{a.x, a.y, b.x};
+    untag((unsigned)__double_as_longlong(b.y), j, cn);
 }
 template <>
-__device__ __forceinline__ void load_geo<double, false>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j,
-                                                        unsigned &vm)
+__device__ __forceinline__ void load_geo<double, false>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j)
 {
     const double2 *g = reinterpret_cast<const double2 *>(s.geo) + 2 * slot;
     const double2 a = g[0], b = g[1];
-    d.x = a.x;
-    d.y = a.y;
-    d.z = b.x;
-    untag(s, (unsigned)__double_as_longlong(b.y), j, cn, vm);
-}
-
-// i's position in the j < i part of j's Verlet row (rows are symmetric: the
-// Verlet predicate is), four entries per load.  Run by the filter of the
-// first step on new rows only; the later steps read the stored result.  The
-// part searched holds plain indices (only entries j > i carry a position).
-__device__ __forceinline__ unsigned mirror_position(const Sys &s, int j, int i)
-{
-    const int *rj = s.vnbr + (size_t)j * s.max_vnb;
-    const int lo = s.vnh[j], hi = s.vnn[j];
-    for (int b = lo & ~3; b < hi; b += 4) {
-        const int4 v = *reinterpret_cast<const int4 *>(rj + b);
-        if (v.x == i && b >= lo) return (unsigned)b;
-        if (v.y == i && b + 1 >= lo && b + 1 < hi) return (unsigned)(b + 1);
-        if (v.z == i && b + 2 >= lo && b + 2 < hi) return (unsigned)(b + 2);
-        if (v.w == i && b + 3 >= lo && b + 3 < hi) return (unsigned)(b + 3);
-    }
-    set_err(s, kErrInternal);  // rows not symmetric: never expected
-    return 0u;
+    d = Vec3<double>{a.x, a.y, b.x};
+    untag((unsigned)__double_as_longlong(b.y), j, cn);
 }
 
 // One exact entry for the gather passes: the neighbour and the switch
@@ -777,69 +756,46 @@ struct alignas(2 * sizeof(real)) JW {
     real w;
 };
 
+// The exact row of atom a.i from its Verlet row: eight candidates a round,
+// compacted by ballot.  The row's indices are kept only where a later pass
+// searches them (FP64, two CVs); everyone else reads j from the tags.
 template <typename real>
 __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
 {
+    const bool rows = sizeof(real) == 8 && s.ncv == 2;
     const int vn = a.ok ? s.vnn[a.i] : 0;
     const int vh = a.ok ? s.vnh[a.i] : 0;
     const float4 pi = a.ok ? s.pos_s[a.i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    int *vrow = s.vnbr + (size_t)(a.ok ? a.i : 0) * s.max_vnb;
-    int *row = s.nbr + (size_t)(a.ok ? a.i : 0) * s.max_nb;
-    unsigned short *vround = s.vround + (s.mirror ? (size_t)(a.ok ? a.i : 0) * s.vround_stride : 0);
-    // mirror slots: each Verlet entry j > i carries i's position in j's
-    // Verlet row in its high bits (searched once on new rows, kept there for
-    // the steps after, read with the entry), and each round records the exact
-    // entries before it and its exact bits
-    if (s.mirror && *s.rows_fresh) {
-        for (int k = a.l; k < vh; k += kG) {
-            const int j = vrow[k] & (int)kMirrorJ;
-            vrow[k] = j | (int)(mirror_position(s, j, a.i) << kMirrorShift);
-        }
-        __syncwarp();
-    }
+    const int *vrow = s.vnbr + (size_t)(a.ok ? a.i : 0) * s.max_vnb;
+    const size_t row0 = (size_t)(a.ok ? a.i : 0) * s.max_nb;
     const unsigned lt = (1u << a.l) - 1u;
-    const unsigned jmask = s.mirror ? kMirrorJ : 0xffffffffu;
     int cnt = 0, nh = 0;
-    unsigned short rec = 0;  // lane r keeps round r's record (rounds below kG)
     // one pass: the Verlet row already has its j > i part first, so accepted
     // entries come out in the same order; nh counts those from that part
     const int vmax = __reduce_max_sync(0xffffffffu, vn);
     for (int base = 0; base < vmax; base += kG) {
         const int k = base + a.l;
         const bool valid = k < vn;
-        const unsigned raw = valid ? (unsigned)vrow[k] : 0u;
-        const int j = (int)(raw & jmask);
-        const unsigned vm = (s.mirror && k < vh) ? raw >> kMirrorShift : 0u;
+        const int j = valid ? vrow[k] : 0;
         const float4 pj = valid ? s.pos_s[j] : pi;
         const Vec3<float> d = displacement_warp(s, pi, pj);  // every lane: a warp vote inside
         const bool in = pair_in_warp(s, valid, pi, pj, d);
         const unsigned gm = group_mask_bits(__ballot_sync(0xffffffffu, in));
-        const int below = min(max(vh - base, 0), kG);  // lanes of this round in the j > i part
         const int at = cnt + __popc(gm & lt);
-        if (s.mirror) {  // only rounds that reach the j < i part are ever looked up
-            const unsigned short r = (unsigned short)(min(cnt, 255) | (gm << 8));
-            const int round = base / kG;
-            if (round < kG) {
-                if (a.l == round) rec = r;
-            } else if (a.l == 0 && base < vn && base + kG > vh) {
-                vround[round] = r;
-            }
-        }
         if (in && at < s.max_nb) {
-            if (!s.mirror) row[at] = j;  // with mirror slots the exact entries' j live in their tags
-            store_geo<real>(s, (size_t)a.i * s.max_nb + at, d, pi, pj, j, vm);
+            if (rows) s.nbr[row0 + at] = j;
+            store_geo<real>(s, row0 + at, d, pi, pj, j);
         }
         cnt += __popc(gm);
-        nh += __popc(gm & ((1u << below) - 1u));
-    }
-    if (s.mirror && a.ok) {
-        const int base = a.l * kG;
-        if (base < vn && base + kG > vh) vround[a.l] = rec;
+        if (rows) {
+            const int below = min(max(vh - base, 0), kG);  // lanes of this round in the j > i part
+            nh += __popc(gm & ((1u << below) - 1u));
+        }
     }
     if (a.ok && a.l == 0) {
         if (cnt > s.max_nb) set_err(s, kErrCapacity);
         s.nn[a.i] = min(cnt, s.max_nb);
-        s.nh[a.i] = min(nh, s.max_nb);
+        if (rows) s.nh[a.i] = min(nh, s.max_nb);
     }
     __syncwarp();
     return min(cnt, s.max_nb);
