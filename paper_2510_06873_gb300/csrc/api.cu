@@ -550,12 +550,12 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
         y.cand_slot = slot;
         return METAD_OK;
     }
-    if ((s = alloc(&y.pos_s, n)) || (s = alloc(&y.perm, n)) || (s = alloc(&y.scell, n)) ||
+    if ((s = alloc(&y.pos_s, n)) || (s = alloc(&y.perm, n)) || (s = alloc(&y.raw, n)) ||
         (s = alloc(&y.ucell, n)) || (s = alloc(&y.uslot, n)) || (s = alloc(&y.cell_count, y.ncell)) ||
         (s = alloc(&y.cell_start, (size_t)y.ncell + 1)) || (s = alloc(&y.scan_part, y.ncell / 4096 + 2)) ||
         (s = alloc(&b.rank_xyz, y.ncell)) || (s = alloc(&b.xyz_rank, y.ncell)) ||
         (s = alloc(&y.nbr, pairs ? rows : 1)) || (s = alloc(&y.nn, n)) || (s = alloc(&y.nh, n)) ||
-        (s = alloc(&y.vnh, n)) || (s = alloc(&b.wlb, two ? 2 * rs * rows : 1)) ||
+        (s = alloc(&b.wlb, two ? 2 * rs * rows : 1)) ||
         (s = alloc(&b.pfb, pairs ? rs * 4 * rows : 1)) || (s = alloc(&b.geob, rs * 4 * rows)) ||
         (s = alloc(&b.crossb, two ? rs * rows : 1)) ||
         (s = alloc(&y.pos_ref, n)) ||
@@ -781,7 +781,6 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
     // the cell counters start at zero; every rebuild's scan leaves them zero
     cudaMemsetAsync(y.cell_count, 0, sizeof(int) * (size_t)c->ncell_alloc, c->stream);
     cudaMemsetAsync(y.nh, 0, sizeof(int) * (size_t)n, c->stream);
-    cudaMemsetAsync(y.vnh, 0, sizeof(int) * (size_t)n, c->stream);
     cudaMemsetAsync(y.vnn, 0, sizeof(int) * (size_t)n, c->stream);
     cudaMemsetAsync(y.rebuilds, 0, sizeof(unsigned long long), c->stream);
     {

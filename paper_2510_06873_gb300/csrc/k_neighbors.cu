@@ -5,8 +5,9 @@
 //   k_gather_check  positions in cell order (wrapped), and a flag when any
 //                   atom moved more than skin/2 since the last rebuild
 //   rebuild chain   (early exit unless flagged) counting sort of the atoms
-//                   into Morton-ranked cells of edge >= rc + skin, stable by
-//                   caller index, and the Verlet list r < rc + skin
+//                   into Morton-ranked cells of edge >= rc + skin (by octant,
+//                   then caller index within a cell), and the Verlet list
+//                   r < rc + skin
 //   filter          exact rows {j : r_ij^2 < rc^2} from the Verlet rows
 //                   (fused into the CV kernel, or k_filter on its own)
 // The exact rows are the FP64 definition bit for bit: while no atom has moved
@@ -91,6 +92,10 @@ __global__ void k_gather_check(Sys s)
     gather_check(s, own_blk());
 }
 
+// Cell of an atom, its slot there, and the octant of the cell it lies in (in
+// the slot's top bits: a cell never holds 2^28 atoms).
+constexpr int kOctShift = 28;
+
 __device__ __forceinline__ void bin_one(const Sys &s, int u)
 {
     bool bad;
@@ -99,8 +104,10 @@ __device__ __forceinline__ void bin_one(const Sys &s, int u)
     int cy = cell_axis(p.y, s.inv_h[1], s.nc[1]);
     int cz = cell_axis(p.z, s.inv_h[2], s.nc[2]);
     int c = s.rank_of_xyz[(cz * s.nc[1] + cy) * s.nc[0] + cx];
+    const int oct = (p.x * s.inv_h[0] - (float)cx >= 0.5f ? 1 : 0) | (p.y * s.inv_h[1] - (float)cy >= 0.5f ? 2 : 0) |
+                    (p.z * s.inv_h[2] - (float)cz >= 0.5f ? 4 : 0);
     s.ucell[u] = c;
-    s.uslot[u] = atomicAdd(&s.cell_count[c], 1);
+    s.uslot[u] = atomicAdd(&s.cell_count[c], 1) | (oct << kOctShift);
 }
 
 __device__ __forceinline__ void bin_count(const Sys &s, Blk k)
@@ -193,41 +200,41 @@ __device__ __forceinline__ void scan_down(const Sys &s, Blk k)
     if (base <= s.ncell - 1 && s.ncell - 1 < base + kScanItems) s.cell_start[s.ncell] = s.n;
 }
 
+// Each cell's atoms, in the order of their atomic slots: octant and caller
+// index, one word each.
 __device__ __forceinline__ void bin_scatter(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
-    for (int u = k.b * blockDim.x + threadIdx.x; u < s.n; u += k.nb * blockDim.x)
-        s.perm[s.cell_start[s.ucell[u]] + s.uslot[u]] = u;
-}
-
-// One thread per cell: order the cell's atoms by caller index (the atomic
-// slots above are not deterministic), gather their wrapped positions and
-// keep them as the reference of the new Verlet list.
-__device__ __forceinline__ void sort_gather_cell(const Sys &s, int c)
-{
-    int a = s.cell_start[c], e = s.cell_start[c + 1];
-    for (int t = a + 1; t < e; ++t) {
-        int v = s.perm[t];
-        int k = t - 1;
-        while (k >= a && s.perm[k] > v) {
-            s.perm[k + 1] = s.perm[k];
-            --k;
-        }
-        s.perm[k + 1] = v;
-    }
-    for (int t = a; t < e; ++t) {
-        bool bad;
-        float4 p = load_wrapped(s, s.perm[t], bad);
-        s.pos_s[t] = p;
-        s.pos_ref[t] = p;
-        s.scell[t] = c;
+    for (int u = k.b * blockDim.x + threadIdx.x; u < s.n; u += k.nb * blockDim.x) {
+        const int v = s.uslot[u];
+        s.raw[s.cell_start[s.ucell[u]] + (v & ((1 << kOctShift) - 1))] =
+            (unsigned)u | ((unsigned)v >> kOctShift << kOctShift);
     }
 }
 
+// The sorted order: within a cell by octant, then caller index (the atomic
+// slots are not deterministic).  Octants put atoms half a cell apart next to
+// each other in memory, so a line of per-atom records holds more atoms that
+// are neighbours of the same atom.  One thread per atom: its place is the
+// number of smaller words in its cell (about eight, read from cache), where
+// one thread sorting a cell by insertion chains its loads (48 us at 1M
+// atoms).  Its wrapped position becomes the reference of the new Verlet list.
 __device__ __forceinline__ void cell_sort_gather(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
-    for (int c = k.b * blockDim.x + threadIdx.x; c < s.ncell; c += k.nb * blockDim.x) sort_gather_cell(s, c);
+    for (int t = k.b * blockDim.x + threadIdx.x; t < s.n; t += k.nb * blockDim.x) {
+        const unsigned v = s.raw[t];
+        const int u = (int)(v & ((1u << kOctShift) - 1u));
+        const int c = s.ucell[u];
+        const int a = s.cell_start[c], e = s.cell_start[c + 1];
+        int at = a;
+        for (int q = a; q < e; ++q) at += s.raw[q] < v ? 1 : 0;
+        bool bad;
+        const float4 p = load_wrapped(s, u, bad);
+        s.perm[at] = u;
+        s.pos_s[at] = p;
+        s.pos_ref[at] = p;
+    }
 }
 
 __device__ __forceinline__ int wrap_cell(int c, int nc)
@@ -243,30 +250,28 @@ __device__ __forceinline__ int axis_span(int nc) { return nc >= 3 ? 3 : nc; }
 __device__ __forceinline__ int axis_off(int nc, int idx) { return nc >= 3 ? idx - 1 : idx; }
 
 // Verlet rows {j : r_ij^2 < (rc + skin)^2 (1 + 1e-4)} over the 27 cells
-// around each atom's own (each distinct cell once): entries with j > i
-// first, then j < i, each part in stencil-cell order (x fastest), atoms in
-// cell order.  Atoms are sorted by cell rank, so a cell ranked above the
-// atom's own holds only j > i and one ranked below only j < i.
+// around each atom's own (each distinct cell once), in stencil-cell order (x
+// fastest), atoms in cell order.
 //
-// One warp per cell A at a time.  The candidates of A's atoms are the same
-// list: the part-0 cells (rank >= A's) then the part-1 cells (rank <= A's),
-// each in stencil order, A itself in both.  The warp stages that list in
-// shared memory with coalesced loads (position, index, stencil cell), then
-// sweeps its 32 lanes over it for each atom of A in turn, compacting the
-// accepted entries with a ballot: the row comes out in its final order, with
-// no per-lane cell search and no divergence between lanes.  A list longer
-// than the buffer is staged and swept in chunks, per atom.
+// One warp per cell at a time.  The candidates of the cell's atoms are the
+// same list; the warp stages it in shared memory (position, index, stencil
+// cell), then gives each of the cell's na atoms 32 / na lanes, which take the
+// list's entries in turn and compact the accepted ones with a ballot: the row
+// comes out in list order whatever na is.  Bound by instruction issue: about
+// 22 a round, and rounds x lanes is the cell's na x candidates (208 at skin 1)
+// whatever their split, where a warp sweeping the list for one atom at a time
+// spent its per-atom and partial-round overheads seven or eight times a cell.
+// A list longer than the buffer is staged and swept in chunks.
 //
 // Displacements: with three or more cells along every axis each stencil cell
 // is a distinct cell at one periodic image, and d = (r_j - r_i) + shift with
 // the cell's image shift (0 or +-L per axis): no minimum-image test per
-// candidate, and since both roundings are sign-symmetric the two directions
-// of a pair give exactly opposite vectors, so the rows stay symmetric.  With
-// fewer cells along an axis, the minimum image per candidate.  The 1e-4
-// margin on the cutoff covers the rounding of either form.
+// candidate.  With fewer cells along an axis, the minimum image per
+// candidate.  The 1e-4 margin on the cutoff covers the rounding of either
+// form.
 constexpr int kStencil = 27;
 constexpr int kVerletWarps = kBlockAtoms / 32;
-constexpr int kCandBuf = 256;  // staged candidates per warp
+constexpr int kCandBuf = 320;  // staged candidates per warp
 
 struct VerletWarpSmem {
     float4 pos[kCandBuf];      // candidate position, index bits in w
@@ -275,88 +280,60 @@ struct VerletWarpSmem {
 };
 
 // Copy the candidates [k0, k0 + len) of the list into the buffer: lane q
-// copies its stencil cell's segments (in part 0 at o0, in part 1 at o1; -1
-// when not in it), so the warp's loads are all independent of one another.
-__device__ __forceinline__ void verlet_stage(const Sys &s, VerletWarpSmem &w, int st, int n, int o0, int o1, int k0,
-                                             int len, int lane)
+// copies its stencil cell's n atoms from st on (list positions from o on), so
+// the warp's loads are all independent of one another.
+__device__ __forceinline__ void verlet_stage(const Sys &s, VerletWarpSmem &w, int st, int n, int o, int k0, int len,
+                                             int lane)
 {
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-        const int o = part == 0 ? o0 : o1;
-        if (o < 0) continue;
-        const int lo = max(o, k0), hi = min(o + n, k0 + len);
+    const int lo = max(o, k0), hi = min(o + n, k0 + len);
 #pragma unroll 4
-        for (int t = lo; t < hi; ++t) {
-            const int j = st + (t - o);
-            float4 pj = s.pos_s[j];
-            pj.w = __int_as_float(j);
-            w.pos[t - k0] = pj;
-            w.q[t - k0] = (unsigned char)lane;
-        }
+    for (int t = lo; t < hi; ++t) {
+        const int j = st + (t - o);
+        float4 pj = s.pos_s[j];
+        pj.w = __int_as_float(j);
+        w.pos[t - k0] = pj;
+        w.q[t - k0] = (unsigned char)lane;
     }
     __syncwarp();
 }
 
-// Sweep atom i over the staged candidates [t0, t1) of the buffer, all in one
-// part (kUp: part 0, j > i; else part 1, j < i), appending to its row.
-// kShift: some stencil cell of this one is a periodic image (a cell on the
-// box faces); interior cells need no shift.
-template <bool kImages, bool kShift, bool kUp>
-__device__ __forceinline__ bool verlet_test(const Sys &s, const VerletWarpSmem &w, int i, float4 pi, int t, int t1,
-                                            int &j)
-{
-    // branch-free: the buffer position is clamped in bounds and the test
-    // masked by t < t1
-    const int tc = min(t, kCandBuf - 1);
-    const float4 cp = w.pos[tc];
-    j = __float_as_int(cp.w);
-    Vec3<float> d;
-    if (!kImages) {
-        d = displacement<float>(s, pi, cp);
-    } else if (kShift) {
-        // past the staged length w.q is stale: keep the index in the table
-        const float4 h = w.shift[min((int)w.q[tc], kStencil - 1)];
-        d.x = (cp.x - pi.x) + h.x;
-        d.y = (cp.y - pi.y) + h.y;
-        d.z = (cp.z - pi.z) + h.z;
-    } else {
-        d.x = cp.x - pi.x;
-        d.y = cp.y - pi.y;
-        d.z = cp.z - pi.z;
-    }
-    return t < t1 && (kUp ? j > i : j < i) && fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)) < s.rv2;
-}
-
-// Sweep atom i over the staged candidates [t0, t1) of the buffer, all in one
-// part (kUp: part 0, j > i; else part 1, j < i), appending to its row, two
-// rounds of 32 per iteration.  kShift: some stencil cell of this one is a
+// Sweep the staged candidates [0, len): lane l of G takes candidates l, l + G,
+// ... for atom i (its position pi; lanes past the atoms have on = false).
+// gsh: the group's first lane.  kShift: some stencil cell of this one is a
 // periodic image (a cell on the box faces); interior cells need no shift.
-template <bool kImages, bool kShift, bool kUp>
-__device__ __forceinline__ void verlet_sweep(const Sys &s, const VerletWarpSmem &w, int i, float4 pi, int t0, int t1,
-                                             int lane, int *vrow, int &total)
-{
-    const unsigned lt = (1u << lane) - 1u;
-    for (int r = t0; r < t1; r += 64) {
-        int ja, jb;
-        const bool ina = verlet_test<kImages, kShift, kUp>(s, w, i, pi, r + lane, t1, ja);
-        const bool inb = verlet_test<kImages, kShift, kUp>(s, w, i, pi, r + 32 + lane, t1, jb);
-        const unsigned ba = __ballot_sync(0xffffffffu, ina), bb = __ballot_sync(0xffffffffu, inb);
-        const int ata = total + __popc(ba & lt);
-        const int atb = total + __popc(ba) + __popc(bb & lt);
-        if (ina && ata < s.max_vnb) vrow[ata] = ja;
-        if (inb && atb < s.max_vnb) vrow[atb] = jb;
-        total += __popc(ba) + __popc(bb);
-    }
-}
-
 template <bool kImages, bool kShift>
-__device__ __forceinline__ void verlet_sweeps(const Sys &s, const VerletWarpSmem &w, int i, float4 pi, int k0, int len,
-                                              int T0, int lane, int *vrow, int &total, int &up)
+__device__ __forceinline__ int verlet_sweep(const Sys &s, const VerletWarpSmem &w, int i, float4 pi, bool on, int l,
+                                            int G, int gsh, int len, int *vrow, int cnt)
 {
-    const int split = min(max(T0 - k0, 0), len);  // buffer positions below it are part 0
-    verlet_sweep<kImages, kShift, true>(s, w, i, pi, 0, split, lane, vrow, total);
-    if (k0 < T0) up = total;
-    verlet_sweep<kImages, kShift, false>(s, w, i, pi, split, len, lane, vrow, total);
+    const unsigned gmask = G == 32 ? 0xffffffffu : (1u << G) - 1u, lt = (1u << l) - 1u;
+#pragma unroll 2
+    for (int r = 0; r < len; r += G) {
+        const int t = r + l;
+        const int tc = min(t, kCandBuf - 1);  // in bounds; masked by t < len
+        const float4 cp = w.pos[tc];
+        const int j = __float_as_int(cp.w);
+        Vec3<float> d;
+        if (!kImages) {
+            d = displacement<float>(s, pi, cp);
+        } else {
+            d.x = cp.x - pi.x;
+            d.y = cp.y - pi.y;
+            d.z = cp.z - pi.z;
+            if (kShift) {
+                // past the staged length w.q is stale: keep the index in the table
+                const float4 h = w.shift[min((int)w.q[tc], kStencil - 1)];
+                d.x += h.x;
+                d.y += h.y;
+                d.z += h.z;
+            }
+        }
+        const bool in = on && t < len && j != i && fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)) < s.rv2;
+        const unsigned m = (__ballot_sync(0xffffffffu, in) >> gsh) & gmask;
+        const int at = cnt + __popc(m & lt);
+        if (in && at < s.max_vnb) vrow[at] = j;
+        cnt += __popc(m);
+    }
+    return cnt;
 }
 
 template <bool kImages>
@@ -372,8 +349,8 @@ __device__ __forceinline__ void verlet_cell(const Sys &s, VerletWarpSmem &w, int
     const int nq = sx * sy * sz;
     // a cell on the box faces has stencil cells at a periodic image
     const bool shifted = cx == 0 || cy == 0 || cz == 0 || cx == s.nc[0] - 1 || cy == s.nc[1] - 1 || cz == s.nc[2] - 1;
-    // the stencil: lane q < nq looks up cell q (x fastest) and its segments
-    int n0 = 0, n1 = 0, st = 0, n = 0;  // lane q's cell: first atom, atoms, its part-0 / part-1 lengths
+    // the stencil: lane q < nq looks up cell q (x fastest)
+    int st = 0, n = 0;
     if (lane < nq) {
         const int ex = lane % sx, ey = (lane / sx) % sy, ez = lane / (sx * sy);
         const int x = cx + axis_off(s.nc[0], ex), y = cy + axis_off(s.nc[1], ey), z = cz + axis_off(s.nc[2], ez);
@@ -385,45 +362,38 @@ __device__ __forceinline__ void verlet_cell(const Sys &s, VerletWarpSmem &w, int
             w.shift[lane] = make_float4(x < 0 ? -s.Lhi[0] : (x >= s.nc[0] ? s.Lhi[0] : 0.0f),
                                         y < 0 ? -s.Lhi[1] : (y >= s.nc[1] ? s.Lhi[1] : 0.0f),
                                         z < 0 ? -s.Lhi[2] : (z >= s.nc[2] ? s.Lhi[2] : 0.0f), 0.0f);
-        n0 = cq >= c ? n : 0;
-        n1 = cq <= c ? n : 0;
     }
-    // exclusive scans of the segment lengths over the stencil (lanes)
-    int i0 = n0, i1 = n1;
+    int o = n;  // inclusive, then exclusive scan of the cells' sizes
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y0 = __shfl_up_sync(0xffffffffu, i0, o), y1 = __shfl_up_sync(0xffffffffu, i1, o);
-        if (lane >= o) {
-            i0 += y0;
-            i1 += y1;
-        }
+    for (int k = 1; k < 32; k <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, o, k);
+        if (lane >= k) o += y;
     }
-    const int T0 = __shfl_sync(0xffffffffu, i0, 31), T1 = __shfl_sync(0xffffffffu, i1, 31);
-    // lane q's segments in the list (-1: not in that part); lanes past the
-    // stencil have none
-    const int o0 = n0 > 0 ? i0 - n0 : -1, o1 = n1 > 0 ? T0 + i1 - n1 : -1;
-    const int T = T0 + T1;
-    const bool one_chunk = T <= kCandBuf;
-    if (one_chunk) verlet_stage(s, w, st, n, o0, o1, 0, T, lane);
-    for (int ia = 0; ia < na; ++ia) {
-        const int i = a0 + ia;
-        const float4 pi = s.pos_s[i];
-        int *vrow = s.vnbr + (size_t)i * s.max_vnb;
-        int total = 0, up = 0;
-        for (int k0 = 0; k0 < T; k0 += kCandBuf) {
-            const int len = min(kCandBuf, T - k0);
-            if (!one_chunk) verlet_stage(s, w, st, n, o0, o1, k0, len, lane);
-            if (shifted) verlet_sweeps<kImages, true>(s, w, i, pi, k0, len, T0, lane, vrow, total, up);
-            else verlet_sweeps<kImages, false>(s, w, i, pi, k0, len, T0, lane, vrow, total, up);
-            if (!one_chunk) __syncwarp();  // the chunk is read before the next is staged
+    const int T = __shfl_sync(0xffffffffu, o, 31);
+    o -= n;
+    // lanes per atom; more than 32 atoms go in batches of 32
+    const int G = na <= 32 ? 32 / na : 1, per = 32 / G;
+    const int g = lane / G, l = lane - g * G, gsh = g * G < 32 ? g * G : 0;
+    for (int k0 = 0; k0 < T; k0 += kCandBuf) {
+        const int len = min(kCandBuf, T - k0);
+        const bool last = k0 + len == T;
+        verlet_stage(s, w, st, n, o, k0, len, lane);
+        for (int ab = 0; ab < na; ab += per) {
+            const bool on = g < per && ab + g < na;
+            const int i = a0 + (on ? ab + g : 0);
+            const float4 pi = s.pos_s[i];
+            int *vrow = s.vnbr + (size_t)i * s.max_vnb;
+            int cnt = k0 > 0 ? s.vnn[i] : 0;  // lane 0 of the group left it there
+            __syncwarp();
+            if (shifted) cnt = verlet_sweep<kImages, true>(s, w, i, pi, on, l, G, gsh, len, vrow, cnt);
+            else cnt = verlet_sweep<kImages, false>(s, w, i, pi, on, l, G, gsh, len, vrow, cnt);
+            if (on && l == 0) {
+                if (last && cnt > s.max_vnb) set_err(s, kErrCapacity);
+                s.vnn[i] = last ? min(cnt, s.max_vnb) : cnt;
+            }
         }
-        if (lane == 0) {
-            if (total > s.max_vnb) set_err(s, kErrCapacity);
-            s.vnn[i] = min(total, s.max_vnb);
-            s.vnh[i] = min(up, s.max_vnb);
-        }
+        __syncwarp();  // the chunk is read (and the counts written) before the next is staged
     }
-    __syncwarp();  // the tables are read before the next cell overwrites them
 }
 
 // End of a rebuild, run once by the last Verlet block to finish: the rows'
@@ -615,7 +585,6 @@ int grid_blocks(const Sys &s, int kind, int persist_cap)
     case GK_ATOM256: return (s.n + 255) / 256;
     case GK_ATOM256_CAP: return capped((s.n + 255) / 256);
     case GK_SCAN_TILES: return (s.ncell + kScanTile - 1) / kScanTile;
-    case GK_CELL128_CAP: return capped((s.ncell + 127) / 128);
     case GK_GROUPS_CAP: return persist_grid(s.n);  // Verlet rows: up to 16 blocks per SM
     case GK_ONE: return 1;
     case GK_GROUPS: {
@@ -677,7 +646,7 @@ void launch_rebuild(const Sys &s, cudaStream_t st)
     chained(k_scan_reduce, grid_blocks(s, GK_SCAN_TILES, 0), kScanThreads, st, s);
     chained(k_scan_down, grid_blocks(s, GK_SCAN_TILES, 0), kScanThreads, st, s);
     chained(k_bin_scatter, grid_blocks(s, GK_ATOM256_CAP, 0), 256, st, s);
-    chained(k_cell_sort_gather, grid_blocks(s, GK_CELL128_CAP, 0), 128, st, s);
+    chained(k_cell_sort_gather, grid_blocks(s, GK_ATOM256_CAP, 0), 256, st, s);
     chained(k_verlet, grid_blocks(s, GK_GROUPS_CAP, 0), kBlockAtoms, st, s);
 }
 
@@ -692,7 +661,7 @@ void launch_batch_rebuild(const BatchView *rows, const int *totals, cudaStream_t
     chained(kb_scan_reduce, totals[GK_SCAN_TILES], kScanThreads, st, rows[GK_SCAN_TILES]);
     chained(kb_scan_down, totals[GK_SCAN_TILES], kScanThreads, st, rows[GK_SCAN_TILES]);
     chained(kb_bin_scatter, totals[GK_ATOM256_CAP], 256, st, rows[GK_ATOM256_CAP]);
-    chained(kb_cell_sort_gather, totals[GK_CELL128_CAP], 128, st, rows[GK_CELL128_CAP]);
+    chained(kb_cell_sort_gather, totals[GK_ATOM256_CAP], 256, st, rows[GK_ATOM256_CAP]);
     chained(kb_verlet, totals[GK_GROUPS_CAP], kBlockAtoms, st, rows[GK_GROUPS_CAP]);
 }
 

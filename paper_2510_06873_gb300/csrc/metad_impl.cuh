@@ -72,7 +72,7 @@ struct Sys {
     const float4 *pos_in;  // caller order
     float4 *pos_s;
     int *perm;             // sorted -> caller
-    int *scell;            // cell of each sorted atom
+    unsigned *raw;         // rebuild: each cell's atoms before they are ordered
     int *ucell, *uslot;    // caller order: cell and slot within it
     int *cell_count;       // [ncell]
     int *cell_start;       // [ncell + 1]
@@ -94,7 +94,6 @@ struct Sys {
     float4 *pos_ref;       // sorted positions at the last rebuild
     int *vnbr;             // [n][max_vnb]
     int *vnn;              // [n]
-    int *vnh;              // [n] Verlet entries with j > i (stored first)
     int max_vnb;
     int *flag;             // 1: rebuild the cell order and Verlet list this step
     float disp_thr2;       // (skin / 2)^2 with margin: rebuild above it
@@ -209,9 +208,8 @@ __device__ __forceinline__ int batch_system(const BatchView &v, Blk &k)
 // Grids of a step, one row of block counts per launch kind.
 enum GridKind : int {
     GK_ATOM256 = 0,    // one thread per atom, 256 per block
-    GK_ATOM256_CAP,    // rebuild: binning and scatter
+    GK_ATOM256_CAP,    // rebuild: binning, scatter and cell sort
     GK_SCAN_TILES,     // rebuild: cell scan
-    GK_CELL128_CAP,    // rebuild: cell sort
     GK_GROUPS_CAP,     // rebuild: Verlet rows
     GK_ONE,            // one block per system
     GK_GROUPS,         // one block per 16 atoms (lane-group kernels); a batch tile caps it
@@ -756,46 +754,53 @@ struct alignas(2 * sizeof(real)) JW {
     real w;
 };
 
-// The exact row of atom a.i from its Verlet row: eight candidates a round,
-// compacted by ballot.  The row's indices are kept only where a later pass
-// searches them (FP64, two CVs); everyone else reads j from the tags.
-template <typename real>
-__device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
+// Eight candidates of a Verlet row a round, the accepted ones compacted by
+// ballot.  kPart: 0 every exact entry, 1 those with j > i, 2 those with j < i.
+template <typename real, int kPart>
+__device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
-    const bool rows = sizeof(real) == 8 && s.ncv == 2;
-    const int vn = a.ok ? s.vnn[a.i] : 0;
-    const int vh = a.ok ? s.vnh[a.i] : 0;
-    const float4 pi = a.ok ? s.pos_s[a.i] : make_float4(0.f, 0.f, 0.f, 0.f);
     const int *vrow = s.vnbr + (size_t)(a.ok ? a.i : 0) * s.max_vnb;
     const size_t row0 = (size_t)(a.ok ? a.i : 0) * s.max_nb;
     const unsigned lt = (1u << a.l) - 1u;
-    int cnt = 0, nh = 0;
-    // one pass: the Verlet row already has its j > i part first, so accepted
-    // entries come out in the same order; nh counts those from that part
-    const int vmax = __reduce_max_sync(0xffffffffu, vn);
     for (int base = 0; base < vmax; base += kG) {
         const int k = base + a.l;
         const bool valid = k < vn;
         const int j = valid ? vrow[k] : 0;
         const float4 pj = valid ? s.pos_s[j] : pi;
         const Vec3<float> d = displacement_warp(s, pi, pj);  // every lane: a warp vote inside
-        const bool in = pair_in_warp(s, valid, pi, pj, d);
+        const bool part = kPart == 0 || (kPart == 1 ? j > a.i : j < a.i);
+        const bool in = pair_in_warp(s, valid && part, pi, pj, d);
         const unsigned gm = group_mask_bits(__ballot_sync(0xffffffffu, in));
         const int at = cnt + __popc(gm & lt);
         if (in && at < s.max_nb) {
-            if (rows) s.nbr[row0 + at] = j;
+            if (kPart != 0) s.nbr[row0 + at] = j;
             store_geo<real>(s, row0 + at, d, pi, pj, j);
         }
         cnt += __popc(gm);
-        if (rows) {
-            const int below = min(max(vh - base, 0), kG);  // lanes of this round in the j > i part
-            nh += __popc(gm & ((1u << below) - 1u));
-        }
+    }
+    return cnt;
+}
+
+// The exact row of atom a.i from its Verlet row.  For the FP64 two-CV pair
+// pass the j > i entries come first, in a sweep of their own, and the row's
+// indices are kept (it searches them); everyone else reads j from the tags.
+template <typename real>
+__device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
+{
+    const int vn = a.ok ? s.vnn[a.i] : 0;
+    const float4 pi = a.ok ? s.pos_s[a.i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int vmax = __reduce_max_sync(0xffffffffu, vn);
+    int cnt;
+    if (sizeof(real) == 8 && s.ncv == 2) {
+        const int nh = filter_sweep<real, 1>(s, a, vn, vmax, pi, 0);
+        cnt = filter_sweep<real, 2>(s, a, vn, vmax, pi, nh);
+        if (a.ok && a.l == 0) s.nh[a.i] = min(nh, s.max_nb);
+    } else {
+        cnt = filter_sweep<real, 0>(s, a, vn, vmax, pi, 0);
     }
     if (a.ok && a.l == 0) {
         if (cnt > s.max_nb) set_err(s, kErrCapacity);
         s.nn[a.i] = min(cnt, s.max_nb);
-        if (rows) s.nh[a.i] = min(nh, s.max_nb);
     }
     __syncwarp();
     return min(cnt, s.max_nb);
