@@ -46,7 +46,7 @@ struct FesGrid {
 // over enough blocks (slices) to fill the GPU, each slice's sums to its own
 // partial array, added in slice order afterwards: a fixed order.
 // Measured: sum-of-hills surface of 101 x 96 bins and 5,000 hills
-// 3,510 -> 238 us; fold of 20,000 hills into 200 x 200 nodes 145.6 -> 10.4 ms.
+// 3,508 -> 155 us; fold of 20,000 hills into 200 x 200 nodes 145.6 -> 6.5 ms.
 struct Axis {
     double lo, step, off;  // point i: lo + (i + off) step
     int n;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kFesThreads) k_fes_vmax(const double *V, long 
 // so a chunk's sums also run in time order.  A lone read-modify-write chain
 // per 32 samples is what bounds it; chunks are short (64 samples) as long as
 // the rows fit the workspace.  Measured (9,696 bins, 20,001 samples):
-// 33,600 -> 30 us with the row sum.
+// 33,600 -> 14 us.
 __global__ void __launch_bounds__(kFesThreads)
     k_fes_accum(const double *S, const double *V, long long T, int ncv, FesGrid g, double beta, const double *bmax,
                 int vblocks, long long per, int chunks, int nbins, double *rows)
