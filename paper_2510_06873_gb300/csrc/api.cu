@@ -456,9 +456,9 @@ metad_status setup_system(metad_ctx *c)
     }
     // FP64 partials: one per block of the CV sums (slot 0: CN, 1: Q6), three
     // per block of the force pass with the virial (slot 1, at most
-    // kPersistBlocks / 2 blocks), up to six per block of the hill kernel (slot
+    // kVirialBlocks blocks), up to six per block of the hill kernel (slot
     // 2), the neighbour statistics (slot 3)
-    y.part_stride = std::max(3 * std::min(metad::force_grid(n, y.ncv, y.pairs), metad::kPersistBlocks / 2),
+    y.part_stride = std::max(3 * std::min(metad::force_grid(n, y.ncv, y.pairs), metad::kVirialBlocks),
                              metad::kMaxBiasBlocks * (metad::kMaxCv + 1));
     return METAD_OK;
 }
@@ -533,7 +533,7 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
     const size_t rs = c->fp64 ? sizeof(double) : sizeof(float);
     const RecSizes r = rec_sizes(c);
     const bool two = c->p.n_cv == 2, pairs = y.pairs != 0;
-    const size_t rows = (size_t)y.max_nb * n;
+    const size_t rows = (size_t)y.max_nb * n, slices = (size_t)y.max_nb * metad::slice_rows(n);
     metad_status s;
     if (c->p.cv_kind != METAD_CV_COORDINATION) {
         // no neighbour list: CV atoms, gradient terms, reductions and hills
@@ -556,8 +556,8 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
         (s = alloc(&b.rank_xyz, y.ncell)) || (s = alloc(&b.xyz_rank, y.ncell)) ||
         (s = alloc(&y.nbr, pairs ? rows : 1)) || (s = alloc(&y.nn, n)) || (s = alloc(&y.nh, n)) ||
         (s = alloc(&b.wlb, two ? 2 * rs * rows : 1)) ||
-        (s = alloc(&b.pfb, pairs ? rs * 4 * rows : 1)) || (s = alloc(&b.geob, rs * 4 * rows)) ||
-        (s = alloc(&b.crossb, two ? rs * rows : 1)) ||
+        (s = alloc(&b.pfb, pairs ? rs * 4 * rows : 1)) || (s = alloc(&b.geob, rs * 4 * slices)) ||
+        (s = alloc(&b.crossb, two ? rs * slices : 1)) ||
         (s = alloc(&y.pos_ref, n)) ||
         (s = alloc(&y.vnbr, (size_t)y.max_vnb * n)) || (s = alloc(&y.vnn, n)) || (s = alloc(&y.flag, 1)) ||
         (s = alloc(&y.rebuilds, 1)) || (s = alloc(&y.Lref, 4)) || (s = alloc(&b.rb, rs * (r.q + r.b + r.h + (size_t)n * 3))) ||

@@ -34,10 +34,8 @@ namespace metad {
 // a float pair so no rounded constant biases the CV.
 // Layout: Y[0] m = 0; Y[2m-1] = P_m C_m; Y[2m] = P_m S_m, m = 1..6.
 struct YlmConst {
-    float pf[7][4];   // P_m(z) coefficients over z^2 powers (highest first)
-    float dpf[7][4];  // dP_m/dz likewise
+    float pf[7][4];  // P_m(z) coefficients over z^2 powers (highest first)
     double pd[7][4];
-    double dpd[7][4];
 };
 __constant__ YlmConst c_ylm;
 
@@ -47,12 +45,6 @@ template <>
 __device__ __forceinline__ float ylm_c<float>(int m, int k) { return c_ylm.pf[m][k]; }
 template <>
 __device__ __forceinline__ double ylm_c<double>(int m, int k) { return c_ylm.pd[m][k]; }
-template <typename real>
-__device__ __forceinline__ real ylm_dc(int m, int k);
-template <>
-__device__ __forceinline__ float ylm_dc<float>(int m, int k) { return c_ylm.dpf[m][k]; }
-template <>
-__device__ __forceinline__ double ylm_dc<double>(int m, int k) { return c_ylm.dpd[m][k]; }
 
 // P_m(z): degree 6 - m with the parity of 6 - m.
 template <typename real>
@@ -67,21 +59,6 @@ __device__ __forceinline__ void legendre_parts(real z, real P[7])
     P[4] = C_(4, 0) * z2 + C_(4, 1);
     P[5] = z * C_(5, 0);
     P[6] = C_(6, 0);
-#undef C_
-}
-
-template <typename real>
-__device__ __forceinline__ void legendre_dparts(real z, real D[7])
-{
-#define C_(m, k) ylm_dc<real>(m, k)
-    real z2 = z * z;
-    D[0] = z * ((C_(0, 0) * z2 + C_(0, 1)) * z2 + C_(0, 2));
-    D[1] = (C_(1, 0) * z2 + C_(1, 1)) * z2 + C_(1, 2);
-    D[2] = z * (C_(2, 0) * z2 + C_(2, 1));
-    D[3] = C_(3, 0) * z2 + C_(3, 1);
-    D[4] = z * C_(4, 0);
-    D[5] = C_(5, 0);
-    D[6] = real(0);
 #undef C_
 }
 
@@ -121,23 +98,32 @@ __device__ __forceinline__ void ylm13_acc(real x, real y, real z, real w, real v
 
 // sum_k h_k Y_k(u) and g = (I - u u^T) grad(sum_k h_k Y_k) / r in one loop,
 // without materialising the harmonics (fewer live registers in the pair pass).
+// dP_m/dz = P_{m+1}, so the parts serve the gradient too, and with
+// e_m = hc_m C_m + hs_m S_m a power adds P_m e_m to the sum and P_{m+1} e_m to
+// its z derivative: 11 operations a power, and none for the parts'
+// derivatives (14 and 12 when each was formed on its own).
 template <typename real>
 __device__ __forceinline__ real ylm13_dot_grad(real x, real y, real z, real inv_r, const real h[kNY], real g[3])
 {
-    real P[7], D[7], C[7], S[7];
+    real P[7], C[7], S[7];
     legendre_parts<real>(z, P);
-    legendre_dparts<real>(z, D);
     cs_powers<real>(x, y, C, S);
     real t = h[0] * P[0];
-    real gx = real(0), gy = real(0), gz = h[0] * D[0];
+    real gx = real(0), gy = real(0), gz = h[0] * P[1];
 #pragma unroll
     for (int m = 1; m <= 6; ++m) {
         const real hc = h[2 * m - 1], hs = h[2 * m];
-        t += hc * (P[m] * C[m]) + hs * (P[m] * S[m]);
-        const real pm = P[m] * real(m);
-        gx += pm * (hc * C[m - 1] + hs * S[m - 1]);
-        gy += pm * (hs * C[m - 1] - hc * S[m - 1]);
-        gz += D[m] * (hc * C[m] + hs * S[m]);
+        const real e = hc * C[m] + hs * S[m];
+        t += P[m] * e;
+        if (m < 6) gz += P[m + 1] * e;
+        if (m == 1) {  // C_0 = 1, S_0 = 0 (not folded by the compiler: y 0 is not 0 for every y)
+            gx += P[1] * hc;
+            gy += P[1] * hs;
+        } else {
+            const real pm = P[m] * real(m);
+            gx += pm * (hc * C[m - 1] + hs * S[m - 1]);
+            gy += pm * (hs * C[m - 1] - hc * S[m - 1]);
+        }
     }
     const real ug = x * gx + y * gy + z * gz;
     g[0] = (gx - ug * x) * inv_r;
@@ -344,12 +330,13 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
     if (a.ok) {
         const int nn = kFilter ? nn_f : s.nn[a.i];
         JW<real> *jwrow = reinterpret_cast<JW<real> *>(s.wl) + (size_t)a.i * s.max_nb;
+        const size_t e0 = entry_base(s, a.i);
         for (int k = a.l; k < nn; k += kG) {
             Vec3<real> d;
             real inv_r, w, dw;
             bool cn;
             int j;
-            cached_geometry<real>(s, (size_t)a.i * s.max_nb + k, d, inv_r, w, dw, cn, j);
+            cached_geometry<real>(s, e0 + entry_off(k), d, inv_r, w, dw, cn, j);
             if (cn) v[14] += w;
             v[13] += w;
             if (s.ncv == 2) {
@@ -573,7 +560,7 @@ __global__ void __launch_bounds__(kSumThreads) kb_cv_sum(BatchView v)
 // components 4l .. 4l + 3 (one 16 B load of each neighbour record per lane),
 // so a warp has eight atoms' gathers in flight.
 constexpr int kG4 = 4;
-static_assert(kRowAtoms * kG4 == kRowThreads, "four lanes per atom");
+static_assert(kRowAtoms * kG4 == kRowThreads && kRowThreads == kBlockAtoms, "four lanes per atom");
 constexpr int kRecQB = 32;  // FP32: q and b side by side, in chunks of four
 
 template <typename real>
@@ -657,10 +644,12 @@ __device__ __forceinline__ void cv_avg_group(const Sys &s, int g)
         inv_D = real(1) / (real(1) + R<real>(s.W)[i]);
         load4<real>(q, i, l, o);
         const JW<real> *jwrow = reinterpret_cast<const JW<real> *>(s.wl) + (size_t)i * s.max_nb;
+        JW<real> n0, n1;  // the entries one round ahead
+        load_jw2<real>(jwrow, 0, n0, n1);
 #pragma unroll 2
         for (int k = 0; k < nn; k += 2) {
-            JW<real> e0, e1;
-            load_jw2<real>(jwrow, k, e0, e1);
+            const JW<real> e0 = n0, e1 = n1;
+            if (k + 2 < nn) load_jw2<real>(jwrow, k + 2, n0, n1);
             const bool two = k + 1 < nn;
             real x[4], y[4] = {real(0), real(0), real(0), real(0)};
             load4<real>(q, e0.j, l, x);
@@ -702,7 +691,8 @@ __device__ __forceinline__ void cv_avg(const Sys &s, Blk k)
     for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_avg_group<real>(s, g);
 }
 
-// At 1M atoms: 10 blocks per SM (48 registers) 145 us, 12 (40) 154 us.
+// Blocks per SM: 10 (48 registers); at 1M atoms 8 / 9 / 10 / 12: 145 / 137 / 129
+// / 135 us, and 145 without the entries one round ahead.
 template <typename real>
 constexpr int kAvgBlocks = sizeof(real) == 4 ? 10 : 0;
 
@@ -770,6 +760,12 @@ __device__ __forceinline__ void store_h(const Sys &s, int i, int l, bool ok, con
 // same bits.  Entries go four at a time; a reduce-scatter over the group
 // leaves entry k0 + l's sum in lane l, so the group stores 16 contiguous
 // bytes.
+//
+// Bound by the latency of the gathered lines: a round's four loads a lane all
+// have to be in flight, which takes 64 registers, and the round's entries are
+// loaded one round ahead.  1M atoms: 197 us with 40 registers, 229 with 40 and
+// the entries after the records, 182 so.  (Eight lanes an atom with 16 B
+// loads, half the L1 wavefronts: 233 to 257 us.)
 __device__ __forceinline__ void adjoint_group(const Sys &s, int g, float)
 {
     const int i = g * kRowAtoms + (threadIdx.x / kG4), l = threadIdx.x & (kG4 - 1);
@@ -780,11 +776,18 @@ __device__ __forceinline__ void adjoint_group(const Sys &s, int g, float)
         load_qb(qb, i, l, q, o);
         const int nn = s.nn[i];
         const JW<float> *jwrow = reinterpret_cast<const JW<float> *>(s.wl) + (size_t)i * s.max_nb;
-        float *crow = R<float>(s.cross) + (size_t)i * s.max_nb;
+        float *crow = R<float>(s.cross) + entry_base(s, i);
+        JW<float> n4[4];  // the entries one round ahead (a row holds at least four)
+        load_jw2<float>(jwrow, 0, n4[0], n4[1]);
+        load_jw2<float>(jwrow, 2, n4[2], n4[3]);
         for (int k0 = 0; k0 < nn; k0 += 4) {
             JW<float> e4[4];
-            load_jw2<float>(jwrow, k0, e4[0], e4[1]);
-            load_jw2<float>(jwrow, k0 + 2, e4[2], e4[3]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e4[u] = n4[u];
+            if (k0 + 4 < nn) {
+                load_jw2<float>(jwrow, k0 + 4, n4[0], n4[1]);
+                load_jw2<float>(jwrow, k0 + 6, n4[2], n4[3]);
+            }
             float p[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -805,7 +808,7 @@ __device__ __forceinline__ void adjoint_group(const Sys &s, int g, float)
                 }
             }
             const float t = group4_reduce_scatter<float>(p, l);
-            if (k0 + l < nn) crow[k0 + l] = t;
+            if (k0 + l < nn) crow[entry_off(k0) + l] = t;
         }
     }
     store_h<float>(s, i, l, ok, acc, o, q);
@@ -824,7 +827,7 @@ __device__ __forceinline__ void adjoint_group(const Sys &s, int g, double)
         load4<double>(R<double>(s.q), i, l, q);
         const int nn = s.nn[i];
         const JW<double> *jwrow = reinterpret_cast<const JW<double> *>(s.wl) + (size_t)i * s.max_nb;
-        double *crow = R<double>(s.cross) + (size_t)i * s.max_nb;
+        double *crow = R<double>(s.cross) + entry_base(s, i);
         for (int k0 = 0; k0 < nn; k0 += 4) {
             JW<double> e4[4];
             load_jw2<double>(jwrow, k0, e4[0], e4[1]);
@@ -844,7 +847,7 @@ __device__ __forceinline__ void adjoint_group(const Sys &s, int g, double)
                 }
             }
             const double t = group4_reduce_scatter<double>(p, l);
-            if (k0 + l < nn) crow[k0 + l] = t;
+            if (k0 + l < nn) crow[entry_off(k0) + l] = t;
         }
     }
     store_h<double>(s, i, l, ok, acc, o, q);
@@ -857,12 +860,12 @@ __device__ __forceinline__ void adjoint(const Sys &s, Blk k)
     for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) adjoint_group(s, g, real(0));
 }
 
-// Resident blocks per SM the adjoint is compiled for (none in FP64): at 1M
-// atoms 12 (40 registers) 200 us, 10 (48) 214 us.  Blocks of 256 / 512 / 1024
-// threads 202 / 206 / 230 us: the neighbours' records are found in L2 either
-// way, and small blocks balance better.
+// Resident blocks per SM the adjoint is compiled for (none in FP64): 1M atoms
+// at 7 / 8 / 9 / 10 / 12: 198 / 182 / 199 / 197 / 324 us (the last two spill).
+// Blocks of 256 / 512 / 1024 threads measured no faster: the neighbours'
+// records are found in L2 either way, and small blocks balance better.
 template <typename real>
-constexpr int kAdjointBlocks = sizeof(real) == 4 ? 12 : 0;
+constexpr int kAdjointBlocks = sizeof(real) == 4 ? 8 : 0;
 
 template <typename real>
 __global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) k_adjoint(Sys s) { adjoint<real>(s, own_blk()); }
@@ -997,11 +1000,11 @@ __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real
 // row and no pass to add the slots up: what bound the half-row form was its
 // scattered line accesses (per pair four for h_j, one each for the mirror
 // entry's place, its cross half and its force slot), and its 32 B of slots
-// per entry were most of the step's DRAM traffic.  Bound by the L1's
-// wavefronts (68% at 262,144 atoms) and instruction issue (54%).
-// Measured against the half-row pass and the slot sums: 1M atoms 300 -> 268
-// us, and the forward pass, without the mirror records, 309 -> 271 us (and
-// 200 us less after a rebuild); 27,648 atoms 36.4 -> 14.3 us.
+// per entry were most of the step's DRAM traffic.  Bound by instruction issue
+// (about 55%) and the latency of the gathered records.  1M atoms: half rows
+// and slot sums 300 us and more, 268 us in a row per atom; 251 with the parts'
+// derivatives shared (ylm13_dot_grad), 235 with the rows of eight atoms
+// interleaved (entry_slot), 214 with the streamed entries one round ahead.
 template <bool kVir>
 __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
 {
@@ -1010,25 +1013,43 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
     const float cn_fac = fac[0], V2 = fac[1];
     const int l = threadIdx.x & (kG4 - 1);
     const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
+    const float *hh = R<float>(s.h);
     RunSum<float> vx, vy, vz;
     for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) {
         const int i = g * kRowAtoms + (threadIdx.x / kG4);
         float fx = 0.0f, fy = 0.0f, fz = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
         if (i < s.n) {
             const int nn = s.nn[i];
-            const float *hh = R<float>(s.h), *crow = R<float>(s.cross) + (size_t)i * s.max_nb;
+            const size_t row = entry_base(s, i) + l;
+            const float4 *grow = reinterpret_cast<const float4 *>(s.geo) + row;
+            const float *crow = R<float>(s.cross) + row;
             float hi[kRec];
             load_rec<float>(hh, i, hi);
+            // the streamed entries one round ahead: their latency is DRAM's
+            float4 geo_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            float cross_next = 0.0f;
+            if (l < nn) {
+                geo_next = __ldcs(grow);
+                cross_next = __ldcs(crow);
+            }
             for (int e = l; e < nn; e += kG4) {
-                Vec3<float> d;
-                float inv_r, w, dw;
-                bool cn;
+                const float4 geo = geo_next;
+                const float cross = cross_next;
                 int j;
-                cached_geometry<float, true>(s, (size_t)i * s.max_nb + e, d, inv_r, w, dw, cn, j);
+                bool cn;
+                untag(__float_as_uint(geo.w), j, cn);
                 float hj[kRec];
                 load_rec<float>(hh, j, hj);
-                const Vec3<float> G =
-                    pair_gradient<float>(d, inv_r, w, dw, cn ? cn_fac * dw : 0.0f, V2, __ldcs(crow + e), hi, hj);
+                if (e + kG4 < nn) {
+                    geo_next = __ldcs(grow + entry_off(e - l + kG4));
+                    cross_next = __ldcs(crow + entry_off(e - l + kG4));
+                }
+                const Vec3<float> d{geo.x, geo.y, geo.z};
+                const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+                const float inv_r = rsqrt_r<float>(r2);
+                float w, dw;
+                switch_eval<float>(s, r2 * inv_r, w, dw);
+                const Vec3<float> G = pair_gradient<float>(d, inv_r, w, dw, cn ? cn_fac * dw : 0.0f, V2, cross, hi, hj);
                 fx += G.x;
                 fy += G.y;
                 fz += G.z;
@@ -1052,10 +1073,12 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
     if (kVir) virial_finish<float>(s, k, vx, vy, vz);
 }
 
-// Resident blocks per SM: at 1M atoms 9 (56 registers) 268 us, 8 (64) 279 us;
-// the virial's instance is left alone.
+// Resident blocks per SM: 8 (64 registers) in the plain pass, 214 us at 1M
+// atoms, 9 (56) 213, 7 (72) 225; with the virial 7 (72): 250,001 atoms 67.7 us,
+// 8 (64, spilling) 69.7, 6 71.2, and 100 when 86 registers left five of the
+// grid's eight blocks per SM resident.
 template <bool kVir>
-constexpr int kForceBlocks = kVir ? 0 : 9;
+constexpr int kForceBlocks = kVir ? 7 : 8;
 
 template <bool kVir>
 __global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) k_force_rows(Sys s) { force_rows<kVir>(s, own_blk()); }
@@ -1122,7 +1145,7 @@ __device__ __forceinline__ void pair_force(const Sys &s, int i, int k, double cn
     double inv_r, w, dw;
     bool cn;
     int j;
-    cached_geometry<double, true>(s, (size_t)i * s.max_nb + k, d, inv_r, w, dw, cn, j);
+    cached_geometry<double, true>(s, entry_slot(s, i, k), d, inv_r, w, dw, cn, j);
     int kk = -1;
     const int nhj = s.nh[j], nnj = s.nn[j];
     const int *rj = nbr_row(s, j);
@@ -1143,7 +1166,7 @@ __device__ __forceinline__ void pair_force(const Sys &s, int i, int k, double cn
     load_rec<double>(hh, j, hj);
     // cross term b_i.q_j + b_j.q_i: the halves the adjoint pass stored
     // in entry ij (b_j.q_i) and in its mirror ji (b_i.q_j)
-    const double cross = cc[(size_t)i * s.max_nb + k] + cc[(size_t)j * s.max_nb + kk];
+    const double cross = cc[entry_slot(s, i, k)] + cc[entry_slot(s, j, kk)];
     const Vec3<double> G = pair_gradient<double>(d, inv_r, w, dw, cn ? cn_fac * dw : 0.0, V2, cross, hi, hj);
     if (kVir) {  // (dV/dd)_a d_a of this pair
         vx.add(G.x * d.x);
@@ -1442,11 +1465,6 @@ void set_ylm_constants(cudaStream_t st)
         for (int p = deg; p >= 0; p -= 2, ++t) {
             h.pd[m][t] = cur[p];
             h.pf[m][t] = (float)cur[p];
-        }
-        t = 0;
-        for (int p = deg; p >= 1; p -= 2, ++t) {
-            h.dpd[m][t] = cur[p] * p;
-            h.dpf[m][t] = (float)(cur[p] * p);
         }
     }
     cudaMemcpyToSymbolAsync(c_ylm, &h, sizeof(h), 0, cudaMemcpyHostToDevice, st);

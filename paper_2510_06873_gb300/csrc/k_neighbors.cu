@@ -534,7 +534,7 @@ __global__ void k_export_pairs(Sys s, long long *pairs, int *count)
         Vec3<real> d;
         bool cn;
         int j;
-        load_geo<real>(s, (size_t)i * s.max_nb + k, d, cn, j);
+        load_geo<real>(s, entry_slot(s, i, k), d, cn, j);
         int uj = s.perm[j];
         if (ui < uj) {
             int slot = atomicAdd(count, 1);
@@ -599,7 +599,7 @@ int grid_blocks(const Sys &s, int kind, int persist_cap)
         // with the virial its grid fixes the order of the virial's partials:
         // by N only, few enough for the last block to add
         const int g = force_grid(s.n, s.ncv, s.pairs);
-        if (s.virial) return g < kPersistBlocks / 2 ? g : kPersistBlocks / 2;
+        if (s.virial) return g < kVirialBlocks ? g : kVirialBlocks;
         return persist_cap > 0 && persist_cap < g ? persist_cap : g;
     }
     case GK_SUM: return sum_blocks(s.n);

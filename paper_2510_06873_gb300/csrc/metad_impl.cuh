@@ -86,10 +86,10 @@ struct Sys {
     int *nh;               // [n] entries with j > i
     void *wl;              // JW<real> [n][max_nb]: neighbour and switch weight of each entry
     void *pairF;           // FP64, two CVs: [n][max_nb][4], G_ij in i's entry of j, -G_ji in the others
-    void *cross;           // real [n][max_nb], two CVs: b_i.q_j + b_j.q_i of each exact entry
+    void *cross;           // two CVs, real of each entry (entry_slot): b_i.q_j + b_j.q_i
                            // (FP64: its half b_j.q_i)
-    void *geo;             // real [n][max_nb][4]: r_j - r_i (minimum image) and the CN mask
-                           // of each exact entry, written by the exact filter
+    void *geo;             // real[4] of each entry (entry_slot): r_j - r_i (minimum image) and
+                           // the CN mask, written by the exact filter
     // Verlet list (cutoff rc + skin, built at the reference positions)
     float4 *pos_ref;       // sorted positions at the last rebuild
     int *vnbr;             // [n][max_vnb]
@@ -583,6 +583,11 @@ __host__ __device__ inline int force_grid(int n, int ncv, int pairs)
 // most kPersistBlocks blocks, walking their work grid-stride.
 constexpr int kPersistBlocks = 152 * 16;
 
+// Blocks of the force pass with the virial, at most: the seven per SM that its
+// registers leave resident, walking their work, so that no part of a second
+// wave is left over and the last block has few partials to add.
+constexpr int kVirialBlocks = 152 * 7;
+
 // The it-th work item (atom group or chunk) of block b of nb: items b,
 // b + nb, b + 2 nb, ...  The items of one sweep form one compact window of
 // the Morton order, so the records they gather stay in L2.  (Mapping the
@@ -746,6 +751,25 @@ __device__ __forceinline__ void load_geo<double, false>(const Sys &s, size_t slo
     untag((unsigned)__double_as_longlong(b.y), j, cn);
 }
 
+// Where the exact rows keep entry k of atom i (geometry, cross terms): the rows
+// of eight consecutive atoms are interleaved by chunks of four entries, so that
+// what the lane groups of a warp read or write at the same k lies together.
+// The L1 serves a warp's access a 128 B line at a time, and with a row per atom
+// each of the eight groups touches a line of its own, for 16 or 64 B of it
+// (force pass, 1M atoms: 254 -> 235 us).  Row capacities are multiples of four, and the arrays
+// hold whole slices of eight atoms.  (The entries of the gather passes, JW,
+// stay a row per atom: a line of a row is then fetched once for sixteen
+// entries, where interleaved pairs fetched one every round: Q6 pass 145 ->
+// 188 us, adjoint 197 -> 313.)
+constexpr int kSlice = 8;
+__host__ __device__ inline size_t slice_rows(int n) { return ((size_t)n + kSlice - 1) / kSlice * kSlice; }
+__device__ __forceinline__ size_t entry_base(const Sys &s, int i)
+{
+    return (size_t)(i & ~(kSlice - 1)) * s.max_nb + 4 * (i & (kSlice - 1));
+}
+__device__ __forceinline__ int entry_off(int k) { return (k >> 2) * (4 * kSlice) + (k & 3); }
+__device__ __forceinline__ size_t entry_slot(const Sys &s, int i, int k) { return entry_base(s, i) + entry_off(k); }
+
 // One exact entry for the gather passes: the neighbour and the switch
 // weight side by side, read with one load.
 template <typename real>
@@ -760,7 +784,8 @@ template <typename real, int kPart>
 __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
     const int *vrow = s.vnbr + (size_t)(a.ok ? a.i : 0) * s.max_vnb;
-    const size_t row0 = (size_t)(a.ok ? a.i : 0) * s.max_nb;
+    const int i = a.ok ? a.i : 0;
+    const size_t e0 = entry_base(s, i), row0 = (size_t)i * s.max_nb;
     const unsigned lt = (1u << a.l) - 1u;
     for (int base = 0; base < vmax; base += kG) {
         const int k = base + a.l;
@@ -774,7 +799,7 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
         const int at = cnt + __popc(gm & lt);
         if (in && at < s.max_nb) {
             if (kPart != 0) s.nbr[row0 + at] = j;
-            store_geo<real>(s, row0 + at, d, pi, pj, j);
+            store_geo<real>(s, e0 + entry_off(at), d, pi, pj, j);
         }
         cnt += __popc(gm);
     }
