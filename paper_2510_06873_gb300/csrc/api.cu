@@ -404,6 +404,10 @@ metad_status setup_system(metad_ctx *c)
     y.rc2_lo = (float)(y.rc2 * (1.0 - 3e-5));
     y.rc2_hi = (float)(y.rc2 * (1.0 + 3e-5));
     {
+        const double half = 0.5 * std::min(c->p.box[0], std::min(c->p.box[1], c->p.box[2]));
+        y.wrap2 = (float)(half * half * (1.0 - 1e-5));
+    }
+    {
         const double rv = c->p.rc + c->p.skin;
         y.rv2 = (float)(rv * rv * (1.0 + 1e-4));
         const double half = 0.5 * c->p.skin * (1.0 - 1e-3);

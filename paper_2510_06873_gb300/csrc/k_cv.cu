@@ -262,14 +262,14 @@ __device__ __forceinline__ void cached_geometry(const Sys &s, size_t slot, Vec3<
     switch_eval<real>(s, r2 * inv_r, w, dw);
 }
 
-// Butterfly reduce-scatter of 16 values over the kG lanes of a group:
-// afterwards lane l holds the group sums of values 2l and 2l + 1 in v[0], v[1].
-template <typename real>
+// Butterfly reduce-scatter of 16 values over the G lanes of a group:
+// afterwards lane l holds the group sums of values l 16/G .. in v[0] ...
+template <typename real, int G>
 __device__ __forceinline__ void reduce_scatter16(real v[kRec], int l)
 {
     int len = kRec;
 #pragma unroll
-    for (int o = kG / 2; o >= 1; o >>= 1) {
+    for (int o = G / 2; o >= 1; o >>= 1) {
         len >>= 1;
         const bool upper = (l & o) != 0;
 #pragma unroll
@@ -293,21 +293,17 @@ __device__ __forceinline__ real group_sum(real v)
     return v;
 }
 
-template <typename real>
-__device__ __forceinline__ real group_get(real v, int src_lane)
+// Components c l .. c l + c - 1 of record i of kLen (c = 2 or 4).
+template <typename real, int kLen, int c>
+__device__ __forceinline__ void store_part(real *base, int i, int l, const real v[])
 {
-    const int base = (threadIdx.x & 31) & ~(kG - 1);
-    return __shfl_sync(0xffffffffu, v, base + src_lane);
-}
-
-// Components (2l, 2l + 1) of a record of kLen.
-template <typename real, int kLen>
-__device__ __forceinline__ void store_pair(real *base, int i, int l, real a, real b)
-{
-    struct alignas(2 * sizeof(real)) P2 {
-        real a, b;
+    struct alignas(c * sizeof(real) < 16 ? c * sizeof(real) : 16) Part {
+        real v[c];
     };
-    reinterpret_cast<P2 *>(base + (size_t)i * kLen)[l] = P2{a, b};
+    Part p;
+#pragma unroll
+    for (int k = 0; k < c; ++k) p.v[k] = v[k];
+    reinterpret_cast<Part *>(base + (size_t)i * kLen)[l] = p;
 }
 
 __device__ __forceinline__ const int *nbr_row(const Sys &s, int i) { return s.nbr + (size_t)i * s.max_nb; }
@@ -319,11 +315,11 @@ __device__ __forceinline__ const int *nbr_row(const Sys &s, int i) { return s.nb
 // With kFilter the exact row is first compacted from the Verlet row.
 constexpr int kCnRec = 8;  // fx fy fz, vx vy vz, 2 unused
 
-template <typename real, bool kFilter>
+template <typename real, bool kFilter, int G>
 __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
 {
     int nn_f = 0;
-    if (kFilter) nn_f = filter_row<real>(s, a);
+    if (kFilter) nn_f = filter_row<real, G>(s, a);
     real v[kRec];  // 0..12: sum w Y_m (one CV: 0..5 as above) ; 13: W ; 14: CN
 #pragma unroll
     for (int m = 0; m < kRec; ++m) v[m] = real(0);
@@ -331,7 +327,7 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
         const int nn = kFilter ? nn_f : s.nn[a.i];
         JW<real> *jwrow = reinterpret_cast<JW<real> *>(s.wl) + (size_t)a.i * s.max_nb;
         const size_t e0 = entry_base(s, a.i);
-        for (int k = a.l; k < nn; k += kG) {
+        for (int k = a.l; k < nn; k += G) {
             Vec3<real> d;
             real inv_r, w, dw;
             bool cn;
@@ -355,33 +351,44 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
             }
         }
     }
-    reduce_scatter16<real>(v, a.l);
-    // lane 6 holds (13: W, ...) in v[1]; lane 7 holds (14: CN, 15) in v[0]
-    const real W = group_get<real>(v[1], 6);
+    reduce_scatter16<real, G>(v, a.l);
+    // lane l holds values c l .. c l + c - 1; 13: W, 14: CN
+    constexpr int c = kRec / G;
+    const real W = __shfl_sync(0xffffffffu, v[13 % c], ((threadIdx.x & 31) & ~(G - 1)) + 13 / c);
     if (a.ok) {
-        if (a.l == 7) R<real>(s.cn)[a.i] = v[0];
+        if (a.l == 14 / c) R<real>(s.cn)[a.i] = v[14 % c];
         if (s.ncv == 2) {
-            if (a.l == 6) R<real>(s.W)[a.i] = W;
+            if (a.l == 13 / c) R<real>(s.W)[a.i] = W;
             const real inv_W = W > real(0) ? real(1) / W : real(0);
-            real q0 = v[0] * inv_W, q1 = v[1] * inv_W;
-            if (a.l == 6) q1 = real(0);
-            if (a.l == 7) q0 = q1 = real(0);
-            store_pair<real, kRec>(R<real>(s.q), a.i, a.l, q0, q1);
-        } else if (a.l < kCnRec / 2) {
-            store_pair<real, kCnRec>(R<real>(s.q), a.i, a.l, v[0], v[1]);
+            real q[c];
+#pragma unroll
+            for (int k = 0; k < c; ++k) q[k] = c * a.l + k < kNY ? v[k] * inv_W : real(0);
+            store_part<real, kRec, c>(R<real>(s.q), a.i, a.l, q);
+        } else if (a.l < kCnRec / c) {
+            store_part<real, kCnRec, c>(R<real>(s.q), a.i, a.l, v);
         }
     }
 }
 
+// Lanes per atom: four in the FP32 pass.  Bound by instruction issue (64 to
+// 69%); with eight lanes the last round of a row leaves more lanes idle and
+// the reduction over the lanes costs twice as much an atom.  1M atoms 264 ->
+// 220 us, 262,144 76 -> 66, 27,648 14.3 -> 14.7 (its warps halve, too few to
+// hide the loads' latency).  FP64 keeps eight: its arithmetic is the bound.
+template <typename real>
+constexpr int kFwdLanes = sizeof(real) == 4 ? 4 : kG;
+
 template <typename real, bool kFilter>
 __device__ __forceinline__ void cv_fwd(const Sys &s, Blk k)
 {
-    const int groups = group_grid(s.n);
-    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_fwd_group<real, kFilter>(s, atom_lane_at(s, g));
+    constexpr int G = kFwdLanes<real>, atoms = kBlockAtoms / G;
+    const int groups = (s.n + atoms - 1) / atoms;
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it)
+        cv_fwd_group<real, kFilter, G>(s, atom_lane_at<G>(s, g));
 }
 
-// Resident blocks per SM: 12 in FP32 (40 registers), none asked for in FP64
-// (40 registers spill there).
+// Resident blocks per SM: 12 in FP32 (40 registers; 10 / 14 / 16: 228 / 230 /
+// 230 us at 1M atoms), none asked for in FP64 (40 registers spill there).
 template <typename real>
 constexpr int kFwdBlocks = sizeof(real) == 4 ? 12 : 0;
 
@@ -1282,7 +1289,7 @@ __global__ void k_per_atom_out(Sys s, double *out)
 
 void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st)
 {
-    const int nb = group_grid(s.n);
+    const int nb = grid_blocks(s, fp64 ? GK_GROUPS : GK_ROWS, 0);  // by kFwdLanes
     if (fp64) {
         if (fused_filter)
             k_cv_fwd<double, true><<<nb, kBlockAtoms, 0, st>>>(s);
@@ -1379,7 +1386,7 @@ void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &
         kb_cv_fwd<double><<<group_total, kBlockAtoms, 0, st>>>(groups);
         if (ncv == 2) kb_cv_avg<double><<<row_total, kRowThreads, 0, st>>>(rows);
     } else {
-        kb_cv_fwd<float><<<group_total, kBlockAtoms, 0, st>>>(groups);
+        kb_cv_fwd<float><<<row_total, kBlockAtoms, 0, st>>>(rows);
         if (ncv == 2) kb_cv_avg<float><<<row_total, kRowThreads, 0, st>>>(rows);
     }
 }

@@ -434,7 +434,7 @@ template <typename real>
 __global__ void __launch_bounds__(kBlockAtoms) k_filter(Sys s)
 {
     const int groups = group_grid(s.n);
-    for (int blk = blockIdx.x; blk < groups; blk += gridDim.x) filter_row<real>(s, atom_lane_at(s, blk));
+    for (int blk = blockIdx.x; blk < groups; blk += gridDim.x) filter_row<real, kG>(s, atom_lane_at(s, blk));
 }
 
 

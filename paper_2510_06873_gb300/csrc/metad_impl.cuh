@@ -57,6 +57,7 @@ struct Sys {
     // neighbour predicate: r^2 < rc^2 decided in FP64 inside the guard band
     double rc2;
     float rc2_lo, rc2_hi;
+    float wrap2;           // below (half the shortest box length)^2, with margin
     // switch
     int sw_n, sw_m, stretch;
     float sw_nf;                 // sw_n and N as floating point: an int
@@ -607,20 +608,22 @@ struct AtomLane {
     bool ok;  // i < n
 };
 
+template <int G = kG>
 __device__ __forceinline__ AtomLane atom_lane_at(const Sys &s, int blk)
 {
     AtomLane a;
-    a.i = blk * kAtomsPerBlock + (threadIdx.x / kG);
-    a.l = threadIdx.x & (kG - 1);
+    a.i = blk * (kBlockAtoms / G) + (threadIdx.x / G);
+    a.l = threadIdx.x & (G - 1);
     a.ok = a.i < s.n;
     return a;
 }
 
 
+template <int G>
 __device__ __forceinline__ unsigned group_mask_bits(unsigned ballot)
 {
-    const int base = (threadIdx.x & 31) & ~(kG - 1);
-    return (ballot >> base) & ((1u << kG) - 1u);
+    const int base = (threadIdx.x & 31) & ~(G - 1);
+    return (ballot >> base) & ((1u << G) - 1u);
 }
 
 // Exact FP64 pair test: r^2 = (dx*dx + dy*dy) + dz*dz < rc^2 on the
@@ -643,18 +646,6 @@ __device__ __forceinline__ bool pair_exact(const Sys &s, float4 pi, float4 pj)
     return pair_exact_fp64(pi, pj, s.L[0], s.L[1], s.L[2], s.rc2);
 }
 
-// displacement<float> for code where the whole warp is converged: the plain
-// difference, and the boundary fix only when some lane of the warp needs it
-// (a vote), instead of both fixes evaluated for every pair.  The same bits:
-// mi_axis returns the plain difference exactly when |d| <= L/2.
-__device__ __forceinline__ Vec3<float> displacement_warp(const Sys &s, float4 pi, float4 pj)
-{
-    Vec3<float> d{pj.x - pi.x, pj.y - pi.y, pj.z - pi.z};
-    const bool wrap = fabsf(d.x) > s.halfL[0] || fabsf(d.y) > s.halfL[1] || fabsf(d.z) > s.halfL[2];
-    if (__any_sync(0xffffffffu, wrap)) d = displacement<float>(s, pi, pj);
-    return d;
-}
-
 // The float32 estimate decides every candidate outside a relative guard band
 // of 3e-5 around rc^2; inside it the FP64 definition decides.  d is the
 // float32 displacement of the pair.
@@ -666,16 +657,23 @@ __device__ __forceinline__ bool pair_in(const Sys &s, float4 pi, float4 pj, cons
     return pair_exact(s, pi, pj);
 }
 
-// pair_in for code where the whole warp is converged: the FP64 decision runs
-// only when some lane of the warp has a candidate inside the guard band (a
-// vote), as a warp-uniform branch.  The same decisions as pair_in.
-__device__ __forceinline__ bool pair_in_warp(const Sys &s, bool valid, float4 pi, float4 pj, const Vec3<float> &d)
+// displacement<float> and pair_in for code where the whole warp is converged:
+// the plain difference decides unless its square lies in the guard band or
+// above wrap2, which it does whenever some axis needs the minimum image; then
+// the full forms run, behind one warp vote.  The same bits and decisions: the
+// full displacement is the plain difference on an axis within half the box,
+// and one beyond it has a square above the band (half the box is at least rc).
+__device__ __forceinline__ bool pair_in_warp(const Sys &s, bool valid, float4 pi, float4 pj, Vec3<float> &d)
 {
+    d = Vec3<float>{pj.x - pi.x, pj.y - pi.y, pj.z - pi.z};
     const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
     bool in = valid && r2 < s.rc2_lo;
-    const bool band = valid && r2 >= s.rc2_lo && r2 <= s.rc2_hi;
-    if (__any_sync(0xffffffffu, band)) {
-        if (band) in = pair_exact(s, pi, pj);
+    const bool full = valid && r2 >= s.rc2_lo && (r2 <= s.rc2_hi || r2 > s.wrap2);
+    if (__any_sync(0xffffffffu, full)) {
+        if (full) {
+            d = displacement<float>(s, pi, pj);
+            in = pair_in(s, pi, pj, d);
+        }
     }
     return in;
 }
@@ -778,24 +776,32 @@ struct alignas(2 * sizeof(real)) JW {
     real w;
 };
 
-// Eight candidates of a Verlet row a round, the accepted ones compacted by
+// G candidates of a Verlet row a round, the accepted ones compacted by
 // ballot.  kPart: 0 every exact entry, 1 those with j > i, 2 those with j < i.
-template <typename real, int kPart>
+// The rows and positions are not written by this kernel (__ldg: the loads need
+// not wait for the stores), and a round's indices are loaded one ahead.
+template <typename real, int kPart, int G>
 __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
-    const int *vrow = s.vnbr + (size_t)(a.ok ? a.i : 0) * s.max_vnb;
     const int i = a.ok ? a.i : 0;
+    const int *vrow = s.vnbr + (size_t)i * s.max_vnb;
     const size_t e0 = entry_base(s, i), row0 = (size_t)i * s.max_nb;
     const unsigned lt = (1u << a.l) - 1u;
-    for (int base = 0; base < vmax; base += kG) {
+    int j1 = a.l < vn ? __ldg(vrow + a.l) : i;
+    float4 p1 = __ldg(s.pos_s + j1);
+    int j2 = a.l + G < vn ? __ldg(vrow + a.l + G) : i;
+    for (int base = 0; base < vmax; base += G) {
         const int k = base + a.l;
         const bool valid = k < vn;
-        const int j = valid ? vrow[k] : 0;
-        const float4 pj = valid ? s.pos_s[j] : pi;
-        const Vec3<float> d = displacement_warp(s, pi, pj);  // every lane: a warp vote inside
+        const int j = j1;
+        const float4 pj = p1;
+        j1 = j2;
+        p1 = __ldg(s.pos_s + j1);
+        j2 = k + 2 * G < vn ? __ldg(vrow + k + 2 * G) : i;
         const bool part = kPart == 0 || (kPart == 1 ? j > a.i : j < a.i);
-        const bool in = pair_in_warp(s, valid && part, pi, pj, d);
-        const unsigned gm = group_mask_bits(__ballot_sync(0xffffffffu, in));
+        Vec3<float> d;
+        const bool in = pair_in_warp(s, valid && part, pi, pj, d);  // every lane: a warp vote inside
+        const unsigned gm = group_mask_bits<G>(__ballot_sync(0xffffffffu, in));
         const int at = cnt + __popc(gm & lt);
         if (in && at < s.max_nb) {
             if (kPart != 0) s.nbr[row0 + at] = j;
@@ -809,7 +815,7 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
 // The exact row of atom a.i from its Verlet row.  For the FP64 two-CV pair
 // pass the j > i entries come first, in a sweep of their own, and the row's
 // indices are kept (it searches them); everyone else reads j from the tags.
-template <typename real>
+template <typename real, int G>
 __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
 {
     const int vn = a.ok ? s.vnn[a.i] : 0;
@@ -817,11 +823,11 @@ __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
     const int vmax = __reduce_max_sync(0xffffffffu, vn);
     int cnt;
     if (sizeof(real) == 8 && s.ncv == 2) {
-        const int nh = filter_sweep<real, 1>(s, a, vn, vmax, pi, 0);
-        cnt = filter_sweep<real, 2>(s, a, vn, vmax, pi, nh);
+        const int nh = filter_sweep<real, 1, G>(s, a, vn, vmax, pi, 0);
+        cnt = filter_sweep<real, 2, G>(s, a, vn, vmax, pi, nh);
         if (a.ok && a.l == 0) s.nh[a.i] = min(nh, s.max_nb);
     } else {
-        cnt = filter_sweep<real, 0>(s, a, vn, vmax, pi, 0);
+        cnt = filter_sweep<real, 0, G>(s, a, vn, vmax, pi, 0);
     }
     if (a.ok && a.l == 0) {
         if (cnt > s.max_nb) set_err(s, kErrCapacity);
