@@ -97,8 +97,9 @@ void drop_graph(metad_ctx::StepGraph &g)
     g.patchable = false;
 }
 
-// The captured kernel nodes that take only the descriptor; false when some
-// kernel node takes other arguments (its buffers cannot be patched).
+// The captured kernel nodes whose buffers a replay has to patch (each patch is
+// two driver calls: four or five nodes, not all 13); false when some kernel
+// node takes other arguments than the descriptor.
 bool collect_step_nodes(cudaGraph_t graph, std::vector<metad_ctx::StepNode> &out)
 {
     size_t count = 0;
@@ -112,10 +113,11 @@ bool collect_step_nodes(cudaGraph_t graph, std::vector<metad_ctx::StepNode> &out
         if (type != cudaGraphNodeTypeKernel) continue;
         cudaKernelNodeParams kp = {};
         if (cudaGraphKernelNodeGetParams(n, &kp) != cudaSuccess || !kp.kernelParams) return false;
-        if (!(metad::sys_kernel_neighbors(kp.func) || metad::sys_kernel_cv(kp.func) ||
-              metad::sys_kernel_bias(kp.func) || metad::sys_kernel_gcv(kp.func)))
-            return false;
-        out.push_back({n, *static_cast<const metad::Sys *>(kp.kernelParams[0])});
+        const int kind = metad::sys_kernel_neighbors(kp.func) | metad::sys_kernel_cv(kp.func) |
+                         metad::sys_kernel_bias(kp.func) | metad::sys_kernel_gcv(kp.func);
+        if (kind == metad::kNotSys) return false;
+        // the others keep the buffers of the capture in their descriptors, unread
+        if (kind == metad::kSysIo) out.push_back({n, *static_cast<const metad::Sys *>(kp.kernelParams[0])});
     }
     return true;
 }

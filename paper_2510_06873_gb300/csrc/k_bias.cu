@@ -21,6 +21,7 @@ namespace {
 // well-tempered hill there as hill s.K.
 __global__ void __launch_bounds__(kBlockBias) k_bias(Sys s)
 {
+    chain_enter();
     hill_sum<kMaxCv>(s, own_blk(), s.bias_x, s.bias_out, s.deposit);
 }
 
@@ -28,6 +29,7 @@ __global__ void __launch_bounds__(kBlockBias) k_bias(Sys s)
 // hill there (deposit 1; only systems with s.deposit have blocks).
 __global__ void __launch_bounds__(kBlockBias) kb_bias(BatchView v, int deposit)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     hill_sum<kMaxCv>(s, k, s.scal + kS0, s.scal + (deposit ? kDepV : kV), deposit);
@@ -95,12 +97,12 @@ void launch_bias(const Sys &s, int K, const double *x_dev, double *out_dev, int 
     t.bias_x = x_dev;
     t.bias_out = out_dev;
     t.deposit = deposit;
-    k_bias<<<bias_blocks(K), kBlockBias, 0, st>>>(t);
+    chained_live(k_bias, bias_blocks(K), kBlockBias, st, t);
 }
 
 void launch_batch_bias(const BatchView &v, int total, int deposit, cudaStream_t st)
 {
-    if (total > 0) kb_bias<<<total, kBlockBias, 0, st>>>(v, deposit);
+    if (total > 0) chained_live(kb_bias, total, kBlockBias, st, v, deposit);
 }
 
 void launch_batch_collect(const BatchView &v, double *out, cudaStream_t st)
@@ -117,14 +119,14 @@ void launch_grid_fold(const Sys &s, int K, cudaStream_t st)
 
 // The kernels of this file whose only argument is the system descriptor
 // (a captured step's nodes of these can take new I/O buffers in place).
-bool sys_kernel_bias(const void *func)
+SysKernel sys_kernel_bias(const void *func)
 {
-    static const void *const kernels[] = {
+    static const void *const rest[] = {
         (const void *)k_bias,
     };
-    for (const void *k : kernels)
-        if (k == func) return true;
-    return false;
+    for (const void *k : rest)
+        if (k == func) return kSysOnly;
+    return kNotSys;
 }
 
 }  // namespace metad

@@ -393,11 +393,16 @@ template <typename real>
 constexpr int kFwdBlocks = sizeof(real) == 4 ? 12 : 0;
 
 template <typename real, bool kFilter>
-__global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) k_cv_fwd(Sys s) { cv_fwd<real, kFilter>(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) k_cv_fwd(Sys s)
+{
+    chain_enter();
+    cv_fwd<real, kFilter>(s, own_blk());
+}
 
 template <typename real>
 __global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) kb_cv_fwd(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     cv_fwd<real, true>(s, k);
@@ -553,11 +558,16 @@ __device__ __forceinline__ void cv_sum(const Sys &s, Blk k)
 }
 
 template <typename real>
-__global__ void __launch_bounds__(kSumThreads) k_cv_sum(Sys s) { cv_sum<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kSumThreads) k_cv_sum(Sys s)
+{
+    chain_enter();
+    cv_sum<real>(s, own_blk());
+}
 
 template <typename real>
 __global__ void __launch_bounds__(kSumThreads) kb_cv_sum(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     cv_sum<real>(s, k);
@@ -704,11 +714,16 @@ template <typename real>
 constexpr int kAvgBlocks = sizeof(real) == 4 ? 10 : 0;
 
 template <typename real>
-__global__ void __launch_bounds__(kRowThreads, kAvgBlocks<real>) k_cv_avg(Sys s) { cv_avg<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kRowThreads, kAvgBlocks<real>) k_cv_avg(Sys s)
+{
+    chain_enter();
+    cv_avg<real>(s, own_blk());
+}
 
 template <typename real>
 __global__ void __launch_bounds__(kRowThreads, kAvgBlocks<real>) kb_cv_avg(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     cv_avg<real>(s, k);
@@ -875,11 +890,16 @@ template <typename real>
 constexpr int kAdjointBlocks = sizeof(real) == 4 ? 8 : 0;
 
 template <typename real>
-__global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) k_adjoint(Sys s) { adjoint<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) k_adjoint(Sys s)
+{
+    chain_enter();
+    adjoint<real>(s, own_blk());
+}
 
 template <typename real>
 __global__ void __launch_bounds__(kRowThreads, kAdjointBlocks<real>) kb_adjoint(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     adjoint<real>(s, k);
@@ -1088,11 +1108,16 @@ template <bool kVir>
 constexpr int kForceBlocks = kVir ? 7 : 8;
 
 template <bool kVir>
-__global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) k_force_rows(Sys s) { force_rows<kVir>(s, own_blk()); }
+__global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) k_force_rows(Sys s)
+{
+    chain_enter();
+    force_rows<kVir>(s, own_blk());
+}
 
 template <bool kVir>
 __global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) kb_force_rows(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     force_rows<kVir>(s, k);
@@ -1123,11 +1148,16 @@ __device__ __forceinline__ void force_cn(const Sys &s, Blk k)
 }
 
 template <typename real, bool kVir>
-__global__ void __launch_bounds__(kBlockAtoms) k_force_cn(Sys s) { force_cn<real, kVir>(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms) k_force_cn(Sys s)
+{
+    chain_enter();
+    force_cn<real, kVir>(s, own_blk());
+}
 
 template <typename real, bool kVir>
 __global__ void __launch_bounds__(kBlockAtoms) kb_force_cn(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     force_cn<real, kVir>(s, k);
@@ -1230,11 +1260,16 @@ __device__ __forceinline__ void force_pairs(const Sys &s, Blk k)
 }
 
 template <bool kVir>
-__global__ void __launch_bounds__(kBlockAtoms) k_force_pairs(Sys s) { force_pairs<kVir>(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms) k_force_pairs(Sys s)
+{
+    chain_enter();
+    force_pairs<kVir>(s, own_blk());
+}
 
 template <bool kVir>
 __global__ void __launch_bounds__(kBlockAtoms) kb_force_pairs(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     force_pairs<kVir>(s, k);
@@ -1265,10 +1300,15 @@ __device__ __forceinline__ void force_gather(const Sys &s, Blk k)
     }
 }
 
-__global__ void __launch_bounds__(kBlockAtoms) k_force_gather(Sys s) { force_gather(s, own_blk()); }
+__global__ void __launch_bounds__(kBlockAtoms) k_force_gather(Sys s)
+{
+    chain_enter();
+    force_gather(s, own_blk());
+}
 
 __global__ void __launch_bounds__(kBlockAtoms) kb_force_gather(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     force_gather(s, k);
@@ -1292,14 +1332,14 @@ void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st)
     const int nb = grid_blocks(s, fp64 ? GK_GROUPS : GK_ROWS, 0);  // by kFwdLanes
     if (fp64) {
         if (fused_filter)
-            k_cv_fwd<double, true><<<nb, kBlockAtoms, 0, st>>>(s);
+            chained_live(k_cv_fwd<double, true>, nb, kBlockAtoms, st, s);
         else
-            k_cv_fwd<double, false><<<nb, kBlockAtoms, 0, st>>>(s);
+            chained_live(k_cv_fwd<double, false>, nb, kBlockAtoms, st, s);
     } else {
         if (fused_filter)
-            k_cv_fwd<float, true><<<nb, kBlockAtoms, 0, st>>>(s);
+            chained_live(k_cv_fwd<float, true>, nb, kBlockAtoms, st, s);
         else
-            k_cv_fwd<float, false><<<nb, kBlockAtoms, 0, st>>>(s);
+            chained_live(k_cv_fwd<float, false>, nb, kBlockAtoms, st, s);
     }
 }
 
@@ -1307,27 +1347,27 @@ void launch_cv_avg(const Sys &s, int fp64, cudaStream_t st)
 {
     const int nb = grid_blocks(s, GK_ROWS, 0);
     if (fp64)
-        k_cv_avg<double><<<nb, kRowThreads, 0, st>>>(s);
+        chained_live(k_cv_avg<double>, nb, kRowThreads, st, s);
     else
-        k_cv_avg<float><<<nb, kRowThreads, 0, st>>>(s);
+        chained_live(k_cv_avg<float>, nb, kRowThreads, st, s);
 }
 
 void launch_cv_sum(const Sys &s, int fp64, cudaStream_t st)
 {
     const int nb = grid_blocks(s, GK_SUM, 0);
     if (fp64)
-        k_cv_sum<double><<<nb, kSumThreads, 0, st>>>(s);
+        chained_live(k_cv_sum<double>, nb, kSumThreads, st, s);
     else
-        k_cv_sum<float><<<nb, kSumThreads, 0, st>>>(s);
+        chained_live(k_cv_sum<float>, nb, kSumThreads, st, s);
 }
 
 void launch_adjoint(const Sys &s, int fp64, cudaStream_t st)
 {
     const int nb = grid_blocks(s, GK_ROWS, 0);
     if (fp64)
-        k_adjoint<double><<<nb, kRowThreads, 0, st>>>(s);
+        chained_live(k_adjoint<double>, nb, kRowThreads, st, s);
     else
-        k_adjoint<float><<<nb, kRowThreads, 0, st>>>(s);
+        chained_live(k_adjoint<float>, nb, kRowThreads, st, s);
 }
 
 namespace {
@@ -1366,7 +1406,7 @@ void launch_forces(const Sys &s, int fp64, float *F, int accumulate, double scal
     t.F_out = F;
     t.accumulate = accumulate;
     t.fscale = scale;
-    force_kernel(fp64, s.ncv, s.virial)<<<grid_blocks(t, GK_FORCE, 0), force_threads(fp64, s.ncv), 0, st>>>(t);
+    chained_live(force_kernel(fp64, s.ncv, s.virial), grid_blocks(t, GK_FORCE, 0), force_threads(fp64, s.ncv), st, t);
 }
 
 void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st)
@@ -1375,7 +1415,7 @@ void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaS
     Sys t = s;
     t.F_out = F;
     t.accumulate = accumulate;
-    k_force_gather<<<group_grid(s.n), kBlockAtoms, 0, st>>>(t);
+    chained_live(k_force_gather, group_grid(s.n), kBlockAtoms, st, t);
 }
 
 void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &rows, int row_total, int fp64, int ncv,
@@ -1383,11 +1423,11 @@ void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &
 {
     if (group_total <= 0) return;
     if (fp64) {
-        kb_cv_fwd<double><<<group_total, kBlockAtoms, 0, st>>>(groups);
-        if (ncv == 2) kb_cv_avg<double><<<row_total, kRowThreads, 0, st>>>(rows);
+        chained_live(kb_cv_fwd<double>, group_total, kBlockAtoms, st, groups);
+        if (ncv == 2) chained_live(kb_cv_avg<double>, row_total, kRowThreads, st, rows);
     } else {
-        kb_cv_fwd<float><<<row_total, kBlockAtoms, 0, st>>>(rows);
-        if (ncv == 2) kb_cv_avg<float><<<row_total, kRowThreads, 0, st>>>(rows);
+        chained_live(kb_cv_fwd<float>, row_total, kBlockAtoms, st, rows);
+        if (ncv == 2) chained_live(kb_cv_avg<float>, row_total, kRowThreads, st, rows);
     }
 }
 
@@ -1395,27 +1435,27 @@ void launch_batch_sum(const BatchView &sums, int sum_total, int fp64, cudaStream
 {
     if (sum_total <= 0) return;
     if (fp64)
-        kb_cv_sum<double><<<sum_total, kSumThreads, 0, st>>>(sums);
+        chained_live(kb_cv_sum<double>, sum_total, kSumThreads, st, sums);
     else
-        kb_cv_sum<float><<<sum_total, kSumThreads, 0, st>>>(sums);
+        chained_live(kb_cv_sum<float>, sum_total, kSumThreads, st, sums);
 }
 
 void launch_batch_adjoint(const BatchView &rows, int total, int fp64, cudaStream_t st)
 {
     if (total <= 0) return;
     if (fp64)
-        kb_adjoint<double><<<total, kRowThreads, 0, st>>>(rows);
+        chained_live(kb_adjoint<double>, total, kRowThreads, st, rows);
     else
-        kb_adjoint<float><<<total, kRowThreads, 0, st>>>(rows);
+        chained_live(kb_adjoint<float>, total, kRowThreads, st, rows);
 }
 
 int launch_batch_forces(const BatchView &force, int force_total, const BatchView &groups, int group_total, int fp64,
                         int ncv, int virial, cudaStream_t st)
 {
     if (force_total <= 0) return 0;
-    batch_force_kernel(fp64, ncv, virial)<<<force_total, force_threads(fp64, ncv), 0, st>>>(force);
+    chained_live(batch_force_kernel(fp64, ncv, virial), force_total, force_threads(fp64, ncv), st, force);
     if (!(fp64 && ncv == 2)) return 1;
-    kb_force_gather<<<group_total, kBlockAtoms, 0, st>>>(groups);
+    chained_live(kb_force_gather, group_total, kBlockAtoms, st, groups);
     return 2;
 }
 
@@ -1480,9 +1520,18 @@ void set_ylm_constants(cudaStream_t st)
 
 // The kernels of this file whose only argument is the system descriptor
 // (a captured step's nodes of these can take new I/O buffers in place).
-bool sys_kernel_cv(const void *func)
+SysKernel sys_kernel_cv(const void *func)
 {
-    static const void *const kernels[] = {
+    static const void *const io[] = {
+        (const void *)k_force_rows<false>,
+        (const void *)k_force_rows<true>,
+        (const void *)k_force_cn<float, false>,
+        (const void *)k_force_cn<float, true>,
+        (const void *)k_force_cn<double, false>,
+        (const void *)k_force_cn<double, true>,
+        (const void *)k_force_gather,
+    };
+    static const void *const rest[] = {
         (const void *)k_cv_fwd<float, true>,
         (const void *)k_cv_fwd<float, false>,
         (const void *)k_cv_fwd<double, true>,
@@ -1493,19 +1542,14 @@ bool sys_kernel_cv(const void *func)
         (const void *)k_cv_sum<double>,
         (const void *)k_adjoint<float>,
         (const void *)k_adjoint<double>,
-        (const void *)k_force_rows<false>,
-        (const void *)k_force_rows<true>,
-        (const void *)k_force_cn<float, false>,
-        (const void *)k_force_cn<float, true>,
-        (const void *)k_force_cn<double, false>,
-        (const void *)k_force_cn<double, true>,
         (const void *)k_force_pairs<false>,
         (const void *)k_force_pairs<true>,
-        (const void *)k_force_gather,
     };
-    for (const void *k : kernels)
-        if (k == func) return true;
-    return false;
+    for (const void *k : io)
+        if (k == func) return kSysIo;
+    for (const void *k : rest)
+        if (k == func) return kSysOnly;
+    return kNotSys;
 }
 
 }  // namespace metad

@@ -474,18 +474,18 @@ void launch_batch_gcv_step(const BatchView &hills, int hill_total, int fp64, cud
 
 // The kernels of this file whose only argument is the system descriptor
 // (a captured step's nodes of these can take new I/O buffers in place).
-bool sys_kernel_gcv(const void *func)
+SysKernel sys_kernel_gcv(const void *func)
 {
-    static const void *const kernels[] = {
+    static const void *const io[] = {
         (const void *)k_gcv_forward<float>,
         (const void *)k_gcv_forward<double>,
         (const void *)k_gcv_forces,
         (const void *)k_gcv_step<float>,
         (const void *)k_gcv_step<double>,
     };
-    for (const void *k : kernels)
-        if (k == func) return true;
-    return false;
+    for (const void *k : io)
+        if (k == func) return kSysIo;
+    return kNotSys;
 }
 
 }  // namespace metad

@@ -51,7 +51,7 @@ __device__ __forceinline__ void gather_check(const Sys &s, Blk k)
     bool move = false;
     float thr2 = s.disp_thr2;
     {
-        const float ex = s.Lhi[0] - __ldg(s.Lref), ey = s.Lhi[1] - __ldg(s.Lref + 1), ez = s.Lhi[2] - __ldg(s.Lref + 2);
+        const float ex = s.Lhi[0] - s.Lref[0], ey = s.Lhi[1] - s.Lref[1], ez = s.Lhi[2] - s.Lref[2];
         const float dL2 = ex * ex + ey * ey + ez * ez;
         if (dL2 > 0.0f) {
             const float half = 0.5f * (s.skin_eff - sqrtf(dL2));
@@ -72,23 +72,9 @@ __device__ __forceinline__ void gather_check(const Sys &s, Blk k)
     if (__any_sync(0xffffffffu, move) && (threadIdx.x & 31) == 0) atomicOr(s.flag, 1);
 }
 
-// Programmatic dependent launch along the rebuild chain.  A kernel of the
-// chain lets the next one be scheduled once all its own blocks have started
-// (so the next launch overlaps its run instead of following it), and waits
-// for the previous kernel to complete, its memory visible, before it reads
-// anything.  A step without a rebuild then pays little more than the
-// blocks' early exits.  (Without a programmatic launch the wait returns at
-// once: the previous kernel has completed.)
-__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void chain_enter()
-{
-    chain_next();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 __global__ void k_gather_check(Sys s)
 {
-    chain_next();
+    chain_enter();
     gather_check(s, own_blk());
 }
 
@@ -473,7 +459,7 @@ __global__ void __launch_bounds__(kBlockAtoms) k_verlet(Sys s)
 // The same kernels over every system of a batch.
 __global__ void kb_gather_check(BatchView v)
 {
-    chain_next();
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     gather_check(s, k);
@@ -611,33 +597,7 @@ int grid_blocks(const Sys &s, int kind, int persist_cap)
 
 void launch_gather_check(const Sys &s, cudaStream_t st)
 {
-    k_gather_check<<<grid_blocks(s, GK_ATOM256, 0), 256, 0, st>>>(s);
-}
-
-// A kernel of the rebuild chain, launched so it may be scheduled while the
-// previous kernel of the stream still runs (it waits for it on the device).
-template <typename Arg>
-void chained(void (*kern)(Arg), int grid, int block, cudaStream_t st, const Arg &arg)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, arg);
-    if (e == cudaErrorNotSupported || e == cudaErrorInvalidValue) {
-        // a stream that refuses the attribute gets a plain launch (the
-        // device-side wait is then already satisfied); the refusal is this
-        // launch's own error, cleared before the retry.  Any other launch
-        // error stays pending for the caller's check.
-        cudaGetLastError();
-        cfg.numAttrs = 0;
-        cudaLaunchKernelEx(&cfg, kern, arg);
-    }
+    chained_live(k_gather_check, grid_blocks(s, GK_ATOM256, 0), 256, st, s);
 }
 
 void launch_rebuild(const Sys &s, cudaStream_t st)
@@ -652,7 +612,7 @@ void launch_rebuild(const Sys &s, cudaStream_t st)
 
 void launch_batch_gather(const BatchView &v, int total, cudaStream_t st)
 {
-    if (total > 0) kb_gather_check<<<total, 256, 0, st>>>(v);
+    if (total > 0) chained_live(kb_gather_check, total, 256, st, v);
 }
 
 void launch_batch_rebuild(const BatchView *rows, const int *totals, cudaStream_t st)
@@ -692,22 +652,26 @@ void launch_export_pairs(const Sys &s, int fp64, long long *pairs, int *count, c
 
 // The kernels of this file whose only argument is the system descriptor
 // (a captured step's nodes of these can take new I/O buffers in place).
-bool sys_kernel_neighbors(const void *func)
+SysKernel sys_kernel_neighbors(const void *func)
 {
-    static const void *const kernels[] = {
+    static const void *const io[] = {
         (const void *)k_gather_check,
         (const void *)k_bin_count,
+        (const void *)k_cell_sort_gather,
+    };
+    static const void *const rest[] = {
         (const void *)k_scan_reduce,
         (const void *)k_scan_down,
         (const void *)k_bin_scatter,
-        (const void *)k_cell_sort_gather,
         (const void *)k_verlet,
         (const void *)k_filter<float>,
         (const void *)k_filter<double>,
     };
-    for (const void *k : kernels)
-        if (k == func) return true;
-    return false;
+    for (const void *k : io)
+        if (k == func) return kSysIo;
+    for (const void *k : rest)
+        if (k == func) return kSysOnly;
+    return kNotSys;
 }
 
 }  // namespace metad

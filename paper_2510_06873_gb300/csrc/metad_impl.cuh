@@ -149,6 +149,21 @@ struct Sys {
     double *gcv;           // [ncv][16] per-CV gradient terms of the last CV pass
 };
 
+// Programmatic dependent launch along the kernels of a step.  A kernel of the
+// chain lets the next one be scheduled once all its own blocks have started
+// (so the next launch overlaps its run instead of following it), and waits
+// for the previous kernel to complete, its memory visible, before it reads or
+// writes anything.  Every kernel that may be launched so waits in every
+// thread that goes on, so completion carries along the chain.  (Without a
+// programmatic launch the wait returns at once: the previous kernel has
+// completed.)  Loads of data that an earlier kernel of the step writes are
+// plain ones: a read-only load (__ldg) may be moved before the wait.
+__device__ __forceinline__ void chain_enter()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The difference s - c a hill sees along CV d: wrapped into [-P/2, P/2]
 // (nearest image) for a periodic CV, x - P rint(x / P), with x / P taken as
 // x * (1 / P) (no division per hill; the two can pick different images only
@@ -227,6 +242,47 @@ enum GridKind : int {
 // lane-group grids (a batch tile setting), 0 keeps the default.
 int grid_blocks(const Sys &s, int kind, int persist_cap);
 
+// A kernel of a step, launched so it may be scheduled while the previous
+// kernel of the stream still runs (it waits for it on the device).
+template <typename... Args>
+void chained(void (*kern)(Args...), int grid, int block, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+    if (e == cudaErrorNotSupported || e == cudaErrorInvalidValue) {
+        // a stream that refuses the attribute gets a plain launch (the
+        // device-side wait is then already satisfied); the refusal is this
+        // launch's own error, cleared before the retry.  Any other launch
+        // error stays pending for the caller's check.
+        cudaGetLastError();
+        cfg.numAttrs = 0;
+        cudaLaunchKernelEx(&cfg, kern, args...);
+    }
+}
+
+// The same for the kernels outside the rebuild chain, but plain in a stream
+// that is being captured: us a step of 1,000 / 27,648 / 100,000 atoms, all
+// launches plain, then chained: launched 46.7 / 62.0 / 120.4, 39.1 / 55.6 /
+// 108.9; replayed from a graph 37.4 / 51.0 / 107.9, 35.6 / 54.1 / 106.4 (at
+// 10,000 41.3, 43.7), so a graph keeps the plain ones.
+template <typename... Args>
+void chained_live(void (*kern)(Args...), int grid, int block, cudaStream_t st, Args... args)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+        chained(kern, grid, block, st, args...);
+    else
+        kern<<<grid, block, 0, st>>>(args...);
+}
+
 // Batched stage launches (one launch each over every system of the view).
 void launch_batch_gather(const BatchView &v, int total, cudaStream_t st);
 void launch_batch_rebuild(const BatchView *rows, const int *totals, cudaStream_t st);
@@ -257,12 +313,13 @@ void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaS
 void configure_kernels();
 void launch_grid_fold(const Sys &s, int K, cudaStream_t st);
 void launch_nn_stats(const Sys &s, unsigned long long *sum, int *mx, cudaStream_t st);
-// Kernels whose only argument is the descriptor, per file (step graphs patch
-// their I/O buffers in place).
-bool sys_kernel_neighbors(const void *func);
-bool sys_kernel_cv(const void *func);
-bool sys_kernel_bias(const void *func);
-bool sys_kernel_gcv(const void *func);
+// Kernels whose only argument is the descriptor, per file, and which of them
+// read the positions or write the forces (step graphs patch those in place).
+enum SysKernel : int { kNotSys = 0, kSysOnly = 1, kSysIo = 2 };
+SysKernel sys_kernel_neighbors(const void *func);
+SysKernel sys_kernel_cv(const void *func);
+SysKernel sys_kernel_bias(const void *func);
+SysKernel sys_kernel_gcv(const void *func);
 void launch_export_pairs(const Sys &s, int fp64, long long *pairs, int *count, cudaStream_t st);
 void launch_per_atom_out(const Sys &s, int fp64, double *out, cudaStream_t st);
 void set_ylm_constants(cudaStream_t st);
@@ -778,8 +835,7 @@ struct alignas(2 * sizeof(real)) JW {
 
 // G candidates of a Verlet row a round, the accepted ones compacted by
 // ballot.  kPart: 0 every exact entry, 1 those with j > i, 2 those with j < i.
-// The rows and positions are not written by this kernel (__ldg: the loads need
-// not wait for the stores), and a round's indices are loaded one ahead.
+// Positions are loaded a round ahead of their use and indices two.
 template <typename real, int kPart, int G>
 __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
@@ -787,17 +843,17 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
     const int *vrow = s.vnbr + (size_t)i * s.max_vnb;
     const size_t e0 = entry_base(s, i), row0 = (size_t)i * s.max_nb;
     const unsigned lt = (1u << a.l) - 1u;
-    int j1 = a.l < vn ? __ldg(vrow + a.l) : i;
-    float4 p1 = __ldg(s.pos_s + j1);
-    int j2 = a.l + G < vn ? __ldg(vrow + a.l + G) : i;
+    int j1 = a.l < vn ? vrow[a.l] : i;
+    float4 p1 = s.pos_s[j1];
+    int j2 = a.l + G < vn ? vrow[a.l + G] : i;
     for (int base = 0; base < vmax; base += G) {
         const int k = base + a.l;
         const bool valid = k < vn;
         const int j = j1;
         const float4 pj = p1;
         j1 = j2;
-        p1 = __ldg(s.pos_s + j1);
-        j2 = k + 2 * G < vn ? __ldg(vrow + k + 2 * G) : i;
+        p1 = s.pos_s[j1];
+        j2 = k + 2 * G < vn ? vrow[k + 2 * G] : i;
         const bool part = kPart == 0 || (kPart == 1 ? j > a.i : j < a.i);
         Vec3<float> d;
         const bool in = pair_in_warp(s, valid && part, pi, pj, d);  // every lane: a warp vote inside
