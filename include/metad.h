@@ -197,6 +197,18 @@ metad_status metad_bias_eval(metad_ctx *ctx, const double *s_host, double *V_hos
  * floating-point atomics. */
 metad_status metad_bias_forces(metad_ctx *ctx, float *forces_dev, int32_t accumulate, double scale);
 
+/* The gradient form of metad_bias_forces, for automatic differentiation (the
+ * paper's forces come from it, Section "Frameworks of GPU-MetaD"): grad_dev
+ * [n_atoms][4] receives g dV_b/dr in the caller's atom order (0 in the species
+ * column), with g = *scale_dev read on the device, so nothing waits for it.
+ * Errors: as metad_bias_forces; METAD_ERR_INVALID (NULL argument). */
+metad_status metad_bias_gradient(metad_ctx *ctx, float *grad_dev, const double *scale_dev);
+
+/* The last bias V_b (Methods, Eq. 2) into device memory: V_dev, one double, on
+ * the context's stream, asynchronous.
+ * Errors: METAD_ERR_STATE (no bias evaluated), METAD_ERR_INVALID (NULL). */
+metad_status metad_bias_value(metad_ctx *ctx, double *V_dev);
+
 /* Atoms of the torsion and nearest-distance CVs, caller indices (host int32):
  *   METAD_CV_TORSION: count = 4 n_cv, quadruplets (a, b, c, d) in CV order;
  *   METAD_CV_NEAREST: count = n_cv + M, the n_cv reference atoms, then the

@@ -27,6 +27,11 @@ class BiasContext(_m.Metad):
         super().__init__(params)
         self.generation = 0
         self.last_pos_ptr = None
+        self._stream = self.stream
+
+    def on_current_stream(self, t: torch.Tensor) -> bool:
+        """Whether torch's current stream for t's device is the context's."""
+        return t.is_cuda and torch.cuda.current_stream(t.device).cuda_stream == self._stream
 
     def evaluate(self, pos: torch.Tensor):
         """Neighbours, CVs and bias for pos (float32 [N, 4] on the device)."""
@@ -51,12 +56,16 @@ class MetadBias(torch.autograd.Function):
             raise ValueError("pos must be float32 [N, 4]")
         pos = pos.contiguous()
         gen = bias_ctx.evaluate(pos)
+        out = None
+        if bias_ctx.on_current_stream(pos):
+            out = torch.empty((), dtype=torch.float64, device=pos.device)
+            _m.metad_bias_value(bias_ctx.ctx, out)
         cv, V, dV = bias_ctx.read_results()
         fctx.save_for_backward(pos)
         fctx.bias_ctx = bias_ctx
         fctx.gen = gen
         fctx.cv = cv
-        return torch.tensor(V, dtype=torch.float64, device=pos.device)
+        return torch.tensor(V, dtype=torch.float64, device=pos.device) if out is None else out
 
     @staticmethod
     def backward(fctx, grad_V: torch.Tensor):
@@ -66,6 +75,13 @@ class MetadBias(torch.autograd.Function):
             # the context moved on: recompute the per-atom state of this frame
             bctx.evaluate(pos)
             fctx.gen = bctx.generation
+        if grad_V.device == pos.device and grad_V.dtype == torch.float64 and bctx.on_current_stream(pos):
+            # one stream orders it all: the gradient is written whole, its
+            # factor read on the device (no round trip to the host, which
+            # left the GPU idle, no second pass over the gradient)
+            grad = torch.empty_like(pos, memory_format=torch.contiguous_format)
+            _m.metad_bias_gradient(bctx.ctx, grad, grad_V.detach())
+            return grad, None
         g = float(grad_V.detach().cpu())
         n = pos.shape[0]
         dVdx = torch.empty((n, 3), dtype=torch.float32, device=pos.device)

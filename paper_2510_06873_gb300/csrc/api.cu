@@ -287,6 +287,21 @@ metad_status sync_and_check(metad_ctx *c)
     return error_word_status(c, *c->err_pinned);
 }
 
+// Copy the scalar block (CVs, bias and its gradient, the error word) to
+// host_pinned and wait: one copy where the results and then the error word
+// took two.
+metad_status read_scalars(metad_ctx *c, const char *what)
+{
+    metad_status s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal, metad::kNumScal * sizeof(double),
+                                                   cudaMemcpyDeviceToHost, c->stream), what);
+    if (s != METAD_OK) return s;
+    s = cuda_check(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+    if (s != METAD_OK) return s;
+    int e;
+    std::memcpy(&e, c->host_pinned + metad::kErrWord, sizeof(e));
+    return error_word_status(c, e);
+}
+
 // Turn a device error word into a status (the context fails on any bit).
 metad_status error_word_status(metad_ctx *c, int e)
 {
@@ -434,6 +449,8 @@ metad_status setup_system(metad_ctx *c)
     y.k_d = sc * y.a_d;
     split(y.a_d, y.a_hi, y.a_lo);
     split(y.k_d, y.k_hi, y.k_lo);
+    y.F_stride = 3;
+    y.fscale_dev = nullptr;
     y.hill_cap = c->p.hill_capacity;
     y.lattice = c->p.lattice_cvs;
     y.virial = c->p.virial || c->p.lattice_cvs;
@@ -546,7 +563,7 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
         int *atoms = nullptr, *slot = nullptr;
         if ((s = alloc(&atoms, 4 * (size_t)2 + n)) || (s = alloc(&slot, n)) || (s = alloc(&y.gcv, 32)) ||
             (s = alloc(&y.part, (size_t)y.part_stride * 4)) || (s = alloc(&y.ticket, 8)) ||
-            (s = alloc(&y.scal, metad::kNumScal)) || (s = alloc(&y.err, 1)) ||
+            (s = alloc(&y.scal, metad::kNumScal)) ||
             (s = alloc(&y.hc, (size_t)y.hstride * ((size_t)y.hill_cap + 1))) ||
             (s = alloc(&y.hw, (size_t)y.hill_cap + 1)) ||
             (s = alloc(&c->stage, (size_t)y.hstride * ((size_t)y.hill_cap + 1))) ||
@@ -568,7 +585,7 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
         (s = alloc(&y.vnbr, (size_t)y.max_vnb * n)) || (s = alloc(&y.vnn, n)) || (s = alloc(&y.flag, 1)) ||
         (s = alloc(&y.rebuilds, 1)) || (s = alloc(&y.Lref, 4)) || (s = alloc(&b.rb, rs * (r.q + r.b + r.h + (size_t)n * 3))) ||
         (s = alloc(&y.part, (size_t)y.part_stride * 4)) || (s = alloc(&y.ticket, 8)) ||
-        (s = alloc(&y.scal, metad::kNumScal)) || (s = alloc(&y.err, 1)) ||
+        (s = alloc(&y.scal, metad::kNumScal)) ||
         (s = alloc(&y.hc, (size_t)y.hstride * ((size_t)y.hill_cap + 1))) ||
         (s = alloc(&y.hw, (size_t)y.hill_cap + 1)) ||
         (s = alloc(&c->stage, (size_t)y.hstride * ((size_t)y.hill_cap + 1))) ||
@@ -733,6 +750,7 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
         metad_destroy(c);
         return s;
     }
+    y.err = reinterpret_cast<int *>(y.scal + metad::kErrWord);
     if (c->p.cv_kind != METAD_CV_COORDINATION) {
         if (cudaMallocHost(&c->host_pinned, 64 * sizeof(double)) != cudaSuccess ||
             cudaMallocHost(&c->err_pinned, sizeof(int)) != cudaSuccess) {
@@ -742,7 +760,6 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
         }
         cudaMemsetAsync(y.ticket, 0, 8 * sizeof(unsigned), c->stream);
         cudaMemsetAsync(y.scal, 0, metad::kNumScal * sizeof(double), c->stream);
-        cudaMemsetAsync(y.err, 0, sizeof(int), c->stream);
         cudaMemsetAsync(y.gcv, 0, 32 * sizeof(double), c->stream);
         cudaMemsetAsync(y.grid, 0, sizeof(double) * (size_t)y.gn[0] * y.gn[1] * 4, c->stream);
         cudaMemsetAsync(const_cast<int *>(y.cand_slot), 0xff, sizeof(int) * (size_t)n, c->stream);  // -1
@@ -781,7 +798,6 @@ metad_status metad_create(const metad_params *p, metad_ctx **out)
     }
     cudaMemsetAsync(y.ticket, 0, 8 * sizeof(unsigned), c->stream);
     cudaMemsetAsync(y.scal, 0, metad::kNumScal * sizeof(double), c->stream);
-    cudaMemsetAsync(y.err, 0, sizeof(int), c->stream);
     cudaMemsetAsync(y.grid, 0, sizeof(double) * (size_t)y.gn[0] * y.gn[1] * 4, c->stream);
     cudaMemsetAsync(y.nn, 0, sizeof(int) * (size_t)n, c->stream);
     // the cell counters start at zero; every rebuild's scan leaves them zero
@@ -877,11 +893,8 @@ metad_status metad_cv_forward(metad_ctx *c, double *cv_host, double *per_atom_de
     c->have_cv = true;
     c->have_bias = false;
     if (cv_host) {
-        s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal + metad::kS0, metad::kMaxCv * sizeof(double),
-                                          cudaMemcpyDeviceToHost, c->stream), "cv copy");
-        if (s) return s;
-        if ((s = sync_and_check(c))) return s;
-        for (int d = 0; d < c->sys.D; ++d) cv_host[d] = c->host_pinned[d];
+        if ((s = read_scalars(c, "cv copy"))) return s;
+        for (int d = 0; d < c->sys.D; ++d) cv_host[d] = c->host_pinned[metad::kS0 + d];
     }
     return METAD_OK;
 }
@@ -911,40 +924,35 @@ metad_status metad_bias_eval(metad_ctx *c, const double *s_host, double *V_host,
     if (s) return s;
     c->have_bias = !s_host ? true : false;
     if (V_host || dVds_host) {
-        s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal + metad::kV, (1 + metad::kMaxCv) * sizeof(double),
-                                          cudaMemcpyDeviceToHost, c->stream), "bias copy");
-        if (s) return s;
-        if ((s = sync_and_check(c))) return s;
-        if (V_host) *V_host = c->host_pinned[0];
+        if ((s = read_scalars(c, "bias copy"))) return s;
+        if (V_host) *V_host = c->host_pinned[metad::kV];
         if (dVds_host)
-            for (int d = 0; d < c->sys.D; ++d) dVds_host[d] = c->host_pinned[1 + d];
+            for (int d = 0; d < c->sys.D; ++d) dVds_host[d] = c->host_pinned[metad::kDV0 + d];
     }
     return METAD_OK;
 }
 
 // a8 on the context stream.
-static void force_passes(metad_ctx *c, float *forces_dev, int accumulate, double scale)
+static void force_passes(metad_ctx *c, const metad::ForceOut &out)
 {
     {
         StageScope t(c, ST_FORCE, 1);
-        metad::launch_forces(c->sys, c->fp64, forces_dev, accumulate, scale, c->stream);
+        metad::launch_forces(c->sys, c->fp64, out, c->stream);
     }
     if (metad::pair_slots(c->sys, c->fp64)) {
         StageScope t(c, ST_FGATHER, 1);
-        metad::launch_force_gather(c->sys, c->fp64, forces_dev, accumulate, c->stream);
+        metad::launch_force_gather(c->sys, c->fp64, out, c->stream);
     }
 }
 
-metad_status metad_bias_forces(metad_ctx *c, float *forces_dev, int32_t accumulate, double scale)
+// Steps a7-a8 after the bias.
+static metad_status forces_after_bias(metad_ctx *c, const metad::ForceOut &out)
 {
-    metad_status s = check_usable(c);
-    if (s) return s;
-    if (!forces_dev) return fail(c, METAD_ERR_INVALID, "forces_dev is NULL");
     if (!c->have_bias || !c->have_cv) return fail(c, METAD_ERR_STATE, "bias_forces before bias_eval");
     if (c->p.cv_kind != METAD_CV_COORDINATION) {
         {
             StageScope t(c, ST_FORCE, 1);
-            metad::launch_gcv_forces(c->sys, forces_dev, accumulate ? 1 : 0, scale, c->stream);
+            metad::launch_gcv_forces(c->sys, out, c->stream);
         }
         return launched(c, "bias_forces");
     }
@@ -953,8 +961,34 @@ metad_status metad_bias_forces(metad_ctx *c, float *forces_dev, int32_t accumula
         StageScope t(c, ST_ADJ, 1);
         metad::launch_adjoint(c->sys, c->fp64, c->stream);
     }
-    force_passes(c, forces_dev, accumulate ? 1 : 0, scale);
+    force_passes(c, out);
     return launched(c, "bias_forces");
+}
+
+metad_status metad_bias_forces(metad_ctx *c, float *forces_dev, int32_t accumulate, double scale)
+{
+    metad_status s = check_usable(c);
+    if (s) return s;
+    if (!forces_dev) return fail(c, METAD_ERR_INVALID, "forces_dev is NULL");
+    return forces_after_bias(c, metad::ForceOut{forces_dev, 3, accumulate ? 1 : 0, scale, nullptr});
+}
+
+metad_status metad_bias_gradient(metad_ctx *c, float *grad_dev, const double *scale_dev)
+{
+    metad_status s = check_usable(c);
+    if (s) return s;
+    if (!grad_dev || !scale_dev) return fail(c, METAD_ERR_INVALID, "NULL gradient argument");
+    return forces_after_bias(c, metad::ForceOut{grad_dev, 4, 0, -1.0, scale_dev});
+}
+
+metad_status metad_bias_value(metad_ctx *c, double *V_dev)
+{
+    metad_status s = check_usable(c);
+    if (s) return s;
+    if (!V_dev) return fail(c, METAD_ERR_INVALID, "V_dev is NULL");
+    if (!c->have_bias) return fail(c, METAD_ERR_STATE, "bias_value before bias_eval");
+    return cuda_check(c, cudaMemcpyAsync(V_dev, c->sys.scal + metad::kV, sizeof(double), cudaMemcpyDeviceToDevice,
+                                         c->stream), "bias copy");
 }
 
 metad_status metad_set_cv_atoms(metad_ctx *c, const int32_t *atoms_host, int32_t count)
@@ -1048,11 +1082,8 @@ metad_status metad_box_gradient(metad_ctx *c, double *dVdL_host)
     if (!dVdL_host) return fail(c, METAD_ERR_INVALID, "output is NULL");
     if (!c->sys.virial) return fail(c, METAD_ERR_INVALID, "needs params.virial or params.lattice_cvs");
     if (!c->forces_done) return fail(c, METAD_ERR_STATE, "box_gradient before bias_forces");
-    if ((s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal + metad::kBoxG0, 3 * sizeof(double),
-                                           cudaMemcpyDeviceToHost, c->stream), "box gradient copy")) ||
-        (s = sync_and_check(c)))
-        return s;
-    for (int a = 0; a < 3; ++a) dVdL_host[a] = c->host_pinned[a];
+    if ((s = read_scalars(c, "box gradient copy"))) return s;
+    for (int a = 0; a < 3; ++a) dVdL_host[a] = c->host_pinned[metad::kBoxG0 + a];
     return METAD_OK;
 }
 
@@ -1080,11 +1111,8 @@ metad_status metad_deposit_hill(metad_ctx *c, const double *center_host, double 
     if (s) return s;
     c->K += 1;
     if (height_host) {
-        s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal + metad::kDepW, sizeof(double),
-                                          cudaMemcpyDeviceToHost, c->stream), "height copy");
-        if (s) return s;
-        if ((s = sync_and_check(c))) return s;
-        *height_host = c->host_pinned[0];
+        if ((s = read_scalars(c, "height copy"))) return s;
+        *height_host = c->host_pinned[metad::kDepW];
     }
     return METAD_OK;
 }
@@ -1300,7 +1328,7 @@ metad_status step_overlapped(metad_ctx *c, const float *pos_dev, float *forces_d
         metad::launch_adjoint(c->sys, c->fp64, c->stream);
     }
     if ((s = cuda_check(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0), "join"))) return s;
-    force_passes(c, forces_dev, accumulate ? 1 : 0, 1.0);
+    force_passes(c, metad::ForceOut{forces_dev, 3, accumulate ? 1 : 0, 1.0, nullptr});
     if ((s = launched(c, "step"))) return s;
     c->have_cv = c->have_bias = true;
     c->forces_done = true;
@@ -1424,10 +1452,7 @@ metad_status metad_step_host(metad_ctx *c, const float *pos_host, float *forces_
     if ((s = cuda_check(c, cudaMemcpyAsync(forces_host, c->force_stage, sizeof(float) * 3 * n,
                                            cudaMemcpyDeviceToHost, c->stream), "force download")))
         return s;
-    if ((s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal, metad::kNumScal * sizeof(double),
-                                           cudaMemcpyDeviceToHost, c->stream), "result copy")))
-        return s;
-    if ((s = sync_and_check(c))) return s;
+    if ((s = read_scalars(c, "result copy"))) return s;
     if (cv_host)
         for (int d = 0; d < c->sys.D; ++d) cv_host[d] = c->host_pinned[metad::kS0 + d];
     if (V_host) *V_host = c->host_pinned[metad::kV];
@@ -1522,10 +1547,7 @@ metad_status metad_read_results(metad_ctx *c, double *cv_host, double *V_host, d
 {
     metad_status s = check_usable(c);
     if (s) return s;
-    s = cuda_check(c, cudaMemcpyAsync(c->host_pinned, c->sys.scal, metad::kNumScal * sizeof(double),
-                                      cudaMemcpyDeviceToHost, c->stream), "result copy");
-    if (s) return s;
-    if ((s = sync_and_check(c))) return s;
+    if ((s = read_scalars(c, "result copy"))) return s;
     for (int d = 0; d < c->sys.D; ++d) {
         if (cv_host) cv_host[d] = c->host_pinned[metad::kS0 + d];
         if (dVds_host) dVds_host[d] = c->host_pinned[metad::kDV0 + d];

@@ -935,8 +935,9 @@ template <typename real>
 __device__ __forceinline__ void chain_factors(const Sys &s, real fac[2])
 {
     if (threadIdx.x == 0) {
-        fac[0] = (real)(s.scal[kDV0] * s.fscale * 2.0 / s.n);
-        fac[1] = s.ncv == 2 ? (real)(s.scal[kDV1] * s.fscale) : real(0);
+        const double scale = force_scale(s);
+        fac[0] = (real)(s.scal[kDV0] * scale * 2.0 / s.n);
+        fac[1] = s.ncv == 2 ? (real)(s.scal[kDV1] * scale) : real(0);
     }
     __syncthreads();
 }
@@ -944,7 +945,7 @@ __device__ __forceinline__ void chain_factors(const Sys &s, real fac[2])
 template <typename real>
 __device__ __forceinline__ void put_force(const Sys &s, int i, int comp, real f)
 {
-    float *o = s.F_out + 3 * (size_t)s.perm[i] + comp;
+    float *o = s.F_out + (size_t)s.F_stride * s.perm[i] + comp;
     *o = s.accumulate ? *o + (float)f : (float)f;
 }
 
@@ -1015,7 +1016,7 @@ __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real
             double t = 0.0;
             for (int w = 0; w < kW; ++w) t += sh[a][w];
             s.scal[kVir0 + a] = t;
-            s.scal[kBoxG0 + a] = (s.lattice ? s.fscale * s.scal[kDV0 + s.ncv + a] : 0.0) + t / s.L[a];
+            s.scal[kBoxG0 + a] = (s.lattice ? force_scale(s) * s.scal[kDV0 + s.ncv + a] : 0.0) + t / s.L[a];
         }
         s.ticket[3] = 0u;
     }
@@ -1090,7 +1091,8 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
         fx = group4_sum<float>(fx);
         fy = group4_sum<float>(fy);
         fz = group4_sum<float>(fz);
-        if (i < s.n && l < 3) put_force<float>(s, i, l, l == 0 ? fx : (l == 1 ? fy : fz));
+        if (i < s.n && l < s.F_stride)
+            put_force<float>(s, i, l, l == 0 ? fx : (l == 1 ? fy : (l == 2 ? fz : 0.0f)));
         if (kVir) {  // each pair is met at both ends
             vx.add(0.5f * wx);
             vy.add(0.5f * wy);
@@ -1137,6 +1139,7 @@ __device__ __forceinline__ void force_cn(const Sys &s, Blk k)
         put_force<real>(s, i, 0, f * r[0]);
         put_force<real>(s, i, 1, f * r[1]);
         put_force<real>(s, i, 2, f * r[2]);
+        if (s.F_stride == 4) put_force<real>(s, i, 3, real(0));
         if (kVir) {  // each pair is met at both ends
             const real hf = real(0.5) * f;
             vx.add(hf * r[3]);
@@ -1296,7 +1299,8 @@ __device__ __forceinline__ void force_gather(const Sys &s, Blk k)
         fx = group_sum<double>(fx);
         fy = group_sum<double>(fy);
         fz = group_sum<double>(fz);
-        if (a.ok && a.l < 3) put_force<double>(s, a.i, a.l, a.l == 0 ? fx : (a.l == 1 ? fy : fz));
+        if (a.ok && a.l < s.F_stride)
+            put_force<double>(s, a.i, a.l, a.l == 0 ? fx : (a.l == 1 ? fy : (a.l == 2 ? fz : 0.0)));
     }
 }
 
@@ -1400,21 +1404,18 @@ Kern<BatchView> batch_force_kernel(int fp64, int ncv, int virial)
 
 }  // namespace
 
-void launch_forces(const Sys &s, int fp64, float *F, int accumulate, double scale, cudaStream_t st)
+void launch_forces(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st)
 {
     Sys t = s;
-    t.F_out = F;
-    t.accumulate = accumulate;
-    t.fscale = scale;
+    out.set(t);
     chained_live(force_kernel(fp64, s.ncv, s.virial), grid_blocks(t, GK_FORCE, 0), force_threads(fp64, s.ncv), st, t);
 }
 
-void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st)
+void launch_force_gather(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st)
 {
     if (!pair_slots(s, fp64)) return;
     Sys t = s;
-    t.F_out = F;
-    t.accumulate = accumulate;
+    out.set(t);
     chained_live(k_force_gather, group_grid(s.n), kBlockAtoms, st, t);
 }
 

@@ -349,9 +349,11 @@ __device__ void gcv_forces(const Sys &s, Blk blk, const double *gterms)
             const double w = exact ? 1.0 : soft_weight(s, r, g[1]) / g[2];
             for (int k = 0; k < 3; ++k) f[k] -= dv * (w * (dd[k] / r));
         }
-        float *out = s.F_out + 3 * (size_t)i;
+        float *out = s.F_out + (size_t)s.F_stride * i;
+        if (s.F_stride == 4) out[3] = 0.0f;
+        const double scale = force_scale(s);
         for (int k = 0; k < 3; ++k) {
-            const float v = (float)(s.fscale * f[k]);
+            const float v = (float)(scale * f[k]);
             out[k] = s.accumulate ? out[k] + v : v;
         }
     }
@@ -424,12 +426,10 @@ void launch_gcv_forward(const Sys &s, int fp64, cudaStream_t st)
         k_gcv_forward<float><<<1, kGcvThreads, 0, st>>>(s);
 }
 
-void launch_gcv_forces(const Sys &s, float *F, int accumulate, double scale, cudaStream_t st)
+void launch_gcv_forces(const Sys &s, const ForceOut &out, cudaStream_t st)
 {
     Sys t = s;
-    t.F_out = F;
-    t.accumulate = accumulate;
-    t.fscale = scale;
+    out.set(t);
     k_gcv_forces<<<grid_blocks(t, GK_ATOM256, 0), kGcvThreads, 0, st>>>(t);
 }
 

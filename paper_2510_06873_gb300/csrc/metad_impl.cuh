@@ -34,6 +34,7 @@ enum Scal : int {
     kDepC0 = 18,                 // the last deposit centre (or a caller's CV point)
     kVir0 = 23,                  // bias virial sum_pairs (dV/dd)_a d_a, a = x, y, z
     kBoxG0 = 26,                 // dV/dL_a at fixed fractional coordinates
+    kErrWord = 31,               // the device error word (an int)
     kNumScal = 32
 };
 
@@ -135,9 +136,11 @@ struct Sys {
     const double *bias_x;  // CV point of the hill kernel
     double *bias_out;      // V, dV/ds1, dV/ds2 of the hill kernel
     int deposit;           // hill kernel: 1 = append a hill at bias_x
-    float *F_out;          // caller's forces [n][3]
+    float *F_out;          // caller's forces [n][F_stride]
+    int F_stride;          // 3, or 4 with the fourth component written as 0
     int accumulate;        // 1: F_out += force, 0: F_out = force
-    double fscale;         // forces are scaled by this
+    double fscale;         // forces are scaled by this, and by *fscale_dev unless NULL
+    const double *fscale_dev;
     // torsion and nearest-distance families (no neighbour list)
     double period[kMaxCv];      // 0, or the period of a periodic CV (2 pi for a torsion)
     double inv_period[kMaxCv];  // 1 / period (0 when not periodic)
@@ -187,6 +190,12 @@ __device__ __forceinline__ float wrap_coord(float x, float Lin, double L)
     float f = (float)w;
     if ((double)f >= L) f = 0.0f;
     return f;
+}
+
+// What the forces are scaled by.
+__device__ __forceinline__ double force_scale(const Sys &s)
+{
+    return s.fscale_dev ? s.fscale * *s.fscale_dev : s.fscale;
 }
 
 // Where a block works: block b of a grid of nb blocks of its system.  A
@@ -305,11 +314,26 @@ void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st);
 void launch_cv_avg(const Sys &s, int fp64, cudaStream_t st);
 void launch_bias(const Sys &s, int K, const double *s_dev, double *out_dev, int deposit, cudaStream_t st);
 void launch_adjoint(const Sys &s, int fp64, cudaStream_t st);
+// Where forces go, and by what they are scaled.
+struct ForceOut {
+    float *F;
+    int stride, accumulate;
+    double scale;
+    const double *scale_dev;
+    void set(Sys &s) const
+    {
+        s.F_out = F;
+        s.F_stride = stride;
+        s.accumulate = accumulate;
+        s.fscale = scale;
+        s.fscale_dev = scale_dev;
+    }
+};
 // The force pass (+ virial if s.virial): one kernel, except that the FP64
 // two-CV one leaves its pair forces for launch_force_gather.
-void launch_forces(const Sys &s, int fp64, float *F, int accumulate, double scale, cudaStream_t st);
+void launch_forces(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st);
 inline bool pair_slots(const Sys &s, int fp64) { return fp64 && s.ncv == 2; }
-void launch_force_gather(const Sys &s, int fp64, float *F, int accumulate, cudaStream_t st);
+void launch_force_gather(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st);
 void configure_kernels();
 void launch_grid_fold(const Sys &s, int K, cudaStream_t st);
 void launch_nn_stats(const Sys &s, unsigned long long *sum, int *mx, cudaStream_t st);
@@ -326,7 +350,7 @@ void set_ylm_constants(cudaStream_t st);
 // Torsion and nearest-distance families: the CV pass (one block per system)
 // and the force pass (one thread per atom).
 void launch_gcv_forward(const Sys &s, int fp64, cudaStream_t st);
-void launch_gcv_forces(const Sys &s, float *F, int accumulate, double scale, cudaStream_t st);
+void launch_gcv_forces(const Sys &s, const ForceOut &out, cudaStream_t st);
 void launch_batch_gcv(const BatchView &one, int one_total, int fp64, cudaStream_t st);
 void launch_batch_gcv_forces(const BatchView &atoms, int atom_total, cudaStream_t st);
 // The whole small-system step in one launch (CVs, hills, deposit, forces),

@@ -54,6 +54,8 @@ _SIGS = {
     "metad_cv_forward": (ctypes.c_int, [_P, _P, _P]),
     "metad_bias_eval": (ctypes.c_int, [_P, _P, _P, _P]),
     "metad_bias_forces": (ctypes.c_int, [_P, _P, ctypes.c_int32, ctypes.c_double]),
+    "metad_bias_gradient": (ctypes.c_int, [_P, _P, _P]),
+    "metad_bias_value": (ctypes.c_int, [_P, _P]),
     "metad_deposit_hill": (ctypes.c_int, [_P, _P, _P]),
     "metad_set_cv_atoms": (ctypes.c_int, [_P, _P, ctypes.c_int32]),
     "metad_set_box": (ctypes.c_int, [_P, _P]),
@@ -197,6 +199,16 @@ def metad_bias_eval(ctx, s=None, want_host=True):
 def metad_bias_forces(ctx, forces, accumulate=False, scale=1.0):
     _check(ctx, lib().metad_bias_forces(ctx, _dptr(forces), int(bool(accumulate)), float(scale)),
            "metad_bias_forces")
+
+
+def metad_bias_gradient(ctx, grad, scale):
+    """grad: float32 [N, 4] device tensor; scale: float64 device scalar."""
+    _check(ctx, lib().metad_bias_gradient(ctx, _dptr(grad), _dptr(scale)), "metad_bias_gradient")
+
+
+def metad_bias_value(ctx, V):
+    """V: float64 device scalar."""
+    _check(ctx, lib().metad_bias_value(ctx, _dptr(V)), "metad_bias_value")
 
 
 def metad_set_cv_atoms(ctx, atoms):

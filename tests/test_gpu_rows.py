@@ -1,0 +1,89 @@
+"""The row passes where their layout changes: atom counts around the slices of
+eight and the blocks of 32 and 16 atoms (interleaved rows, four and eight lanes
+an atom), rows at their capacity; and the gradient written whole with its
+factor read on the device, against the forces."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from parity_util import check_bias, check_cv, check_forces, kbdt, setup_hills
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_06873_gb300 import build
+    build.build()
+    d = torch.device("cuda:0")
+    torch.cuda.set_stream(torch.cuda.Stream(d))
+    return d
+
+
+def _params(dev, n, box, mp, **kw):
+    from paper_2510_06873_gb300 import metad
+    return metad.params_for(n, box, n_cv=mp.n_cv, sigma=mp.sigma, stream=torch.cuda.current_stream(dev).cuda_stream,
+                            hill_capacity=256, **kw)
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 1031, 1047])
+def test_step_at_slice_and_block_edges(dev, n, fp64):
+    """The common tolerances against the oracle, with rows just long enough
+    for the longest one."""
+    from paper_2510_06873_gb300 import metad
+    system = synth.wurtzite_system(n, cfg=93)
+    mp = synth.MethodParams(n_cv=2)
+    frame = synth.perturbed_frame(system, 2)
+    p = oracle.params_from(mp, system.box)
+    pairs = oracle.pairs_cells(frame, system.box, 3.5)
+    longest = int(np.bincount(pairs.ravel(), minlength=n).max())
+    c, _ = setup_hills(system, mp, 50, cfg=93)
+    w = oracle.deposit_sequence(c, mp.sigma, mp.w0, kbdt(mp))
+    ref = oracle.step(frame, p, c, w, mp.sigma)
+    ctx = metad.Metad(_params(dev, n, system.box, mp, fp64=fp64, max_neighbors=longest))
+    ctx.load_hills(c, w)
+    F = torch.full((n + 1, 3), 7.0, dtype=torch.float32, device=dev)
+    ctx.step(torch.from_numpy(frame).to(dev), F)
+    s, V, dV = ctx.read_results()
+    assert bool((F[n] == 7.0).all())
+    check_cv(s, ref["s"])
+    check_bias(V, dV, ref["V"], ref["dV"], mp)
+    check_forces(F[:n].cpu().numpy(), ref["F"])
+    ctx.close()
+
+
+@pytest.mark.parametrize("kind,n_cv,fp64", [("coordination", 1, False), ("coordination", 1, True),
+                                            ("coordination", 2, False), ("coordination", 2, True),
+                                            ("torsion", 2, False)])
+def test_gradient_is_the_scaled_force(dev, kind, n_cv, fp64):
+    """bias_gradient with factor g equals bias_forces scaled by -g bit for bit,
+    and writes 0 in the species column."""
+    from paper_2510_06873_gb300 import metad
+    system = synth.wurtzite_system(1001, cfg=94)
+    mp = synth.MethodParams(n_cv=n_cv, sigma=(0.05, 0.02)[:n_cv])
+    ctx = metad.Metad(_params(dev, system.n, system.box, mp, fp64=fp64, cv_kind=kind))
+    if kind == "torsion":
+        ctx.set_cv_atoms([0, 1, 2, 3, 1, 2, 3, 4])
+    frame = synth.perturbed_frame(system, 0)
+    pos = torch.from_numpy(frame).to(dev)
+    ctx.build_neighbors(pos)
+    s = ctx.cv_forward()
+    ctx.load_hills([np.asarray(s) + 0.01], [1.0])
+    ctx.bias_eval()
+    F = torch.zeros((system.n, 3), dtype=torch.float32, device=dev)
+    ctx.bias_forces(F, scale=-0.7)
+    grad = torch.full((system.n, 4), 9.0, dtype=torch.float32, device=dev)
+    g = torch.tensor(0.7, dtype=torch.float64, device=dev)
+    metad.metad_bias_gradient(ctx.ctx, grad, g)
+    V = torch.zeros((), dtype=torch.float64, device=dev)
+    metad.metad_bias_value(ctx.ctx, V)
+    _, V_host, _ = ctx.read_results()
+    assert float(V) == V_host
+    assert float(F.abs().max()) > 0.0
+    assert torch.equal(grad[:, :3], F) and bool((grad[:, 3] == 0.0).all())
+    ctx.close()
