@@ -79,8 +79,10 @@ __global__ void k_gather_check(Sys s)
 }
 
 // Cell of an atom, its slot there, and the octant of the cell it lies in (in
-// the slot's top bits: a cell never holds 2^28 atoms).
-constexpr int kOctShift = 28;
+// the top bits of the slot, and of the caller index where the cells are
+// sorted; systems of 2^28 atoms and more need those bits and have no octants).
+__device__ __forceinline__ int oct_shift(const Sys &s) { return s.n <= 1 << 28 ? 28 : 31; }
+__device__ __forceinline__ unsigned low_bits(unsigned v, int shift) { return v & ((1u << shift) - 1u); }
 
 __device__ __forceinline__ void bin_one(const Sys &s, int u)
 {
@@ -90,10 +92,13 @@ __device__ __forceinline__ void bin_one(const Sys &s, int u)
     int cy = cell_axis(p.y, s.inv_h[1], s.nc[1]);
     int cz = cell_axis(p.z, s.inv_h[2], s.nc[2]);
     int c = s.rank_of_xyz[(cz * s.nc[1] + cy) * s.nc[0] + cx];
-    const int oct = (p.x * s.inv_h[0] - (float)cx >= 0.5f ? 1 : 0) | (p.y * s.inv_h[1] - (float)cy >= 0.5f ? 2 : 0) |
-                    (p.z * s.inv_h[2] - (float)cz >= 0.5f ? 4 : 0);
+    const int shift = oct_shift(s);
+    unsigned oct = 0;
+    if (shift == 28)
+        oct = (p.x * s.inv_h[0] - (float)cx >= 0.5f ? 1u : 0u) | (p.y * s.inv_h[1] - (float)cy >= 0.5f ? 2u : 0u) |
+              (p.z * s.inv_h[2] - (float)cz >= 0.5f ? 4u : 0u);
     s.ucell[u] = c;
-    s.uslot[u] = atomicAdd(&s.cell_count[c], 1) | (oct << kOctShift);
+    s.uslot[u] = (int)((unsigned)atomicAdd(&s.cell_count[c], 1) | (oct << shift));
 }
 
 __device__ __forceinline__ void bin_count(const Sys &s, Blk k)
@@ -191,10 +196,10 @@ __device__ __forceinline__ void scan_down(const Sys &s, Blk k)
 __device__ __forceinline__ void bin_scatter(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
+    const int shift = oct_shift(s);
     for (int u = k.b * blockDim.x + threadIdx.x; u < s.n; u += k.nb * blockDim.x) {
-        const int v = s.uslot[u];
-        s.raw[s.cell_start[s.ucell[u]] + (v & ((1 << kOctShift) - 1))] =
-            (unsigned)u | ((unsigned)v >> kOctShift << kOctShift);
+        const unsigned v = (unsigned)s.uslot[u], slot = low_bits(v, shift);
+        s.raw[s.cell_start[s.ucell[u]] + slot] = (unsigned)u | (v - slot);
     }
 }
 
@@ -208,9 +213,10 @@ __device__ __forceinline__ void bin_scatter(const Sys &s, Blk k)
 __device__ __forceinline__ void cell_sort_gather(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
+    const int shift = oct_shift(s);
     for (int t = k.b * blockDim.x + threadIdx.x; t < s.n; t += k.nb * blockDim.x) {
         const unsigned v = s.raw[t];
-        const int u = (int)(v & ((1u << kOctShift) - 1u));
+        const int u = (int)low_bits(v, shift);
         const int c = s.ucell[u];
         const int a = s.cell_start[c], e = s.cell_start[c + 1];
         int at = a;
