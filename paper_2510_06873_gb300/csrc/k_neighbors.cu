@@ -101,12 +101,6 @@ __device__ __forceinline__ void bin_one(const Sys &s, int u)
     s.uslot[u] = (int)((unsigned)atomicAdd(&s.cell_count[c], 1) | (oct << shift));
 }
 
-__device__ __forceinline__ void bin_count(const Sys &s, Blk k)
-{
-    if (!*s.flag) return;
-    for (int u = k.b * blockDim.x + threadIdx.x; u < s.n; u += k.nb * blockDim.x) bin_one(s, u);
-}
-
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
@@ -140,6 +134,52 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int &
     return r;
 }
 
+// The cell starts of a grid of at most kScanOne cells, by the 256 threads of
+// one block, each 16 consecutive cells.
+constexpr int kBinThreads = 256;
+constexpr int kScanOne = kBinThreads * 16;
+__device__ __forceinline__ void scan_one(const Sys &s, int *ws)
+{
+    const int base = threadIdx.x * 16;
+    int c[16], v = 0;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        c[t] = base + t < s.ncell ? __ldcg(s.cell_count + base + t) : 0;
+        v += c[t];
+    }
+    if (threadIdx.x < 32) ws[threadIdx.x] = 0;  // the scan sums 32 warps; a block has eight
+    __syncthreads();
+    int total;
+    int ex = block_exclusive_scan(v, ws, total);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        if (base + t < s.ncell) s.cell_start[base + t] = ex;
+        ex += c[t];
+    }
+    if (threadIdx.x == 0) s.cell_start[s.ncell] = s.n;
+}
+
+// kScan: the grid has at most kScanOne cells, and the last block to finish
+// scans them (two kernels fewer in the chain, which a step without a rebuild
+// pays for too).
+template <bool kScan>
+__device__ __forceinline__ void bin_count(const Sys &s, Blk k)
+{
+    if (!*s.flag) return;
+    for (int u = k.b * blockDim.x + threadIdx.x; u < s.n; u += k.nb * blockDim.x) bin_one(s, u);
+    if (!kScan) return;
+    __shared__ int ws[33];
+    __shared__ bool am_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) am_last = atomicAdd(&s.ticket[5], 1u) == (unsigned)k.nb - 1u;
+    __syncthreads();
+    if (!am_last) return;
+    __threadfence();
+    scan_one(s, ws);
+    if (threadIdx.x == 0) s.ticket[5] = 0u;
+}
+
 __device__ __forceinline__ void scan_reduce(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
@@ -154,12 +194,27 @@ __device__ __forceinline__ void scan_reduce(const Sys &s, Blk k)
     if (threadIdx.x == 0) s.scan_part[k.b] = total;
 }
 
+// kDirect: a block adds the counts before its tile itself (a grid of few
+// tiles), else the tiles' sums of scan_reduce.
+constexpr int kDirectTiles = 48;
+template <bool kDirect>
 __device__ __forceinline__ void scan_down(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
     __shared__ int ws[33];
     __shared__ int prefix;
-    if (threadIdx.x < 32) {
+    if (kDirect) {
+        const int4 *c4 = reinterpret_cast<const int4 *>(s.cell_count);
+        int acc = 0;
+#pragma unroll 4
+        for (int q = threadIdx.x; q < k.b * (kScanTile / 4); q += kScanThreads) {
+            const int4 v = c4[q];
+            acc += (v.x + v.y) + (v.z + v.w);
+        }
+        int total;
+        block_exclusive_scan(acc, ws, total);
+        if (threadIdx.x == 0) prefix = total;
+    } else if (threadIdx.x < 32) {
         int acc = 0;
         for (int b = threadIdx.x; b < k.b; b += 32) acc += s.scan_part[b];
 #pragma unroll
@@ -170,15 +225,9 @@ __device__ __forceinline__ void scan_down(const Sys &s, Blk k)
     int base = k.b * kScanTile + threadIdx.x * kScanItems;
     int c[kScanItems];
     int v = 0;
-    // the counters' last reader: they are left zero for the next rebuild
-    // (zero from creation on, so no pass of their own clears them)
 #pragma unroll
     for (int t = 0; t < kScanItems; ++t) {
-        c[t] = 0;
-        if (base + t < s.ncell) {
-            c[t] = s.cell_count[base + t];
-            s.cell_count[base + t] = 0;
-        }
+        c[t] = base + t < s.ncell ? s.cell_count[base + t] : 0;
         v += c[t];
     }
     int total;
@@ -192,7 +241,8 @@ __device__ __forceinline__ void scan_down(const Sys &s, Blk k)
 }
 
 // Each cell's atoms, in the order of their atomic slots: octant and caller
-// index, one word each.
+// index, one word each.  The scanned counters are left zero for the next
+// rebuild (zero from creation on, so no pass of their own clears them).
 __device__ __forceinline__ void bin_scatter(const Sys &s, Blk k)
 {
     if (!*s.flag) return;
@@ -201,6 +251,7 @@ __device__ __forceinline__ void bin_scatter(const Sys &s, Blk k)
         const unsigned v = (unsigned)s.uslot[u], slot = low_bits(v, shift);
         s.raw[s.cell_start[s.ucell[u]] + slot] = (unsigned)u | (v - slot);
     }
+    for (int c = k.b * blockDim.x + threadIdx.x; c < s.ncell; c += k.nb * blockDim.x) s.cell_count[c] = 0;
 }
 
 // The sorted order: within a cell by octant, then caller index (the atomic
@@ -431,20 +482,22 @@ __global__ void __launch_bounds__(kBlockAtoms) k_filter(Sys s)
 
 
 // Single-system kernels of the rebuild chain.
-__global__ void k_bin_count(Sys s)
+template <bool kScan>
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(Sys s)
 {
     chain_enter();
-    bin_count(s, own_blk());
+    bin_count<kScan>(s, own_blk());
 }
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(Sys s)
 {
     chain_enter();
     scan_reduce(s, own_blk());
 }
+template <bool kDirect>
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(Sys s)
 {
     chain_enter();
-    scan_down(s, own_blk());
+    scan_down<kDirect>(s, own_blk());
 }
 __global__ void k_bin_scatter(Sys s)
 {
@@ -475,7 +528,7 @@ __global__ void kb_bin_count(BatchView v)
     chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
-    bin_count(s, k);
+    bin_count<false>(s, k);
 }
 __global__ void __launch_bounds__(kScanThreads) kb_scan_reduce(BatchView v)
 {
@@ -489,7 +542,7 @@ __global__ void __launch_bounds__(kScanThreads) kb_scan_down(BatchView v)
     chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
-    scan_down(s, k);
+    scan_down<false>(s, k);
 }
 __global__ void kb_bin_scatter(BatchView v)
 {
@@ -577,7 +630,10 @@ int grid_blocks(const Sys &s, int kind, int persist_cap)
     case GK_ATOM256: return (s.n + 255) / 256;
     case GK_ATOM256_CAP: return capped((s.n + 255) / 256);
     case GK_SCAN_TILES: return (s.ncell + kScanTile - 1) / kScanTile;
-    case GK_GROUPS_CAP: return persist_grid(s.n);  // Verlet rows: up to 16 blocks per SM
+    case GK_GROUPS_CAP: {  // Verlet rows: a warp per cell, up to 16 blocks per SM
+        const int g = (s.ncell + kVerletWarps - 1) / kVerletWarps;
+        return g < kPersistBlocks ? g : kPersistBlocks;
+    }
     case GK_ONE: return 1;
     case GK_GROUPS: {
         const int g = group_grid(s.n);
@@ -606,11 +662,21 @@ void launch_gather_check(const Sys &s, cudaStream_t st)
     chained_live(k_gather_check, grid_blocks(s, GK_ATOM256, 0), 256, st, s);
 }
 
+// The cell scan's kernels, fewer for small grids: none up to kScanOne cells
+// (about 36,000 atoms), one up to kDirectTiles tiles (about 1.8 million).
+inline int scan_kernels(const Sys &s)
+{
+    return s.ncell <= kScanOne ? 0 : (grid_blocks(s, GK_SCAN_TILES, 0) <= kDirectTiles ? 1 : 2);
+}
+
+int rebuild_kernels(const Sys &s) { return 4 + scan_kernels(s); }
+
 void launch_rebuild(const Sys &s, cudaStream_t st)
 {
-    chained(k_bin_count, grid_blocks(s, GK_ATOM256_CAP, 0), 256, st, s);
-    chained(k_scan_reduce, grid_blocks(s, GK_SCAN_TILES, 0), kScanThreads, st, s);
-    chained(k_scan_down, grid_blocks(s, GK_SCAN_TILES, 0), kScanThreads, st, s);
+    const int scans = scan_kernels(s), tiles = grid_blocks(s, GK_SCAN_TILES, 0);
+    chained(scans == 0 ? k_bin_count<true> : k_bin_count<false>, grid_blocks(s, GK_ATOM256_CAP, 0), kBinThreads, st, s);
+    if (scans == 2) chained(k_scan_reduce, tiles, kScanThreads, st, s);
+    if (scans > 0) chained(scans == 1 ? k_scan_down<true> : k_scan_down<false>, tiles, kScanThreads, st, s);
     chained(k_bin_scatter, grid_blocks(s, GK_ATOM256_CAP, 0), 256, st, s);
     chained(k_cell_sort_gather, grid_blocks(s, GK_ATOM256_CAP, 0), 256, st, s);
     chained(k_verlet, grid_blocks(s, GK_GROUPS_CAP, 0), kBlockAtoms, st, s);
@@ -662,12 +728,14 @@ SysKernel sys_kernel_neighbors(const void *func)
 {
     static const void *const io[] = {
         (const void *)k_gather_check,
-        (const void *)k_bin_count,
+        (const void *)k_bin_count<true>,
+        (const void *)k_bin_count<false>,
         (const void *)k_cell_sort_gather,
     };
     static const void *const rest[] = {
         (const void *)k_scan_reduce,
-        (const void *)k_scan_down,
+        (const void *)k_scan_down<true>,
+        (const void *)k_scan_down<false>,
         (const void *)k_bin_scatter,
         (const void *)k_verlet,
         (const void *)k_filter<float>,

@@ -309,6 +309,7 @@ void launch_batch_collect(const BatchView &v, double *out, cudaStream_t st);
 // Launch entry points (stream-ordered, no host synchronisation).
 void launch_gather_check(const Sys &s, cudaStream_t st);
 void launch_rebuild(const Sys &s, cudaStream_t st);  // kernels early-exit unless *flag
+int rebuild_kernels(const Sys &s);                   // how many they are
 void launch_filter(const Sys &s, int fp64, cudaStream_t st);
 void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st);
 void launch_cv_avg(const Sys &s, int fp64, cudaStream_t st);
@@ -676,12 +677,6 @@ constexpr int kVirialBlocks = 152 * 7;
 // blocks that share an SM to consecutive items, for L1 reuse, measured
 // slower: the gather kernels lost more to L2 misses than they won in L1.)
 __device__ __forceinline__ int work_item(Blk k, int it) { return k.b + it * k.nb; }
-
-__host__ __device__ inline int persist_grid(int n)
-{
-    const int g = group_grid(n);
-    return g < kPersistBlocks ? g : kPersistBlocks;
-}
 
 struct AtomLane {
     int i;    // atom (sorted index), may be >= n for idle groups

@@ -1,7 +1,8 @@
 """The row passes where their layout changes: atom counts around the slices of
 eight and the blocks of 32 and 16 atoms (interleaved rows, four and eight lanes
-an atom), rows at their capacity; and the gradient written whole with its
-factor read on the device, against the forces."""
+an atom), rows at their capacity; cell grids around the sizes where the scan
+takes none, one or two kernels; and the gradient written whole with its factor
+read on the device, against the forces."""
 import numpy as np
 import pytest
 
@@ -86,4 +87,27 @@ def test_gradient_is_the_scaled_force(dev, kind, n_cv, fp64):
     assert float(V) == V_host
     assert float(F.abs().max()) > 0.0
     assert torch.equal(grad[:, :3], F) and bool((grad[:, 3] == 0.0).all())
+    ctx.close()
+
+
+@pytest.mark.parametrize("cells", [(15, 16, 16), (16, 16, 16), (17, 16, 16), (48, 64, 64), (49, 64, 64)])
+def test_cell_scan_edges(dev, cells):
+    """Few atoms in pairs within rc, spread over grids of 4,096 cells and one
+    layer fewer and more, and of 48 and 49 tiles of 4,096: exact pairs after a
+    first build, and after a rebuild on moved positions."""
+    from paper_2510_06873_gb300 import metad
+    g = np.random.default_rng(sum(cells))
+    box = np.array(cells) * (4.5 * 1.0002)
+    mp = synth.MethodParams(n_cv=1, sigma=(0.05,))
+    ctx = metad.Metad(_params(dev, 600, box, mp))
+    for _ in range(2):
+        a = g.uniform(0.0, 1.0, (300, 3)) * box
+        xyz = np.concatenate([a, a + g.normal(0.0, 1.6, (300, 3))])
+        pos = np.zeros((600, 4), np.float32)
+        pos[:, :3] = synth.wrap_to_box(xyz, box)
+        pos[::2, 3] = 1.0
+        ctx.build_neighbors(torch.from_numpy(pos).to(dev))
+        ref = oracle.pairs_brute(pos, box, 3.5)
+        assert len(ref) > 100 and np.array_equal(ctx.export_neighbors(), ref)
+    assert ctx.rebuild_count == 2
     ctx.close()
