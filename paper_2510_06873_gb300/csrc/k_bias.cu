@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kBlockBias) kb_bias(BatchView v, int deposit)
 // word, for one copy to the host.
 __global__ void kb_collect(const Sys *sys, int nsys, double *out)
 {
+    chain_enter();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nsys) return;
     const Sys &s = sys[k];
@@ -107,7 +108,7 @@ void launch_batch_bias(const BatchView &v, int total, int deposit, cudaStream_t 
 
 void launch_batch_collect(const BatchView &v, double *out, cudaStream_t st)
 {
-    kb_collect<<<(v.nsys + 127) / 128, 128, 0, st>>>(v.sys, v.nsys, out);
+    chained_live(kb_collect, (v.nsys + 127) / 128, 128, st, v.sys, v.nsys, out);
 }
 
 void launch_grid_fold(const Sys &s, int K, cudaStream_t st)

@@ -41,7 +41,7 @@ __device__ __forceinline__ double min_image(double d, double L)
 // Caller atom i, wrapped into the box; flags a non-finite input.
 __device__ __forceinline__ void atom_posf(const Sys &s, int i, float p[3], bool &bad)
 {
-    const float4 q = __ldg(s.pos_in + i);
+    const float4 q = s.pos_in[i];
     bad |= !(isfinite(q.x) && isfinite(q.y) && isfinite(q.z));
     p[0] = wrap_coord(isfinite(q.x) ? q.x : 0.0f, s.Lin[0], s.L[0]);
     p[1] = wrap_coord(isfinite(q.y) ? q.y : 0.0f, s.Lin[1], s.L[1]);
@@ -175,28 +175,47 @@ __device__ void torsion(const Sys &s, int d, bool &bad, double *xo, double *go)
     }
 }
 
-// Block reductions over the kGcvThreads threads in a fixed tree.
-__device__ __forceinline__ void block_argmin(double &v, int &arg, double *shv, int *sha)
+// The smallest (v, arg) over the block's threads, ties to the lower arg, in
+// every thread; v >= 0 or infinite, compared as integers (no FP64
+// instruction).  Threads with nothing pass an infinite v.
+__device__ __forceinline__ void block_argmin(double &v, int &arg)
 {
+    __shared__ long long shv[kGcvThreads / 32];
+    __shared__ int sha[kGcvThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long none = 0x7ff0000000000000ll;  // infinity
+    long long b = __double_as_longlong(v);
+    if (__any_sync(0xffffffffu, b != none)) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_down_sync(0xffffffffu, v, o);
-        const int oa = __shfl_down_sync(0xffffffffu, arg, o);
-        if (ov < v || (ov == v && oa < arg)) { v = ov; arg = oa; }
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ob = __shfl_down_sync(0xffffffffu, b, o);
+            const int oa = __shfl_down_sync(0xffffffffu, arg, o);
+            if (ob < b || (ob == b && oa < arg)) { b = ob; arg = oa; }
+        }
     }
-    if (lane == 0) { shv[wid] = v; sha[wid] = arg; }
+    __syncthreads();  // an earlier call's results are read
+    if (lane == 0) { shv[wid] = b; sha[wid] = arg; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kGcvThreads / 32; ++w)
-            if (shv[w] < v || (shv[w] == v && sha[w] < arg)) { v = shv[w]; arg = sha[w]; }
-        shv[0] = v;
-        sha[0] = arg;
-    }
-    __syncthreads();
-    v = shv[0];
+    b = shv[0];
     arg = sha[0];
+#pragma unroll
+    for (int w = 1; w < kGcvThreads / 32; ++w)
+        if (shv[w] < b || (shv[w] == b && sha[w] < arg)) { b = shv[w]; arg = sha[w]; }
+    v = __longlong_as_double(b);
+}
+
+// The smallest v over the block's threads, v >= 0 (or infinite).
+__device__ __forceinline__ float block_min(float v)
+{
+    __shared__ unsigned sh[kGcvThreads / 32];
+    const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(v));
+    __syncthreads();  // an earlier call's results are read
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
     __syncthreads();
+    unsigned r = sh[0];
+#pragma unroll
+    for (int w = 1; w < kGcvThreads / 32; ++w) r = min(r, sh[w]);
+    return __uint_as_float(r);
 }
 
 // Four sums at once; the totals land in thread 0 only.
@@ -228,39 +247,76 @@ __device__ __forceinline__ double soft_weight(const Sys &s, double r, double rmi
     return exp(-s.sm_beta * (r - rmin));
 }
 
+// Squared distance of a candidate in FP32, within 2e-5 of the FP64 one
+// relative and 1e-10 absolute: each component is one correctly rounded
+// difference (across the box faces of exact ones, mi_axis).
+__device__ __forceinline__ float sq_dist_f(const Sys &s, const float a[3], const float b[3])
+{
+    float r2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float d = mi_axis(b[k], a[k], s.halfL[k], s.Lhi[k], s.Llo[k]);
+        r2 = fmaf(d, d, r2);
+    }
+    return r2;
+}
+
 // Nearest-distance CV d (all threads of the block): go[16 d] holds the
 // nearest slot, r_min, the soft-minimum normaliser Z and d s/d r_ref.
+//
+// The nearest candidate is decided on FP64 squared distances, but only those
+// whose FP32 estimate lies within the estimates' error of the smallest one
+// are formed: FP64 takes 16 cycles a warp instruction on this part, about 30
+// of them a candidate.
 __device__ void nearest(const Sys &s, int d, bool &bad, double *xo, double *go)
 {
-    __shared__ double shv[kGcvThreads / 32];
-    __shared__ int sha[kGcvThreads / 32];
+    __shared__ double dsh[3];
     const int o = s.cv_atoms[d];
     const int *cand = s.cv_atoms + s.ncv;
-    double po[3];
-    atom_pos(s, o, po, bad);
-    double best = DBL_MAX;
-    int arg = INT_MAX;
+    float pof[3];
+    atom_posf(s, o, pof, bad);
+    const double po[3] = {(double)pof[0], (double)pof[1], (double)pof[2]};
+    float est = INFINITY;
     for (int m = threadIdx.x; m < s.n_cand; m += kGcvThreads) {
-        double pj[3], dv[3];
-        atom_pos(s, cand[m], pj, bad);
-        disp(s, po, pj, dv);
-        const double r2 = sq_dist(dv);
-        if (r2 < best) { best = r2; arg = m; }
+        float pj[3];
+        atom_posf(s, cand[m], pj, bad);
+        est = fminf(est, sq_dist_f(s, pof, pj));
     }
-    block_argmin(best, arg, shv, sha);
+    const float lim = block_min(est) * (1.0f + 5e-5f) + 1e-9f;
+    double best = INFINITY, dv[3] = {0.0, 0.0, 0.0};
+    int arg = INT_MAX;
+    if (est <= lim) {
+        for (int m = threadIdx.x; m < s.n_cand; m += kGcvThreads) {
+            float pf[3];
+            atom_posf(s, cand[m], pf, bad);
+            if (sq_dist_f(s, pof, pf) > lim) continue;
+            const double pj[3] = {(double)pf[0], (double)pf[1], (double)pf[2]};
+            double t[3];
+            disp(s, po, pj, t);
+            const double r2 = sq_dist(t);
+            if (r2 < best) {
+                best = r2;
+                arg = m;
+                for (int k = 0; k < 3; ++k) dv[k] = t[k];
+            }
+        }
+    }
+    const int mine = arg;
+    block_argmin(best, arg);
     const double rmin = sqrt(best);
     double *g = go + 16 * d;
     if (s.sm_beta <= 0.0) {
+        if (mine == arg)  // one thread: a candidate belongs to one
+            for (int k = 0; k < 3; ++k) dsh[k] = dv[k];
+        __syncthreads();
+        if (threadIdx.x < 3) g[3 + threadIdx.x] = rmin > 0.0 ? -dsh[threadIdx.x] / rmin : 0.0;
         if (threadIdx.x == 0) {
-            double pj[3], dv[3];
-            atom_pos(s, cand[arg], pj, bad);
-            disp(s, po, pj, dv);
             xo[d] = rmin;
             g[0] = (double)arg;
             g[1] = rmin;
             g[2] = 1.0;
-            for (int k = 0; k < 3; ++k) g[3 + k] = rmin > 0.0 ? -dv[k] / rmin : 0.0;
         }
+        __syncthreads();  // dsh is read before the next CV's
         return;
     }
     __shared__ double sh4[4][kGcvThreads / 32];
@@ -314,10 +370,9 @@ __device__ void gcv_forward(const Sys &s)
 
 // F_i = (accumulate ? F_i : 0) - scale sum_d dV/ds_d ds_d/dr_i, with the
 // gradient terms gterms of the CV pass.
-__device__ void gcv_forces(const Sys &s, Blk blk, const double *gterms)
+__device__ __forceinline__ void gcv_force(const Sys &s, int i, const double *gterms)
 {
-    const int *cand = s.cv_atoms + s.ncv;
-    for (int i = blk.b * kGcvThreads + threadIdx.x; i < s.n; i += blk.nb * kGcvThreads) {
+        const int *cand = s.cv_atoms + s.ncv;
         double f[3] = {0.0, 0.0, 0.0};
         for (int d = 0; d < s.ncv; ++d) {
             const double dv = s.scal[kDV0 + d];
@@ -356,7 +411,26 @@ __device__ void gcv_forces(const Sys &s, Blk blk, const double *gterms)
             const float v = (float)(scale * f[k]);
             out[k] = s.accumulate ? out[k] + v : v;
         }
+}
+
+__device__ void gcv_forces(const Sys &s, Blk blk, const double *gterms)
+{
+    for (int i = blk.b * kGcvThreads + threadIdx.x; i < s.n; i += blk.nb * kGcvThreads) gcv_force(s, i, gterms);
+}
+
+// Whether atom i can have a force with these gradient terms (an atom of a
+// torsion; a reference; the nearest candidate, or any with the soft minimum).
+__device__ __forceinline__ bool gcv_moves(const Sys &s, int i, const double *gterms)
+{
+    bool in = false;
+    if (s.kind == kKindTorsion) {
+        for (int q = 0; q < 4 * s.ncv; ++q) in |= s.cv_atoms[q] == i;
+        return in;
     }
+    const int m = s.cand_slot[i];
+    for (int d = 0; d < s.ncv; ++d)
+        in |= s.cv_atoms[d] == i || (m >= 0 && (s.sm_beta > 0.0 || m == (int)gterms[16 * d]));
+    return in;
 }
 
 template <typename real>
@@ -368,9 +442,11 @@ __global__ void __launch_bounds__(kGcvThreads) k_gcv_forces(Sys s) { gcv_forces(
 // block evaluates the CVs (a few atoms, or one pass over the candidates)
 // into shared memory and sums its share of the hills there; block 0
 // publishes the CVs; the last block to finish the hill sum (which also
-// deposits, if asked) writes every atom's force from its own copy of the
-// CV gradient terms.  The same arithmetic as the three-kernel path, so the
-// same bits.
+// deposits, if asked) writes the forces from its own copy of the CV gradient
+// terms.  Atoms that no gradient term reaches get their zero (or, when
+// accumulating, nothing) before the hill sum, from all blocks, off the chain
+// that a lone step waits for.  The same arithmetic as the three-kernel path,
+// so the same bits.
 template <typename real>
 __device__ void gcv_step(const Sys &s, Blk blk)
 {
@@ -385,17 +461,40 @@ __device__ void gcv_step(const Sys &s, Blk blk)
         if (threadIdx.x < kMaxCv) s.scal[kS0 + threadIdx.x] = xs[threadIdx.x];
         if (threadIdx.x < 16 * s.ncv) s.gcv[threadIdx.x] = gs[threadIdx.x];
     }
+    if (!s.accumulate)
+        for (int i = blk.b * kGcvThreads + threadIdx.x; i < s.n; i += blk.nb * kGcvThreads)
+            if (!gcv_moves(s, i, gs))
+                for (int k = 0; k < 3; ++k) s.F_out[3 * (size_t)i + k] = 0.0f;
     if (!hill_sum<2>(s, blk, xs, s.scal + kV, s.deposit)) return;
     __syncthreads();  // thread 0 of this block wrote dV/ds
-    gcv_forces(s, Blk{0, 1}, gs);
+    // the atoms that move: each of the few, or the soft minimum's candidates
+    const int *list = s.cv_atoms;
+    const bool exact = s.kind == kKindNearest && s.sm_beta <= 0.0;
+    const int refs = s.kind == kKindTorsion ? 4 * s.ncv : s.ncv;
+    const int count = refs + (s.kind == kKindTorsion ? 0 : (exact ? s.ncv : s.n_cand));
+    for (int q = threadIdx.x; q < count; q += kGcvThreads) {
+        const int at = q >= refs && exact ? s.ncv + (int)gs[16 * (q - refs)] : q;
+        const int i = list[at];
+        bool first = true;  // an atom may serve both CVs
+        for (int p = 0; p < min(q, 8); ++p) {
+            const int pt = p >= refs && exact ? s.ncv + (int)gs[16 * (p - refs)] : p;
+            first = first && (p >= refs && !exact ? true : list[pt] != i);
+        }
+        if (first) gcv_force(s, i, gs);
+    }
 }
 
 template <typename real>
-__global__ void __launch_bounds__(kGcvThreads) k_gcv_step(Sys s) { gcv_step<real>(s, own_blk()); }
+__global__ void __launch_bounds__(kGcvThreads) k_gcv_step(Sys s)
+{
+    chain_enter();
+    gcv_step<real>(s, own_blk());
+}
 
 template <typename real>
 __global__ void __launch_bounds__(kGcvThreads, 4) kb_gcv_step(BatchView v)
 {
+    chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     gcv_step<real>(s, k);
@@ -457,18 +556,18 @@ void launch_gcv_step(const Sys &s, int K, float *F, int accumulate, int deposit,
     t.deposit = deposit;
     const int nb = bias_blocks(K);
     if (fp64)
-        k_gcv_step<double><<<nb, kGcvThreads, 0, st>>>(t);
+        chained_live(k_gcv_step<double>, nb, kGcvThreads, st, t);
     else
-        k_gcv_step<float><<<nb, kGcvThreads, 0, st>>>(t);
+        chained_live(k_gcv_step<float>, nb, kGcvThreads, st, t);
 }
 
 void launch_batch_gcv_step(const BatchView &hills, int hill_total, int fp64, cudaStream_t st)
 {
     if (hill_total <= 0) return;
     if (fp64)
-        kb_gcv_step<double><<<hill_total, kGcvThreads, 0, st>>>(hills);
+        chained_live(kb_gcv_step<double>, hill_total, kGcvThreads, st, hills);
     else
-        kb_gcv_step<float><<<hill_total, kGcvThreads, 0, st>>>(hills);
+        chained_live(kb_gcv_step<float>, hill_total, kGcvThreads, st, hills);
 }
 
 

@@ -215,14 +215,19 @@ struct BatchView {
     int nsys;
 };
 
+// The warp's lanes probe the table together, 32 entries a round (two dependent
+// loads up to 1,024 systems where a search by halves chains ten).  The whole
+// warp calls it.
 __device__ __forceinline__ int batch_system(const BatchView &v, Blk &k)
 {
-    const int x = (int)blockIdx.x;
-    int lo = 0, hi = v.nsys - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(v.pre + mid) <= x) lo = mid;
-        else hi = mid - 1;
+    const int x = (int)blockIdx.x, lane = threadIdx.x & 31;
+    int lo = 0, n = v.nsys;  // the system is one of lo .. lo + n - 1
+    while (n > 1) {
+        const int step = (n + 31) >> 5, at = lo + lane * step;
+        const bool in = at < lo + n && __ldg(v.pre + at) <= x;  // true for a prefix of the lanes, lane 0 among them
+        const int last = __popc(__ballot_sync(0xffffffffu, in)) - 1;
+        n = min(step, lo + n - (lo + last * step));
+        lo += last * step;
     }
     const int p0 = __ldg(v.pre + lo);
     k.b = x - p0;
