@@ -873,7 +873,7 @@ metad_status metad_cv_forward(metad_ctx *c, double *cv_host, double *per_atom_de
     {
         StageScope t(c, ST_CV_FWD, 1);
         metad::launch_cv_fwd(c->sys, c->fp64, c->filter_pending ? 1 : 0, c->stream);
-        c->filter_pending = false;
+        if (metad::stores_rows(c->sys, c->fp64)) c->filter_pending = false;
     }
     if (c->p.n_cv == 2) {
         StageScope t(c, ST_CV_AVG, 1);
@@ -1426,7 +1426,7 @@ metad_status step_graph(metad_ctx *c, const float *pos_dev, float *forces_dev, i
         c->sys.pos_in = reinterpret_cast<const float4 *>(pos_dev);
         c->have_nbr = c->have_cv = c->have_bias = true;
         c->forces_done = c->p.cv_kind == METAD_CV_COORDINATION;
-        c->filter_pending = false;
+        c->filter_pending = !metad::stores_rows(c->sys, c->fp64);
         if (deposit) c->K += 1;
     }
     c->launches += g.kernels;
@@ -1789,7 +1789,7 @@ metad_status metad_batch_step(metad_batch *b, const float *const *pos_dev, float
         metad_ctx *c = b->ctx[k];
         c->have_nbr = c->have_cv = c->have_bias = true;
         c->forces_done = b->kind == METAD_CV_COORDINATION;
-        c->filter_pending = false;
+        c->filter_pending = !metad::stores_rows(c->sys, c->fp64);
         if (deposit && deposit[k]) c->K += 1;
     }
     b->stepped = true;

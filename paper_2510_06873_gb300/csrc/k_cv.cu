@@ -318,6 +318,7 @@ constexpr int kCnRec = 8;  // fx fy fz, vx vy vz, 2 unused
 template <typename real, bool kFilter, int G>
 __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
 {
+    const bool two = sizeof(real) == 4 || s.ncv == 2;  // FP32 with one CV: cv_cn
     int nn_f = 0;
     if (kFilter) nn_f = filter_row<real, G>(s, a);
     real v[kRec];  // 0..12: sum w Y_m (one CV: 0..5 as above) ; 13: W ; 14: CN
@@ -335,7 +336,7 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
             cached_geometry<real>(s, e0 + entry_off(k), d, inv_r, w, dw, cn, j);
             if (cn) v[14] += w;
             v[13] += w;
-            if (s.ncv == 2) {
+            if (two) {
                 jwrow[k] = JW<real>{j, w};
                 ylm13_acc<real>(d.x * inv_r, d.y * inv_r, d.z * inv_r, w, v);
             } else if (cn) {
@@ -357,7 +358,7 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
     const real W = __shfl_sync(0xffffffffu, v[13 % c], ((threadIdx.x & 31) & ~(G - 1)) + 13 / c);
     if (a.ok) {
         if (a.l == 14 / c) R<real>(s.cn)[a.i] = v[14 % c];
-        if (s.ncv == 2) {
+        if (two) {
             if (a.l == 13 / c) R<real>(s.W)[a.i] = W;
             const real inv_W = W > real(0) ? real(1) / W : real(0);
             real q[c];
@@ -368,6 +369,73 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
             store_part<real, kCnRec, c>(R<real>(s.q), a.i, a.l, v);
         }
     }
+}
+
+// a4 for FP32 and one CV: CN_i and the force and virial sums straight from the
+// candidates, a pair evaluated where it is found.  No row is written (16 B an
+// entry, most of the pass's DRAM traffic) or read back; a round evaluates for
+// the pairs counted alone, where compacted rows held all.
+__device__ __forceinline__ void cv_cn_group(const Sys &s, const AtomLane a)
+{
+    const int i = a.ok ? a.i : 0, vn = a.ok ? s.vnn[i] : 0;
+    const float4 pi = s.pos_s[i];
+    const int vmax = __reduce_max_sync(0xffffffffu, vn);
+    float v[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // force, virial, CN
+    int cnt = 0;
+    sweep_candidates<4>(s, i, a.l, vn, vmax, [&](bool valid, int, float4 pj) {
+        Vec3<float> d;
+        const bool in = pair_in_warp(s, valid, pi, pj, d);
+        cnt += in ? 1 : 0;
+        if (in && (!s.cn_unlike || pj.w != pi.w)) {
+            const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+            const float inv_r = rsqrt_r<float>(r2);
+            float w, dw;
+            switch_eval<float>(s, r2 * inv_r, w, dw);
+            const float gx = dw * inv_r * d.x, gy = dw * inv_r * d.y, gz = dw * inv_r * d.z;
+            v[0] += gx;
+            v[1] += gy;
+            v[2] += gz;
+            if (s.virial) {
+                v[3] += gx * d.x;
+                v[4] += gy * d.y;
+                v[5] += gz * d.z;
+            }
+            v[6] += w;
+        }
+    });
+#pragma unroll
+    for (int o = 2; o >= 1; o >>= 1) {
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+#pragma unroll
+        for (int k = 0; k < 7; ++k)
+            if (k < 3 || k == 6 || s.virial) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    }
+    if (!a.ok) return;
+    float4 *q = reinterpret_cast<float4 *>(R<float>(s.q) + (size_t)i * kCnRec);
+    if (a.l == 0) q[0] = make_float4(v[0], v[1], v[2], v[3]);
+    if (a.l == 1) q[1] = make_float4(v[4], v[5], 0.0f, 0.0f);
+    if (a.l == 2) R<float>(s.cn)[i] = v[6];
+    if (a.l == 3 && cnt > s.max_nb) set_err(s, kErrCapacity);
+}
+
+__device__ __forceinline__ void cv_cn(const Sys &s, Blk k)
+{
+    const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_cn_group(s, atom_lane_at<4>(s, g));
+}
+
+__global__ void __launch_bounds__(kBlockAtoms, 12) k_cv_cn(Sys s)
+{
+    chain_enter();
+    cv_cn(s, own_blk());
+}
+
+__global__ void __launch_bounds__(kBlockAtoms, 12) kb_cv_cn(BatchView v)
+{
+    chain_enter();
+    Blk k;
+    const Sys &s = v.sys[batch_system(v, k)];
+    cv_cn(s, k);
 }
 
 // Lanes per atom: four in the FP32 pass.  Bound by instruction issue (64 to
@@ -1334,6 +1402,10 @@ __global__ void k_per_atom_out(Sys s, double *out)
 void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st)
 {
     const int nb = grid_blocks(s, fp64 ? GK_GROUPS : GK_ROWS, 0);  // by kFwdLanes
+    if (!stores_rows(s, fp64)) {
+        chained_live(k_cv_cn, nb, kBlockAtoms, st, s);
+        return;
+    }
     if (fp64) {
         if (fused_filter)
             chained_live(k_cv_fwd<double, true>, nb, kBlockAtoms, st, s);
@@ -1426,6 +1498,8 @@ void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &
     if (fp64) {
         chained_live(kb_cv_fwd<double>, group_total, kBlockAtoms, st, groups);
         if (ncv == 2) chained_live(kb_cv_avg<double>, row_total, kRowThreads, st, rows);
+    } else if (ncv == 1) {
+        chained_live(kb_cv_cn, row_total, kBlockAtoms, st, rows);
     } else {
         chained_live(kb_cv_fwd<float>, row_total, kBlockAtoms, st, rows);
         if (ncv == 2) chained_live(kb_cv_avg<float>, row_total, kRowThreads, st, rows);
@@ -1533,6 +1607,7 @@ SysKernel sys_kernel_cv(const void *func)
         (const void *)k_force_gather,
     };
     static const void *const rest[] = {
+        (const void *)k_cv_cn,
         (const void *)k_cv_fwd<float, true>,
         (const void *)k_cv_fwd<float, false>,
         (const void *)k_cv_fwd<double, true>,

@@ -339,6 +339,9 @@ struct ForceOut {
 // two-CV one leaves its pair forces for launch_force_gather.
 void launch_forces(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st);
 inline bool pair_slots(const Sys &s, int fp64) { return fp64 && s.ncv == 2; }
+// Whether the CV pass leaves the exact rows behind it (the FP32 pass of one CV
+// goes over the candidates without them; whoever wants them runs the filter).
+inline bool stores_rows(const Sys &s, int fp64) { return fp64 || s.ncv == 2; }
 void launch_force_gather(const Sys &s, int fp64, const ForceOut &out, cudaStream_t st);
 void configure_kernels();
 void launch_grid_fold(const Sys &s, int K, cudaStream_t st);
@@ -857,27 +860,37 @@ struct alignas(2 * sizeof(real)) JW {
     real w;
 };
 
-// G candidates of a Verlet row a round, the accepted ones compacted by
-// ballot.  kPart: 0 every exact entry, 1 those with j > i, 2 those with j < i.
-// Positions are loaded a round ahead of their use and indices two.
-template <typename real, int kPart, int G>
-__device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
+// The candidates of atom i's Verlet row (vn of them; vmax the warp's most), G
+// a round: each(valid, j, pj) in every lane of the warp, lane l of G taking
+// candidates l, l + G, ...  Positions are loaded a round ahead of their use
+// and indices two.
+template <int G, typename F>
+__device__ __forceinline__ void sweep_candidates(const Sys &s, int i, int l, int vn, int vmax, F &&each)
 {
-    const int i = a.ok ? a.i : 0;
     const int *vrow = s.vnbr + (size_t)i * s.max_vnb;
-    const size_t e0 = entry_base(s, i), row0 = (size_t)i * s.max_nb;
-    const unsigned lt = (1u << a.l) - 1u;
-    int j1 = a.l < vn ? vrow[a.l] : i;
+    int j1 = l < vn ? vrow[l] : i;
     float4 p1 = s.pos_s[j1];
-    int j2 = a.l + G < vn ? vrow[a.l + G] : i;
+    int j2 = l + G < vn ? vrow[l + G] : i;
     for (int base = 0; base < vmax; base += G) {
-        const int k = base + a.l;
-        const bool valid = k < vn;
-        const int j = j1;
+        const int k = base + l, j = j1;
         const float4 pj = p1;
         j1 = j2;
         p1 = s.pos_s[j1];
         j2 = k + 2 * G < vn ? vrow[k + 2 * G] : i;
+        each(k < vn, j, pj);
+    }
+}
+
+// The accepted candidates of atom a.i's Verlet row compacted by ballot from
+// entry cnt on.  kPart: 0 every exact entry, 1 those with j > i, 2 those with
+// j < i.
+template <typename real, int kPart, int G>
+__device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
+{
+    const int i = a.ok ? a.i : 0;
+    const size_t e0 = entry_base(s, i), row0 = (size_t)i * s.max_nb;
+    const unsigned lt = (1u << a.l) - 1u;
+    sweep_candidates<G>(s, i, a.l, vn, vmax, [&](bool valid, int j, float4 pj) {
         const bool part = kPart == 0 || (kPart == 1 ? j > a.i : j < a.i);
         Vec3<float> d;
         const bool in = pair_in_warp(s, valid && part, pi, pj, d);  // every lane: a warp vote inside
@@ -888,7 +901,7 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
             store_geo<real>(s, e0 + entry_off(at), d, pi, pj, j);
         }
         cnt += __popc(gm);
-    }
+    });
     return cnt;
 }
 

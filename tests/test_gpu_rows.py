@@ -111,3 +111,33 @@ def test_cell_scan_edges(dev, cells):
         assert len(ref) > 100 and np.array_equal(ctx.export_neighbors(), ref)
     assert ctx.rebuild_count == 2
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [1023, 1025])
+def test_one_cv_rows_on_demand(dev, n):
+    """With one CV in FP32 the CV pass writes no rows: the export and the
+    statistics make them, the CV pass before and after gives the same bits, and
+    a row longer than its capacity is still refused."""
+    from paper_2510_06873_gb300 import metad
+    system = synth.wurtzite_system(n, cfg=92)
+    mp = synth.MethodParams(n_cv=1, sigma=(0.05,))
+    frame = synth.perturbed_frame(system, 1)
+    pos = torch.from_numpy(frame).to(dev)
+    pairs = oracle.pairs_cells(frame, system.box, 3.5)
+    longest = int(np.bincount(pairs.ravel(), minlength=n).max())
+    ctx = metad.Metad(_params(dev, n, system.box, mp, max_neighbors=longest))
+    ctx.load_hills([[2.0]], [1.0])
+    F = torch.zeros((n, 3), dtype=torch.float32, device=dev)
+    ctx.step(pos, F)
+    first = ctx.read_results()
+    assert np.array_equal(ctx.export_neighbors(), pairs)
+    assert ctx.neighbor_stats() == (2 * len(pairs), longest)
+    again = ctx.cv_forward()
+    check_cv(first[0], oracle.cv(frame, oracle.params_from(mp, system.box))[0])
+    assert np.array_equal(first[0], again)
+    ctx.close()
+    short = metad.Metad(_params(dev, n, system.box, mp, max_neighbors=longest - 4 - longest % 4))
+    with pytest.raises(metad.MetadError):
+        short.step(pos, F)
+        short.read_results()
+    short.close()
