@@ -1721,13 +1721,12 @@ metad_status metad_batch_step(metad_batch *b, const float *const *pos_dev, float
         metad_ctx *c = b->ctx[k];
         const bool on = !active || active[k];
         if (on) c->sys.pos_in = reinterpret_cast<const float4 *>(pos_dev[k]);
-        Sys y = c->sys;
+        Sys &y = hs[k] = c->sys;  // one copy, into the table that is uploaded
         y.K = c->K;
         y.deposit = on && deposit && deposit[k] ? 1 : 0;
         y.F_out = on ? forces_dev[k] : nullptr;
         y.accumulate = accumulate ? 1 : 0;
         y.fscale = 1.0;
-        hs[k] = y;
         for (int g = 0; g < metad::kGridKinds; ++g)
             pre[g * (n + 1) + k + 1] = pre[g * (n + 1) + k] + (on ? metad::grid_blocks(y, g, b->persist_cap) : 0);
     }

@@ -8,6 +8,7 @@ raises: there is no CPU fallback.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -151,6 +152,15 @@ def _dptr(t):
     if isinstance(t, int):
         return t
     return t.data_ptr()
+
+
+def _dptr_table(tensors):
+    """Device pointers of many tensors (or None, or addresses) as one array.
+    A batched launch of 256 walkers waits for 512 of them."""
+    try:
+        return array.array("Q", [t.data_ptr() for t in tensors])
+    except AttributeError:
+        return array.array("Q", [_dptr(t) or 0 for t in tensors])
 
 
 def _hptr(a):
@@ -634,12 +644,11 @@ def metad_batch_set_tile(batch, blocks_per_system):
 
 def metad_batch_step(batch, pos_list, force_list, accumulate=False, deposit=None, active=None):
     """pos_list / force_list: one tensor (or None when inactive) per system."""
-    n = len(pos_list)
-    pos = (ctypes.c_void_p * n)(*[_dptr(t) for t in pos_list])
-    frc = (ctypes.c_void_p * n)(*[_dptr(t) for t in force_list])
+    pos, frc = _dptr_table(pos_list), _dptr_table(force_list)
     dep_a = None if deposit is None else np.ascontiguousarray(np.asarray(deposit, dtype=np.int32))
     act_a = None if active is None else np.ascontiguousarray(np.asarray(active, dtype=np.int32))
-    _bcheck(batch, lib().metad_batch_step(batch, pos, frc, 1 if accumulate else 0, _hptr(dep_a), _hptr(act_a)),
+    _bcheck(batch, lib().metad_batch_step(batch, pos.buffer_info()[0], frc.buffer_info()[0], 1 if accumulate else 0,
+                                          _hptr(dep_a), _hptr(act_a)),
             "metad_batch_step")
 
 
