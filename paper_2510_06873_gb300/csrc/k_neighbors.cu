@@ -94,9 +94,9 @@ __device__ __forceinline__ void bin_one(const Sys &s, int u)
     int c = s.rank_of_xyz[(cz * s.nc[1] + cy) * s.nc[0] + cx];
     const int shift = oct_shift(s);
     unsigned oct = 0;
-    if (shift == 28)
-        oct = (p.x * s.inv_h[0] - (float)cx >= 0.5f ? 1u : 0u) | (p.y * s.inv_h[1] - (float)cy >= 0.5f ? 2u : 0u) |
-              (p.z * s.inv_h[2] - (float)cz >= 0.5f ? 4u : 0u);
+    if (shift == 28)  // explicit multiply-adds: single and batched kernels decide alike
+        oct = (fmaf(p.x, s.inv_h[0], -(float)cx) >= 0.5f ? 1u : 0u) | (fmaf(p.y, s.inv_h[1], -(float)cy) >= 0.5f ? 2u : 0u) |
+              (fmaf(p.z, s.inv_h[2], -(float)cz) >= 0.5f ? 4u : 0u);
     s.ucell[u] = c;
     s.uslot[u] = (int)((unsigned)atomicAdd(&s.cell_count[c], 1) | (oct << shift));
 }

@@ -141,3 +141,39 @@ def test_one_cv_rows_on_demand(dev, n):
         short.step(pos, F)
         short.read_results()
     short.close()
+
+
+def test_octant_edges_sort_alike_in_a_batch(dev):
+    """Atoms within an ulp or two of their cell's middle: the single and the
+    batched kernels put them into the same octants, so the rows have one order
+    and a batched step gives the single step's bits."""
+    from paper_2510_06873_gb300 import metad
+    g = np.random.default_rng(8)
+    edge, planes, side = 4.567, 9, 16
+    box = np.array([planes * edge, 2.55 * side, 2.55 * side])
+    k, a, b = np.meshgrid(np.arange(planes), np.arange(side), np.arange(side), indexing="ij")
+    pos = np.zeros((k.size, 4), np.float32)
+    mid = ((k.ravel() + 0.5) * edge).astype(np.float32)
+    for ulps in (1, 2):
+        mid = np.where(g.random(k.size) < 0.4, np.nextafter(mid, np.float32(g.choice([0.0, 99.0]))), mid)
+    pos[:, 0] = mid
+    pos[:, 1] = (a.ravel() + 0.5) * 2.55 + g.uniform(-0.3, 0.3, k.size)
+    pos[:, 2] = (b.ravel() + 0.5) * 2.55 + g.uniform(-0.3, 0.3, k.size)
+    pos[:, 3] = g.integers(0, 2, k.size)
+    pos = torch.from_numpy(pos[g.permutation(k.size)]).to(dev)
+    mp = synth.MethodParams(n_cv=2)
+    s_ref, _, _ = oracle.cv(pos.cpu().numpy(), oracle.params_from(mp, box))
+    ctxs = [metad.Metad(_params(dev, k.size, box, mp)) for _ in range(2)]
+    F = [torch.zeros((k.size, 3), dtype=torch.float32, device=dev) for _ in range(2)]
+    for ctx in ctxs:
+        ctx.load_hills([s_ref + 0.01], [1.0])
+    ctxs[0].step(pos, F[0])
+    s0 = ctxs[0].read_results()
+    batch = metad.Batch(ctxs[1:])
+    batch.step([pos], F[1:])
+    s1 = ctxs[1].read_results()
+    assert np.array_equal(s0[0], s1[0]) and s0[1] == s1[1] and np.array_equal(s0[2], s1[2])
+    assert torch.equal(F[0], F[1]) and float(F[0].abs().max()) > 0.0
+    batch.close()
+    for ctx in ctxs:
+        ctx.close()
