@@ -151,9 +151,10 @@ def dist_env():
 # Sources that make up the per-atom kernels; a profile summary records their
 # SHA-1 when its counters were taken.
 KERNEL_SOURCES = ("paper_2510_06873_gb300/csrc/k_cv.cu", "paper_2510_06873_gb300/csrc/metad_impl.cuh")
-# The kernel each timed stage launches (its ncu summary is profiles/<kernel>.md).
-STAGE_KERNEL = {"cv_fwd": "k_cv_fwd", "cv_avg": "k_cv_avg", "adjoint": "k_adjoint", "force_pairs": "k_force_pairs",
-                "force_gather": "k_force_gather", "neighbors": "k_verlet", "gather": "k_gather_check", "bias": "k_bias"}
+# The kernel each timed stage launches (its DRAM bytes: profiles/<kernel>.md, if there).
+STAGE_KERNEL = {"cv_fwd": "k_cv_fwd", "cv_avg": "k_cv_avg", "cv_sum": "k_cv_sum", "adjoint": "k_adjoint",
+                "force_pairs": "k_force_rows", "force_gather": "k_force_gather", "neighbors": "k_verlet",
+                "gather": "k_gather_check", "bias": "k_bias"}
 
 
 def kernel_sources_sha1() -> str:
