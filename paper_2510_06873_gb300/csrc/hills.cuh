@@ -124,6 +124,7 @@ static __device__ __forceinline__ bool hill_sum(const Sys &s, Blk blk, const dou
         out_v[2] += gg1;
     }
     for (int i = 0; i <= kMaxCv; ++i) out[i] = i <= kD ? out_v[i] : 0.0;
+    if (out == s.scal + kV) s.scal[kCnFac] = out_v[1] * 2.0 / s.n;
     if (blk.nb > 1) s.ticket[2] = 0u;
     if (deposit) {
         const double w = s.w0 * exp(-out_v[0] / s.kbdt);

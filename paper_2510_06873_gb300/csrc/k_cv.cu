@@ -997,17 +997,20 @@ __device__ __forceinline__ Vec3<real> pair_gradient(const Vec3<real> &d, real in
     return Vec3<real>{vw * gY[0] + radial * ux, vw * gY[1] + radial * uy, vw * gY[2] + radial * uz};
 }
 
-// The chain-rule factors of the two CVs, 2 V1 scale / N and V2 scale, formed
-// once per block: an FP64 chain is long and its pipe narrow on this part.
+// The chain-rule factors of the two CVs, 2 V1 scale / N and V2 scale.  The
+// division is the hill kernel's (an FP64 chain is long and its pipe narrow on
+// this part); plain forces take no FP64 arithmetic here.
 template <typename real>
 __device__ __forceinline__ void chain_factors(const Sys &s, real fac[2])
 {
-    if (threadIdx.x == 0) {
+    double f0 = s.scal[kCnFac], f1 = s.ncv == 2 ? s.scal[kDV1] : 0.0;
+    if (s.fscale_dev || s.fscale != 1.0) {
         const double scale = force_scale(s);
-        fac[0] = (real)(s.scal[kDV0] * scale * 2.0 / s.n);
-        fac[1] = s.ncv == 2 ? (real)(s.scal[kDV1] * scale) : real(0);
+        f0 *= scale;
+        f1 *= scale;
     }
-    __syncthreads();
+    fac[0] = (real)f0;
+    fac[1] = (real)f1;
 }
 
 template <typename real>
@@ -1100,11 +1103,13 @@ __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real
 // (about 55%) and the latency of the gathered records.  1M atoms: half rows
 // and slot sums 300 us and more, 268 us in a row per atom; 251 with the parts'
 // derivatives shared (ylm13_dot_grad), 235 with the rows of eight atoms
-// interleaved (entry_slot), 214 with the streamed entries one round ahead.
+// interleaved (entry_slot), 214 with the streamed entries one round ahead, 198
+// without a division, a barrier and shared memory in every block
+// (chain_factors).
 template <bool kVir>
 __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
 {
-    __shared__ float fac[2];
+    float fac[2];
     chain_factors<float>(s, fac);
     const float cn_fac = fac[0], V2 = fac[1];
     const int l = threadIdx.x & (kG4 - 1);
@@ -1198,7 +1203,7 @@ __global__ void __launch_bounds__(kRowThreads, kForceBlocks<kVir>) kb_force_rows
 template <typename real, bool kVir>
 __device__ __forceinline__ void force_cn(const Sys &s, Blk k)
 {
-    __shared__ real fac[2];
+    real fac[2];
     chain_factors<real>(s, fac);
     const real f = fac[0];
     RunSum<real> vx, vy, vz;
@@ -1292,7 +1297,7 @@ __device__ __forceinline__ void pair_force(const Sys &s, int i, int k, double cn
 template <bool kVir>
 __device__ __forceinline__ void force_pairs(const Sys &s, Blk k)
 {
-    __shared__ double fac[2];
+    double fac[2];
     chain_factors<double>(s, fac);
     const double cn_fac = fac[0], V2 = fac[1];
     // each warp takes its own chunk of atoms (a block is one work item): no barrier
@@ -1535,10 +1540,7 @@ int launch_batch_forces(const BatchView &force, int force_total, const BatchView
 }
 
 // The gather kernels without shared memory prefer the SM's unified storage
-// as L1.  (Kernels with even a small static shared array, the pair pass's
-// two chain-rule factors among them, are left to the driver: a minimal
-// shared carve-out caps how many of their blocks fit, 7 where the pair
-// pass's registers allow 9.)
+// as L1.  (It makes no difference to the force pass.)
 void configure_kernels()
 {
     const int l1 = cudaSharedmemCarveoutMaxL1;

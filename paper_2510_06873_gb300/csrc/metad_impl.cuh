@@ -34,6 +34,7 @@ enum Scal : int {
     kDepC0 = 18,                 // the last deposit centre (or a caller's CV point)
     kVir0 = 23,                  // bias virial sum_pairs (dV/dd)_a d_a, a = x, y, z
     kBoxG0 = 26,                 // dV/dL_a at fixed fractional coordinates
+    kCnFac = 29,                 // 2 dV/ds1 / N, left by the hill kernel for the force pass
     kErrWord = 31,               // the device error word (an int)
     kNumScal = 32
 };
