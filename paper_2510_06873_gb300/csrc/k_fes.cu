@@ -74,7 +74,19 @@ __global__ void __launch_bounds__(kFesThreads) k_axis_factors(Sys s, int k0, int
     }
 }
 
+// t + v with the rounding error gathered in c (Knuth's TwoSum).
+__device__ __forceinline__ void add_exact(double &t, double &c, double v)
+{
+    const double n = t + v, b = n - t;
+    c += (t - (n - b)) + (v - b);
+    t = n;
+}
+
 // Slice z of the chunk's hills: part[z][point][kOut] (+)= the tile's sums.
+// A stage's 32 products are summed on their own, then added to the slice's
+// sum: a slice's hundreds of products in one chain gather several roundings of
+// the whole sum (up to 8e-16 of the surface, where one sum per thread and a
+// tree over the threads left 3e-16).
 // kOut 1: V; 4: V, dV/dx0, dV/dx1, d2V/dx0dx1.
 template <int kOut>
 __global__ void __launch_bounds__(kSepTile * kSepTile)
@@ -99,15 +111,18 @@ __global__ void __launch_bounds__(kSepTile * kSepTile)
             }
         }
         __syncthreads();
+        double sub[kOut] = {};
 #pragma unroll 8
         for (int c = 0; c < kSepK; ++c) {
-            acc[0] = fma(A[0][ty][c], B[0][tx][c], acc[0]);
+            sub[0] = fma(A[0][ty][c], B[0][tx][c], sub[0]);
             if (kOut == 4) {
-                acc[kOut - 3] = fma(A[kT - 1][ty][c], B[0][tx][c], acc[kOut - 3]);
-                acc[kOut - 2] = fma(A[0][ty][c], B[kT - 1][tx][c], acc[kOut - 2]);
-                acc[kOut - 1] = fma(A[kT - 1][ty][c], B[kT - 1][tx][c], acc[kOut - 1]);
+                sub[kOut - 3] = fma(A[kT - 1][ty][c], B[0][tx][c], sub[kOut - 3]);
+                sub[kOut - 2] = fma(A[0][ty][c], B[kT - 1][tx][c], sub[kOut - 2]);
+                sub[kOut - 1] = fma(A[kT - 1][ty][c], B[kT - 1][tx][c], sub[kOut - 1]);
             }
         }
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) acc[o] += sub[o];
         __syncthreads();
     }
     if (a0 + ty >= n0 || b0 + tx >= n1) return;
@@ -121,9 +136,9 @@ __global__ void k_fold_add(double *grid, const double *part, int values, int sli
 {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= values) return;
-    double t = 0.0;
-    for (int z = 0; z < slices; ++z) t += part[(size_t)z * values + v];
-    grid[v] += t;
+    double t = 0.0, c = 0.0;
+    for (int z = 0; z < slices; ++z) add_exact(t, c, part[(size_t)z * values + v]);
+    grid[v] += t + c;
 }
 
 // Block-wide minimum and sum in a fixed order, in every thread.
@@ -155,7 +170,9 @@ __global__ void __launch_bounds__(kFesThreads)
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < M; b += gridDim.x * blockDim.x) {
         double v = 0.0;
         if (slices > 0) {
-            for (int z = 0; z < slices; ++z) v += part[(size_t)z * M + b];
+            double c = 0.0;
+            for (int z = 0; z < slices; ++z) add_exact(v, c, part[(size_t)z * M + b]);
+            v += c;
             const int i0 = b / g.n[1], i1 = b % g.n[1];
             double gv, g0, g1;
             grid_value(s, g.lo[0] + (i0 + 0.5) * ((g.hi[0] - g.lo[0]) / g.n[0]),
