@@ -1175,8 +1175,9 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
     if (kVir) virial_finish<float>(s, k, vx, vy, vz);
 }
 
-// Resident blocks per SM: 8 (64 registers) in the plain pass, 214 us at 1M
-// atoms, 9 (56) 213, 7 (72) 225; with the virial 7 (72): 250,001 atoms 67.7 us,
+// Resident blocks per SM: 8 (64 registers) in the plain pass, 198 us at 1M
+// atoms and 28.6 at 100,000; 9 (56) 196 and 29.3, 7 (72) 210 and 28.7, 10 259
+// and 36.7 (spilling); with the virial 7 (72): 250,001 atoms 67.7 us,
 // 8 (64, spilling) 69.7, 6 71.2, and 100 when 86 registers left five of the
 // grid's eight blocks per SM resident.
 template <bool kVir>

@@ -640,8 +640,7 @@ __device__ __forceinline__ void grid_value(const Sys &s, double x0, double x1, d
 constexpr int kG = 8;
 constexpr int kAtomsPerBlock = kBlockAtoms / kG;
 
-// Grid of every lane-group kernel; the FP64 partial-sum slots are sized from
-// it, so launches and allocations can never disagree.
+// Grid of the eight-lane kernels.
 __host__ __device__ inline int group_grid(int n) { return (n + kAtomsPerBlock - 1) / kAtomsPerBlock; }
 
 // The CV sums run in their own kernel: kSumThreads threads per block, one
