@@ -643,10 +643,17 @@ def metad_batch_set_tile(batch, blocks_per_system):
 
 
 def metad_batch_step(batch, pos_list, force_list, accumulate=False, deposit=None, active=None):
-    """pos_list / force_list: one tensor (or None when inactive) per system."""
-    pos, frc = _dptr_table(pos_list), _dptr_table(force_list)
+    """pos_list / force_list: one tensor (or None when inactive) per system;
+    deposit / active: one flag per system, or None."""
+    n = len(pos_list)
     dep_a = None if deposit is None else np.ascontiguousarray(np.asarray(deposit, dtype=np.int32))
     act_a = None if active is None else np.ascontiguousarray(np.asarray(active, dtype=np.int32))
+    # the C side reads one entry per system of each
+    for what, m in (("force_list", len(force_list)), ("deposit", n if dep_a is None else dep_a.size),
+                    ("active", n if act_a is None else act_a.size)):
+        if m != n:
+            raise MetadError(METAD_ERR_INVALID, "metad_batch_step", f"{what} has {m} entries for {n} systems")
+    pos, frc = _dptr_table(pos_list), _dptr_table(force_list)
     _bcheck(batch, lib().metad_batch_step(batch, pos.buffer_info()[0], frc.buffer_info()[0], 1 if accumulate else 0,
                                           _hptr(dep_a), _hptr(act_a)),
             "metad_batch_step")
@@ -693,6 +700,8 @@ class Batch:
         metad_batch_set_tile(self.batch, blocks_per_system)
 
     def step(self, pos_list, force_list, accumulate=False, deposit=None, active=None):
+        if len(pos_list) != self.n:
+            raise MetadError(METAD_ERR_INVALID, "Batch.step", f"{len(pos_list)} position buffers for {self.n} systems")
         metad_batch_step(self.batch, pos_list, force_list, accumulate, deposit, active)
 
     def collect(self, out_host):

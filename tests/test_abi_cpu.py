@@ -132,6 +132,26 @@ def test_batch_entry_points_reject_null_without_a_gpu(metad):
     assert L.metad_batch_destroy(None) == metad.METAD_OK
 
 
+@pytest.mark.parametrize("pos,frc,dep,act", [(3, 2, None, None), (3, 4, None, None), (2, 3, None, None),
+                                             (2, 2, None, None), (4, 4, None, None), (3, 3, 2, None), (3, 3, 4, None),
+                                             (3, 3, None, 2), (3, 3, None, 4), (3, 3, 0, None)])
+def test_batch_step_refuses_lists_of_another_length(metad, monkeypatch, pos, frc, dep, act):
+    """The library reads one entry per system of every list: another length is
+    refused before the library is called."""
+    class Library:  # stands in for the library, and must not be reached
+        def __init__(self, L):
+            self.metad_status_string = L.metad_status_string
+
+    monkeypatch.setattr(metad, "_lib", Library(metad.lib()))
+    batch = metad.Batch.__new__(metad.Batch)
+    batch.n, batch.batch = 3, None
+    buf = [4096 * (k + 1) for k in range(4)]  # addresses
+    with pytest.raises(metad.MetadError) as e:
+        batch.step(buf[:pos], buf[:frc], deposit=None if dep is None else [0] * dep,
+                   active=None if act is None else [1] * act)
+    assert e.value.status == metad.METAD_ERR_INVALID
+
+
 @pytest.mark.parametrize("kind,field,value", [("torsion", "n_atoms", 3), ("torsion", "grid_on", 1),
                                               ("nearest", "softmin_beta", -1.0), ("nearest", "box", 0.0),
                                               ("coordination", "cv_kind", 3)])
