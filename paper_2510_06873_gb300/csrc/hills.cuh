@@ -105,7 +105,7 @@ static __device__ __forceinline__ bool hill_sum(const Sys &s, Blk blk, const dou
         // l, l + 32, ... of value q in order, then the same tree
         if (q <= D) {
             a = 0.0;
-            for (int b = lane; b < blk.nb; b += 32) a += __ldcg(part + (D + 1) * b + q);
+            for (int b = lane; b < blk.nb; b += 32) a += ld_l2(part + (D + 1) * b + q);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
         }

@@ -567,7 +567,7 @@ __device__ void finish_cv_sums(const Sys &s, Blk k, double sum, int which)
         __threadfence();
         if (which < 2) {
             sum = 0.0;
-            for (int b = lane; b < k.nb; b += 32) sum += __ldcg(part + b);
+            for (int b = lane; b < k.nb; b += 32) sum += ld_l2(part + b);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
         }
@@ -687,10 +687,7 @@ __device__ __forceinline__ void store4<double>(double *base, int i, int l, const
 // Chunk l of record i of the FP32 q-and-b records: q then b, one 32 B load.
 __device__ __forceinline__ void load_qb(const float *base, int i, int l, float q[4], float b[4])
 {
-    const float *p = base + (size_t)i * kRecQB + 8 * l;
-    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(q[0]), "=f"(q[1]), "=f"(q[2]), "=f"(q[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
-        : "l"(p));
+    ld_8(base + (size_t)i * kRecQB + 8 * l, q, b);
 }
 
 __device__ __forceinline__ void store_b(const Sys &s, int i, int l, const float q[4], const float b[4])
@@ -1068,7 +1065,7 @@ __device__ void virial_finish(const Sys &s, Blk k, RunSum<real> &vx, RunSum<real
             const int b = b0 + r * blockDim.x;
             if (b < k.nb) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) acc[a][r] += __ldcg(part + 3 * b + a);
+                for (int a = 0; a < 3; ++a) acc[a][r] += ld_l2(part + 3 * b + a);
             }
         }
     }
@@ -1130,8 +1127,8 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
             float4 geo_next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             float cross_next = 0.0f;
             if (l < nn) {
-                geo_next = __ldcs(grow);
-                cross_next = __ldcs(crow);
+                geo_next = ld_stream(grow);
+                cross_next = ld_stream(crow);
             }
             for (int e = l; e < nn; e += kG4) {
                 const float4 geo = geo_next;
@@ -1142,8 +1139,8 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
                 float hj[kRec];
                 load_rec<float>(hh, j, hj);
                 if (e + kG4 < nn) {
-                    geo_next = __ldcs(grow + entry_off(e - l + kG4));
-                    cross_next = __ldcs(crow + entry_off(e - l + kG4));
+                    geo_next = ld_stream(grow + entry_off(e - l + kG4));
+                    cross_next = ld_stream(crow + entry_off(e - l + kG4));
                 }
                 const Vec3<float> d{geo.x, geo.y, geo.z};
                 const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
@@ -1364,7 +1361,7 @@ __device__ __forceinline__ void force_gather(const Sys &s, Blk k)
             const int nn = s.nn[a.i];
             const double2 *pf = reinterpret_cast<const double2 *>(s.pairF) + 2 * (size_t)a.i * s.max_nb;
             for (int e = a.l; e < nn; e += kG) {
-                const double2 u = __ldcs(pf + 2 * e), v = __ldcs(pf + 2 * e + 1);
+                const double2 u = ld_stream(pf + 2 * e), v = ld_stream(pf + 2 * e + 1);
                 fx += u.x;
                 fy += u.y;
                 fz += v.x;

@@ -144,7 +144,7 @@ __device__ __forceinline__ void scan_one(const Sys &s, int *ws)
     int c[16], v = 0;
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
-        c[t] = base + t < s.ncell ? __ldcg(s.cell_count + base + t) : 0;
+        c[t] = base + t < s.ncell ? ld_l2(s.cell_count + base + t) : 0;
         v += c[t];
     }
     if (threadIdx.x < 32) ws[threadIdx.x] = 0;  // the scan sums 32 warps; a block has eight

@@ -88,9 +88,9 @@ __global__ void __launch_bounds__(kNoAllocThreads)
     __threadfence();
     double a = 0.0, b = 0.0, cc = 0.0;
     for (int q = 0; q < (int)gridDim.x; ++q) {
-        a += __ldcg(scratch + 3 * q);
-        b += __ldcg(scratch + 3 * q + 1);
-        cc += __ldcg(scratch + 3 * q + 2);
+        a += metad::ld_l2(scratch + 3 * q);
+        b += metad::ld_l2(scratch + 3 * q + 1);
+        cc += metad::ld_l2(scratch + 3 * q + 2);
     }
     out[0] = a;
     out[1] = b;

@@ -161,11 +161,57 @@ struct Sys {
 // thread that goes on, so completion carries along the chain.  (Without a
 // programmatic launch the wait returns at once: the previous kernel has
 // completed.)  Loads of data that an earlier kernel of the step writes are
-// plain ones: a read-only load (__ldg) may be moved before the wait.
+// plain ones or the ld_* below: a read-only load (__ldg) may be moved before
+// the wait, and so may assembly that is neither volatile nor marked as
+// touching memory (to the compiler a function of its address alone), which
+// the toolkit's cache-hint loads (__ldcs, __ldcg) need not be.
 __device__ __forceinline__ void chain_enter()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Loads with a cache hint or of 32 B, kept in program order with the wait
+// above, fences and stores by "volatile" and the memory clobber.  ld_stream:
+// evict-first, for data read for the last time; ld_l2: past the L1, for what
+// other blocks of the same kernel wrote.
+__device__ __forceinline__ float ld_stream(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_stream(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double2 ld_stream(const double2 *p)
+{
+    double2 v;
+    asm volatile("ld.global.cs.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_l2(const double *p)
+{
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_l2(const int *p)
+{
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void ld_8(const float *p, float a[4], float b[4])
+{
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
+                 : "l"(p)
+                 : "memory");
 }
 
 // The difference s - c a hill sees along CV d: wrapped into [-P/2, P/2]
@@ -812,7 +858,7 @@ __device__ __forceinline__ void load_geo<float, false>(const Sys &s, size_t slot
 template <>
 __device__ __forceinline__ void load_geo<float, true>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j)
 {
-    const float4 g = __ldcs(reinterpret_cast<const float4 *>(s.geo) + slot);
+    const float4 g = ld_stream(reinterpret_cast<const float4 *>(s.geo) + slot);
     d = Vec3<float>{g.x, g.y, g.z};
     untag(__float_as_uint(g.w), j, cn);
 }
@@ -820,7 +866,7 @@ template <>
 __device__ __forceinline__ void load_geo<double, true>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j)
 {
     const double2 *g = reinterpret_cast<const double2 *>(s.geo) + 2 * slot;
-    const double2 a = __ldcs(g), b = __ldcs(g + 1);
+    const double2 a = ld_stream(g), b = ld_stream(g + 1);
     d = Vec3<double>{a.x, a.y, b.x};
     untag((unsigned)__double_as_longlong(b.y), j, cn);
 }
