@@ -1756,7 +1756,7 @@ metad_status metad_batch_step(metad_batch *b, const float *const *pos_dev, float
     metad::launch_batch_gather(rows[metad::GK_ATOM256], totals[metad::GK_ATOM256], b->stream);
     metad::launch_batch_rebuild(rows, totals, b->stream);
     metad::launch_batch_cv(rows[metad::GK_GROUPS], totals[metad::GK_GROUPS], rows[metad::GK_ROWS],
-                           totals[metad::GK_ROWS], b->fp64, b->ncv, b->stream);
+                           totals[metad::GK_ROWS], b->fp64, b->ncv, b->ctx[0]->sys.virial, b->stream);
     // two CVs: the CV sums and the hill kernel on the side stream, concurrent
     // with the adjoint
     const bool fork = b->ncv == 2;

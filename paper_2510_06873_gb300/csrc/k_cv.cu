@@ -308,12 +308,83 @@ __device__ __forceinline__ void store_part(real *base, int i, int l, const real 
 
 __device__ __forceinline__ const int *nbr_row(const Sys &s, int i) { return s.nbr + (size_t)i * s.max_nb; }
 
+// Per-thread running sum of a per-atom CV or of pairs' virials.  With FP32
+// records it is a compensated pair (Knuth's TwoSum: s + c holds the sum with
+// only c's own rounding), so no FP64 instruction runs per atom (their pipe is
+// narrow on this part); it enters the FP64 block and grid sums once per thread.
+template <typename real>
+struct RunSum;
+template <>
+struct RunSum<float> {
+    float s = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float t = s + x;
+        const float bp = t - s;
+        c += (s - (t - bp)) + (x - bp);
+        s = t;
+    }
+    // f (hi + lo), the product's rounding error kept
+    __device__ __forceinline__ void add_scaled(float f, float hi, float lo)
+    {
+        const float p = f * hi;
+        add(p);
+        c += fmaf(f, lo, fmaf(f, hi, -p));
+    }
+    __device__ __forceinline__ void halve()
+    {
+        s *= 0.5f;
+        c *= 0.5f;
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+template <>
+struct RunSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add_scaled(double f, double hi, double) { s += f * hi; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+
+// Warp tree over RunSum values (lane 0 ends with the warp's sum): FP32
+// pairs combine by TwoSum on s and a plain sum of the c terms.
+__device__ __forceinline__ void warp_sum(RunSum<float> &v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float os = __shfl_down_sync(0xffffffffu, v.s, o);
+        const float oc = __shfl_down_sync(0xffffffffu, v.c, o);
+        const float t = v.s + os;
+        const float bp = t - v.s;
+        v.c += oc + ((v.s - (t - bp)) + (os - bp));
+        v.s = t;
+    }
+}
+__device__ __forceinline__ void warp_sum(RunSum<double> &v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v.s += __shfl_down_sync(0xffffffffu, v.s, o);
+}
+// The sums of four consecutive lanes, the same bits in each.
+__device__ __forceinline__ void group4_sum(RunSum<float> &v)
+{
+#pragma unroll
+    for (int o = 2; o >= 1; o >>= 1) {
+        const float os = __shfl_xor_sync(0xffffffffu, v.s, o);
+        const float oc = __shfl_xor_sync(0xffffffffu, v.c, o);
+        const float t = v.s + os;
+        const float bp = t - v.s;
+        v.c = (v.c + oc) + ((v.s - (t - bp)) + (os - bp));
+        v.s = t;
+    }
+}
+
 // a4: CN_i, W_i and q_m(i) = sum_j w_ij Y_m(rhat_ij) / W_i.  With one CV, CN_i
 // and what its force and virial need: sum_j w' d / r and sum_j w' d_a^2 / r
 // over the counted pairs (the force on an atom is 2 V1 / N times the first,
 // so no later pass walks the rows).
 // With kFilter the exact row is first compacted from the Verlet row.
-constexpr int kCnRec = 8;  // fx fy fz, vx vy vz, 2 unused
+constexpr int kCnRec = 8;  // fx fy fz, vx vy vz; FP32: the error terms of vx vy (that of vz lies in W)
 
 template <typename real, bool kFilter, int G>
 __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
@@ -374,13 +445,16 @@ __device__ __forceinline__ void cv_fwd_group(const Sys &s, const AtomLane a)
 // a4 for FP32 and one CV: CN_i and the force and virial sums straight from the
 // candidates, a pair evaluated where it is found.  No row is written (16 B an
 // entry, most of the pass's DRAM traffic) or read back; a round evaluates for
-// the pairs counted alone, where compacted rows held all.
+// the pairs counted alone, where compacted rows held all.  Each pair's virial
+// enters a compensated sum (kVir).
+template <bool kVir>
 __device__ __forceinline__ void cv_cn_group(const Sys &s, const AtomLane a)
 {
     const int i = a.ok ? a.i : 0, vn = a.ok ? s.vnn[i] : 0;
     const float4 pi = s.pos_s[i];
     const int vmax = __reduce_max_sync(0xffffffffu, vn);
-    float v[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // force, virial, CN
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // force, CN
+    RunSum<float> vir[3];
     int cnt = 0;
     sweep_candidates<4>(s, i, a.l, vn, vmax, [&](bool valid, int, float4 pj) {
         Vec3<float> d;
@@ -395,47 +469,63 @@ __device__ __forceinline__ void cv_cn_group(const Sys &s, const AtomLane a)
             v[0] += gx;
             v[1] += gy;
             v[2] += gz;
-            if (s.virial) {
-                v[3] += gx * d.x;
-                v[4] += gy * d.y;
-                v[5] += gz * d.z;
+            if (kVir) {
+                vir[0].add(gx * d.x);
+                vir[1].add(gy * d.y);
+                vir[2].add(gz * d.z);
             }
-            v[6] += w;
+            v[3] += w;
         }
     });
 #pragma unroll
     for (int o = 2; o >= 1; o >>= 1) {
         cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
 #pragma unroll
-        for (int k = 0; k < 7; ++k)
-            if (k < 3 || k == 6 || s.virial) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    }
+    if (kVir) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) group4_sum(vir[k]);
     }
     if (!a.ok) return;
     float4 *q = reinterpret_cast<float4 *>(R<float>(s.q) + (size_t)i * kCnRec);
-    if (a.l == 0) q[0] = make_float4(v[0], v[1], v[2], v[3]);
-    if (a.l == 1) q[1] = make_float4(v[4], v[5], 0.0f, 0.0f);
-    if (a.l == 2) R<float>(s.cn)[i] = v[6];
+    if (a.l == 0) q[0] = make_float4(v[0], v[1], v[2], vir[0].s);
+    if (kVir && a.l == 1) {
+        q[1] = make_float4(vir[1].s, vir[2].s, vir[0].c, vir[1].c);
+        R<float>(s.W)[i] = vir[2].c;
+    }
+    if (a.l == 2) R<float>(s.cn)[i] = v[3];
     if (a.l == 3 && cnt > s.max_nb) set_err(s, kErrCapacity);
 }
 
+template <bool kVir>
 __device__ __forceinline__ void cv_cn(const Sys &s, Blk k)
 {
     const int groups = (s.n + kRowAtoms - 1) / kRowAtoms;
-    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_cn_group(s, atom_lane_at<4>(s, g));
+    for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) cv_cn_group<kVir>(s, atom_lane_at<4>(s, g));
 }
 
-__global__ void __launch_bounds__(kBlockAtoms, 12) k_cv_cn(Sys s)
+// Resident blocks per SM: 12 without the virial; with its compensated sums 8:
+// 30,000 / 900,000 atoms a step 42.5 / 218.8 us, 12: 45.1 / 219.3, 9: 43.0 /
+// 226.7.  (The row's virial as a plain float32 sum: 43.6 / 199.8, and three
+// times the error of rows of 450.)
+template <bool kVir>
+constexpr int kCnBlocks = kVir ? 8 : 12;
+
+template <bool kVir>
+__global__ void __launch_bounds__(kBlockAtoms, kCnBlocks<kVir>) k_cv_cn(Sys s)
 {
     chain_enter();
-    cv_cn(s, own_blk());
+    cv_cn<kVir>(s, own_blk());
 }
 
-__global__ void __launch_bounds__(kBlockAtoms, 12) kb_cv_cn(BatchView v)
+template <bool kVir>
+__global__ void __launch_bounds__(kBlockAtoms, kCnBlocks<kVir>) kb_cv_cn(BatchView v)
 {
     chain_enter();
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
-    cv_cn(s, k);
+    cv_cn<kVir>(s, k);
 }
 
 // Lanes per atom: four in the FP32 pass.  Bound by instruction issue (64 to
@@ -474,51 +564,6 @@ __global__ void __launch_bounds__(kBlockAtoms, kFwdBlocks<real>) kb_cv_fwd(Batch
     Blk k;
     const Sys &s = v.sys[batch_system(v, k)];
     cv_fwd<real, true>(s, k);
-}
-
-// Per-thread running sum of a per-atom CV.  With FP32 records it is a
-// compensated pair (Knuth's TwoSum: s + c holds the sum with only c's own
-// rounding), so no FP64 instruction runs per atom (their pipe is narrow on
-// this part); it enters the FP64 block and grid sums once per thread.
-template <typename real>
-struct RunSum;
-template <>
-struct RunSum<float> {
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float t = s + x;
-        const float bp = t - s;
-        c += (s - (t - bp)) + (x - bp);
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-template <>
-struct RunSum<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ double value() const { return s; }
-};
-
-// Warp tree over RunSum values (lane 0 ends with the warp's sum): FP32
-// pairs combine by TwoSum on s and a plain sum of the c terms.
-__device__ __forceinline__ void warp_sum(RunSum<float> &v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float os = __shfl_down_sync(0xffffffffu, v.s, o);
-        const float oc = __shfl_down_sync(0xffffffffu, v.c, o);
-        const float t = v.s + os;
-        const float bp = t - v.s;
-        v.c += oc + ((v.s - (t - bp)) + (os - bp));
-        v.s = t;
-    }
-}
-__device__ __forceinline__ void warp_sum(RunSum<double> &v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v.s += __shfl_down_sync(0xffffffffu, v.s, o);
 }
 
 // Row entries k and k + 1 (k even, so k + 1 lies inside the row's capacity,
@@ -1115,7 +1160,7 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
     RunSum<float> vx, vy, vz;
     for (int it = 0, g; (g = work_item(k, it)) < groups; ++it) {
         const int i = g * kRowAtoms + (threadIdx.x / kG4);
-        float fx = 0.0f, fy = 0.0f, fz = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
+        float fx = 0.0f, fy = 0.0f, fz = 0.0f;
         if (i < s.n) {
             const int nn = s.nn[i];
             const size_t row = entry_base(s, i) + l;
@@ -1152,9 +1197,9 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
                 fy += G.y;
                 fz += G.z;
                 if (kVir) {
-                    wx += G.x * d.x;
-                    wy += G.y * d.y;
-                    wz += G.z * d.z;
+                    vx.add(G.x * d.x);
+                    vy.add(G.y * d.y);
+                    vz.add(G.z * d.z);
                 }
             }
         }
@@ -1163,20 +1208,21 @@ __device__ __forceinline__ void force_rows(const Sys &s, Blk k)
         fz = group4_sum<float>(fz);
         if (i < s.n && l < s.F_stride)
             put_force<float>(s, i, l, l == 0 ? fx : (l == 1 ? fy : (l == 2 ? fz : 0.0f)));
-        if (kVir) {  // each pair is met at both ends
-            vx.add(0.5f * wx);
-            vy.add(0.5f * wy);
-            vz.add(0.5f * wz);
-        }
     }
-    if (kVir) virial_finish<float>(s, k, vx, vy, vz);
+    if (kVir) {  // each pair is met at both ends
+        vx.halve();
+        vy.halve();
+        vz.halve();
+        virial_finish<float>(s, k, vx, vy, vz);
+    }
 }
 
 // Resident blocks per SM: 8 (64 registers) in the plain pass, 198 us at 1M
 // atoms and 28.6 at 100,000; 9 (56) 196 and 29.3, 7 (72) 210 and 28.7, 10 259
-// and 36.7 (spilling); with the virial 7 (72): 250,001 atoms 67.7 us,
-// 8 (64, spilling) 69.7, 6 71.2, and 100 when 86 registers left five of the
-// grid's eight blocks per SM resident.
+// and 36.7 (spilling); with the virial 7 (72): 250,001 atoms 69.2 us.  (With a
+// lane's share of a row's virial summed plainly 67.2, where 8 blocks (64,
+// spilling) took 69.7, 6 71.2, and 100 when 86 registers left five of the
+// grid's eight blocks per SM resident.)
 template <bool kVir>
 constexpr int kForceBlocks = kVir ? 7 : 8;
 
@@ -1213,9 +1259,9 @@ __device__ __forceinline__ void force_cn(const Sys &s, Blk k)
         if (s.F_stride == 4) put_force<real>(s, i, 3, real(0));
         if (kVir) {  // each pair is met at both ends
             const real hf = real(0.5) * f;
-            vx.add(hf * r[3]);
-            vy.add(hf * r[4]);
-            vz.add(hf * r[5]);
+            vx.add_scaled(hf, r[3], r[6]);
+            vy.add_scaled(hf, r[4], r[7]);
+            vz.add_scaled(hf, r[5], sizeof(real) == 4 ? R<real>(s.W)[i] : real(0));
         }
     }
     if (kVir) virial_finish<real>(s, k, vx, vy, vz);
@@ -1406,7 +1452,7 @@ void launch_cv_fwd(const Sys &s, int fp64, int fused_filter, cudaStream_t st)
 {
     const int nb = grid_blocks(s, fp64 ? GK_GROUPS : GK_ROWS, 0);  // by kFwdLanes
     if (!stores_rows(s, fp64)) {
-        chained_live(k_cv_cn, nb, kBlockAtoms, st, s);
+        chained_live(s.virial ? k_cv_cn<true> : k_cv_cn<false>, nb, kBlockAtoms, st, s);
         return;
     }
     if (fp64) {
@@ -1495,14 +1541,14 @@ void launch_force_gather(const Sys &s, int fp64, const ForceOut &out, cudaStream
 }
 
 void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &rows, int row_total, int fp64, int ncv,
-                     cudaStream_t st)
+                     int virial, cudaStream_t st)
 {
     if (group_total <= 0) return;
     if (fp64) {
         chained_live(kb_cv_fwd<double>, group_total, kBlockAtoms, st, groups);
         if (ncv == 2) chained_live(kb_cv_avg<double>, row_total, kRowThreads, st, rows);
     } else if (ncv == 1) {
-        chained_live(kb_cv_cn, row_total, kBlockAtoms, st, rows);
+        chained_live(virial ? kb_cv_cn<true> : kb_cv_cn<false>, row_total, kBlockAtoms, st, rows);
     } else {
         chained_live(kb_cv_fwd<float>, row_total, kBlockAtoms, st, rows);
         if (ncv == 2) chained_live(kb_cv_avg<float>, row_total, kRowThreads, st, rows);
@@ -1607,7 +1653,8 @@ SysKernel sys_kernel_cv(const void *func)
         (const void *)k_force_gather,
     };
     static const void *const rest[] = {
-        (const void *)k_cv_cn,
+        (const void *)k_cv_cn<false>,
+        (const void *)k_cv_cn<true>,
         (const void *)k_cv_fwd<float, true>,
         (const void *)k_cv_fwd<float, false>,
         (const void *)k_cv_fwd<double, true>,

@@ -105,7 +105,7 @@ struct Sys {
     float rv2;             // (rc + skin)^2 with margin: Verlet cutoff
     int always_rebuild;    // skin == 0
     unsigned long long *rebuilds;  // number of rebuilds done
-    void *cn, *W, *qb6;    // real-typed per-atom scalars
+    void *cn, *W, *qb6;    // real-typed per-atom scalars (one CV, FP32, virial: W holds an error term, see k_cv.cu)
     void *q, *b, *h;       // real-typed per-atom records [n][16]: q_m; b_m, beta; h_m, gamma.
                            // FP32: b is [n][32], q and b side by side in chunks of four
                            // (q0..3 b0..3 q4..7 ...).  One CV: q is [n][8], the sums of
@@ -348,7 +348,7 @@ void chained_live(void (*kern)(Args...), int grid, int block, cudaStream_t st, A
 void launch_batch_gather(const BatchView &v, int total, cudaStream_t st);
 void launch_batch_rebuild(const BatchView *rows, const int *totals, cudaStream_t st);
 void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &rows, int row_total, int fp64, int ncv,
-                     cudaStream_t st);
+                     int virial, cudaStream_t st);
 void launch_batch_sum(const BatchView &sums, int sum_total, int fp64, cudaStream_t st);
 void launch_cv_sum(const Sys &s, int fp64, cudaStream_t st);
 void launch_batch_bias(const BatchView &v, int total, int deposit, cudaStream_t st);

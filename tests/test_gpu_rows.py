@@ -177,3 +177,46 @@ def test_octant_edges_sort_alike_in_a_batch(dev):
     batch.close()
     for ctx in ctxs:
         ctx.close()
+
+
+@pytest.mark.parametrize("n_cv", [1, 2])
+def test_every_pair_enters_a_compensated_virial_sum(dev, n_cv):
+    """Box gradient of rows of some 450 neighbours against FP64 sums, with
+    factors that are exact in float32 (r0 a power of two, no stretch) and no
+    force from the second CV, so that what is left is each pair's own rounding,
+    unbiased, and the sums'.  The same arithmetic in numpy leaves 0.014 units of
+    2^-24 (rms, relative, over boxes and axes) where the sums add nothing, and
+    0.043 with plain float32 sums of a lane's share of a row."""
+    from paper_2510_06873_gb300 import metad
+    n, L, r0, rc = 1100, np.array([7.25, 7.5, 8.0]), 2.0, 3.5
+    p = metad.params_for(n, L, n_cv=n_cv, sigma=(0.5, 0.02)[:n_cv], virial=True, max_neighbors=560, r0=r0, rc=rc,
+                         stream=torch.cuda.current_stream(dev).cuda_stream, hill_capacity=4)
+    p.stretch, p.cn_pairs = 0, 0
+    ctx = metad.Metad(p)
+    F = torch.zeros((n, 3), dtype=torch.float32, device=dev)
+    rel = []
+    for seed in range(24):
+        r = np.random.default_rng(seed)
+        g = (np.stack(np.meshgrid(*[np.arange(11)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.5) / 11
+        x = (((g[r.permutation(1331)[:n]] + r.uniform(-0.3, 0.3, (n, 3)) / 11) % 1.0) * L).astype(np.float32)
+        x = np.where(x >= L, np.float32(0.0), x)
+        ctx.build_neighbors(torch.from_numpy(np.concatenate([x, np.zeros((n, 1), np.float32)], 1)).to(dev))
+        s = np.asarray(ctx.cv_forward())
+        c = s.copy()
+        c[0] += 0.3
+        ctx.load_hills([c], [1.0])
+        _, dV = ctx.bias_eval()
+        assert n_cv == 1 or dV[1] == 0.0
+        ctx.bias_forces(F)
+        d = x[None].astype(np.float64) - x[:, None].astype(np.float64)
+        d -= L * np.rint(d / L)
+        r2 = (d * d).sum(2)
+        np.fill_diagonal(r2, rc * rc)
+        d, rr = d[r2 < rc * rc], np.sqrt(r2[r2 < rc * rc])
+        assert rr.size > 440 * n
+        q = rr / r0
+        dw = -6.0 * q**5 / (1.0 + q**6) ** 2 / r0
+        ref = 0.5 * float(np.float32(dV[0] * 2.0 / n)) * ((dw / rr)[:, None] * d * d).sum(0) / L
+        rel.append(ctx.box_gradient() / ref - 1.0)
+    ctx.close()
+    assert np.sqrt(np.mean(np.square(rel))) <= 0.025 * 2.0**-24
