@@ -266,7 +266,11 @@ metad_status metad_load_hills(metad_ctx *ctx, const double *centers_host, const 
 metad_status metad_get_hills(metad_ctx *ctx, double *centers_host, double *heights_host, int32_t cap, int32_t *K);
 
 /* Fold every live hill into the bias grid (node values V, dV/ds1, dV/ds2,
- * d2V/ds1ds2 as exact FP64 sums) and empty the live list.  Needs grid_on. */
+ * d2V/ds1ds2 as exact FP64 sums) and empty the live list.  Needs grid_on.
+ * Asynchronous, allocates nothing: its workspace (some 14 MB for 200 x 200
+ * nodes) belongs to the context from creation on.  A grid whose workspace
+ * would pass 256 MB (about 8 million nodes) has none and is folded node by
+ * node, which takes longer. */
 metad_status metad_fold_hills(metad_ctx *ctx);
 
 /* Copy the grid nodes out: double [grid_n0][grid_n1][4].  Synchronises. */
@@ -316,8 +320,8 @@ metad_status metad_rebuild_count(metad_ctx *ctx, int64_t *count);
  * Errors: those of metad_create's parameter checks. */
 metad_status metad_estimate_bytes(const metad_params *params, int64_t *bytes);
 
-/* Device bytes this context has requested so far (creation plus the
- * buffers allocated on first use by export and host-buffer steps). */
+/* Device bytes this context holds (creation plus the buffers allocated on
+ * first use by export, host-buffer steps and the free-energy calls). */
 int64_t metad_device_bytes(const metad_ctx *ctx);
 
 /* Turn the CUDA-graph replay of metad_step on (1) or off (0) after creation

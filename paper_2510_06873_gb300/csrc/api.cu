@@ -51,7 +51,9 @@ struct metad_ctx {
     std::vector<int> prof_stage;
     int64_t launches = 0;
     int64_t device_bytes = 0;  // requested by cudaMalloc for this context
-    // workspace of the fold and free-energy passes: grown on use, kept up to
+    // workspace of the fold (from creation on; NULL: the fold needs none)
+    double *fold = nullptr;
+    // workspace of the free-energy calls: grown on use, kept up to
     // kScratchKeep bytes, freed with the context
     static constexpr size_t kScratchKeep = 256u << 20;
     double *scratch = nullptr;
@@ -218,19 +220,19 @@ metad_status dalloc(metad_ctx *c, T **ptr, size_t count)
     return METAD_OK;
 }
 
-// The context's workspace with room for `doubles`, or NULL: more than is kept,
-// no memory, or a growth asked for while the stream is being captured.  Work
-// on it is ordered by the context stream; growing frees the old one, which
-// waits for the device.
+// The workspace of the synchronising calls with room for `doubles`, or NULL:
+// more than is kept, no memory, or a stream that is being captured (a graph
+// would outlive it).  Work on it is ordered by the context stream; growing
+// frees the old one, which waits for the device.
 double *kept_scratch(metad_ctx *c, size_t doubles)
 {
-    if (doubles <= c->scratch_doubles) return c->scratch;
     if (doubles * sizeof(double) > metad_ctx::kScratchKeep) return nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
         return nullptr;
     }
+    if (doubles <= c->scratch_doubles) return c->scratch;
     void *p = nullptr;
     if (cudaMalloc(&p, doubles * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
@@ -557,7 +559,9 @@ metad_status state_buffers(metad_ctx *c, Buffers &b, Alloc &&alloc)
     const RecSizes r = rec_sizes(c);
     const bool two = c->p.n_cv == 2, pairs = y.pairs != 0;
     const size_t rows = (size_t)y.max_nb * n, slices = (size_t)y.max_nb * metad::slice_rows(n);
+    const size_t fold = metad::fold_doubles(y);
     metad_status s;
+    if (fold && (s = alloc(&c->fold, fold))) return s;
     if (c->p.cv_kind != METAD_CV_COORDINATION) {
         // no neighbour list: CV atoms, gradient terms, reductions and hills
         int *atoms = nullptr, *slot = nullptr;
@@ -1195,12 +1199,9 @@ metad_status metad_fold_hills(metad_ctx *c)
     if (s) return s;
     if (!c->p.grid_on) return fail(c, METAD_ERR_INVALID, "fold_hills needs grid_on");
     if (c->K > 0) {
-        // the contraction needs a workspace; without one (see kept_scratch)
-        // every node evaluates every hill
-        double *work = kept_scratch(c, metad::fold_doubles(c->sys, c->K));
         StageScope t(c, ST_OTHER, 0);
-        if (work) {
-            c->launches += metad::launch_fold_separable(c->sys, c->K, work, c->stream);
+        if (c->fold) {
+            c->launches += metad::launch_fold_separable(c->sys, c->K, c->fold, c->stream);
         } else {
             metad::launch_grid_fold(c->sys, c->K, c->stream);
             c->launches += 1;

@@ -49,8 +49,8 @@ __global__ void kb_collect(const Sys *sys, int nsys, double *out)
     out[4 * k + 3] = (double)*s.err;
 }
 
-// One thread per grid node: exact sums over hills [0, K).  (Used when there is
-// no workspace for the contraction of k_fes.cu.)
+// One thread per grid node: exact sums over hills [0, K).  (For grids too
+// large for the contraction's workspace, fold_doubles.)
 __global__ void k_grid_fold(Sys s, int K)
 {
     const int node = blockIdx.x * blockDim.x + threadIdx.x;

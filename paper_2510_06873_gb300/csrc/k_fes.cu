@@ -46,7 +46,7 @@ struct FesGrid {
 // over enough blocks (slices) to fill the GPU, each slice's sums to its own
 // partial array, added in slice order afterwards: a fixed order.
 // Measured: sum-of-hills surface of 101 x 96 bins and 5,000 hills
-// 3,508 -> 155 us; fold of 20,000 hills into 200 x 200 nodes 145.6 -> 6.5 ms.
+// 3,508 -> 155 us; fold of 20,000 hills into 200 x 200 nodes 145.6 -> 7.0 ms.
 struct Axis {
     double lo, step, off;  // point i: lo + (i + off) step
     int n;
@@ -374,14 +374,17 @@ int fes_blocks(long long items)
 struct SepPlan {
     int chunk, slices, per, ld;
     size_t tab, part;  // doubles
+    size_t most;       // of both together, for any number of hills up to K
 };
 
 SepPlan sep_plan(int K, int n0, int n1, int out)
 {
     SepPlan p;
     const long long rows = (long long)(n0 + n1) * (out == 4 ? 2 : 1);
-    // the table stays near 32 MB (it then lives in L2)
-    long long chunk = (4LL << 20) / rows / kSepK * kSepK;
+    // the table stays near 32 MB (it then lives in L2); a fold's near 8 MB, as
+    // every context with a grid holds one (20,000 hills into 200 x 200 nodes
+    // 7.00 ms, with 32 MB 6.89)
+    long long chunk = (out == 4 ? 1LL << 20 : 4LL << 20) / rows / kSepK * kSepK;
     if (chunk < kSepK) chunk = kSepK;
     if (chunk > K) chunk = K;
     p.chunk = (int)chunk;
@@ -396,6 +399,7 @@ SepPlan sep_plan(int K, int n0, int n1, int out)
     p.slices = (p.chunk + p.per - 1) / p.per;
     p.tab = (size_t)rows * p.ld;
     p.part = (size_t)p.slices * n0 * n1 * out;
+    p.most = p.tab + (size_t)sl * n0 * n1 * out;  // table and sl grow with the chunk, and slices <= sl
     return p;
 }
 
@@ -459,10 +463,14 @@ int launch_fes_points(const Sys &s, int K, const double *lo, const double *hi, c
     return launched;
 }
 
-size_t fold_doubles(const Sys &s, int K)
+// A grid whose workspace would pass 256 MB (from about 8M nodes, or 500,000
+// along both axes together) is folded node by node instead (k_grid_fold).  By
+// the grid and the capacity alone, so that a context always sums alike.
+size_t fold_doubles(const Sys &s)
 {
-    const SepPlan p = sep_plan(K, s.gn[0], s.gn[1], 4);
-    return p.tab + p.part;
+    if (!s.grid_on) return 0;
+    const size_t most = sep_plan(s.hill_cap, s.gn[0], s.gn[1], 4).most;
+    return most * sizeof(double) <= (256u << 20) ? most : 0;
 }
 
 int launch_fold_separable(const Sys &s, int K, double *work, cudaStream_t st)

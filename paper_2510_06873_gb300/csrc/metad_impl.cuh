@@ -430,8 +430,10 @@ int launch_fes_points(const Sys &s, int K, const double *lo, const double *hi, c
 size_t reweight_doubles(long long T, int ncv, int nbins, size_t rows);
 int launch_fes_reweight(const double *S, const double *V, long long T, int ncv, const double *lo, const double *hi,
                         const int *n, double beta, size_t rows, double *work, double *F, cudaStream_t st);
-// Fold of the live hills into the grid through the contraction.
-size_t fold_doubles(const Sys &s, int K);
+// Fold of the live hills into the grid through the contraction; the doubles
+// its workspace takes for any number of hills the context holds, 0: the fold
+// runs node by node, without one (launch_grid_fold).
+size_t fold_doubles(const Sys &s);
 int launch_fold_separable(const Sys &s, int K, double *work, cudaStream_t st);
 
 // ----------------------------------------------------------------- device math

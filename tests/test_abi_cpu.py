@@ -118,6 +118,21 @@ def test_row_capacity_is_a_multiple_of_four(metad):
     assert est(0) == est(64) == est(61)
 
 
+@pytest.mark.parametrize("kind", ["coordination", "nearest"])
+def test_estimate_counts_the_fold_workspace(metad, kind):
+    """A context with a grid holds the fold's workspace from creation on: a
+    table of axis factors and at least one more array of node values; none
+    where it would pass 256 MB."""
+    def est(n):
+        p = metad.params_for(2000, [30.0, 30.0, 30.0], cv_kind=kind, hill_capacity=20000,
+                             grid=None if n is None else (n, (0.0, 0.0), (1.0, 1.0)))
+        return metad.metad_estimate_bytes(p) - (32 * (4 if n is None else n[0] * n[1]))
+
+    none, nodes = est(None), 200 * 200
+    assert none + 32 * nodes < est((200, 200)) < none + (16 << 20)
+    assert est((2, 600_000)) == none == est((3000, 3000))
+
+
 def test_batch_entry_points_reject_null_without_a_gpu(metad):
     import ctypes
     L = metad.lib()

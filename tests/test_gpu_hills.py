@@ -160,3 +160,81 @@ def test_reweight_chunk_edges(dev, T, n):
         ref -= ref.min()
         fin = acc > 0
         assert np.allclose(F[fin], ref[fin], rtol=1e-11, atol=1e-11)
+
+
+def _fold_sums(ax, c, w, sig):
+    """Node sums of V, dV/dx, dV/dy, d2V/dxdy and of the terms' magnitudes."""
+    ref, scale = (np.zeros((ax[0].size, ax[1].size, 4)) for _ in range(2))
+    for k in range(0, len(w), 500):
+        dx = [ax[d][:, None] - c[None, k:k + 500, d] for d in range(2)]
+        e = [dx[d] ** 2 / (2 * sig[d] ** 2) for d in range(2)]
+        g = w[k:k + 500] * np.exp(-(e[0][:, None, :] + e[1][None, :, :]))
+        u, v = (dx[0] / sig[0] ** 2)[:, None, :], (dx[1] / sig[1] ** 2)[None, :, :]
+        for q, t in enumerate((g, -g * u, -g * v, g * u * v)):
+            ref[..., q] += t.sum(2)
+            scale[..., q] += np.abs(t).sum(2)
+    return ref, scale
+
+
+@pytest.mark.parametrize("n,K", [((60, 35), 5505), ((60, 35), 11009), ((2, 600_000), 3)])
+def test_fold_over_several_tables_and_node_by_node(dev, n, K):
+    """One hill more than fits one table of factors, and two; a grid too long
+    for the contraction's workspace."""
+    r = np.random.default_rng(K)
+    sig, ctr = np.array([0.05, 0.02]), np.array([2.0, 0.3])
+    lo, hi = ctr - 8 * sig, ctr + 8 * sig
+    ctx = _ctx(dev, 2, sig, grid=(n, lo, hi), hill_capacity=K)
+    c, w = ctr + sig * r.uniform(-6, 6, (K, 2)), r.uniform(0.1, 1.0, K)
+    ctx.load_hills(c, w)
+    ctx.fold_hills()
+    ref, scale = _fold_sums([lo[d] + np.arange(n[d]) * ((hi[d] - lo[d]) / (n[d] - 1)) for d in range(2)], c, w, sig)
+    tol = (6 * 196 + 60 + 14 * 2 * 2.4 / 0.05 * 2) * U  # as test_fold_tile_edges
+    assert np.all(np.abs(ctx.get_grid() - ref) <= tol * scale + 1e-300)
+
+
+def test_fold_allocates_nothing_and_its_capture_outlives_other_calls(dev):
+    """The fold's workspace is the context's own from creation on: a fold in
+    the middle of a run allocates nothing, and a captured one can be replayed
+    after calls that need a larger workspace."""
+    sig, ctr = np.array([0.05, 0.02]), np.array([2.0, 0.3])
+    lo, hi = ctr - 8 * sig, ctr + 8 * sig
+    r = np.random.default_rng(5)
+    c, w = ctr + sig * r.uniform(-6, 6, (300, 2)), r.uniform(0.1, 1.0, 300)
+    kw = dict(grid=((40, 30), lo, hi), hill_capacity=500)
+    a, b = _ctx(dev, 2, sig, **kw), _ctx(dev, 2, sig, **kw)
+    held = a.device_bytes
+    a.load_hills(c, w)
+    a.fold_hills()
+    assert a.device_bytes == held
+    once = a.get_grid()
+    a.load_hills(c, w)
+    a.fold_hills()  # adds to the first
+    b.load_hills(c, w)
+    b.fes_grid(lo, hi, (16, 16))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.current_stream(dev)):
+        b.fold_hills()
+    assert not b.get_grid().any()  # captured, not run
+    b.fes_grid(lo, hi, (900, 900))
+    graph.replay()
+    assert np.array_equal(b.get_grid(), once)
+    graph.replay()
+    assert np.array_equal(b.get_grid(), a.get_grid())
+
+
+@pytest.mark.parametrize("K", [2753, 5600])
+def test_free_energy_grid_over_several_tables(dev, K):
+    """1,500 x 8 points: a table of factors holds 2,752 hills."""
+    n = (1500, 8)
+    r = np.random.default_rng(K)
+    sig, ctr = np.array([0.05, 0.02]), np.array([2.0, 0.3])
+    c, w = ctr + sig * r.uniform(-6, 6, (K, 2)), r.uniform(0.1, 1.0, K)
+    ctx = _ctx(dev, 2, sig)
+    ctx.load_hills(c, w)
+    lo, hi = ctr - 8 * sig, ctr + 7 * sig
+    F = ctx.fes_grid(lo, hi, n)
+    ax = [lo[d] + (np.arange(n[d]) + 0.5) * ((hi[d] - lo[d]) / n[d]) for d in range(2)]
+    ref = -(10.0 / 9.0) * _fold_sums(ax, c, w, sig)[0][..., 0]
+    # as test_free_energy_grid_tile_edges
+    assert np.abs(F - (ref - ref.min())).max() <= 2 * (6 * 196 + 10 + 40) * U * np.abs(ref).max()
+    assert F.min() == 0.0
