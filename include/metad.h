@@ -475,8 +475,11 @@ int64_t metad_batch_launch_count(const metad_batch *batch);
 const char *metad_batch_last_error(const metad_batch *batch);
 
 /* -------------------------------------------------------------- free energy
- * Analysis passes (not per step; each call allocates a device buffer for
- * its own use and synchronises).  The grid is regular: n[d] bins over
+ * Analysis passes (not per step; each call synchronises).  metad_fes_grid and
+ * metad_fes_reweight share a workspace that the context keeps once they have
+ * grown it, up to 256 MB, until it is destroyed (growing waits for the
+ * device); a call that needs more, and every metad_cv_trajectory, allocates a
+ * buffer for itself.  The grid is regular: n[d] bins over
  * [lo[d], hi[d]) per CV (n[1], lo[1], hi[1] unused when n_cv == 1), laid
  * out row-major with the first CV slowest; F_host is double [n0 (x n1)].
  *
@@ -492,10 +495,13 @@ const char *metad_batch_last_error(const metad_batch *batch);
  * each, as a biased run records them),
  *     P_b = sum_{t in b} exp(beta V_t) / sum_{t inside the grid} exp(beta V_t),
  *     F_b = -(1/beta) log P_b,  beta = 1 / (params.kB params.temperature),
- * shifted to minimum 0 over the non-empty bins; empty bins are +inf.  Every
- * sum runs in sample order (bit-reproducible).
+ * shifted to minimum 0 over the non-empty bins; empty bins are +inf.  The
+ * order of every sum follows from T and the number of bins (chunks of
+ * consecutive samples, each added in sample order, then the chunks' sums), and
+ * in metad_fes_grid from the hills' and points' numbers: bit-reproducible.
  * Errors: METAD_ERR_INVALID (NULL pointers, n < 1, hi <= lo, more than 2^24
- * bins, T < 1), METAD_ERR_OOM / METAD_ERR_CUDA. */
+ * bins, T < 1), METAD_ERR_OOM (no memory for the workspace; the context stays
+ * usable), METAD_ERR_CUDA. */
 metad_status metad_fes_grid(metad_ctx *ctx, const double *lo, const double *hi, const int32_t *n, double *F_host);
 
 /* CVs of a stored trajectory (offline analysis, no bias or forces; the

@@ -1873,14 +1873,19 @@ struct Scratch {
 };
 
 // A workspace for one synchronising call: the kept one, or a buffer of the
-// call's own.
-cudaError_t call_scratch(metad_ctx *c, size_t doubles, Scratch &own, double **out)
+// call's own.  No form with less memory stands in for a missing one: it would
+// add in another order, and the same input give other bits.
+metad_status call_scratch(metad_ctx *c, size_t doubles, Scratch &own, double **out)
 {
     *out = kept_scratch(c, doubles);
-    if (*out) return cudaSuccess;
+    if (*out) return METAD_OK;
     const cudaError_t e = cudaMalloc(&own.p, sizeof(double) * doubles);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return fail(c, METAD_ERR_OOM, "workspace of " + std::to_string(sizeof(double) * doubles) + " bytes");
+    }
     *out = static_cast<double *>(own.p);
-    return e;
+    return cuda_check(c, e, "workspace");
 }
 
 }  // namespace
@@ -1895,14 +1900,8 @@ metad_status metad_fes_grid(metad_ctx *c, const double *lo, const double *hi, co
     const int nn[2] = {n[0], c->p.n_cv == 2 ? n[1] : 1};
     Scratch own;
     double *work = nullptr;
-    bool separable = metad::fes_separable(c->sys, c->K, nn);
-    if (separable && call_scratch(c, metad::fes_points_doubles(c->sys, c->K, nn, true), own, &work) != cudaSuccess) {
-        cudaGetLastError();
-        separable = false;
-    }
-    if (!separable && (s = cuda_check(c, call_scratch(c, metad::fes_points_doubles(c->sys, c->K, nn, false), own, &work),
-                                      "fes buffer")))
-        return s;
+    const bool separable = metad::fes_separable(c->sys, c->K, nn);
+    if ((s = call_scratch(c, metad::fes_points_doubles(c->sys, c->K, nn, separable), own, &work))) return s;
     const double fac = std::isinf(c->p.biasfactor) ? 1.0 : c->p.biasfactor / (c->p.biasfactor - 1.0);
     c->launches += metad::launch_fes_points(c->sys, c->K, lo, hi, nn, work, separable, fac, c->stream);
     if ((s = launched(c, "fes_grid"))) return s;
@@ -1921,17 +1920,9 @@ metad_status metad_fes_reweight(metad_ctx *c, const double *samples_host, const 
     if ((s = fes_grid_args(c, lo, hi, n, bins))) return s;
     if (T < 1 || !samples_host || !V_host || !F_host) return fail(c, METAD_ERR_INVALID, "bad samples");
     const int ncv = c->p.n_cv;
-    constexpr size_t kRows = 8u << 20;  // 64 MB of chunk rows
-    size_t rows = kRows;
     Scratch own;
     double *S = nullptr;
-    if (call_scratch(c, metad::reweight_doubles(T, ncv, (int)bins, rows), own, &S) != cudaSuccess) {
-        cudaGetLastError();
-        rows = 0;  // one row
-        if ((s = cuda_check(c, call_scratch(c, metad::reweight_doubles(T, ncv, (int)bins, rows), own, &S),
-                            "reweight buffer")))
-            return s;
-    }
+    if ((s = call_scratch(c, metad::reweight_doubles(T, ncv, (int)bins), own, &S))) return s;
     double *V = S + (size_t)T * ncv, *F = V + T, *work = F + bins;
     if ((s = cuda_check(c, cudaMemcpyAsync(S, samples_host, sizeof(double) * T * ncv, cudaMemcpyHostToDevice,
                                            c->stream), "sample upload")) ||
@@ -1940,7 +1931,7 @@ metad_status metad_fes_reweight(metad_ctx *c, const double *samples_host, const 
         return s;
     const int nn[2] = {n[0], ncv == 2 ? n[1] : 1};
     const double beta = 1.0 / (c->p.kB * c->p.temperature);
-    c->launches += metad::launch_fes_reweight(S, V, T, ncv, lo, hi, nn, beta, rows, work, F, c->stream);
+    c->launches += metad::launch_fes_reweight(S, V, T, ncv, lo, hi, nn, beta, work, F, c->stream);
     if ((s = launched(c, "fes_reweight"))) return s;
     if ((s = cuda_check(c, cudaMemcpyAsync(F_host, F, sizeof(double) * bins, cudaMemcpyDeviceToHost, c->stream),
                         "fes copy")))

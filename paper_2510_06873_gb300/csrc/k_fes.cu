@@ -262,13 +262,14 @@ __global__ void __launch_bounds__(kFesThreads) k_fes_vmax(const double *V, long 
 // Walking all samples for every bin costs bins x samples bin computations
 // (FP64 divides); here each sample is binned once.  The samples are cut into
 // chunks of `per` in time order, one warp and one row of bins per chunk, and
-// the rows are added in chunk order (k_fes_bin_sum).  A warp takes 32 samples
-// at a time: the lanes of one bin are found by a match vote, their lowest
-// lane adds their weights in lane order and adds the sum to the chunk's row,
-// so a chunk's sums also run in time order.  A lone read-modify-write chain
-// per 32 samples is what bounds it; chunks are short (64 samples) as long as
-// the rows fit the workspace.  Measured (9,696 bins, 20,001 samples):
-// 33,600 -> 14 us.
+// the rows are added by k_fes_bin_sum, in an order that follows from their
+// number.  A warp takes 32 samples at a time: the lanes of one bin are found by
+// a match vote, their lowest lane adds their weights in lane order and adds the
+// sum to the chunk's row.  A lone read-modify-write chain per 32 samples is
+// what bounds it; chunks are short (64 samples) as long as the rows fit 64 MB
+// (rw_per).  Measured (9,696 bins, 20,001 samples): 33,600 -> 14 us.  Fine
+// grids leave few chunks, one warp each, and the pass turns serial: a million
+// samples 0.15 ms at 9,696 bins, 14 at 1M (eight chunks), 95 at 2^24 (one).
 __global__ void __launch_bounds__(kFesThreads)
     k_fes_accum(const double *S, const double *V, long long T, int ncv, FesGrid g, double beta, const double *bmax,
                 int vblocks, long long per, int chunks, int nbins, double *rows)
@@ -306,9 +307,9 @@ __global__ void __launch_bounds__(kFesThreads)
 }
 
 // Bin sums over the chunks' rows, and each block's total of them.  A block
-// takes 32 bins at a time: its warp g adds rows g, g + 8, ... (32 neighbouring
-// bins a load, four loads in flight), then warp 0 adds the eight sums in
-// order.  (One thread walking all the rows of a bin: 139 us for 313 rows of
+// takes 32 bins at a time: its warp g adds rows g, g + 8, ... in order (32
+// neighbouring bins a load, four loads in flight), then warp 0 adds the eight
+// sums in order.  (One thread walking all the rows of a bin: 139 us for 313 rows of
 // 9,696 bins.)
 __global__ void __launch_bounds__(kFesThreads) k_fes_bin_sum(const double *rows, int chunks, int nbins, double *acc, double *btot)
 {
@@ -483,26 +484,28 @@ int launch_fold_separable(const Sys &s, int K, double *work, cudaStream_t st)
     return 1 + 2 * ((K + p.chunk - 1) / p.chunk);
 }
 
-// Samples per chunk: 64, or as many as keep the chunks' rows within `rows`
-// doubles (at least one row).
-static long long rw_per(long long T, int nbins, size_t rows)
+// Samples per chunk: 64, or as many as keep the chunks' rows within 64 MB (at
+// least one row).  By T and the bins alone: the chunks decide the order of the
+// sums, which must not depend on the memory that happens to be free.
+static long long rw_per(long long T, int nbins)
 {
+    constexpr long long kRows = 8 << 20;  // doubles
     long long chunks = (T + 63) / 64;
     if (chunks > 2048) chunks = 2048;  // the rows' sum walks them one after another
-    const long long most = (long long)(rows / (size_t)nbins);
+    const long long most = kRows / nbins;
     if (chunks > most) chunks = most;
     if (chunks < 1) chunks = 1;
     return ((T + chunks - 1) / chunks + 31) / 32 * 32;
 }
 
-size_t reweight_doubles(long long T, int ncv, int nbins, size_t rows)
+size_t reweight_doubles(long long T, int ncv, int nbins)
 {
-    const long long per = rw_per(T, nbins, rows), chunks = (T + per - 1) / per;
+    const long long per = rw_per(T, nbins), chunks = (T + per - 1) / per;
     return (size_t)T * (ncv + 1) + 2 * (size_t)nbins + 2 * kFesBlocks + (chunks > 1 ? (size_t)chunks * nbins : 0);
 }
 
 int launch_fes_reweight(const double *S, const double *V, long long T, int ncv, const double *lo, const double *hi,
-                        const int *n, double beta, size_t rows_cap, double *work, double *F, cudaStream_t st)
+                        const int *n, double beta, double *work, double *F, cudaStream_t st)
 {
     FesGrid g{};
     int nbins = 1;
@@ -512,7 +515,7 @@ int launch_fes_reweight(const double *S, const double *V, long long T, int ncv, 
         g.n[d] = n[d];
         nbins *= n[d];
     }
-    const long long per = rw_per(T, nbins, rows_cap);
+    const long long per = rw_per(T, nbins);
     const int chunks = (int)((T + per - 1) / per);
     double *acc = work, *b0 = acc + nbins, *b1 = b0 + kFesBlocks;
     double *rows = chunks > 1 ? b1 + kFesBlocks : acc;  // a lone row is the bins' sums itself

@@ -426,10 +426,9 @@ bool fes_separable(const Sys &s, int K, const int *n);
 size_t fes_points_doubles(const Sys &s, int K, const int *n, bool separable);
 int launch_fes_points(const Sys &s, int K, const double *lo, const double *hi, const int *n, double *scratch,
                       bool separable, double fac, cudaStream_t st);
-// rows: doubles the chunks' rows of bins may take (at least one row is used).
-size_t reweight_doubles(long long T, int ncv, int nbins, size_t rows);
+size_t reweight_doubles(long long T, int ncv, int nbins);
 int launch_fes_reweight(const double *S, const double *V, long long T, int ncv, const double *lo, const double *hi,
-                        const int *n, double beta, size_t rows, double *work, double *F, cudaStream_t st);
+                        const int *n, double beta, double *work, double *F, cudaStream_t st);
 // Fold of the live hills into the grid through the contraction; the doubles
 // its workspace takes for any number of hills the context holds, 0: the fold
 // runs node by node, without one (launch_grid_fold).

@@ -238,3 +238,36 @@ def test_free_energy_grid_over_several_tables(dev, K):
     # as test_free_energy_grid_tile_edges
     assert np.abs(F - (ref - ref.min())).max() <= 2 * (6 * 196 + 10 + 40) * U * np.abs(ref).max()
     assert F.min() == 0.0
+
+
+@pytest.mark.parametrize("T,n", [(140_000, (9, 7)), (5000, (2000, 1500)), (700, (3000, 3000))])
+def test_reweight_with_few_or_long_chunks(dev, T, n):
+    """More samples than 2,048 chunks of 64 hold; grids whose rows leave two
+    chunks and one."""
+    r = np.random.default_rng(T)
+    S, V = np.column_stack([r.normal(2.0, 0.1, T), r.normal(0.3, 0.03, T)]), r.uniform(0.0, 15.0, T)
+    lo, hi = np.array([1.8, 0.22]), np.array([2.2, 0.38])
+    F = _ctx(dev, 2, (0.05, 0.02)).fes_reweight(S, V, lo, hi, n)
+    idx = np.floor((S - lo) / ((hi - lo) / np.array(n))).astype(int)
+    ok = np.all((S >= lo) & (S < hi) & (idx < np.array(n)), axis=1)
+    beta = 1.0 / (0.0083144626 * 300.0)
+    acc = np.zeros(n)
+    np.add.at(acc, tuple(idx[ok].T), np.exp(beta * (V[ok] - V.max())))
+    fin = acc > 0
+    assert np.array_equal(np.isfinite(F), fin)
+    ref = -np.log(acc[fin] / acc.sum()) / beta
+    assert np.allclose(F[fin], ref - ref.min(), rtol=1e-11, atol=1e-11)
+
+
+def test_reweight_without_memory_is_refused(dev):
+    """A workspace no device has: METAD_ERR_OOM before any host array is read
+    (no other order of summation stands in), and the context goes on."""
+    from paper_2510_06873_gb300 import metad
+    ctx = _ctx(dev, 2, (0.05, 0.02))
+    S, V, F = np.full((1, 2), 2.0), np.zeros(1), np.zeros(64)
+    lo, hi, n = np.array([1.8, 1.8]), np.array([2.2, 2.2]), np.array([8, 8], dtype=np.int32)
+    call = lambda T: metad.lib().metad_fes_reweight(ctx.ctx, S.ctypes.data, V.ctypes.data, T, lo.ctypes.data,  # noqa: E731
+                                                    hi.ctypes.data, n.ctypes.data, F.ctypes.data)
+    assert call(1 << 40) == metad.METAD_ERR_OOM
+    assert call(1) == metad.METAD_OK
+    assert F.min() == 0.0 and np.isinf(F).sum() == 63
