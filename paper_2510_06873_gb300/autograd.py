@@ -75,7 +75,10 @@ class MetadBias(torch.autograd.Function):
             # the context moved on: recompute the per-atom state of this frame
             bctx.evaluate(pos)
             fctx.gen = bctx.generation
-        if grad_V.device == pos.device and grad_V.dtype == torch.float64 and bctx.on_current_stream(pos):
+        # a lazily negated factor's memory holds its opposite, a zero tensor has none
+        plain = not (grad_V.is_neg() or grad_V._is_zerotensor())
+        if (plain and grad_V.device == pos.device and grad_V.dtype == torch.float64
+                and bctx.on_current_stream(pos)):
             # one stream orders it all: the gradient is written whole, its
             # factor read on the device (no round trip to the host, which
             # left the GPU idle, no second pass over the gradient)

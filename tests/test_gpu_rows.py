@@ -220,3 +220,26 @@ def test_every_pair_enters_a_compensated_virial_sum(dev, n_cv):
         rel.append(ctx.box_gradient() / ref - 1.0)
     ctx.close()
     assert np.sqrt(np.mean(np.square(rel))) <= 0.025 * 2.0**-24
+
+
+def test_gradient_factors_that_are_not_plain_memory(dev):
+    """A factor that autograd negates lazily (through a conjugate) and one
+    without memory (a zero tensor) give what their values say."""
+    from paper_2510_06873_gb300 import autograd
+    system = synth.wurtzite_system(1001, cfg=95)
+    mp = synth.MethodParams(n_cv=2)
+    ctx = autograd.BiasContext(_params(dev, system.n, system.box, mp))
+    pos = torch.from_numpy(synth.perturbed_frame(system, 0)).to(dev).requires_grad_(True)
+    ctx.build_neighbors(pos.detach())
+    ctx.load_hills([np.asarray(ctx.cv_forward()) + 0.01], [1.0])
+    grads, negated = [], []
+    for wrap in (lambda V: V, lambda V: torch.complex(torch.zeros_like(V), V).conj().abs()):
+        V = autograd.bias(pos, ctx)
+        V.register_hook(lambda g: negated.append(g.is_neg()))
+        grads += torch.autograd.grad(wrap(V), pos)  # V > 0: |V| has the gradient of V
+    assert negated == [False, True]
+    assert bool(grads[0].any()) and torch.equal(grads[0], grads[1])
+    V = autograd.bias(pos, ctx)
+    (zero,) = torch.autograd.grad(V, pos, torch._efficientzerotensor((), dtype=torch.float64, device=dev))
+    assert not bool(zero.any())
+    ctx.close()
