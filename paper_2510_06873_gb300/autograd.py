@@ -33,6 +33,15 @@ class BiasContext(_m.Metad):
         """Whether torch's current stream for t's device is the context's."""
         return t.is_cuda and torch.cuda.current_stream(t.device).cuda_stream == self._stream
 
+    def after_current_stream(self, t: torch.Tensor):
+        """Where torch's current stream for t's device is another one, order
+        the context's after it (which writes t) and return it; else None."""
+        if not t.is_cuda or self.on_current_stream(t):
+            return None
+        own = torch.cuda.ExternalStream(self._stream, device=t.device)
+        own.wait_stream(torch.cuda.current_stream(t.device))
+        return own
+
     def evaluate(self, pos: torch.Tensor):
         """Neighbours, CVs and bias for pos (float32 [N, 4] on the device)."""
         self.build_neighbors(pos)
@@ -55,6 +64,7 @@ class MetadBias(torch.autograd.Function):
         if pos.dtype != torch.float32 or pos.dim() != 2 or pos.shape[1] != 4:
             raise ValueError("pos must be float32 [N, 4]")
         pos = pos.contiguous()
+        bias_ctx.after_current_stream(pos)
         gen = bias_ctx.evaluate(pos)
         out = None
         if bias_ctx.on_current_stream(pos):
@@ -71,6 +81,7 @@ class MetadBias(torch.autograd.Function):
     def backward(fctx, grad_V: torch.Tensor):
         (pos,) = fctx.saved_tensors
         bctx: BiasContext = fctx.bias_ctx
+        own = bctx.after_current_stream(pos)
         if bctx.generation != fctx.gen or bctx.last_pos_ptr != pos.data_ptr():
             # the context moved on: recompute the per-atom state of this frame
             bctx.evaluate(pos)
@@ -90,6 +101,8 @@ class MetadBias(torch.autograd.Function):
         dVdx = torch.empty((n, 3), dtype=torch.float32, device=pos.device)
         # forces are -dV/dx: scale by -g to get g * dV/dx
         bctx.bias_forces(dVdx, accumulate=False, scale=-g)
+        if own is not None:  # the context's stream wrote dVdx and reads pos
+            torch.cuda.current_stream(pos.device).wait_stream(own)
         grad = torch.zeros_like(pos)
         grad[:, :3] = dVdx
         return grad, None

@@ -243,3 +243,35 @@ def test_gradient_factors_that_are_not_plain_memory(dev):
     (zero,) = torch.autograd.grad(V, pos, torch._efficientzerotensor((), dtype=torch.float64, device=dev))
     assert not bool(zero.any())
     ctx.close()
+
+
+def test_autograd_on_another_stream_than_the_context(dev):
+    """Positions still being written on torch's current stream when the
+    forward pass is called, and a context's stream that is behind when the
+    gradient is read: both are waited for."""
+    from paper_2510_06873_gb300 import autograd, metad
+    system = synth.wurtzite_system(1001, cfg=96)
+    mp = synth.MethodParams(n_cv=2)
+    ctx = autograd.BiasContext(metad.params_for(system.n, system.box, n_cv=2, sigma=mp.sigma, hill_capacity=16))
+    own = torch.cuda.ExternalStream(ctx.stream, device=dev)
+    base = torch.from_numpy(synth.perturbed_frame(system, 0)).to(dev)
+    torch.cuda.synchronize(dev)
+    ctx.build_neighbors(base)
+    ctx.load_hills([np.asarray(ctx.cv_forward()) + 0.01], [1.0])
+    ref = base.clone().requires_grad_(True)
+    torch.cuda.synchronize(dev)
+    V_ref = autograd.bias(ref, ctx)
+    V_ref.backward()
+    torch.cuda.synchronize(dev)
+    for _ in range(2):
+        late = torch.zeros_like(base)
+        torch.cuda.synchronize(dev)
+        torch.cuda._sleep(20_000_000)  # some 10 ms
+        late.copy_(base)
+        late.requires_grad_(True)
+        V = autograd.bias(late, ctx)
+        with torch.cuda.stream(own):
+            torch.cuda._sleep(20_000_000)
+        (g,) = torch.autograd.grad(V, late)
+        assert float(V.detach()) == float(V_ref.detach()) and torch.equal(g, ref.grad)
+    ctx.close()
