@@ -930,7 +930,7 @@ __device__ __forceinline__ void sweep_candidates(const Sys &s, int i, int l, int
 
 // The accepted candidates of atom a.i's Verlet row compacted by ballot from
 // entry cnt on.  kPart: 0 every exact entry, 1 those with j > i, 2 those with
-// j < i.
+// j < i (their indices alone).
 template <typename real, int kPart, int G>
 __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
@@ -945,7 +945,7 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
         const int at = cnt + __popc(gm & lt);
         if (in && at < s.max_nb) {
             if (kPart != 0) s.nbr[row0 + at] = j;
-            store_geo<real>(s, e0 + entry_off(at), d, pi, pj, j);
+            else store_geo<real>(s, e0 + entry_off(at), d, pi, pj, j);
         }
         cnt += __popc(gm);
     });
@@ -955,6 +955,9 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
 // The exact row of atom a.i from its Verlet row.  For the FP64 two-CV pair
 // pass the j > i entries come first, in a sweep of their own, and the row's
 // indices are kept (it searches them); everyone else reads j from the tags.
+// Its FP64 displacements follow from the compacted indices, every lane with an
+// entry: in the sweeps few lanes of a round have one, and the warp pays for all
+// (250,001 atoms, build and filter: 584 -> 341 us, a step 2,984 -> 2,665).
 template <typename real, int G>
 __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
 {
@@ -966,6 +969,13 @@ __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
         const int nh = filter_sweep<real, 1, G>(s, a, vn, vmax, pi, 0);
         cnt = filter_sweep<real, 2, G>(s, a, vn, vmax, pi, nh);
         if (a.ok && a.l == 0) s.nh[a.i] = min(nh, s.max_nb);
+        __syncwarp();  // the group's lanes wrote the indices
+        const int nn = a.ok ? min(cnt, s.max_nb) : 0;
+        for (int k = a.l; k < nn; k += G) {
+            const int j = s.nbr[(size_t)a.i * s.max_nb + k];
+            const float4 pj = s.pos_s[j];
+            store_geo<real>(s, entry_slot(s, a.i, k), Vec3<float>{}, pi, pj, j);
+        }
     } else {
         cnt = filter_sweep<real, 0, G>(s, a, vn, vmax, pi, 0);
     }

@@ -130,7 +130,7 @@ def test_one_cv_rows_on_demand(dev, n):
     F = torch.zeros((n, 3), dtype=torch.float32, device=dev)
     ctx.step(pos, F)
     first = ctx.read_results()
-    assert np.array_equal(ctx.export_neighbors(), pairs)
+    assert np.array_equal(ctx.export_neighbors(), pairs[np.lexsort((pairs[:, 1], pairs[:, 0]))])
     assert ctx.neighbor_stats() == (2 * len(pairs), longest)
     again = ctx.cv_forward()
     check_cv(first[0], oracle.cv(frame, oracle.params_from(mp, system.box))[0])
@@ -274,4 +274,35 @@ def test_autograd_on_another_stream_than_the_context(dev):
             torch.cuda._sleep(20_000_000)
         (g,) = torch.autograd.grad(V, late)
         assert float(V.detach()) == float(V_ref.detach()) and torch.equal(g, ref.grad)
+    ctx.close()
+
+
+@pytest.mark.parametrize("skin", [0.0, 1.0])
+def test_fp64_geometry_from_compacted_indices(dev, skin):
+    """The FP64 two-CV filter forms its displacements from the row's compacted
+    indices: long rows, the longest just fitting, of few and many candidates."""
+    from paper_2510_06873_gb300 import metad
+    n, L, rc = 1100, np.array([7.25, 7.5, 8.0]), 2.0
+    r = np.random.default_rng(7)
+    g = (np.stack(np.meshgrid(*[np.arange(11)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.5) / 11
+    x = (((g[r.permutation(1331)[:n]] + r.uniform(-0.3, 0.3, (n, 3)) / 11) % 1.0) * L).astype(np.float32)
+    frame = np.concatenate([np.where(x >= L, np.float32(0.0), x), r.integers(0, 2, (n, 1)).astype(np.float32)], 1)
+    mp = synth.MethodParams(n_cv=2, rc=rc, r0=1.5)
+    p = oracle.params_from(mp, L)
+    pairs = oracle.pairs_cells(frame, L, rc)
+    s0, _, _ = oracle.cv(frame, p)
+    c = (np.asarray(s0) + 0.01)[None]
+    w = oracle.deposit_sequence(c, mp.sigma, mp.w0, kbdt(mp))
+    ref = oracle.step(frame, p, c, w, mp.sigma)
+    ctx = metad.Metad(_params(dev, n, L, mp, fp64=True, max_neighbors=int(np.bincount(pairs.ravel()).max()), rc=rc, r0=1.5,
+                            skin=skin))
+    ctx.load_hills(c, w)
+    F = torch.zeros((n, 3), dtype=torch.float32, device=dev)
+    pos = torch.from_numpy(frame).to(dev)
+    ctx.step(pos, F)
+    assert np.array_equal(ctx.export_neighbors(), pairs[np.lexsort((pairs[:, 1], pairs[:, 0]))])
+    s, V, dV = ctx.read_results()
+    check_cv(s, ref["s"])
+    check_bias(V, dV, ref["V"], ref["dV"], mp)
+    check_forces(F.cpu().numpy(), ref["F"])
     ctx.close()
