@@ -465,7 +465,10 @@ __device__ __forceinline__ void cv_cn_group(const Sys &s, const AtomLane a)
             const float inv_r = rsqrt_r<float>(r2);
             float w, dw;
             switch_eval<float>(s, r2 * inv_r, w, dw);
-            const float gx = dw * inv_r * d.x, gy = dw * inv_r * d.y, gz = dw * inv_r * d.z;
+            // products of their own rounding in both instances: the same forces
+            // with the virial and without
+            const float g = dw * inv_r;
+            const float gx = __fmul_rn(g, d.x), gy = __fmul_rn(g, d.y), gz = __fmul_rn(g, d.z);
             v[0] += gx;
             v[1] += gy;
             v[2] += gz;

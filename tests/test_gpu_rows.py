@@ -306,3 +306,26 @@ def test_fp64_geometry_from_compacted_indices(dev, skin):
     check_bias(V, dV, ref["V"], ref["dV"], mp)
     check_forces(F.cpu().numpy(), ref["F"])
     ctx.close()
+
+
+def test_one_cv_forces_do_not_depend_on_the_virial(dev):
+    """The same bits with the virial asked for and without, and in a batch."""
+    from paper_2510_06873_gb300 import metad
+    system = synth.wurtzite_system(5003, cfg=97)
+    mp = synth.MethodParams(n_cv=1, sigma=(0.05,))
+    pos = torch.from_numpy(synth.perturbed_frame(system, 0)).to(dev)
+    out = []
+    for virial in (False, True):
+        ctx = metad.Metad(_params(dev, system.n, system.box, mp, virial=virial))
+        ctx.build_neighbors(pos)
+        ctx.load_hills([np.asarray(ctx.cv_forward()) + 0.01], [1.0])
+        batch = metad.Batch([ctx])
+        for step in (lambda F: ctx.step(pos, F), lambda F: batch.step([pos], [F])):
+            F = torch.zeros((system.n, 3), dtype=torch.float32, device=dev)
+            step(F)
+            s, V, _ = ctx.read_results()
+            out.append((F, s[0], V))
+        batch.close()
+        ctx.close()
+    for F, s, V in out[1:]:
+        assert torch.equal(F, out[0][0]) and (s, V) == out[0][1:]
