@@ -1554,7 +1554,7 @@ void launch_batch_cv(const BatchView &groups, int group_total, const BatchView &
         chained_live(virial ? kb_cv_cn<true> : kb_cv_cn<false>, row_total, kBlockAtoms, st, rows);
     } else {
         chained_live(kb_cv_fwd<float>, row_total, kBlockAtoms, st, rows);
-        if (ncv == 2) chained_live(kb_cv_avg<float>, row_total, kRowThreads, st, rows);
+        chained_live(kb_cv_avg<float>, row_total, kRowThreads, st, rows);
     }
 }
 

@@ -857,13 +857,6 @@ __device__ __forceinline__ void load_geo<float, false>(const Sys &s, size_t slot
     untag(__float_as_uint(g.w), j, cn);
 }
 template <>
-__device__ __forceinline__ void load_geo<float, true>(const Sys &s, size_t slot, Vec3<float> &d, bool &cn, int &j)
-{
-    const float4 g = ld_stream(reinterpret_cast<const float4 *>(s.geo) + slot);
-    d = Vec3<float>{g.x, g.y, g.z};
-    untag(__float_as_uint(g.w), j, cn);
-}
-template <>
 __device__ __forceinline__ void load_geo<double, true>(const Sys &s, size_t slot, Vec3<double> &d, bool &cn, int &j)
 {
     const double2 *g = reinterpret_cast<const double2 *>(s.geo) + 2 * slot;
