@@ -649,10 +649,10 @@ def metad_batch_step(batch, pos_list, force_list, accumulate=False, deposit=None
     dep_a = None if deposit is None else np.ascontiguousarray(np.asarray(deposit, dtype=np.int32))
     act_a = None if active is None else np.ascontiguousarray(np.asarray(active, dtype=np.int32))
     # the C side reads one entry per system of each
-    for what, m in (("force_list", len(force_list)), ("deposit", n if dep_a is None else dep_a.size),
-                    ("active", n if act_a is None else act_a.size)):
-        if m != n:
-            raise MetadError(METAD_ERR_INVALID, "metad_batch_step", f"{what} has {m} entries for {n} systems")
+    if (len(force_list) != n or (dep_a is not None and dep_a.size != n)
+            or (act_a is not None and act_a.size != n)):
+        raise MetadError(METAD_ERR_INVALID, "metad_batch_step",
+                         f"force_list, deposit and active take one entry for each of the {n} systems")
     pos, frc = _dptr_table(pos_list), _dptr_table(force_list)
     _bcheck(batch, lib().metad_batch_step(batch, pos.buffer_info()[0], frc.buffer_info()[0], 1 if accumulate else 0,
                                           _hptr(dep_a), _hptr(act_a)),
