@@ -31,12 +31,13 @@ class BiasContext(_m.Metad):
 
     def on_current_stream(self, t: torch.Tensor) -> bool:
         """Whether torch's current stream for t's device is the context's."""
-        return t.is_cuda and torch.cuda.current_stream(t.device).cuda_stream == self._stream
+        # (torch.cuda.current_stream builds a Stream object of the same handle)
+        return t.is_cuda and torch._C._cuda_getCurrentRawStream(t.device.index) == self._stream
 
     def after_current_stream(self, t: torch.Tensor):
-        """Where torch's current stream for t's device is another one, order
-        the context's after it (which writes t) and return it; else None."""
-        if not t.is_cuda or self.on_current_stream(t):
+        """Order the context's stream after torch's current one for t's device,
+        which writes t; the context's (None for a host tensor)."""
+        if not t.is_cuda:
             return None
         own = torch.cuda.ExternalStream(self._stream, device=t.device)
         own.wait_stream(torch.cuda.current_stream(t.device))
@@ -64,10 +65,12 @@ class MetadBias(torch.autograd.Function):
         if pos.dtype != torch.float32 or pos.dim() != 2 or pos.shape[1] != 4:
             raise ValueError("pos must be float32 [N, 4]")
         pos = pos.contiguous()
-        bias_ctx.after_current_stream(pos)
+        one_stream = bias_ctx.on_current_stream(pos)
+        if not one_stream:
+            bias_ctx.after_current_stream(pos)
         gen = bias_ctx.evaluate(pos)
         out = None
-        if bias_ctx.on_current_stream(pos):
+        if one_stream:
             out = torch.empty((), dtype=torch.float64, device=pos.device)
             _m.metad_bias_value(bias_ctx.ctx, out)
         cv, V, dV = bias_ctx.read_results()
@@ -81,15 +84,15 @@ class MetadBias(torch.autograd.Function):
     def backward(fctx, grad_V: torch.Tensor):
         (pos,) = fctx.saved_tensors
         bctx: BiasContext = fctx.bias_ctx
-        own = bctx.after_current_stream(pos)
+        one_stream = bctx.on_current_stream(pos)
+        own = None if one_stream else bctx.after_current_stream(pos)
         if bctx.generation != fctx.gen or bctx.last_pos_ptr != pos.data_ptr():
             # the context moved on: recompute the per-atom state of this frame
             bctx.evaluate(pos)
             fctx.gen = bctx.generation
         # a lazily negated factor's memory holds its opposite, a zero tensor has none
         plain = not (grad_V.is_neg() or grad_V._is_zerotensor())
-        if (plain and grad_V.device == pos.device and grad_V.dtype == torch.float64
-                and bctx.on_current_stream(pos)):
+        if one_stream and plain and grad_V.device == pos.device and grad_V.dtype == torch.float64:
             # one stream orders it all: the gradient is written whole, its
             # factor read on the device (no round trip to the host, which
             # left the GPU idle, no second pass over the gradient)
