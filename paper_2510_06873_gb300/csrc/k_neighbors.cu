@@ -664,6 +664,12 @@ void launch_gather_check(const Sys &s, cudaStream_t st)
 
 // The cell scan's kernels, fewer for small grids: none up to kScanOne cells
 // (about 36,000 atoms), one up to kDirectTiles tiles (about 1.8 million).
+// Adding up the tiles before its own, a block reads more the larger the grid: a
+// step that rebuilds, one / two scan kernels, 100,000 atoms 108.4 / 109.5 us,
+// 800,000 559 / 557, 1.6 million 1,084 / 1,081, 3 million 2,028 / 2,023; one that
+// does not (nine in ten) is a launch shorter: 42.9 / 44.0, 158.5 / 159.9, 287.5 /
+// 289.0, 522.0 / 523.5.  That passes the loss at all of these; the line bounds
+// what the last tile reads (0.8 MB).
 inline int scan_kernels(const Sys &s)
 {
     return s.ncell <= kScanOne ? 0 : (grid_blocks(s, GK_SCAN_TILES, 0) <= kDirectTiles ? 1 : 2);
