@@ -701,8 +701,10 @@ __host__ __device__ inline int sum_blocks(int n)
 }
 
 // Atoms per warp of the FP64 pair pass: 32 keep its lanes full, but leave a
-// small system on few SMs (1,000 atoms: 8 blocks, 39.6 us).
-__host__ __device__ inline int pair_chunk(int n) { return n < 20000 ? 8 : 32; }
+// small system on few SMs.  A step in us with 8 / 32 atoms (and with the
+// virial): 2,000 atoms 103 / 172, 20,000 298 / 341 (298 / 349), 60,000 717 / 741
+// (745 / 757), 80,000 935 / 950 (983 / 968), 150,000 1,692 / 1,661 (1,784 / 1,673).
+__host__ __device__ inline int pair_chunk(int n) { return n < 70000 ? 8 : 32; }
 
 // The row passes (Q6 average, adjoint, FP32 force) give an atom four lanes and
 // a block kRowAtoms consecutive atoms.

@@ -308,6 +308,27 @@ def test_fp64_geometry_from_compacted_indices(dev, skin):
     ctx.close()
 
 
+@pytest.mark.parametrize("n", [69_999, 70_000])
+def test_fp64_pair_pass_where_its_chunks_change(dev, n):
+    """Eight atoms a warp below 70,000 atoms, 32 from there on."""
+    from paper_2510_06873_gb300 import metad
+    system = synth.wurtzite_system(n, cfg=93)
+    mp = synth.MethodParams(n_cv=2)
+    frame = synth.perturbed_frame(system, 1)
+    c, _ = setup_hills(system, mp, 20, cfg=93)
+    w = oracle.deposit_sequence(c, mp.sigma, mp.w0, kbdt(mp))
+    ref = oracle.step(frame, oracle.params_from(mp, system.box), c, w, mp.sigma)
+    ctx = metad.Metad(_params(dev, n, system.box, mp, fp64=True))
+    ctx.load_hills(c, w)
+    F = torch.zeros((n, 3), dtype=torch.float32, device=dev)
+    ctx.step(torch.from_numpy(frame).to(dev), F)
+    s, V, dV = ctx.read_results()
+    check_cv(s, ref["s"])
+    check_bias(V, dV, ref["V"], ref["dV"], mp)
+    check_forces(F.cpu().numpy(), ref["F"])
+    ctx.close()
+
+
 def test_one_cv_forces_do_not_depend_on_the_virial(dev):
     """The same bits with the virial asked for and without, and in a batch."""
     from paper_2510_06873_gb300 import metad
