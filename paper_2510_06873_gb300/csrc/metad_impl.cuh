@@ -824,23 +824,15 @@ __device__ __forceinline__ unsigned make_tag(const Sys &s, int j, float4 pi, flo
     return (unsigned)j | ((!s.cn_unlike || pj.w != pi.w) ? kCnBit : 0u);
 }
 
-template <typename real>
-__device__ __forceinline__ void store_geo(const Sys &s, size_t slot, const Vec3<float> &df, float4 pi, float4 pj,
-                                          int j);
-template <>
-__device__ __forceinline__ void store_geo<float>(const Sys &s, size_t slot, const Vec3<float> &df, float4 pi,
-                                                 float4 pj, int j)
+// An accepted candidate of the filter: FP32 writes the record whole, FP64 its
+// tag alone (the displacement follows from it, fill_geo).
+__device__ __forceinline__ void store_entry(const Sys &s, float, size_t slot, const Vec3<float> &df, unsigned tag)
 {
-    reinterpret_cast<float4 *>(s.geo)[slot] = make_float4(df.x, df.y, df.z, __uint_as_float(make_tag(s, j, pi, pj)));
+    reinterpret_cast<float4 *>(s.geo)[slot] = make_float4(df.x, df.y, df.z, __uint_as_float(tag));
 }
-template <>
-__device__ __forceinline__ void store_geo<double>(const Sys &s, size_t slot, const Vec3<float> &, float4 pi,
-                                                  float4 pj, int j)
+__device__ __forceinline__ void store_entry(const Sys &s, double, size_t slot, const Vec3<float> &, unsigned tag)
 {
-    const Vec3<double> d = displacement<double>(s, pi, pj);
-    double2 *g = reinterpret_cast<double2 *>(s.geo) + 2 * slot;
-    g[0] = make_double2(d.x, d.y);
-    g[1] = make_double2(d.z, __longlong_as_double((long long)make_tag(s, j, pi, pj)));
+    reinterpret_cast<double *>(s.geo)[4 * slot + 3] = __longlong_as_double((long long)tag);
 }
 
 __device__ __forceinline__ void untag(unsigned tag, int &j, bool &cn)
@@ -925,7 +917,7 @@ __device__ __forceinline__ void sweep_candidates(const Sys &s, int i, int l, int
 
 // The accepted candidates of atom a.i's Verlet row compacted by ballot from
 // entry cnt on.  kPart: 0 every exact entry, 1 those with j > i, 2 those with
-// j < i (their indices alone).
+// j < i.
 template <typename real, int kPart, int G>
 __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int vn, int vmax, float4 pi, int cnt)
 {
@@ -940,19 +932,34 @@ __device__ __forceinline__ int filter_sweep(const Sys &s, const AtomLane &a, int
         const int at = cnt + __popc(gm & lt);
         if (in && at < s.max_nb) {
             if (kPart != 0) s.nbr[row0 + at] = j;
-            else store_geo<real>(s, e0 + entry_off(at), d, pi, pj, j);
+            store_entry(s, real(0), e0 + entry_off(at), d, make_tag(s, j, pi, pj));
         }
         cnt += __popc(gm);
     });
     return cnt;
 }
 
+// FP64: the displacements of atom i's first nn entries from their tags, every
+// lane with an entry.  Formed in the sweeps, few lanes of a round have one, and
+// the warp pays for all (250,001 atoms, a step: one CV 906 -> 813 us, two 2,984 ->
+// 2,665; build and filter 385 -> 322, 584 -> 324).
+__device__ __forceinline__ void fill_geo(const Sys &s, int i, int l, int G, int nn, float4 pi)
+{
+    const size_t e0 = entry_base(s, i);
+    for (int k = l; k < nn; k += G) {
+        double *g = reinterpret_cast<double *>(s.geo) + 4 * (e0 + entry_off(k));
+        int j;
+        bool cn;
+        untag((unsigned)__double_as_longlong(g[3]), j, cn);
+        const Vec3<double> d = displacement<double>(s, pi, s.pos_s[j]);
+        reinterpret_cast<double2 *>(g)[0] = make_double2(d.x, d.y);
+        g[2] = d.z;
+    }
+}
+
 // The exact row of atom a.i from its Verlet row.  For the FP64 two-CV pair
 // pass the j > i entries come first, in a sweep of their own, and the row's
 // indices are kept (it searches them); everyone else reads j from the tags.
-// Its FP64 displacements follow from the compacted indices, every lane with an
-// entry: in the sweeps few lanes of a round have one, and the warp pays for all
-// (250,001 atoms, build and filter: 584 -> 341 us, a step 2,984 -> 2,665).
 template <typename real, int G>
 __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
 {
@@ -964,13 +971,6 @@ __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
         const int nh = filter_sweep<real, 1, G>(s, a, vn, vmax, pi, 0);
         cnt = filter_sweep<real, 2, G>(s, a, vn, vmax, pi, nh);
         if (a.ok && a.l == 0) s.nh[a.i] = min(nh, s.max_nb);
-        __syncwarp();  // the group's lanes wrote the indices
-        const int nn = a.ok ? min(cnt, s.max_nb) : 0;
-        for (int k = a.l; k < nn; k += G) {
-            const int j = s.nbr[(size_t)a.i * s.max_nb + k];
-            const float4 pj = s.pos_s[j];
-            store_geo<real>(s, entry_slot(s, a.i, k), Vec3<float>{}, pi, pj, j);
-        }
     } else {
         cnt = filter_sweep<real, 0, G>(s, a, vn, vmax, pi, 0);
     }
@@ -978,8 +978,13 @@ __device__ __forceinline__ int filter_row(const Sys &s, const AtomLane &a)
         if (cnt > s.max_nb) set_err(s, kErrCapacity);
         s.nn[a.i] = min(cnt, s.max_nb);
     }
-    __syncwarp();
-    return min(cnt, s.max_nb);
+    __syncwarp();  // the group's lanes wrote the row
+    cnt = min(cnt, s.max_nb);
+    if (sizeof(real) == 8) {
+        fill_geo(s, a.i, a.l, G, a.ok ? cnt : 0, pi);
+        __syncwarp();
+    }
+    return cnt;
 }
 
 }  // namespace metad

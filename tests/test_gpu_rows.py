@@ -277,21 +277,22 @@ def test_autograd_on_another_stream_than_the_context(dev):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_cv", [1, 2])
 @pytest.mark.parametrize("skin", [0.0, 1.0])
-def test_fp64_geometry_from_compacted_indices(dev, skin):
-    """The FP64 two-CV filter forms its displacements from the row's compacted
-    indices: long rows, the longest just fitting, of few and many candidates."""
+def test_fp64_geometry_from_compacted_rows(dev, skin, n_cv):
+    """The FP64 filter forms its displacements from the row's compacted tags:
+    long rows, the longest just fitting, of few and many candidates."""
     from paper_2510_06873_gb300 import metad
     n, L, rc = 1100, np.array([7.25, 7.5, 8.0]), 2.0
     r = np.random.default_rng(7)
     g = (np.stack(np.meshgrid(*[np.arange(11)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.5) / 11
     x = (((g[r.permutation(1331)[:n]] + r.uniform(-0.3, 0.3, (n, 3)) / 11) % 1.0) * L).astype(np.float32)
     frame = np.concatenate([np.where(x >= L, np.float32(0.0), x), r.integers(0, 2, (n, 1)).astype(np.float32)], 1)
-    mp = synth.MethodParams(n_cv=2, rc=rc, r0=1.5)
+    mp = synth.MethodParams(n_cv=n_cv, sigma=(0.05, 0.02)[:n_cv], rc=rc, r0=1.5)
     p = oracle.params_from(mp, L)
     pairs = oracle.pairs_cells(frame, L, rc)
     s0, _, _ = oracle.cv(frame, p)
-    c = (np.asarray(s0) + 0.01)[None]
+    c = (np.asarray(s0)[:n_cv] + 0.01)[None]
     w = oracle.deposit_sequence(c, mp.sigma, mp.w0, kbdt(mp))
     ref = oracle.step(frame, p, c, w, mp.sigma)
     ctx = metad.Metad(_params(dev, n, L, mp, fp64=True, max_neighbors=int(np.bincount(pairs.ravel()).max()), rc=rc, r0=1.5,
